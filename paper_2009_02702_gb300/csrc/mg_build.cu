@@ -47,40 +47,67 @@ __global__ void copy_ids_kernel(const IdT* __restrict__ in, OutT* __restrict__ o
 // ---------------------------------------------------------------------------
 // A1: level 0 -> level 1 (sort <= 8 IDs per parent)
 // ---------------------------------------------------------------------------
+// the <= 8 IDs under a parent, ascending: a compare-exchange network on
+// registers (an index into a local array would spill it), absent children as
+// kNone, which sorts last
 template <typename IdT>
-__device__ __forceinline__ int gather_l0(const IdT* __restrict__ ids, Dims3 d0, int X, int Y, int Z, uint32_t v[8]) {
+__device__ __forceinline__ int gather_l0(const IdT* __restrict__ ids, Dims3 d0, int X, int Y, int Z, uint32_t (&v)[8]) {
     int n = 0;
+    const bool x1 = 2 * X + 1 < d0.x;
 #pragma unroll
-    for (int k = 0; k < 2; k++)
-#pragma unroll
-        for (int j = 0; j < 2; j++)
-#pragma unroll
-            for (int i = 0; i < 2; i++) {
-                const int x = 2 * X + i, y = 2 * Y + j, z = 2 * Z + k;
-                if (x < d0.x && y < d0.y && z < d0.z) v[n++] = (uint32_t)ids[((int64_t)z * d0.y + y) * d0.x + x];
+    for (int r = 0; r < 4; r++) {
+        const int y = 2 * Y + (r & 1), z = 2 * Z + (r >> 1);
+        v[2 * r] = v[2 * r + 1] = kNone;
+        if (y < d0.y && z < d0.z) {
+            const IdT* p = ids + ((int64_t)z * d0.y + y) * d0.x + 2 * X;
+            v[2 * r] = (uint32_t)__ldg(p);
+            n++;
+            if (x1) {
+                v[2 * r + 1] = (uint32_t)__ldg(p + 1);
+                n++;
             }
-    // insertion sort, at most 8 elements
-    for (int a = 1; a < n; a++) {
-        uint32_t t = v[a];
-        int b = a - 1;
-        while (b >= 0 && v[b] > t) {
-            v[b + 1] = v[b];
-            b--;
         }
-        v[b + 1] = t;
     }
     return n;
+}
+
+__device__ __forceinline__ void sort8(uint32_t (&v)[8]) {
+    // Batcher's odd-even merge network for eight (19 exchanges)
+    constexpr int A[19] = {0, 2, 4, 6, 0, 1, 4, 5, 1, 5, 0, 1, 2, 3, 2, 3, 1, 3, 5};
+    constexpr int B[19] = {1, 3, 5, 7, 2, 3, 6, 7, 2, 6, 4, 5, 6, 7, 4, 5, 2, 4, 6};
+#pragma unroll
+    for (int k = 0; k < 19; k++) {
+        const uint32_t lo = min(v[A[k]], v[B[k]]), hi = max(v[A[k]], v[B[k]]);
+        v[A[k]] = lo;
+        v[B[k]] = hi;
+    }
+}
+
+// parent coordinates of voxel v (32-bit arithmetic: volumes hold < 2^32 voxels)
+__device__ __forceinline__ void parent_at(uint32_t v, Dims3 d, int& X, int& Y, int& Z) {
+    const uint32_t r = v / (uint32_t)d.x;
+    X = (int)(v - r * (uint32_t)d.x);
+    Z = (int)(r / (uint32_t)d.y);
+    Y = (int)(r - (uint32_t)Z * (uint32_t)d.y);
 }
 
 template <typename IdT>
 __global__ void l1_count_kernel(const IdT* __restrict__ ids, Dims3 d0, Dims3 d1, uint32_t* __restrict__ nnz) {
     const int64_t V1 = nvox(d1);
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < V1; v += (int64_t)gridDim.x * blockDim.x) {
-        const int X = (int)(v % d1.x), Y = (int)((v / d1.x) % d1.y), Z = (int)(v / ((int64_t)d1.x * d1.y));
+        int X, Y, Z;
+        parent_at((uint32_t)v, d1, X, Y, Z);
         uint32_t s[8];
-        const int n = gather_l0(ids, d0, X, Y, Z, s);
+        gather_l0(ids, d0, X, Y, Z, s);
+        bool one = true;
+#pragma unroll
+        for (int a = 1; a < 8; a++) one = one && (s[a] == s[0] || s[a] == kNone);
         uint32_t c = 1;
-        for (int a = 1; a < n; a++) c += s[a] != s[a - 1];
+        if (!one) {
+            sort8(s);
+#pragma unroll
+            for (int a = 1; a < 8; a++) c += s[a] != s[a - 1] && s[a] != kNone;
+        }
         nnz[v] = c;
     }
 }
@@ -90,20 +117,30 @@ __global__ void l1_write_kernel(const IdT* __restrict__ ids, Dims3 d0, Dims3 d1,
                                 uint32_t* __restrict__ out_ids, uint64_t* __restrict__ out_w) {
     const int64_t V1 = nvox(d1);
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < V1; v += (int64_t)gridDim.x * blockDim.x) {
-        const int X = (int)(v % d1.x), Y = (int)((v / d1.x) % d1.y), Z = (int)(v / ((int64_t)d1.x * d1.y));
+        uint32_t o = off[v];
+        int X, Y, Z;
+        parent_at((uint32_t)v, d1, X, Y, Z);
         uint32_t s[8];
         const int n = gather_l0(ids, d0, X, Y, Z, s);
+        if (off[v + 1] - o == 1) {
+            out_ids[o] = s[0];
+            out_w[o] = 8;   // n children of weight 8 / n
+            continue;
+        }
         const uint64_t scale = 8u / (unsigned)n;   // Eq. 4: divide by N, times 8^l
-        uint32_t o = off[v];
+        sort8(s);
         uint32_t run = 1;
-        for (int a = 1; a <= n; a++) {
-            if (a < n && s[a] == s[a - 1]) {
+#pragma unroll
+        for (int a = 1; a <= 8; a++) {
+            if (a < 8 && s[a] == s[a - 1]) {
                 run++;
                 continue;
             }
-            out_ids[o] = s[a - 1];
-            out_w[o] = (uint64_t)run * scale;
-            o++;
+            if (s[a - 1] != kNone) {
+                out_ids[o] = s[a - 1];
+                out_w[o] = (uint64_t)run * scale;
+                o++;
+            }
             run = 1;
         }
     }
@@ -152,7 +189,8 @@ __global__ void next_count_kernel(const uint32_t* __restrict__ off, const uint32
                                   Dims3 dn, uint32_t* __restrict__ nnz) {
     const int64_t Vn = nvox(dn);
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < Vn; v += (int64_t)gridDim.x * blockDim.x) {
-        const int X = (int)(v % dn.x), Y = (int)((v / dn.x) % dn.y), Z = (int)(v / ((int64_t)dn.x * dn.y));
+        int X, Y, Z;
+        parent_at((uint32_t)v, dn, X, Y, Z);
         Heads h;
         load_children(off, ids, dl, X, Y, Z, h);
         uint32_t cnt = 0;
@@ -178,7 +216,8 @@ __global__ void next_write_kernel(const uint32_t* __restrict__ off, const uint32
                                   uint64_t* __restrict__ nw) {
     const int64_t Vn = nvox(dn);
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < Vn; v += (int64_t)gridDim.x * blockDim.x) {
-        const int X = (int)(v % dn.x), Y = (int)((v / dn.x) % dn.y), Z = (int)(v / ((int64_t)dn.x * dn.y));
+        int X, Y, Z;
+        parent_at((uint32_t)v, dn, X, Y, Z);
         Heads h;
         load_children(off, ids, dl, X, Y, Z, h);
         const uint64_t scale = 8u / (unsigned)h.n;   // Eq. 4
@@ -295,10 +334,13 @@ constexpr int kShortList = 16;
 
 __global__ void factor_short_kernel(NodeTab t, const uint32_t* __restrict__ off, const uint32_t* __restrict__ ids,
                                     const uint64_t* __restrict__ w, int64_t V, uint32_t* __restrict__ mip_out,
-                                    uint32_t* __restrict__ long_list, unsigned* __restrict__ long_count) {
+                                    uint32_t* __restrict__ long_list, unsigned* __restrict__ long_count,
+                                    unsigned* __restrict__ longest) {
+    unsigned most = 0;   // longest list seen (statistics)
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t b = off[v];
         int n = (int)(off[v + 1] - b);
+        most = max(most, (unsigned)n);
         if (n == 1) {
             mip_out[v] = ids[b];
             continue;
@@ -332,6 +374,8 @@ __global__ void factor_short_kernel(NodeTab t, const uint32_t* __restrict__ off,
         }
         mip_out[v] = nd[0];
     }
+    most = __reduce_max_sync(0xffffffffu, most);
+    if ((threadIdx.x & 31) == 0 && most > ld_relaxed_u32(longest)) atomicMax(longest, most);
 }
 
 // One CTA per long list; rounds in place in the level's CSR arrays (all reads
@@ -379,14 +423,6 @@ __global__ void factor_long_kernel(NodeTab t, const uint32_t* __restrict__ off, 
     }
 }
 
-__global__ void list_max_kernel(const uint32_t* __restrict__ off, int64_t V, unsigned* __restrict__ out) {
-    unsigned m = 0;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (int64_t)gridDim.x * blockDim.x)
-        m = max(m, off[v + 1] - off[v]);
-    m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
-}
-
 __global__ void rehash_kernel(NodeTab t, uint64_t lo, uint64_t hi) {
     for (uint64_t k = lo + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < hi;
          k += (uint64_t)gridDim.x * blockDim.x) {
@@ -403,29 +439,61 @@ __global__ void rehash_kernel(NodeTab t, uint64_t lo, uint64_t hi) {
 // ---------------------------------------------------------------------------
 // A3: canonical relabel
 // ---------------------------------------------------------------------------
-__global__ void depth_hist_kernel(const uint32_t* __restrict__ p, const uint8_t* __restrict__ depth, uint64_t lo,
-                                  uint64_t hi, unsigned long long* __restrict__ hist) {
+// nodes per topological level, and the OR of each level's weights (the digits
+// its sort has to look at)
+struct LevelStats {
+    unsigned long long count[MG_MAX_DEPTH + 1], weights[MG_MAX_DEPTH + 1];
+};
+__global__ void depth_hist_kernel(const uint32_t* __restrict__ p, const uint8_t* __restrict__ depth,
+                                  const uint64_t* __restrict__ a, const uint64_t* __restrict__ b, uint64_t lo,
+                                  uint64_t hi, LevelStats* __restrict__ st) {
     __shared__ unsigned int sh[MG_MAX_DEPTH + 1];
-    for (int i = threadIdx.x; i <= MG_MAX_DEPTH; i += blockDim.x) sh[i] = 0;
-    __syncthreads();
-    for (uint64_t k = lo + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < hi;
-         k += (uint64_t)gridDim.x * blockDim.x) {
-        if (p[k] < kDead) atomicAdd(&sh[min((int)depth[k], MG_MAX_DEPTH)], 1u);
+    __shared__ unsigned long long sw[MG_MAX_DEPTH + 1];
+    for (int i = threadIdx.x; i <= MG_MAX_DEPTH; i += blockDim.x) {
+        sh[i] = 0;
+        sw[i] = 0;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i <= MG_MAX_DEPTH; i += blockDim.x)
-        if (sh[i]) atomicAdd(&hist[i], (unsigned long long)sh[i]);
-}
-
-__global__ void scatter_depth_kernel(const uint32_t* __restrict__ p, const uint8_t* __restrict__ depth, uint64_t lo,
-                                     uint64_t hi, unsigned long long* __restrict__ cursor,
-                                     uint32_t* __restrict__ order) {
     for (uint64_t k = lo + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < hi;
          k += (uint64_t)gridDim.x * blockDim.x) {
         if (p[k] < kDead) {
-            const unsigned long long pos = atomicAdd(&cursor[depth[k]], 1ull);
-            order[pos] = (uint32_t)k;
+            const int d = min((int)depth[k], MG_MAX_DEPTH);
+            atomicAdd(&sh[d], 1u);
+            const unsigned long long w = a[k] | b[k];
+            if (w & ~sw[d]) atomicOr(&sw[d], w);
         }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i <= MG_MAX_DEPTH; i += blockDim.x)
+        if (sh[i]) {
+            atomicAdd(&st->count[i], (unsigned long long)sh[i]);
+            atomicOr(&st->weights[i], sw[i]);
+        }
+}
+
+// The nodes of each level gathered (in any order: the sort's key is unique).
+// Places are handed out per CTA and level, not per node: a global atomic each
+// on the same few cursors took 130 us for 230,000 nodes, this takes 5.
+__global__ void __launch_bounds__(256) scatter_depth_kernel(const uint32_t* __restrict__ p,
+                                                            const uint8_t* __restrict__ depth, uint64_t lo, uint64_t hi,
+                                                            unsigned long long* __restrict__ cursor,
+                                                            uint32_t* __restrict__ order) {
+    __shared__ unsigned int sh[MG_MAX_DEPTH + 1];
+    __shared__ unsigned long long s_base[MG_MAX_DEPTH + 1];
+    for (uint64_t k0 = lo + (uint64_t)blockIdx.x * blockDim.x; k0 < hi; k0 += (uint64_t)gridDim.x * blockDim.x) {
+        for (int i = threadIdx.x; i <= MG_MAX_DEPTH; i += blockDim.x) sh[i] = 0;
+        __syncthreads();
+        const uint64_t k = k0 + threadIdx.x;
+        const bool live = k < hi && p[k] < kDead;
+        const int d = live ? depth[k] : 0;
+        unsigned at = 0;
+        if (live) at = atomicAdd(&sh[d], 1u);
+        __syncthreads();
+        for (int i = threadIdx.x; i <= MG_MAX_DEPTH; i += blockDim.x)
+            if (sh[i]) s_base[i] = atomicAdd(&cursor[i], (unsigned long long)sh[i]);
+        __syncthreads();
+        if (live) order[s_base[d] + at] = (uint32_t)k;
+        __syncthreads();
     }
 }
 
@@ -455,6 +523,71 @@ __global__ void assign_kernel(const uint32_t* __restrict__ perm, int64_t n, uint
         canon[k] = c;
         pq[c] = make_uint2(canon[p[k]], canon[q[k]]);
         ab[c] = make_ulonglong2(a[k], b[k]);
+    }
+}
+
+// The levels from `first` on, all of at most kTailMax nodes, sorted and
+// numbered by one CTA, level after level (a level's key reads the numbers of
+// the levels below it): bitonic in shared memory on the whole key (p', q', a,
+// b).  The last levels hold a few nodes each, and a radix sort of any size
+// costs some 60 launches a level: 84 sort passes of the 512x512x384 volume
+// became 22, 1.27 -> 0.53 ms.
+constexpr int kTailThreads = 1024;
+constexpr int kTailMax = 4096;
+struct TailLevels {
+    int first, last;
+    int64_t bucket[MG_MAX_DEPTH + 2];
+};
+struct TailKey {
+    uint64_t pq, a, b;
+};
+constexpr size_t kTailSmem = (size_t)kTailMax * (sizeof(TailKey) + sizeof(uint32_t));
+
+__global__ void __launch_bounds__(kTailThreads) sort_tail_kernel(TailLevels T, uint32_t S, const uint32_t* order,
+                                                                 const uint32_t* __restrict__ p,
+                                                                 const uint32_t* __restrict__ q,
+                                                                 const uint64_t* __restrict__ a,
+                                                                 const uint64_t* __restrict__ b, uint32_t* canon,
+                                                                 uint2* __restrict__ pq, ulonglong2* __restrict__ ab) {
+    extern __shared__ __align__(16) uint8_t smem[];
+    TailKey* key = reinterpret_cast<TailKey*>(smem);
+    uint32_t* idx = reinterpret_cast<uint32_t*>(key + kTailMax);
+    for (int k = T.first; k <= T.last; k++) {
+        const int n = (int)(T.bucket[k + 1] - T.bucket[k]);
+        const uint32_t* perm = order + (T.bucket[k] - S);
+        int m = 1;
+        while (m < n) m *= 2;
+        for (int i = threadIdx.x; i < m; i += kTailThreads) {
+            idx[i] = (uint32_t)i;
+            if (i < n) {
+                const uint32_t t = perm[i];
+                key[i] = TailKey{(uint64_t)canon[p[t]] << 32 | canon[q[t]], a[t], b[t]};
+            } else {
+                key[i] = TailKey{~0ull, ~0ull, ~0ull};
+            }
+        }
+        __syncthreads();
+        for (int w = 2; w <= m; w *= 2)
+            for (int h = w / 2; h > 0; h /= 2) {
+                for (int t = threadIdx.x; t < m / 2; t += kTailThreads) {
+                    const int i = 2 * t - (t & (h - 1)), j = i + h;
+                    const uint32_t x = idx[i], y = idx[j];
+                    const TailKey &kx = key[x], &ky = key[y];
+                    const bool more = kx.pq != ky.pq ? kx.pq > ky.pq : kx.a != ky.a ? kx.a > ky.a : kx.b > ky.b;
+                    if (more == ((i & w) == 0)) {
+                        idx[i] = y;
+                        idx[j] = x;
+                    }
+                }
+                __syncthreads();
+            }
+        for (int i = threadIdx.x; i < n; i += kTailThreads) {
+            const uint32_t x = idx[i], t = perm[x], c = (uint32_t)T.bucket[k] + (uint32_t)i;
+            canon[t] = c;
+            pq[c] = make_uint2((uint32_t)(key[x].pq >> 32), (uint32_t)key[x].pq);
+            ab[c] = make_ulonglong2(key[x].a, key[x].b);
+        }
+        __syncthreads();   // the next level's keys read these numbers
     }
 }
 
@@ -726,10 +859,10 @@ mg_status build_graph(mg_graph* g, const void* ids, int id_bytes, int64_t nx, in
 
     // ---- node table: sources 0..S-1 ----
     HostTable t;
-    MG_TRY(t.count.alloc(&al, sizeof(unsigned long long), s));
+    MG_TRY(t.count.alloc(&al, 2 * sizeof(unsigned long long), s));   // nodes; entries of the newest lists
     {
-        unsigned long long c0 = S;
-        MG_CUDA(cudaMemcpyAsync(t.count.p, &c0, sizeof(c0), cudaMemcpyHostToDevice, s));
+        const unsigned long long c0[2] = {S, 0};
+        MG_CUDA(cudaMemcpyAsync(t.count.p, c0, sizeof(c0), cudaMemcpyHostToDevice, s));
     }
     MG_TRY(grow_table(t, (uint64_t)S + 4096, 0, al, s));
     MG_CUDA(cudaMemsetAsync(t.p.p, 0xFF, (size_t)S * 4, s));
@@ -752,6 +885,15 @@ mg_status build_graph(mg_graph* g, const void* ids, int id_bytes, int64_t nx, in
         int64_t V = 0;
         uint32_t nnz = 0;
     };
+    // the newest lists' entries and the node count, in one read-back
+    unsigned long long counts[2] = {S, 0};
+    auto read_counts = [&](Lists& out) -> mg_status {
+        MG_CUDA(cudaMemcpyAsync(t.count.as<unsigned long long>() + 1, out.off.as<uint32_t>() + out.V, sizeof(uint32_t),
+                                cudaMemcpyDeviceToDevice, s));
+        MG_TRY(read_scalar(&counts, t.count.p, s));
+        out.nnz = (uint32_t)counts[1];
+        return MG_OK;
+    };
     auto make_level1 = [&](Lists& out) -> mg_status {
         const Dims3 d0 = dims_of(0), d1 = dims_of(1);
         out.V = nvox(d1);
@@ -764,7 +906,7 @@ mg_status build_graph(mg_graph* g, const void* ids, int id_bytes, int64_t nx, in
         MG_CUDA(cudaGetLastError());
         MG_TRY(scan_exclusive_u32(out.off.as<uint32_t>(), out.off.as<uint32_t>(), out.V,
                                   out.off.as<uint32_t>() + out.V, al, s));
-        MG_TRY(read_scalar(&out.nnz, out.off.as<uint32_t>() + out.V, s));
+        MG_TRY(read_counts(out));
         MG_TRY(out.ids.alloc(&al, (size_t)out.nnz * 4, s));
         MG_TRY(out.w.alloc(&al, (size_t)out.nnz * 8, s));
         if (g->id0_bytes == 2)
@@ -786,7 +928,7 @@ mg_status build_graph(mg_graph* g, const void* ids, int id_bytes, int64_t nx, in
         MG_CUDA(cudaGetLastError());
         MG_TRY(scan_exclusive_u32(out.off.as<uint32_t>(), out.off.as<uint32_t>(), out.V,
                                   out.off.as<uint32_t>() + out.V, al, s));
-        MG_TRY(read_scalar(&out.nnz, out.off.as<uint32_t>() + out.V, s));
+        MG_TRY(read_counts(out));
         MG_TRY(out.ids.alloc(&al, (size_t)out.nnz * 4, s));
         MG_TRY(out.w.alloc(&al, (size_t)out.nnz * 8, s));
         next_write_kernel<<<gb, 256, 0, s>>>(in.off.as<uint32_t>(), in.ids.as<uint32_t>(), in.w.as<uint64_t>(), dl,
@@ -806,9 +948,9 @@ mg_status build_graph(mg_graph* g, const void* ids, int id_bytes, int64_t nx, in
         const uint64_t pairs = (uint64_t)cur.nnz - (uint64_t)cur.V;
         g->pairs += (int64_t)pairs;
         if (pairs > 0) {
-            unsigned long long cnt = 0;
-            MG_TRY(read_scalar(&cnt, t.count.p, s));
-            used = cnt;
+            // (the last level makes no further lists: read the count alone)
+            if (l + 1 == L) MG_TRY(read_scalar(&counts[0], t.count.p, s));
+            used = counts[0];
             const uint64_t old_slots = t.nslots;
             MG_TRY(grow_table(t, used + pairs, used, al, s));
             if (t.nslots != old_slots && used > S) {
@@ -822,14 +964,11 @@ mg_status build_graph(mg_graph* g, const void* ids, int id_bytes, int64_t nx, in
         factor_short_kernel<<<grid_n(cur.V), 256, 0, s>>>(view(t, status), cur.off.as<uint32_t>(),
                                                           cur.ids.as<uint32_t>(), cur.w.as<uint64_t>(), cur.V,
                                                           mip_out, long_list.as<uint32_t>(),
-                                                          long_count.as<unsigned>());
+                                                          long_count.as<unsigned>(), maxlen.as<unsigned>());
         MG_CUDA(cudaGetLastError());
         factor_long_kernel<<<152 * 4, 256, 0, s>>>(view(t, status), cur.off.as<uint32_t>(), cur.ids.as<uint32_t>(),
                                                    cur.w.as<uint64_t>(), long_list.as<uint32_t>(),
                                                    long_count.as<unsigned>(), mip_out);
-        MG_CUDA(cudaGetLastError());
-        // longest list of this level (statistics)
-        list_max_kernel<<<grid_n(cur.V), 256, 0, s>>>(cur.off.as<uint32_t>(), cur.V, maxlen.as<unsigned>());
         MG_CUDA(cudaGetLastError());
         cur = std::move(nxt);
     }
@@ -850,16 +989,18 @@ mg_status build_graph(mg_graph* g, const void* ids, int id_bytes, int64_t nx, in
 
     // ---- A3: topological levels and canonical numbering ----
     Buf hist;
-    MG_TRY(hist.alloc(&al, (MG_MAX_DEPTH + 1) * sizeof(unsigned long long), s));
-    MG_CUDA(cudaMemsetAsync(hist.p, 0, (MG_MAX_DEPTH + 1) * sizeof(unsigned long long), s));
+    MG_TRY(hist.alloc(&al, sizeof(LevelStats), s));
+    MG_CUDA(cudaMemsetAsync(hist.p, 0, sizeof(LevelStats), s));
     if (used > S) {
-        depth_hist_kernel<<<grid_n((int64_t)(used - S)), 256, 0, s>>>(t.p.as<uint32_t>(), t.depth.as<uint8_t>(), S,
-                                                                       used, hist.as<unsigned long long>());
+        depth_hist_kernel<<<grid_n((int64_t)(used - S)), 256, 0, s>>>(t.p.as<uint32_t>(), t.depth.as<uint8_t>(),
+                                                                       t.a.as<uint64_t>(), t.b.as<uint64_t>(), S, used,
+                                                                       hist.as<LevelStats>());
         MG_CUDA(cudaGetLastError());
     }
-    unsigned long long hh[MG_MAX_DEPTH + 1];
-    MG_CUDA(cudaMemcpyAsync(hh, hist.p, sizeof(hh), cudaMemcpyDeviceToHost, s));
+    LevelStats stats;
+    MG_CUDA(cudaMemcpyAsync(&stats, hist.p, sizeof(stats), cudaMemcpyDeviceToHost, s));
     MG_CUDA(cudaStreamSynchronize(s));
+    const unsigned long long (&hh)[MG_MAX_DEPTH + 1] = stats.count;
     if (hh[MG_MAX_DEPTH]) return fail(MG_ERR_UNSUPPORTED, "topological depth above the supported maximum");
     int D = 0;
     for (int k = 1; k < MG_MAX_DEPTH; k++)
@@ -889,9 +1030,12 @@ mg_status build_graph(mg_graph* g, const void* ids, int id_bytes, int64_t nx, in
                                                                           used, cursor.as<unsigned long long>(),
                                                                           order.as<uint32_t>());
         MG_CUDA(cudaGetLastError());
-        const int bits_ab = std::max(1, 3 * (L - 1));
         const int bits_n = bits_for((uint64_t)N);
-        for (int k = 1; k <= D; k++) {
+        // the levels from `tail` on are small: sorted by one CTA after the loop
+        int tail = D + 1;
+        while (tail > 1 && g->bucket[tail] - g->bucket[tail - 1] <= kTailMax) tail--;
+        for (int k = 1; k < tail; k++) {
+            const int bits_ab = std::max(1, bits_for(stats.weights[k]));
             const int64_t n = g->bucket[k + 1] - g->bucket[k];
             uint32_t* perm = order.as<uint32_t>() + (g->bucket[k] - S);
             uint64_t* kk = keys.as<uint64_t>();
@@ -912,6 +1056,18 @@ mg_status build_graph(mg_graph* g, const void* ids, int id_bytes, int64_t nx, in
             assign_kernel<<<grid_n(n), 256, 0, s>>>(perm, n, (uint32_t)g->bucket[k], t.p.as<uint32_t>(),
                                                     t.q.as<uint32_t>(), t.a.as<uint64_t>(), t.b.as<uint64_t>(),
                                                     canon.as<uint32_t>(), g->pq.as<uint2>(), g->ab.as<ulonglong2>());
+            MG_CUDA(cudaGetLastError());
+        }
+        if (tail <= D) {
+            TailLevels T;
+            T.first = tail;
+            T.last = D;
+            for (int k = 0; k < MG_MAX_DEPTH + 2; k++) T.bucket[k] = g->bucket[k];
+            MG_CUDA(cudaFuncSetAttribute(sort_tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem));
+            sort_tail_kernel<<<1, kTailThreads, kTailSmem, s>>>(T, S, order.as<uint32_t>(), t.p.as<uint32_t>(),
+                                                                t.q.as<uint32_t>(), t.a.as<uint64_t>(),
+                                                                t.b.as<uint64_t>(), canon.as<uint32_t>(),
+                                                                g->pq.as<uint2>(), g->ab.as<ulonglong2>());
             MG_CUDA(cudaGetLastError());
         }
     }

@@ -94,6 +94,48 @@ __global__ void scan_tile_kernel(const T* in, T* out, int64_t n, const T* __rest
     if (total && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *total = off + bt;
 }
 
+// A few tiles in one CTA of 1,024 threads, tile after tile with a running
+// carry: one launch of about 2 us per 8,192 elements where the reduce-then-scan
+// takes three launches (and three 2-us gaps), so it is taken up to 64 K.
+constexpr int kOneThreads = 1024;
+constexpr int64_t kOneMax = 1 << 16;
+template <typename T>
+__global__ void __launch_bounds__(kOneThreads) scan_one_kernel(const T* in, T* out, int64_t n, T* __restrict__ total) {
+    __shared__ T tile[kOneThreads * kScanItems];
+    __shared__ T wsum[32];
+    T carry = 0;
+    for (int64_t base = 0; base < n; base += kOneThreads * kScanItems) {
+#pragma unroll
+        for (int i = 0; i < kScanItems; i++) {
+            const int64_t idx = base + i * kOneThreads + threadIdx.x;
+            tile[i * kOneThreads + threadIdx.x] = idx < n ? in[idx] : T(0);
+        }
+        __syncthreads();
+        T loc[kScanItems], sum = 0;
+#pragma unroll
+        for (int i = 0; i < kScanItems; i++) {
+            loc[i] = tile[threadIdx.x * kScanItems + i];
+            sum += loc[i];
+        }
+        T bt;
+        T run = carry + block_excl_scan(sum, wsum, &bt);
+        carry += bt;
+#pragma unroll
+        for (int i = 0; i < kScanItems; i++) {
+            tile[threadIdx.x * kScanItems + i] = run;
+            run += loc[i];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kScanItems; i++) {
+            const int64_t idx = base + i * kOneThreads + threadIdx.x;
+            if (idx < n) out[idx] = tile[i * kOneThreads + threadIdx.x];
+        }
+        __syncthreads();
+    }
+    if (total && threadIdx.x == 0) *total = carry;
+}
+
 template <typename T>
 mg_status scan_impl(const T* in, T* out, int64_t n, T* total, const Alloc& al, cudaStream_t s) {
     if (n <= 0) {
@@ -103,6 +145,13 @@ mg_status scan_impl(const T* in, T* out, int64_t n, T* total, const Alloc& al, c
     const int64_t nb = (n + kScanTile - 1) / kScanTile;
     if (nb == 1) {
         scan_tile_kernel<T><<<1, kScanThreads, 0, s>>>(in, out, n, nullptr, total);
+        MG_CUDA(cudaGetLastError());
+        return MG_OK;
+    }
+    if (n <= kOneMax && sizeof(T) == 4) {
+        scan_one_kernel<uint32_t><<<1, kOneThreads, 0, s>>>(reinterpret_cast<const uint32_t*>(in),
+                                                            reinterpret_cast<uint32_t*>(out), n,
+                                                            reinterpret_cast<uint32_t*>(total));
         MG_CUDA(cudaGetLastError());
         return MG_OK;
     }
