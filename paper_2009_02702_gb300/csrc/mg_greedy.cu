@@ -916,9 +916,11 @@ extern "C" MG_API mg_status mg_graph_from_greedy(const mg_greedy* r, const mg_al
     MG_CUDA(cudaMemcpyAsync(g->dw.p, dw.data(), (size_t)N * 8, cudaMemcpyHostToDevice, s));
     MG_CUDA(cudaMemsetAsync(g->status.p, 0, 4, s));
     MG_TRY(build_query_copies(g.get(), s));
+    MG_TRY(build_tiles(g.get(), s));
     MG_CUDA(cudaStreamSynchronize(s));   // the host staging above is freed on return
     for (Buf* b : {&g->mip0, &g->mip, &g->pq, &g->ab, &g->ab32, &g->alpha, &g->wq, &g->dw, &g->status}) b->s = nullptr;
     for (int c = 0; c < 3; c++) g->mip0x[c].s = g->mipx[c].s = nullptr;
+    g->tiles.s = g->tile_pool.s = g->lut_rec.s = nullptr;
     *out = g.release();
     return MG_OK;
 }

@@ -118,6 +118,21 @@ struct LevelGeom {
     int64_t off[MG_MAX_LEVELS];   // offset of level l (l >= 1) in the concatenated mip array
 };
 
+// Tiles of the box queries (mg_tiles.cu).  Kinds of level l: 0 and 1, plane
+// tiles of edge 8 and 16; 2, lines of 16.  The records of copy c start at
+// off[l][kind][c], with strides 1, st1, st2 along the copy's axes.
+constexpr int kTileLevels = 4;
+constexpr int kTileStages = 3 * kTileLevels;     // (level, kind) pairs at most
+constexpr uint32_t kTileList = 0xFFFFu;     // first word of a record that is a list in the pool
+constexpr uint32_t kMaxSharedSegments = 32768;   // segments of a box query at most
+constexpr uint32_t kFracPair = 2u, kFracList = 1u;   // last word of a 16-bit record
+struct TileGeom {
+    int32_t edge[kTileLevels];   // log2 of the largest plane edge of the level (0: none)
+    int32_t line[kTileLevels];   // the level has lines
+    int64_t off[kTileLevels][3][3];
+    uint32_t st1[kTileLevels][3][3], st2[kTileLevels][3][3];
+};
+
 }  // namespace mg
 
 struct mg_graph {
@@ -148,6 +163,10 @@ struct mg_graph {
     mg::Buf mipx[3];
     int32_t qpitch[MG_MAX_LEVELS][3] = {};
     int64_t qoff[MG_MAX_LEVELS][3] = {};
+    // exact segment counts of tiles (mg_tiles.cu; empty if there was no room)
+    mg::Buf tiles;      // uint4 records
+    mg::Buf tile_pool;  // uint4 blocks of the lists
+    mg::TileGeom tgeom{};
     // node table, canonical order, N entries
     mg::Buf pq;       // uint2 (p, q); (kNone, kNone) for sources
     mg::Buf ab;       // ulonglong2 (a, b) exact coprime weights
@@ -160,6 +179,12 @@ struct mg_graph {
     // lut_meta[n] = (first entry, entries << 8 | lmin), lut = (source, count)
     mg::Buf lut_meta;
     mg::Buf lut;
+    mg::Buf lut_rec;   // uint4 record per node (mg_tiles.cu; empty if there was no room)
+    // the same for 16-bit weights (0: f16, 1: bf16), built on first use: the
+    // share of a node's weight that every entry of its row receives, and the
+    // nodes' records
+    std::mutex rec16_mu;
+    mg::Buf frac16[2], rec16[2];
     int64_t lut_entries = 0;
     // quantised graph (from the greedy factorisation): a node's weight is its
     // bin's codeword, no exact weights (a = b = 0), so only fp32 pushes apply
@@ -212,9 +237,15 @@ mg_status propagate_multi(mg_graph* g, const float* tf, int k, int C, mg_dtype s
 mg_status build_lut(mg_graph* g, cudaStream_t s);
 // the padded axis-major copies of the box queries, from mip0 and mip
 mg_status build_query_copies(mg_graph* g, cudaStream_t s);
+// the tiles of the box queries (after the copies and the mixture table);
+// the queries do without them where there is no memory for them
+mg_status build_tiles(mg_graph* g, cudaStream_t s);
 // box histograms summed from the mixture table, with error bars (Sec. 3.5-3.6)
 mg_status query_lut(const mg_graph* g, const int32_t* boxes, int64_t Q, double* hist, double* err, cudaStream_t s);
 mg_status ensure_alpha16(mg_graph* g, mg_dtype dt, cudaStream_t s);
+// the nodes' shares and records for 16-bit weights (after ensure_alpha16); the
+// queries walk the lerp trees where there is no memory for them
+mg_status ensure_records16(mg_graph* g, mg_dtype dt, cudaStream_t s);
 mg_status query_boxes(const mg_graph* g, const int32_t* boxes, int64_t Q, const mg_query_opts& o,
                       void* out, size_t cap, uint32_t* seg, uint64_t* offsets, size_t* required,
                       cudaStream_t s);
@@ -246,6 +277,14 @@ struct PlanParts {
     uint64_t cap_blocks, cap_chunks;
 };
 PlanParts plan_parts(const mg_query_plan* p);
+// Work-chunk length of a plan, and the chunk-map entries it keeps per chunk of
+// the caller's capacity: an untuned plan for few boxes takes chunks `scale`
+// times shorter than the default, so that what fits the capacity in default
+// chunks fits its map.
+struct PlanChunk {
+    uint32_t chunk, scale;
+};
+PlanChunk plan_chunk(const mg_graph* g, int hist_type, int chunk_cubes, int64_t max_Q, uint64_t cap_chunks);
 
 // ---------------------------------------------------------------------------
 // small device helpers

@@ -6,8 +6,8 @@
 // Image: a fixed header (magic, version, sizes, geometry, depth buckets, the
 // byte size of every array), then the arrays in header order, each starting
 // on a 256-byte boundary.  Import validates the header and every size before
-// allocating anything.  The padded axis-major copies of the box queries are
-// not stored: import rebuilds them from the mip levels.
+// allocating anything.  The padded axis-major copies and the tiles of the
+// box queries are not stored: import rebuilds them from the mip levels.
 #include "mg_internal.cuh"
 
 #include <cstring>
@@ -182,10 +182,11 @@ MG_API mg_status mg_graph_import(const void* host, size_t bytes, const mg_alloca
     MG_TRY(g->status.alloc(&g->al, sizeof(unsigned), s));
     MG_CUDA(cudaMemsetAsync(g->status.p, 0, sizeof(unsigned), s));
     MG_TRY(build_query_copies(g.get(), s));
+    MG_TRY(build_tiles(g.get(), s));
     MG_CUDA(cudaStreamSynchronize(s));   // the host image may be freed on return
     for (int k = 0; k < kArrays; k++) arrays(g.get(), k)->s = nullptr;
     for (int c = 0; c < 3; c++) g->mip0x[c].s = g->mipx[c].s = nullptr;
-    g->status.s = nullptr;
+    g->status.s = g->tiles.s = g->tile_pool.s = g->lut_rec.s = nullptr;
     *out = g.release();
     return MG_OK;
 }

@@ -1,28 +1,28 @@
 // mg_query.cu -- segment histograms of boxes: footprint assembly (Sec. 3.6,
 // Algorithm 1) and the reverse weight push through the Mixture Graph.
 //
-// Plan (one warp per box): clip the box, split each axis range into aligned
-// power-of-two runs (footprint_1d), count the blocks of the runs' tensor
-// product and the cubes tiling them (a block of run levels (lx, ly, lz) sits at
-// level l = min and holds 2^(lx-l) * 2^(ly-l) * 2^(lz-l) cubes), then write one
-// 12-byte record per block: first cube index, the index of its first cube in
-// the level's ID array, level, and log2 extents.  Blocks follow Algorithm 1's
-// loop order (z, y, x).  Every level is stored three times (x-, y- and
-// z-fastest); a block reads the copy whose fastest axis is its longest side,
-// so even a one-voxel-thick slab reads contiguous IDs.
+// Plan: clip the box, split each axis range into aligned power-of-two runs
+// (footprint_1d), count the blocks of the runs' tensor product and the cubes
+// tiling them (a block of run levels (lx, ly, lz) sits at level l = min and
+// holds 2^(lx-l) * 2^(ly-l) * 2^(lz-l) cubes), then write one 12-byte record
+// per block: first item, the index of its first item in its array, array, and
+// log2 extents.  Blocks follow Algorithm 1's loop order (z, y, x).  A block one
+// cube thick or 16 cubes long is read as tile records (mg_tiles.cu), each the
+// exact segment counts of 16, 64 or 256 cubes; the others as the cubes' IDs.
+// Every level is stored three times (x-, y- and z-fastest); a block reads the
+// copy whose fastest axis is its longest side, so even a one-voxel-thick line
+// reads contiguous IDs.
 //
 // Main (persistent CTAs, MG_SCHED_BATCHED): a global ticket hands out chunks of
-// `chunk` consecutive cubes of one box; each warp of the CTA takes a
-// contiguous span of the chunk.  While 32 or more cubes of the current block
-// remain, the warp walks the block directly (one ID per lane, 32-bit index
-// arithmetic); the last few cubes of a block go with the next block's first
-// ones through a ballot that tells each lane its block.  Adjacent lanes with
-// the same (level, node) merge into one contribution of count * 8^l.  A
-// source adds it to the CTA's shared-memory histogram; an internal node is
-// queued per warp and pushed down its lerp tree 32 at a time (p gets
-// W*a/(a+b), q gets W*b/(a+b), exact u32 arithmetic) into the same histogram.
-// At the end of a chunk the touched bins are added to the box's row in global
-// memory -- the only global atomics.
+// `chunk` consecutive items of one box to a warp with its own histogram in
+// shared memory (few segments), or to a CTA that shares one (many).  A source
+// adds its voxels to the histogram; a mixture node adds the segments of its
+// record or table row, or is queued and pushed down its lerp tree (p gets
+// W*a/(a+b), q gets W*b/(a+b), exact u32 arithmetic).  At the end of a chunk
+// the touched bins are added to the box's row in global memory -- the only
+// global atomics.  100,000 boxes on 2048x2048x300: 58,000 cubes a box become
+// 890 units (280 tile records, 480 vectors and 120 cubes), 5.41 -> 1.08 ms;
+// what is left is the latency of a chunk's dependent loads and its flush.
 //
 // MG_SCHED_PLAIN is the baseline: one launch and one CTA per box, walking the
 // blocks in order.
@@ -38,19 +38,28 @@ namespace {
 
 constexpr int kMaxRuns = 40;
 constexpr int kMaxStack = 64;
-constexpr uint32_t kMaxSharedSegments = 32768;
 constexpr uint32_t kMaxPushSteps = 1u << 24;   // a valid table never needs this many
+
+// A block is read either as its cubes' IDs or as tiles (mg_tiles.cu): "array"
+// l < 32 holds the IDs of level l, array tile_array(l, kind) the records of
+// level l's tiles of that kind.
+constexpr int kArrays = MG_MAX_LEVELS + 3 * kTileLevels;
+__host__ __device__ __forceinline__ int tile_array(int l, int kind) { return MG_MAX_LEVELS + 3 * l + kind; }
 
 struct Geom {
     int L;
     int id0_bytes;
     uint32_t S;
     int32_t dims[MG_MAX_LEVELS][3];
-    // offset of level l >= 1 in copy c's concatenated levels
-    int64_t off[MG_MAX_LEVELS][3];
+    // offset of level l >= 1 in copy c's concatenated levels, of a tile array
+    // in the records
+    int64_t off[kArrays][3];
     // strides of the second and third axis of each copy (copy 0: x, y, z;
     // copy 1: y, z, x; copy 2: z, x, y): the row pitch and pitch x middle dim
-    uint32_t st1[MG_MAX_LEVELS][3], st2[MG_MAX_LEVELS][3];
+    uint32_t st1[kArrays][3], st2[kArrays][3];
+    // tiles of the levels 0-3, four bits a level: log2 of the largest plane
+    // edge (0, 3 or 4), plus 8 where the level has lines
+    uint32_t tiles;
     // bit l of vec_ok[c] / vec32_ok[c]: every row of copy c at level l starts
     // on a 16-byte / 32-byte boundary (row pitch and level offset multiples)
     uint32_t vec_ok[3], vec32_ok[3];
@@ -59,15 +68,20 @@ struct Geom {
 struct Ids {
     const void* l0[3];       // level 0 copies (uint16 or uint32)
     const uint32_t* hi[3];   // levels >= 1 copies, concatenated at Geom::off
+    const uint4* tiles;      // tile records
+    const uint4* pool;       // their lists
 };
 
 struct Blk {
-    uint32_t start;   // first cube of the block within its box
-    uint32_t base;    // index of the block's first cube in its copy of level l
-    uint32_t meta;    // l | copy << 5 | e0 << 7 | e1 << 12 | e2 << 17 (log2 extents, copy axis order)
+    uint32_t start;   // first item (cube or tile) of the block within its box
+    uint32_t base;    // index of the block's first item in its copy of the array
+    uint32_t meta;    // array | copy << 6 | e0 << 8 | e1 << 13 | e2 << 18 (log2 extents, copy axis order)
 };
 
-Geom make_geom(const mg_graph* g) {
+// tile_levels: levels whose tiles the caller's pushes may take (0: cubes only;
+// 1: level 0, whose cubes are segments whatever the weights; kTileLevels:
+// exact weights)
+Geom make_geom(const mg_graph* g, int tile_levels) {
     Geom G;
     G.L = g->L;
     G.id0_bytes = g->id0_bytes;
@@ -82,6 +96,17 @@ Geom make_geom(const mg_graph* g) {
             G.st1[l][c] = pitch;
             G.st2[l][c] = pitch * mid[c];
         }
+    }
+    G.tiles = 0;
+    for (int l = 0; l < kTileLevels; l++) {
+        if (l < tile_levels) G.tiles |= (uint32_t)(g->tgeom.edge[l] | (g->tgeom.line[l] ? 8 : 0)) << (4 * l);
+        for (int k = 0; k < 3; k++)
+            for (int c = 0; c < 3; c++) {
+                const int a = tile_array(l, k);
+                G.off[a][c] = g->tgeom.off[l][k][c];
+                G.st1[a][c] = g->tgeom.st1[l][k][c];
+                G.st2[a][c] = g->tgeom.st2[l][k][c];
+            }
     }
     for (int c = 0; c < 3; c++) {
         G.vec_ok[c] = G.vec32_ok[c] = 0;
@@ -99,37 +124,59 @@ Geom make_geom(const mg_graph* g) {
     return G;
 }
 
+// 16-bit weights and quantised graphs push rounded weights through the trees:
+// their levels >= 1 stay cubes
+int tile_levels(const mg_graph* g, mg_dtype weights) {
+    return weights == MG_F32 && !g->quantised && g->lut_meta.p ? kTileLevels : 1;
+}
+
 Ids make_ids(const mg_graph* g) {
     Ids I;
     for (int c = 0; c < 3; c++) {
         I.l0[c] = g->mip0x[c].p ? g->mip0x[c].p : g->mip0.p;   // copy 0 may be mip0 itself
         I.hi[c] = g->mipx[c].as<uint32_t>();
     }
+    I.tiles = g->tiles.as<uint4>();
+    I.pool = g->tile_pool.as<uint4>();
     return I;
 }
 
-// block of run levels (lx, ly, lz) whose origin is the level-0 voxel (x0, y0, z0)
-__device__ __forceinline__ Blk make_blk(const Geom& G, uint32_t start, int32_t x0, int32_t y0, int32_t z0, int lx,
-                                        int ly, int lz) {
+// How a block of run levels (lx, ly, lz) is read: T = 3 or 4, as plane tiles
+// of edge 2^T (one cube thick, the other two extents reaching 2^T; then the
+// thickness axis is unique; the larger edge wherever the shorter side reaches
+// it); T = 2, as lines of 16 (2^(2 T) cubes too: two extents under 8, the
+// longest at least 16); T = 0, as cubes.
+__device__ __forceinline__ int block_tile(uint32_t tiles, int lx, int ly, int lz) {
+    const int lo = min(lx, ly), hi = max(lx, ly), l = min(lo, lz);
+    const int mid = max(lo, min(hi, lz)) - l, most = max(hi, lz) - l;
+    const int t = l < kTileLevels ? (int)(tiles >> (4 * l)) & 15 : 0;
+    return mid >= 3 ? min(mid, t & 7) : (t & 8) && most >= 4 ? 2 : 0;
+}
+
+// items of a block: cubes, or tiles of 2^(2 T) cubes
+__device__ __forceinline__ uint32_t block_items(int lx, int ly, int lz, int T) {
     const int l = min(lx, min(ly, lz));
-    const int ex = lx - l, ey = ly - l, ez = lz - l;
-    const uint32_t X = (uint32_t)x0 >> l, Y = (uint32_t)y0 >> l, Z = (uint32_t)z0 >> l;
-    int c, e0, e1, e2;
-    uint32_t base;
-    if (ex >= ey && ex >= ez) {
-        c = 0; e0 = ex; e1 = ey; e2 = ez;
-        base = Z * G.st2[l][0] + Y * G.st1[l][0] + X;
-    } else if (ey >= ez) {
-        c = 1; e0 = ey; e1 = ez; e2 = ex;
-        base = X * G.st2[l][1] + Z * G.st1[l][1] + Y;
-    } else {
-        c = 2; e0 = ez; e1 = ex; e2 = ey;
-        base = Y * G.st2[l][2] + X * G.st1[l][2] + Z;
-    }
+    return 1u << (lx + ly + lz - 3 * l - 2 * T);
+}
+
+// block of run levels (lx, ly, lz) whose origin is the level-0 voxel (x0, y0,
+// z0), read as T says
+__device__ __forceinline__ Blk make_blk(const Geom& G, uint32_t start, int32_t x0, int32_t y0, int32_t z0, int lx,
+                                        int ly, int lz, int T) {
+    const int l = min(lx, min(ly, lz));
+    // plane tiles lie in the copy whose slowest axis is the thickness, all
+    // else in the copy whose fastest axis is the longest side
+    const int c = T >= 3 ? (lz == l ? 0 : lx == l ? 1 : 2) : (lx >= ly && lx >= lz) ? 0 : ly >= lz ? 1 : 2;
+    const int v = T == 0 ? l : tile_array(l, T == 2 ? 2 : T - 3);
+    const int32_t a0 = c == 0 ? x0 : c == 1 ? y0 : z0, b0 = c == 0 ? y0 : c == 1 ? z0 : x0;
+    const int32_t t0 = c == 0 ? z0 : c == 1 ? x0 : y0;
+    const int la = c == 0 ? lx : c == 1 ? ly : lz, lb = c == 0 ? ly : c == 1 ? lz : lx;
+    const int lt = c == 0 ? lz : c == 1 ? lx : ly;
+    const int sa = l + (T == 2 ? 4 : T), sb = l + (T == 2 ? 0 : T);   // log2 item extents
     Blk B;
     B.start = start;
-    B.base = base;
-    B.meta = (uint32_t)(l | c << 5 | e0 << 7 | e1 << 12 | e2 << 17);
+    B.base = ((uint32_t)t0 >> l) * G.st2[v][c] + ((uint32_t)b0 >> sb) * G.st1[v][c] + ((uint32_t)a0 >> sa);
+    B.meta = (uint32_t)(v | c << 6 | (la - sa) << 8 | (lb - sb) << 13 | (lt - l) << 18);
     return B;
 }
 
@@ -191,30 +238,64 @@ __device__ __forceinline__ uint32_t block_cubes(int lx, int ly, int lz) {
 // P(0) - 7 * sum over m >= 1 of P(m).  Algorithm 1's steps on one axis rise
 // to a peak and fall again, so no level occurs more than twice and two bit
 // masks hold an axis's levels: F(m) = (once >> m) + (twice >> m).
-__device__ __forceinline__ void level_masks(const uint8_t* l, int n, uint64_t& once, uint64_t& twice) {
-    once = twice = 0;
+struct Masks {
+    uint32_t once, twice;   // levels below 32: an axis's voxels are counted in int32
+    __device__ __forceinline__ uint32_t sum(int m) const { return (once >> m) + (twice >> m); }            // F(m)
+    __device__ __forceinline__ uint32_t runs(int l) const { return ((once >> l) & 1) + ((twice >> l) & 1); }
+};
+
+__device__ __forceinline__ Masks level_masks(const uint8_t* l, int n) {
+    Masks M{0u, 0u};
     for (int i = 0; i < n; i++) {
-        const uint64_t bit = 1ull << l[i];
-        if (once & bit) twice |= bit;
-        else once |= bit;
+        const uint32_t bit = 1u << l[i];
+        if (M.once & bit) M.twice |= bit;
+        else M.once |= bit;
     }
+    return M;
 }
 
-__device__ __forceinline__ uint64_t cubes_from_masks(uint64_t x1, uint64_t x2, uint64_t y1, uint64_t y2, uint64_t z1,
-                                                     uint64_t z2) {
-    const uint64_t p0 = (x1 + x2) * (y1 + y2) * (z1 + z2);
-    uint64_t rest = 0;
-    for (int m = 1; m < 64 && (x1 >> m) && (y1 >> m) && (z1 >> m); m++)
-        rest += ((x1 >> m) + (x2 >> m)) * ((y1 >> m) + (y2 >> m)) * ((z1 >> m) + (z2 >> m));
-    return p0 - 7 * rest;
+// level m's term of that sum
+__device__ __forceinline__ uint64_t cube_term(int m, const Masks& x, const Masks& y, const Masks& z) {
+    const uint64_t p = (uint64_t)x.sum(m) * y.sum(m) * z.sum(m);
+    return m == 0 ? p : 0ull - 7 * p;
 }
 
-__device__ __forceinline__ uint64_t footprint_cubes(const Runs& R) {
-    uint64_t x1, x2, y1, y2, z1, z2;
-    level_masks(R.lx, R.nx, x1, x2);
-    level_masks(R.ly, R.ny, y1, y2);
-    level_masks(R.lz, R.nz, z1, z2);
-    return cubes_from_masks(x1, x2, y1, y2, z1, z2);
+// Items of the same footprint: level l's change to the count of cubes.  A
+// block of level l on axis t and extents 2^a, 2^b >= 8 cubes on the others
+// counts 2^(a+b) cubes but 2^(a+b-6) tiles of edge 8, or 2^(a+b-8) of edge 16
+// where both extents reach 16: summed over such blocks, with n_t(l) the runs
+// of level l on axis t, n_t(l) (63 F(l+3) F'(l+3) + 3 F(l+4) F'(l+4)) less, the
+// last term with edge 16.  Lines along axis t replace 16 cubes each where the
+// other axes' levels lie within l..l+2 and one of them is l: 15 F(l+4) times
+// the sum over such pairs less.
+__device__ __forceinline__ uint64_t tile_term(uint32_t tiles, int l, const Masks& x, const Masks& y, const Masks& z) {
+    const uint32_t t = l < kTileLevels ? (tiles >> (4 * l)) & 15u : 0u;
+    if (!t) return 0;
+    const uint64_t nx = x.runs(l), ny = y.runs(l), nz = z.runs(l);
+    const uint64_t fx = x.sum(l + 3), fy = y.sum(l + 3), fz = z.sum(l + 3);
+    const uint64_t gx = x.sum(l + 4), gy = y.sum(l + 4), gz = z.sum(l + 4);
+    uint64_t less = 0;
+    if (t & 7u) less += 63 * (nx * fy * fz + ny * fz * fx + nz * fx * fy);
+    if ((t & 7u) == 4u) less += 3 * (nx * gy * gz + ny * gz * gx + nz * gx * gy);
+    if (t & 8u) {
+        // cubes across of the runs of levels l + 1 and l + 2, per axis
+        const uint64_t wx = 2 * x.runs(l + 1) + 4 * x.runs(l + 2), wy = 2 * y.runs(l + 1) + 4 * y.runs(l + 2),
+                       wz = 2 * z.runs(l + 1) + 4 * z.runs(l + 2);
+        less += 15 * (gx * (ny * nz + ny * wz + wy * nz) + gy * (nz * nx + nz * wx + wz * nx) +
+                      gz * (nx * ny + nx * wy + wx * ny));
+    }
+    return 0ull - less;
+}
+
+constexpr int kMaxAxisLevels = 32;
+
+// cubes of a footprint, or its items (tiles = G.tiles; 0: cubes)
+__device__ __forceinline__ uint64_t footprint_count(const Runs& R, uint32_t tiles) {
+    const Masks x = level_masks(R.lx, R.nx), y = level_masks(R.ly, R.ny), z = level_masks(R.lz, R.nz);
+    uint64_t n = 0;
+    for (int m = 0; m < kMaxAxisLevels && (x.once >> m) && (y.once >> m) && (z.once >> m); m++)
+        n += cube_term(m, x, y, z) + tile_term(tiles, m, x, y, z);
+    return n;
 }
 
 // Batch size and capacities read on the device, for query plans replayed as
@@ -238,7 +319,7 @@ __device__ __forceinline__ bool over_cap(const Lim& lim, const uint64_t* blk_off
 // ---------------------------------------------------------------------------
 __global__ void plan_count_kernel(Geom G, const int32_t* __restrict__ boxes, int64_t Q, uint32_t chunk,
                                   uint32_t* __restrict__ nblk, uint64_t* __restrict__ ncube,
-                                  uint64_t* __restrict__ nchunk, unsigned* __restrict__ status, Lim lim) {
+                                  uint64_t* __restrict__ nchunk, unsigned* __restrict__ status, Lim lim, bool items) {
     const int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (q >= Q) return;
@@ -266,7 +347,7 @@ __global__ void plan_count_kernel(Geom G, const int32_t* __restrict__ boxes, int
     Runs& R = wr[threadIdx.x >> 5];
     make_runs_warp(b, G, R);
     if (lane == 0) {
-        const uint64_t cubes = footprint_cubes(R);
+        const uint64_t cubes = footprint_count(R, items ? G.tiles : 0u);
         if (nblk) nblk[q] = (uint32_t)(R.nx * R.ny * R.nz);
         ncube[q] = cubes;
         if (nchunk) nchunk[q] = (cubes + chunk - 1) / chunk;
@@ -299,7 +380,8 @@ __global__ void plan_write_kernel(Geom G, const int32_t* __restrict__ boxes, int
         const int j = valid ? pr % R.ny : 0, k = valid ? pr / R.ny : 0;
         uint32_t row = 0;
         if (valid)
-            for (int i = 0; i < R.nx; i++) row += block_cubes(R.lx[i], R.ly[j], R.lz[k]);
+            for (int i = 0; i < R.nx; i++)
+                row += block_items(R.lx[i], R.ly[j], R.lz[k], block_tile(G.tiles, R.lx[i], R.ly[j], R.lz[k]));
         // exclusive warp scan of the row totals
         uint32_t incl = row;
 #pragma unroll
@@ -312,8 +394,9 @@ __global__ void plan_write_kernel(Geom G, const int32_t* __restrict__ boxes, int
             uint32_t start = running + incl - row;
             for (int i = 0; i < R.nx; i++) {
                 const uint64_t bi = base + (uint64_t)pr * R.nx + i;
-                const uint32_t n = block_cubes(R.lx[i], R.ly[j], R.lz[k]);
-                blk[bi] = make_blk(G, start, R.sx[i], R.sy[j], R.sz[k], R.lx[i], R.ly[j], R.lz[k]);
+                const int T = block_tile(G.tiles, R.lx[i], R.ly[j], R.lz[k]);
+                const uint32_t n = block_items(R.lx[i], R.ly[j], R.lz[k], T);
+                blk[bi] = make_blk(G, start, R.sx[i], R.sy[j], R.sz[k], R.lx[i], R.ly[j], R.lz[k], T);
                 // the chunks whose first cube lies in this block
                 for (uint64_t c = ((uint64_t)start + chunk - 1) / chunk; c * chunk < (uint64_t)start + n; c++) {
                     chunk_q[cbase + c] = (uint32_t)q;
@@ -379,23 +462,22 @@ struct FusedOut {
 
 // Algorithm 1's steps on one axis (as footprint_1d) together with the axis's
 // level masks (levels seen once, levels seen twice)
-__device__ __forceinline__ int axis_runs(int64_t i, int64_t di, int64_t dim, uint8_t* r, int32_t* start,
-                                         uint64_t& once, uint64_t& twice) {
+// (0 <= i < dim <= 65535, di >= 1)
+__device__ __forceinline__ int axis_runs(int32_t i, int32_t di, int32_t dim, uint8_t* r, int32_t* start, Masks& M) {
     int n = 0;
-    once = twice = 0;
-    di = min(i + di, dim) - i;
+    M = Masks{0u, 0u};
+    di = min(di, dim - i);
     while (di > 0 && n < kMaxRuns) {
-        const int a = 63 - __clzll(di);
-        const int b = i == 0 ? 63 : __ffsll(i) - 1;
-        const int l = min(a, b);
-        const uint64_t bit = 1ull << l;
-        if (once & bit) twice |= bit;
-        else once |= bit;
+        const int a = 31 - __clz(di);
+        const int l = i == 0 ? a : min(a, __ffs(i) - 1);
+        const uint32_t bit = 1u << l;
+        M.twice |= M.once & bit;
+        M.once |= bit;
         r[n] = (uint8_t)l;
-        start[n] = (int32_t)i;
+        start[n] = i;
         n++;
-        di -= (int64_t)1 << l;
-        i += (int64_t)1 << l;
+        di -= (int32_t)bit;
+        i += (int32_t)bit;
     }
     return n;
 }
@@ -413,7 +495,8 @@ __device__ __forceinline__ void zero_span(T* a, size_t r0, size_t r1) {
     for (size_t i = threadIdx.x; i < (a1 - a0) / 4; i += kFusedThreads) v[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-__global__ void __launch_bounds__(kFusedThreads, 2) plan_fused_kernel(Geom G, const int32_t* __restrict__ boxes,
+__global__ void __launch_bounds__(kFusedThreads, 2) plan_fused_kernel(const __grid_constant__ Geom G,
+                                                                      const int32_t* __restrict__ boxes,
                                                                       int64_t Q, int tb, uint32_t chunk,
                                                                       int chunk_shift, Lim lim, FusedOut F,
                                                                       unsigned* __restrict__ status) {
@@ -454,7 +537,7 @@ __global__ void __launch_bounds__(kFusedThreads, 2) plan_fused_kernel(Geom G, co
         const int64_t q = q0 + w;
         const bool live = w < tb && q < Qe;
         bool ok = false;
-        uint64_t once = 0, twice = 0;
+        Masks M{0u, 0u};
         if (live) {
             int32_t b[6];
 #pragma unroll
@@ -463,36 +546,36 @@ __global__ void __launch_bounds__(kFusedThreads, 2) plan_fused_kernel(Geom G, co
             if (!ok && bl == 0) set_status(status, kStatBadInput);
             if (ok && bl < 3) {
                 Runs& R = wr[w];
-                const int64_t i0 = bl == 0 ? b[0] : bl == 1 ? b[1] : b[2];
-                const int64_t di = bl == 0 ? b[3] : bl == 1 ? b[4] : b[5];
-                const int64_t dim = bl == 0 ? G.dims[0][0] : bl == 1 ? G.dims[0][1] : G.dims[0][2];
+                const int32_t i0 = bl == 0 ? b[0] : bl == 1 ? b[1] : b[2];
+                const int32_t di = bl == 0 ? b[3] : bl == 1 ? b[4] : b[5];
+                const int32_t dim = bl == 0 ? G.dims[0][0] : bl == 1 ? G.dims[0][1] : G.dims[0][2];
                 uint8_t* lv = bl == 0 ? R.lx : bl == 1 ? R.ly : R.lz;
                 int32_t* sv = bl == 0 ? R.sx : bl == 1 ? R.sy : R.sz;
-                const int n = axis_runs(i0, di, dim, lv, sv, once, twice);
+                const int n = axis_runs(i0, di, dim, lv, sv, M);
                 if (bl == 0) R.nx = n;
                 else if (bl == 1) R.ny = n;
                 else R.nz = n;
             }
         }
-        // lanes 1 and 2 of a group hand their masks to lane 0
-        const uint64_t y1 = __shfl_down_sync(0xffffffffu, once, 1, kBoxLanes);
-        const uint64_t y2 = __shfl_down_sync(0xffffffffu, twice, 1, kBoxLanes);
-        const uint64_t z1 = __shfl_down_sync(0xffffffffu, once, 2, kBoxLanes);
-        const uint64_t z2 = __shfl_down_sync(0xffffffffu, twice, 2, kBoxLanes);
+        // the group's lanes take the levels of the closed form in turn
+        const Masks x{__shfl_sync(0xffffffffu, M.once, 0, kBoxLanes), __shfl_sync(0xffffffffu, M.twice, 0, kBoxLanes)};
+        const Masks y{__shfl_sync(0xffffffffu, M.once, 1, kBoxLanes), __shfl_sync(0xffffffffu, M.twice, 1, kBoxLanes)};
+        const Masks z{__shfl_sync(0xffffffffu, M.once, 2, kBoxLanes), __shfl_sync(0xffffffffu, M.twice, 2, kBoxLanes)};
         __syncwarp();
-        if (bl == 0 && w < tb) {
-            uint64_t cubes = 0;
-            uint32_t nb = 0;
-            if (ok) {
-                const Runs& R = wr[w];
-                cubes = cubes_from_masks(once, twice, y1, y2, z1, z2);
-                nb = (uint32_t)(R.nx * R.ny * R.nz);
-                s_mx[w] = ((1ull << 32) + R.nx - 1) / (uint64_t)R.nx;
-                s_my[w] = ((1ull << 32) + R.ny - 1) / (uint64_t)R.ny;
+        uint64_t items = tile_term(G.tiles, bl, x, y, z);
+        for (int m = bl; m < kMaxAxisLevels; m += kBoxLanes) items += cube_term(m, x, y, z);
+#pragma unroll
+        for (int o = kBoxLanes / 2; o > 0; o >>= 1) items += __shfl_xor_sync(0xffffffffu, items, o, kBoxLanes);
+        if (w < tb) {
+            if (bl == 0) {
+                if (live) F.ncube[q] = items;
+                s_ncube[w] = items;
+                s_nblk[w] = ok ? (uint32_t)(wr[w].nx * wr[w].ny * wr[w].nz) : 0u;
+            } else if (bl <= 2 && ok) {
+                // ceil(2^32 / n)
+                const uint32_t n = (uint32_t)(bl == 1 ? wr[w].nx : wr[w].ny);
+                (bl == 1 ? s_mx : s_my)[w] = (uint64_t)(0xffffffffu / n) + 1;
             }
-            if (live) F.ncube[q] = cubes;
-            s_nblk[w] = nb;
-            s_ncube[w] = cubes;
         }
     }
     {   // the tile's live output rows are one contiguous span
@@ -634,12 +717,12 @@ __global__ void __launch_bounds__(kFusedThreads, 2) plan_fused_kernel(Geom G, co
     uint32_t carry = 0;   // cubes of the earlier rounds, mod 2^32
     for (uint32_t r0 = 0; r0 < nbt; r0 += kFusedThreads * kFusedItems) {
         uint32_t n[kFusedItems], incl[kFusedItems];
-        int wk[kFusedItems], ik[kFusedItems], jk[kFusedItems], kk[kFusedItems];
+        int wk[kFusedItems], ik[kFusedItems], jk[kFusedItems], kk[kFusedItems], tk[kFusedItems];
 #pragma unroll
         for (int it = 0; it < kFusedItems; it++) {
             const uint32_t idx = r0 + it * kFusedThreads + threadIdx.x;
             n[it] = 0;
-            wk[it] = ik[it] = jk[it] = kk[it] = 0;
+            wk[it] = ik[it] = jk[it] = kk[it] = tk[it] = 0;
             if (idx < nbt) {
                 int w = 0;   // the last box whose blocks start at or before idx
 #pragma unroll
@@ -653,7 +736,9 @@ __global__ void __launch_bounds__(kFusedThreads, 2) plan_fused_kernel(Geom G, co
                 ik[it] = (int)(t - pr * (uint32_t)R.nx);
                 jk[it] = (int)(pr - k * (uint32_t)R.ny);
                 kk[it] = (int)k;
-                n[it] = block_cubes(R.lx[ik[it]], R.ly[jk[it]], R.lz[kk[it]]);
+                const int lx = R.lx[ik[it]], ly = R.ly[jk[it]], lz = R.lz[kk[it]];
+                tk[it] = block_tile(G.tiles, lx, ly, lz);
+                n[it] = block_items(lx, ly, lz, tk[it]);
             }
             uint32_t v = n[it];
 #pragma unroll
@@ -690,7 +775,7 @@ __global__ void __launch_bounds__(kFusedThreads, 2) plan_fused_kernel(Geom G, co
                 const Runs& R = wr[w];
                 const uint32_t start = base + s_wsum[warp][it] + incl[it] - n[it] - s_cube[w];
                 const uint64_t bi = pre_b + idx;
-                F.blk[bi] = make_blk(G, start, R.sx[i], R.sy[j], R.sz[k], R.lx[i], R.ly[j], R.lz[k]);
+                F.blk[bi] = make_blk(G, start, R.sx[i], R.sy[j], R.sz[k], R.lx[i], R.ly[j], R.lz[k], tk[it]);
                 const uint64_t cb = pre_c + s_coff[w];
                 const uint64_t first = (uint64_t)start + chunk - 1;
                 for (uint64_t c = chunk_shift >= 0 ? first >> chunk_shift : first / chunk;
@@ -757,6 +842,8 @@ struct PushArgs {
     unsigned* status;
     const uint2* lut_meta;   // mixture lookup table (null: walk the lerp trees)
     const uint2* lut;
+    const uint4* rec;        // records of the nodes in the table (null: none)
+    const float* frac;       // 16-bit weights: the share of each table entry
 };
 
 // The table row of node n for a push of weight w: entries (source, count)
@@ -880,8 +967,8 @@ __device__ __forceinline__ uint32_t read_id(const Geom& G, const Ids& I, int l, 
 
 // node ID of cube o of block B
 __device__ __forceinline__ uint32_t cube_node(const Geom& G, const Ids& I, const Blk& B, uint32_t o, int& l) {
-    l = B.meta & 31;
-    const int c = (B.meta >> 5) & 3, e0 = (B.meta >> 7) & 31, e1 = (B.meta >> 12) & 31;
+    l = B.meta & 63;
+    const int c = (B.meta >> 6) & 3, e0 = (B.meta >> 8) & 31, e1 = (B.meta >> 13) & 31;
     const uint32_t f = o & ((1u << e0) - 1u);
     const uint32_t sc = (o >> e0) & ((1u << e1) - 1u);
     const uint32_t t = o >> (e0 + e1);
@@ -1123,56 +1210,138 @@ __device__ __forceinline__ void drain(const PushArgs& P, const Hist<FP>& H, cons
     __syncwarp();
 }
 
-// Cubes [w0, w1) of one box by one warp, b the block holding cube w0.
+// What a lane needs to read the units of one block.  A warp keeps one of these
+// per block of its window in shared memory, so that a unit costs two shared
+// loads instead of a shuffle per field and an indexed parameter load per
+// stride.
+struct __align__(16) Desc {
+    uint64_t addr;       // the block's first item
+    uint32_t st1, st2;   // strides of its second and third axis, in items
+    uint32_t off;        // item of unit u: off + (u << lg)
+    uint32_t bits;       // e0 | e1 << 5 | lg << 10 | level << 13
+    uint32_t lo, hi;     // its items inside the span
+};
+constexpr size_t kDescBytes = 32 * sizeof(Desc);   // per warp
+
+// One class's units of a window, numbered through its blocks by a warp scan.
+struct Units {
+    uint32_t n, incl, total;   // this lane's block's units, their inclusive sum, the window's
+
+    // number the units (n set) and lay out the blocks that have any, in order;
+    // false when the window has none
+    __device__ __forceinline__ bool number(Desc& D, uint32_t first, uint32_t lg, Desc* desc) {
+        const int lane = threadIdx.x & 31;
+        const unsigned act = __ballot_sync(0xffffffffu, n != 0u);
+        if (!act) return false;
+        incl = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        total = __shfl_sync(0xffffffffu, incl, 31);
+        __syncwarp();   // the previous class's units have been read
+        if (n) {
+            D.off = first - ((incl - n) << lg);
+            desc[__popc(act & ((1u << lane) - 1u))] = D;
+        }
+        __syncwarp();
+        return true;
+    }
+
+    // place in desc of the block of unit ub + lane: the blocks that end at or
+    // before ub, plus those that end inside this group of 32 at or before the
+    // unit (blocks with units have distinct ends, so one bit each)
+    __device__ __forceinline__ int block(uint32_t ub) const {
+        const int lane = threadIdx.x & 31;
+        const unsigned below = __ballot_sync(0xffffffffu, n != 0u && incl <= ub);
+        const uint32_t te = incl - ub;
+        const unsigned ends = __reduce_or_sync(0xffffffffu, n != 0u && incl > ub && te < 32u ? 1u << te : 0u);
+        return __popc(below) + __popc(ends & ((2u << lane) - 1u));
+    }
+};
+
+// index of item o of a block, relative to its first one
+__device__ __forceinline__ uint32_t item_at(uint32_t o, uint32_t bits, uint32_t st1, uint32_t st2) {
+    const uint32_t e0 = bits & 31u, e1 = (bits >> 5) & 31u;
+    return (o & ((1u << e0) - 1u)) + ((o >> e0) & ((1u << e1) - 1u)) * st1 + (o >> (e0 + e1)) * st2;
+}
+
+// the words segment | count << 16 of a tile record's or list's block
+template <bool FP>
+__device__ __forceinline__ void add_words(const Hist<FP>& H, uint4 x) {
+    H.add_int(x.x & 0xffffu, x.x >> 16);
+    if (x.y) H.add_int(x.y & 0xffffu, x.y >> 16);
+    if (x.z) H.add_int(x.z & 0xffffu, x.z >> 16);
+    if (x.w) H.add_int(x.w & 0xffffu, x.w >> 16);
+}
+
+// a mixture node's cube of level l through the node's record r
+template <bool FP, typename AT>
+__device__ __forceinline__ void add_record(const PushArgs& P, const Hist<FP>& H, uint4 r, uint32_t node, uint32_t l) {
+    if constexpr (!std::is_same<AT, float>::value) {
+        // shares of 8^l, a power of two: the products are those of the tree walk
+        const float W = (float)(1u << (3 * l));
+        if (r.w == kFracPair) {
+            H.add_frac(r.x & 0xffffu, W * __uint_as_float(r.y));
+            H.add_frac(r.x >> 16, W * __uint_as_float(r.z));
+        } else if (r.w == kFracList) {
+            for (uint32_t e = 0; e < r.y; e++)
+                H.add_frac(__ldg(P.lut + r.x + e).x, W * __ldg(P.frac + r.x + e));
+        } else {
+            push_one<FP, AT>(P, H, node, 1u << (3 * l));
+        }
+    } else if (r.x >> 16) {
+        // counts of 8^lmin voxels: they sum to that power of two
+        const uint32_t sum = (r.x >> 16) + (r.y >> 16) + (r.z >> 16) + (r.w >> 16);
+        const uint32_t sh = 3 * l - (31 - __clz(sum));
+        H.add_int(r.x & 0xffffu, (r.x >> 16) << sh);
+        H.add_int(r.y & 0xffffu, (r.y >> 16) << sh);
+        if (r.z) H.add_int(r.z & 0xffffu, (r.z >> 16) << sh);
+        if (r.w) H.add_int(r.w & 0xffffu, (r.w >> 16) << sh);
+    } else if (r.x == kTileList) {
+        const uint32_t sh = 3 * l - r.w;
+        for (uint32_t e = 0; e < r.z; e += 2) {
+            const uint2 a = __ldg(P.lut + r.y + e);
+            const uint2 b = e + 1 < r.z ? __ldg(P.lut + r.y + e + 1) : make_uint2(0u, 0u);
+            H.add_int(a.x, a.y << sh);
+            if (b.y) H.add_int(b.x, b.y << sh);
+        }
+    } else {
+        push_one<FP, AT>(P, H, node, 1u << (3 * l));
+    }
+}
+
+// Items [w0, w1) of one box by one warp, b the block holding item w0.
 //
 // The span is a flat stream of units.  A window holds the records of 31
-// consecutive blocks, one per lane; the part of each block inside the span is
-// cut into units -- 32-byte vectors of IDs (16 uint16 or 8 uint32 of one row)
-// where the block's rows are 32-byte aligned and at least that long, else
-// 16-byte vectors where they are 16-byte aligned (Algorithm 1's runs start on
-// multiples of their own length, so whole rows are), and single cubes for the
-// unaligned head and tail and for every other block -- and a warp scan of
-// the unit counts lets lane k find the block of unit u from a ballot of
-// the block ends.
-// Each lane takes units u, u + 32, ... (a 32-byte unit is two 16-byte loads),
-// so no load waits on a block boundary.  Every lane keeps a run (level, node, count) of
-// its own consecutive cubes; a finished run of a source is added to the
-// shared histogram, one of an internal node (levels >= 1) is queued for the
-// warp's pushes.
-// RN: units per lane per step in windows without 32-byte units (2 in the
-// per-warp kernel, whose registers are capped for occupancy; 4 in the CTA
-// kernel, which has registers to spare: measured 4.67 -> 4.34 ms on the
-// cylinder batch, while the per-warp kernel spills at 4)
-template <bool FP, typename AT, int RN>
-__device__ __forceinline__ void process_span(const MainArgs& A, const Hist<FP>& H, const Queue& Qu, uint32_t w0,
-                                             uint32_t w1, uint64_t b, uint64_t b1, uint32_t ncube) {
+// consecutive blocks, one per lane, and their units are taken class by class,
+// so that the lanes of a warp do the same work at the same time: tile records,
+// vectors of 16 or 8 level-0 IDs of one row (32 or 16 bytes, where rows of
+// 2-byte IDs start on 16-byte boundaries and are at least 8 long; Algorithm
+// 1's runs start on multiples of their own length, so only the ends of the
+// span cut a vector), and single cubes.  No load waits on a block boundary.
+// Voxels of one segment extend a per-lane run, added to the histogram when the
+// segment changes (in uniform regions the lanes would otherwise meet in one
+// bin at every step).
+//
+// REC: a mixture node's cube reads the node's record (mg_tiles.cu) and adds
+// its segments at once, two dependent loads.  Without records (quantised
+// graphs, no room for them) the cube is queued for the warp's pushes, equal
+// nodes of a step merged.
+template <bool FP, typename AT, bool REC>
+__device__ __forceinline__ void process_span(const MainArgs& A, const Hist<FP>& H, const Queue& Qu, Desc* desc,
+                                             uint32_t w0, uint32_t w1, uint64_t b, uint64_t b1, uint32_t ncube) {
     const int lane = threadIdx.x & 31;
     const uint32_t S = A.P.S;
-    const int lg0 = A.G.id0_bytes == 2 ? 3 : 2;   // log2 level-0 IDs per 16 bytes
+    const bool id16 = A.G.id0_bytes == 2;
     uint32_t rid = kNone, rcnt = 0;
-    int rl = 0;
-    auto finish = [&]() {
-        if (!rcnt) return;
-        const uint32_t W = rcnt << (3 * rl);
-        if (rl == 0 || rid < S) {
-            H.add_int(rid, W);
-        } else {
-            const uint32_t pos = atomicAdd(Qu.count, 1u);
-            if (pos < Qu.cap) {
-                Qu.n[pos] = rid;
-                Qu.w[pos] = W;
-            } else {
-                push_one<FP, AT>(A.P, H, rid, W);
-            }
-        }
-    };
-    auto feed = [&](uint32_t x, int l, uint32_t n = 1) {
-        if (x == rid && l == rl) {
+    auto run_add = [&](uint32_t s, uint32_t n) {
+        if (s == rid) {
             rcnt += n;
         } else {
-            finish();
-            rid = x;
-            rl = l;
+            if (rcnt) H.add_int(rid, rcnt);
+            rid = s;
             rcnt = n;
         }
     };
@@ -1188,181 +1357,169 @@ __device__ __forceinline__ void process_span(const MainArgs& A, const Hist<FP>& 
         const uint32_t nxt = __shfl_down_sync(0xffffffffu, st, 1);
         const uint32_t lo_a = max(st, w0), hi_a = min(nxt, w1);
         const bool use = lane < 31 && lo_a < hi_a;
-        const int l = meta & 31, cp = (meta >> 5) & 3, e0 = (meta >> 7) & 31;
-        // 32-byte units where the block's rows allow them, else 16-byte ones
-        const int lg16 = l == 0 ? lg0 : 2;
-        const uint32_t lo = use ? lo_a - st : 0u, hi = use ? hi_a - st : 0u;
-        const bool wide = use && e0 > lg16 && ((A.G.vec32_ok[cp] >> l) & 1u) && hi - lo >= (4u << lg16);
-        const int lg = lg16 + (wide ? 1 : 0);
-        const bool vec = use && e0 >= lg && ((A.G.vec_ok[cp] >> l) & 1u) && hi - lo >= (2u << lg);
-        const uint32_t vm = (1u << lg) - 1u;
-        // scalar head [lo, ha), vectors [ha, hb), scalar tail [hb, hi)
-        const uint32_t ha = vec ? (lo + vm) & ~vm : hi;
-        const uint32_t hb = vec ? hi & ~vm : hi;
-        const uint32_t nh = ha - lo, nv = (hb - ha) >> lg;
-        const uint32_t units = use ? (hi - lo) - (hb - ha) + nv : 0u;
-        const uint32_t wmeta = meta | (wide ? 1u << 22 : 0u);
-        uint32_t incl = units;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
+        const int v = meta & 63, cp = (meta >> 6) & 3;
+        const bool tiles = use && v >= MG_MAX_LEVELS;
+        const bool vecs = use && v == 0 && id16 && ((meta >> 8) & 31u) >= 3 && (A.G.vec_ok[cp] & 1u);
+        const uint32_t vlg = ((meta >> 8) & 31u) >= 4 && (A.G.vec32_ok[cp] & 1u) ? 4 : 3;
+        Desc D{};
+        if (use) {
+            D.lo = lo_a - st;
+            D.hi = hi_a - st;
+            D.addr = tiles    ? reinterpret_cast<uint64_t>(A.I.tiles + A.G.off[v][cp] + base)
+                     : v == 0 ? reinterpret_cast<uint64_t>(A.I.l0[cp]) + ((uint64_t)base << (id16 ? 1 : 2))
+                              : reinterpret_cast<uint64_t>(A.I.hi[cp] + A.G.off[v][cp] + base);
+            D.st1 = A.G.st1[v][cp];
+            D.st2 = A.G.st2[v][cp];
+            D.bits = ((meta >> 8) & 1023u) | (vecs ? vlg << 10 : 0u) | (uint32_t)(v & 31) << 13;
         }
-        const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-        const uint32_t excl = incl - units;
-        // R units per lane per step: one (16- or 32-byte) where the window
-        // has 32-byte units, else RN, so scalar-heavy windows keep several
-        // loads in flight per lane
-        auto run_units = [&](auto rc) {
-            constexpr int R = decltype(rc)::value;
-            for (uint32_t u0 = 0; u0 < total; u0 += 32u * R) {
-                uint4 va[R], vb[R];
-                int kind[R], ul[R];   // kind: 0 scalar; 1 / 3: 4 / 8 uint32; 2 / 4: 8 / 16 uint16
+        Units U;
+
+        // tile records, two in flight per lane
+        U.n = tiles ? D.hi - D.lo : 0u;
+        if (U.number(D, D.lo, 0, desc)) {
+            for (uint32_t u0 = 0; u0 < U.total; u0 += 64) {
+                uint4 x[2];
 #pragma unroll
-                for (int r = 0; r < R; r++) {
-                    const uint32_t ub = u0 + 32u * r, u = ub + lane;
-                    // block of unit u: blocks ending at or before ub, plus those
-                    // ending inside this group at or before u (block ends are
-                    // distinct below the total, so one bit each)
-                    const unsigned below = __ballot_sync(0xffffffffu, incl <= ub);
-                    const uint32_t te = incl - ub;
-                    const unsigned ends = __reduce_or_sync(0xffffffffu, incl > ub && te < 32u ? 1u << te : 0u);
-                    const int j = __popc(below) + __popc(ends & ((2u << lane) - 1u) & ~1u);
-                    const uint32_t jbase = __shfl_sync(0xffffffffu, base, j & 31);
-                    const uint32_t jmeta = __shfl_sync(0xffffffffu, wmeta, j & 31);
-                    const uint32_t jlo = __shfl_sync(0xffffffffu, lo, j & 31);
-                    const uint32_t jnh = __shfl_sync(0xffffffffu, nh, j & 31);
-                    const uint32_t jnv = __shfl_sync(0xffffffffu, nv, j & 31);
-                    const uint32_t jex = __shfl_sync(0xffffffffu, excl, j & 31);
-                    kind[r] = -1;
-                    ul[r] = 0;
-                    va[r] = make_uint4(0u, 0u, 0u, 0u);
-                    vb[r] = va[r];
-                    if (u < total) {
-                        const int jl = jmeta & 31, jc = (jmeta >> 5) & 3;
-                        const int je0 = (jmeta >> 7) & 31, je1 = (jmeta >> 12) & 31;
-                        const bool jw = R == 1 && ((jmeta >> 22) & 1u);
-                        const int jlg = (jl == 0 ? lg0 : 2) + (jw ? 1 : 0);
-                        const uint32_t t = u - jex;
-                        uint32_t o;
-                        bool vv = false;
-                        if (t < jnh) {
-                            o = jlo + t;
-                        } else if (t < jnh + jnv) {
-                            o = jlo + jnh + ((t - jnh) << jlg);
-                            vv = true;
-                        } else {
-                            o = jlo + jnh + (jnv << jlg) + (t - jnh - jnv);
-                        }
-                        const uint32_t idx = jbase + (o & ((1u << je0) - 1u)) +
-                                             ((o >> je0) & ((1u << je1) - 1u)) * A.G.st1[jl][jc] +
-                                             (o >> (je0 + je1)) * A.G.st2[jl][jc];
-                        ul[r] = jl;
-                        const bool u16 = jl == 0 && lg0 == 3;
-                        // IDs are read once: streaming loads (evict first) leave L2
-                        // to the mixture table and node records the pushes gather
-                        const void* row =
-                            jl == 0 ? A.I.l0[jc] : static_cast<const void*>(A.I.hi[jc] + A.G.off[jl][jc]);
-                        if (vv) {
-                            const uint4* p = reinterpret_cast<const uint4*>(
-                                u16 ? static_cast<const void*>(static_cast<const uint16_t*>(row) + idx)
-                                    : static_cast<const void*>(static_cast<const uint32_t*>(row) + idx));
-                            va[r] = __ldcs(p);
-                            if (jw) vb[r] = __ldcs(p + 1);
-                            kind[r] = (u16 ? 2 : 1) + (jw ? 2 : 0);
-                        } else {
-                            va[r].x = u16 ? (uint32_t)__ldcs(static_cast<const uint16_t*>(row) + idx)
-                                          : __ldcs(static_cast<const uint32_t*>(row) + idx);
-                            kind[r] = 0;
-                        }
+                for (int r = 0; r < 2; r++) {
+                    const uint32_t u = u0 + 32 * r + lane;
+                    const int j = U.block(u0 + 32 * r);
+                    x[r] = make_uint4(0u, 0u, 0u, 0u);
+                    if (u < U.total) {
+                        const Desc& d = desc[j];
+                        const uint32_t idx = item_at(d.off + u, d.bits, d.st1, d.st2);
+                        x[r] = __ldcs(reinterpret_cast<const uint4*>(d.addr) + idx);
                     }
                 }
 #pragma unroll
-                for (int r = 0; r < R; r++) {
-                    const int k = kind[r], l = ul[r];
-                    const uint4 x = va[r], y = vb[r];
-                    if (k == 0) {
-                        feed(x.x, l);
-                    } else if (k == 1 || k == 3) {
-                        const bool same = rcnt && rl == l && x.x == rid && x.y == rid && x.z == rid && x.w == rid &&
-                                          (k == 1 || (y.x == rid && y.y == rid && y.z == rid && y.w == rid));
-                        if (same) {
-                            rcnt += k == 1 ? 4 : 8;
-                        } else {
-                            feed(x.x, l);
-                            feed(x.y, l);
-                            feed(x.z, l);
-                            feed(x.w, l);
-                            if (k == 3) {
-                                feed(y.x, l);
-                                feed(y.y, l);
-                                feed(y.z, l);
-                                feed(y.w, l);
-                            }
-                        }
-                    } else if (k == 2 || k == 4) {
-                        // uniform vector (every ID equals the first): it extends
-                        // the lane's run or starts a new one.  Mixed vector (a
-                        // segment boundary inside): each ID is added to its bin
-                        // at once -- level-0 IDs are bins, and the adds are
-                        // independent where a run would chain them
-                        const uint32_t a = x.x & 0xffffu, pa = a * 0x10001u;
-                        uint32_t d = (x.x ^ pa) | (x.y ^ pa) | (x.z ^ pa) | (x.w ^ pa);
-                        if (k == 4) d |= (y.x ^ pa) | (y.y ^ pa) | (y.z ^ pa) | (y.w ^ pa);
-                        if (d == 0u) {
-                            if (rcnt && rl == 0 && rid == a) {
-                                rcnt += k == 2 ? 8 : 16;
-                            } else {
-                                finish();
-                                rid = a;
-                                rl = 0;
-                                rcnt = k == 2 ? 8 : 16;
-                            }
-                        } else {
-                            const uint32_t w4[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-                            for (int q = 0; q < 8; q++) H.add_int((w4[q >> 1] >> (16 * (q & 1))) & 0xffffu, 1u);
-                            if (k == 4) {
-                                const uint32_t x4[4] = {y.x, y.y, y.z, y.w};
-#pragma unroll
-                                for (int q = 0; q < 8; q++) H.add_int((x4[q >> 1] >> (16 * (q & 1))) & 0xffffu, 1u);
-                            }
-                        }
+                for (int r = 0; r < 2; r++) {
+                    if (x[r].x == kTileList) {
+                        const uint4* t = A.I.pool + x[r].y;
+                        for (uint32_t k = 0; k < x[r].z; k++) add_words(H, __ldg(t + k));
+                    } else if (x[r].y) {
+                        add_words(H, x[r]);
+                    } else if (x[r].x) {
+                        run_add(x[r].x & 0xffffu, x[r].x >> 16);
                     }
                 }
-                __syncwarp();
-                if (*Qu.count >= 32) drain<FP, AT>(A.P, H, Qu, false);
             }
-        };
-        if (__any_sync(0xffffffffu, wide)) run_units(std::integral_constant<int, 1>{});
-        else run_units(std::integral_constant<int, RN>{});
+        }
+
+        // level-0 vectors
+        U.n = vecs ? ((D.hi + (1u << vlg) - 1) >> vlg) - (D.lo >> vlg) : 0u;
+        if (U.number(D, D.lo >> vlg << vlg, vlg, desc)) {
+            for (uint32_t u0 = 0; u0 < U.total; u0 += 32) {
+                const uint32_t u = u0 + lane;
+                const int j = U.block(u0);
+                if (u < U.total) {
+                    const Desc& d = desc[j];
+                    const uint32_t lg = (d.bits >> 10) & 7u, o = d.off + (u << lg);
+                    const uint4* p = reinterpret_cast<const uint4*>(
+                        d.addr + 2ull * item_at(o, d.bits, d.st1, d.st2));
+                    // IDs are read once: streaming loads (evict first) leave L2
+                    // to the records and table rows
+                    const uint4 x = __ldcs(p);
+                    uint4 y = x;
+                    if (lg == 4) y = __ldcs(p + 1);
+                    const uint32_t a = x.x & 0xffffu, pa = a * 0x10001u;
+                    const uint32_t m = (x.x ^ pa) | (x.y ^ pa) | (x.z ^ pa) | (x.w ^ pa) | (y.x ^ pa) | (y.y ^ pa) |
+                                       (y.z ^ pa) | (y.w ^ pa);
+                    const uint32_t k0 = d.lo > o ? d.lo - o : 0u, k1 = min(d.hi - o, 1u << lg);   // IDs of the span
+                    if (m == 0u) {
+                        run_add(a, k1 - k0);
+                    } else {
+                        // a segment boundary inside: each ID is added to its
+                        // bin at once, independent adds where a run would
+                        // chain them
+                        const uint32_t w[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+#pragma unroll
+                        for (uint32_t q = 0; q < 16; q++)
+                            if (q >= k0 && q < k1) H.add_int((w[q >> 1] >> (16 * (q & 1))) & 0xffffu, 1u);
+                    }
+                }
+            }
+        }
+
+        // single cubes, R in flight per lane
+        constexpr int R = 2;
+        U.n = use && !tiles && !vecs ? D.hi - D.lo : 0u;
+        if (U.number(D, D.lo, 0, desc)) {
+            for (uint32_t u0 = 0; u0 < U.total; u0 += 32 * R) {
+                uint32_t id[R], lv[R];
+#pragma unroll
+                for (int r = 0; r < R; r++) {
+                    const uint32_t u = u0 + 32 * r + lane;
+                    const int j = U.block(u0 + 32 * r);
+                    id[r] = kNone;
+                    lv[r] = 0;
+                    if (u < U.total) {
+                        const Desc& d = desc[j];
+                        const uint32_t idx = item_at(d.off + u, d.bits, d.st1, d.st2);
+                        lv[r] = d.bits >> 13;
+                        id[r] = lv[r] == 0 && id16 ? (uint32_t)__ldcs(reinterpret_cast<const uint16_t*>(d.addr) + idx)
+                                                   : __ldcs(reinterpret_cast<const uint32_t*>(d.addr) + idx);
+                    }
+                }
+                if constexpr (REC) {
+                    uint4 rec[R];
+#pragma unroll
+                    for (int r = 0; r < R; r++) {
+                        rec[r] = make_uint4(0u, 0u, 0u, 0u);
+                        if (id[r] >= S && id[r] != kNone) rec[r] = __ldg(A.P.rec + id[r]);
+                    }
+#pragma unroll
+                    for (int r = 0; r < R; r++) {
+                        if (id[r] < S) run_add(id[r], 1u << (3 * lv[r]));
+                        else if (id[r] != kNone) add_record<FP, AT>(A.P, H, rec[r], id[r], lv[r]);
+                    }
+                } else {
+#pragma unroll
+                    for (int r = 0; r < R; r++) {
+                        const bool node = id[r] >= S && id[r] != kNone;
+                        if (id[r] < S) run_add(id[r], 1u << (3 * lv[r]));
+                        // one queue entry for the equal nodes of the step
+                        const unsigned peers =
+                            __match_any_sync(0xffffffffu, node ? (uint64_t)lv[r] << 32 | id[r] : ~0ull);
+                        if (node && lane == __ffs(peers) - 1) {
+                            const uint32_t W = (uint32_t)__popc(peers) << (3 * lv[r]);
+                            const uint32_t pos = atomicAdd(Qu.count, 1u);
+                            if (pos < Qu.cap) {
+                                Qu.n[pos] = id[r];
+                                Qu.w[pos] = W;
+                            } else {
+                                push_one<FP, AT>(A.P, H, id[r], W);
+                            }
+                        }
+                    }
+                    __syncwarp();
+                    if (*Qu.count >= 32) drain<FP, AT>(A.P, H, Qu, false);
+                }
+            }
+        }
         const uint32_t st31 = __shfl_sync(0xffffffffu, st, 31);
         if (bb + 31 >= b1 || st31 >= w1) break;
     }
-    finish();
+    if (rcnt) H.add_int(rid, rcnt);
     __syncwarp();
 }
 
 // Few segments: every warp owns a histogram in shared memory and takes whole
 // chunks from the global ticket, so warps never wait for each other.
 // Register budget by CTA size NT: 256 threads, at most 51 registers (5 CTAs
-// per SM): the loop is bound by load latency, and 40 resident warps per SM
-// beat 32 at 63 registers even with a few spilled values (0.40 vs 0.42 ms on
-// the 10,000-box batch).  128 threads, at most 56 registers (9 CTAs): where
-// shared memory holds 9-10 CTAs of 4 warps anyway (1,182 segments), fewer
-// spills beat the tenth CTA (7.04 vs 7.25 ms on the 100,000-box batch; 64
-// registers and 8 CTAs: 7.41 ms).
+// per SM); 128 threads, at most 56 (9 CTAs).  The loop is bound by load
+// latency, so resident warps count; neither spills.
 template <int NT> struct WarpKernelBounds;
 template <> struct WarpKernelBounds<128> { static constexpr int min_ctas = 9; };
 template <> struct WarpKernelBounds<256> { static constexpr int min_ctas = 5; };
 
-template <bool FP, typename AT, int NT>
-__global__ void __launch_bounds__(NT, WarpKernelBounds<NT>::min_ctas) query_warp_kernel(MainArgs A) {
+template <bool FP, typename AT, int NT, bool REC>
+__global__ void __launch_bounds__(NT, WarpKernelBounds<NT>::min_ctas) query_warp_kernel(
+    const __grid_constant__ MainArgs A) {
     extern __shared__ __align__(16) uint8_t smem[];
     const uint32_t S = A.P.S;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t hist_bytes = (size_t)S * 4 * (FP ? 2 : 1);
-    uint8_t* mine = smem + warp * (hist_bytes + queue_bytes(A.qcap));
+    Desc* desc = reinterpret_cast<Desc*>(smem + warp * kDescBytes);
+    uint8_t* mine = smem + (blockDim.x >> 5) * kDescBytes + warp * (hist_bytes + (REC ? 0 : queue_bytes(A.qcap)));
     Hist<FP> H;
     H.h = reinterpret_cast<uint32_t*>(mine);
     H.hf = FP ? reinterpret_cast<float*>(H.h + S) : nullptr;
@@ -1374,7 +1531,8 @@ __global__ void __launch_bounds__(NT, WarpKernelBounds<NT>::min_ctas) query_warp
         H.h[i] = 0;
         if constexpr (FP) H.hf[i] = 0.f;
     }
-    clear_queue(Qu);
+    if constexpr (!REC) clear_queue(Qu);
+    __syncwarp();
     grid_dependency_wait();
     uint32_t* acc;
     float* accf;
@@ -1389,8 +1547,8 @@ __global__ void __launch_bounds__(NT, WarpKernelBounds<NT>::min_ctas) query_warp
         const uint32_t ncube = (uint32_t)A.ncube[q];
         const uint32_t c0 = (uint32_t)(c - A.chunk_off[q]) * A.chunk;
         const uint32_t c1 = min(c0 + A.chunk, ncube);
-        process_span<FP, AT, 2>(A, H, Qu, c0, c1, __ldg(A.chunk_b + c), A.blk_off[q + 1], ncube);
-        drain<FP, AT>(A.P, H, Qu, true);
+        process_span<FP, AT, REC>(A, H, Qu, desc, c0, c1, __ldg(A.chunk_b + c), A.blk_off[q + 1], ncube);
+        if constexpr (!REC) drain<FP, AT>(A.P, H, Qu, true);
         for (uint32_t s = lane; s < S; s += 32) {
             const uint32_t v = H.h[s];
             if (v) {
@@ -1411,16 +1569,17 @@ __global__ void __launch_bounds__(NT, WarpKernelBounds<NT>::min_ctas) query_warp
 
 // Many segments: one histogram per CTA; the CTA takes a chunk and its warps
 // take sub-spans of it (about two each) from a shared counter.
-template <bool FP, typename AT>
-__global__ void __launch_bounds__(512) query_batched_kernel(MainArgs A) {
+template <bool FP, typename AT, bool REC>
+__global__ void __launch_bounds__(512, 2) query_batched_kernel(const __grid_constant__ MainArgs A) {
     extern __shared__ __align__(16) uint8_t smem[];
     __shared__ uint32_t s_ntouched;
     __shared__ unsigned long long s_chunk;
     __shared__ uint32_t s_q;
     __shared__ uint32_t s_next;
     const uint32_t S = A.P.S;
-    const Hist<FP> H = carve<FP>(smem, S, &s_ntouched);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    Desc* desc = reinterpret_cast<Desc*>(smem + warp * kDescBytes);
+    const Hist<FP> H = carve<FP>(smem + nw * kDescBytes, S, &s_ntouched);
     // per-warp queues follow the touched list
     const size_t touched_bytes = (size_t)S * 2 * (FP ? 2 : 1);
     uint8_t* qbase = reinterpret_cast<uint8_t*>(H.touched) + ((touched_bytes + 15) & ~(size_t)15);
@@ -1430,7 +1589,7 @@ __global__ void __launch_bounds__(512) query_batched_kernel(MainArgs A) {
         if constexpr (FP) H.hf[i] = 0.f;
     }
     if (threadIdx.x == 0) s_ntouched = 0;
-    clear_queue(Qu);
+    if constexpr (!REC) clear_queue(Qu);
     grid_dependency_wait();
     uint32_t* acc;
     float* accf;
@@ -1472,9 +1631,9 @@ __global__ void __launch_bounds__(512) query_batched_kernel(MainArgs A) {
             }
             b = __shfl_sync(0xffffffffu, b, 0);
             bhint = b;
-            process_span<FP, AT, 4>(A, H, Qu, w0, w1, b, b1, ncube);
+            process_span<FP, AT, REC>(A, H, Qu, desc, w0, w1, b, b1, ncube);
         }
-        drain<FP, AT>(A.P, H, Qu, true);
+        if constexpr (!REC) drain<FP, AT>(A.P, H, Qu, true);
         __syncthreads();
         flush<FP>(H, S, q, acc, accf);
         __syncthreads();
@@ -1519,7 +1678,7 @@ __global__ void __launch_bounds__(256) query_plain_kernel(MainArgs A, const int3
                 const uint32_t n = block_cubes(R.lx[i], R.ly[j], R.lz[k]);
                 const uint64_t lo = max(start, c0), hi = min(start + n, c1);
                 if (lo < hi) {
-                    const Blk B = make_blk(A.G, 0, R.sx[i], R.sy[j], R.sz[k], R.lx[i], R.ly[j], R.lz[k]);
+                    const Blk B = make_blk(A.G, 0, R.sx[i], R.sy[j], R.sz[k], R.lx[i], R.ly[j], R.lz[k], 0);
                     for (uint64_t base = lo - start; base < hi - start; base += blockDim.x) {
                         const uint32_t o = (uint32_t)base + threadIdx.x;
                         const bool valid = o < hi - start;
@@ -1876,6 +2035,22 @@ int sm_count(int dev) {
     return cache[dev] ? cache[dev] : 1;
 }
 
+// Items per work chunk of an untuned batch of Q boxes.  A small batch is bound
+// by the latency of the longest chunk (one warp walks it alone), so its chunks
+// shrink until the batch holds a few per resident warp.  Histogram kernel, us
+// at 128 / 256 / 512 / 1,024 / 2,048 items a chunk: 1,000 boxes of a 64^3
+// volume 16 / 18 / 24 / 35 / 46; 777 of a 251x187x113 volume 20 / 24 / 28 / 37
+// / 61; 2,000 with 16-bit weights on 512x512x384 - / 120 / 106 / 118 / 151;
+// 10,000 there 205 / 135 / 104 / 104 / 121; 100,000 on 2048x2048x300 - / - /
+// 1580 / 1290 / 1120.  Below 128 the per-chunk flush outweighs it.  A histogram
+// shared by a CTA (many segments) has 16 warps on a chunk already.
+constexpr uint32_t kDefaultChunk = 2048, kMinChunk = 128;
+uint32_t default_chunk(uint32_t S, int64_t Q) {
+    uint32_t c = kDefaultChunk;
+    while (S <= kWarpHistMax && c > kMinChunk && (int64_t)c > Q * 2 / 7) c /= 2;
+    return c;
+}
+
 template <typename K>
 mg_status prepare_kernel(K kernel, size_t smem) {
     MG_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -1919,7 +2094,7 @@ mg_status launch_main(const mg_graph* g, const MainArgs& A, const mg_query_opts&
         Buf cubes;
         MG_TRY(cubes.alloc(scratch, (size_t)A.Q * 8, s));
         plan_count_kernel<<<grid_for(A.Q * 32, kPlanThreads), kPlanThreads, 0, s>>>(
-            A.G, boxes, A.Q, 1, nullptr, cubes.as<uint64_t>(), nullptr, A.P.status, Lim{nullptr, 0, 0});
+            A.G, boxes, A.Q, 1, nullptr, cubes.as<uint64_t>(), nullptr, A.P.status, Lim{nullptr, 0, 0}, false);
         MG_CUDA(cudaGetLastError());
         std::vector<uint64_t> nc((size_t)A.Q);
         MG_CUDA(cudaMemcpyAsync(nc.data(), cubes.p, (size_t)A.Q * 8, cudaMemcpyDeviceToHost, s));
@@ -1937,18 +2112,29 @@ mg_status launch_main(const mg_graph* g, const MainArgs& A, const mg_query_opts&
         return MG_OK;
     }
     // few segments: a private histogram per warp; else one per CTA (smem
-    // is then the histogram's part, the warps' queues come on top)
-    const int warps = threads / 32;
+    // is then the histogram's part); the warps' block descriptors and, without
+    // node records, their queues come on top
+    int warps = threads / 32;
     const size_t hist_w = (size_t)g->S * 4 * (FP ? 2 : 1);
+    const bool rec = A.P.rec != nullptr;
     const bool warp_mode =
         g->S <= kWarpHistMax && threads <= 256 && (hist_w + queue_bytes(kQueueShort)) * warps <= 96 * 1024;
-    auto k = !warp_mode ? query_batched_kernel<FP, AT>
-             : threads <= 128 ? query_warp_kernel<FP, AT, 128> : query_warp_kernel<FP, AT, 256>;
+    auto k = !warp_mode       ? (rec ? query_batched_kernel<FP, AT, true> : query_batched_kernel<FP, AT, false>)
+             : threads <= 128 ? (rec ? query_warp_kernel<FP, AT, 128, true> : query_warp_kernel<FP, AT, 128, false>)
+                              : (rec ? query_warp_kernel<FP, AT, 256, true> : query_warp_kernel<FP, AT, 256, false>);
     auto smem_for = [&](uint32_t cap) {
-        return warp_mode ? (hist_w + queue_bytes(cap)) * warps : smem + warps * queue_bytes(cap);
+        const size_t each = kDescBytes + (rec ? 0 : queue_bytes(cap));
+        return warp_mode ? (hist_w + each) * warps : smem + warps * each;
     };
     int per_sm = 0, per_long = 0;
-    if (smem_for(kQueueShort) > kMaxDynSmem) return fail(MG_ERR_UNSUPPORTED, "query kernel does not fit on an SM");
+    if (!warp_mode) {
+        // the shape asked for has to fit with its queues alone; the descriptors
+        // of the last few segment counts that do take fewer warps
+        if (smem + warps * queue_bytes(kQueueShort) > kMaxDynSmem)
+            return fail(MG_ERR_UNSUPPORTED, "query kernel does not fit on an SM");
+        while (warps > 1 && smem_for(kQueueShort) > kMaxDynSmem) warps /= 2;
+        threads = warps * 32;
+    }
     MG_TRY(prepare_kernel(k, smem_for(kQueueShort)));
     MG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem_for(kQueueShort)));
     if (per_sm < 1) return fail(MG_ERR_UNSUPPORTED, "query kernel does not fit on an SM");
@@ -2026,7 +2212,7 @@ __global__ void __launch_bounds__(256) query_lut_kernel(Geom G, Ids I, const int
         };
         for (int bi = warp; bi < nb; bi += nwarps) {
             const int i = bi % R.nx, j = (bi / R.nx) % R.ny, k = bi / (R.nx * R.ny);
-            const Blk B = make_blk(G, 0, R.sx[i], R.sy[j], R.sz[k], R.lx[i], R.ly[j], R.lz[k]);
+            const Blk B = make_blk(G, 0, R.sx[i], R.sy[j], R.sz[k], R.lx[i], R.ly[j], R.lz[k], 0);
             const uint32_t n = block_cubes(R.lx[i], R.ly[j], R.lz[k]);
             const uint32_t per = (n + 31) / 32, o0 = min(n, lane * per), o1 = min(n, o0 + per);
             for (uint32_t o = o0; o < o1; o++) {
@@ -2059,7 +2245,7 @@ mg_status query_lut(const mg_graph* g, const int32_t* boxes, int64_t Q, double* 
     if (sm > 200 * 1024) return fail(MG_ERR_UNSUPPORTED, "too many segments for the shared fp64 accumulators");
     if (Q == 0) return MG_OK;
     MG_CUDA(cudaFuncSetAttribute(query_lut_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    query_lut_kernel<<<(unsigned)Q, 256, sm, s>>>(make_geom(g), make_ids(g), boxes, g->err_off.as<uint64_t>(),
+    query_lut_kernel<<<(unsigned)Q, 256, sm, s>>>(make_geom(g, 0), make_ids(g), boxes, g->err_off.as<uint64_t>(),
                                                    g->err_src.as<uint32_t>(), g->err_mu.as<double>(),
                                                    g->err_dmu.as<double>(), hist, err, g->status.as<unsigned>());
     MG_CUDA(cudaGetLastError());
@@ -2067,9 +2253,9 @@ mg_status query_lut(const mg_graph* g, const int32_t* boxes, int64_t Q, double* 
 }
 
 mg_status count_cubes(const mg_graph* g, const int32_t* boxes, int64_t Q, uint64_t* cubes, cudaStream_t s) {
-    const Geom G = make_geom(g);
+    const Geom G = make_geom(g, 0);
     plan_count_kernel<<<grid_for(Q * 32, kPlanThreads), kPlanThreads, 0, s>>>(G, boxes, Q, 1, nullptr, cubes, nullptr,
-                                                            g->status.as<unsigned>(), Lim{nullptr, 0, 0});
+                                                            g->status.as<unsigned>(), Lim{nullptr, 0, 0}, false);
     MG_CUDA(cudaGetLastError());
     return MG_OK;
 }
@@ -2090,11 +2276,18 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
         if (csr) MG_CUDA(cudaMemsetAsync(offsets, 0, sizeof(uint64_t), s));
         return MG_OK;
     }
-    if (FP && o.alpha_dtype != MG_F32) MG_TRY(ensure_alpha16(const_cast<mg_graph*>(g), (mg_dtype)o.alpha_dtype, s));
+    if (FP && o.alpha_dtype != MG_F32) {
+        MG_TRY(ensure_alpha16(const_cast<mg_graph*>(g), (mg_dtype)o.alpha_dtype, s));
+        MG_TRY(ensure_records16(const_cast<mg_graph*>(g), (mg_dtype)o.alpha_dtype, s));
+    }
     const int tuned_c = g->tuned_chunk[FP ? 1 : 0], tuned_t = g->tuned_threads[FP ? 1 : 0];
-    const uint32_t chunk = o.chunk_cubes > 0 ? (uint32_t)o.chunk_cubes : tuned_c > 0 ? (uint32_t)tuned_c : 2048u;
+    // a fixed pool keeps the long chunks: its room is counted in them
+    const uint32_t chunk = o.chunk_cubes > 0 ? (uint32_t)o.chunk_cubes
+                           : tuned_c > 0     ? (uint32_t)tuned_c
+                           : room            ? kDefaultChunk
+                                             : default_chunk(S, Q);
     const int threads = o.block_threads > 0 ? o.block_threads : tuned_t > 0 ? tuned_t : 256;
-    const Geom G = make_geom(g);
+    const Geom G = make_geom(g, tile_levels(g, (mg_dtype)o.alpha_dtype));
     unsigned* status = g->status.as<unsigned>();
     mg_graph* gm = const_cast<mg_graph*>(g);
     const bool timed = o.timing != 0;
@@ -2125,6 +2318,7 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
         }
     }
 
+    const mg_dtype weights = (mg_dtype)o.alpha_dtype;
     MainArgs A;
     A.G = G;
     A.I = make_ids(g);
@@ -2132,6 +2326,9 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
     A.P.ab32 = g->ab32.as<uint2>();
     A.P.lut_meta = g->lut_meta.as<uint2>();
     A.P.lut = g->lut.as<uint2>();
+    const int w16 = weights == MG_BF16;
+    A.P.rec = weights == MG_F32 ? g->lut_rec.as<uint4>() : g->rec16[w16].as<uint4>();
+    A.P.frac = weights == MG_F32 ? nullptr : g->frac16[w16].as<float>();
     A.P.alpha = o.alpha_dtype == MG_F16 ? g->alpha16.p : o.alpha_dtype == MG_BF16 ? g->alphab16.p : g->alpha.p;
     A.P.S = S;
     A.P.status = status;
@@ -2164,7 +2361,7 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
         MG_TRY(ticket.alloc(&al, 8, s));
         plan_count_kernel<<<grid_for(Q * 32, kPlanThreads), kPlanThreads, 0, s>>>(G, boxes, Q, chunk, nblk.as<uint32_t>(),
                                                                 ncube.as<uint64_t>(), nchunk.as<uint64_t>(),
-                                                                status, Lim{nullptr, 0, 0});
+                                                                status, Lim{nullptr, 0, 0}, true);
         MG_CUDA(cudaGetLastError());
         if (Q <= kFusedScanMax) {
             plan_scan_kernel<<<1, kScanThreads, 0, s>>>(nblk.as<uint32_t>(), nchunk.as<uint64_t>(), Q,
@@ -2435,7 +2632,10 @@ mg_status plan_enqueue(mg_query_plan* p, const Alloc& al, cudaStream_t s) {
     const mg_graph* g = p->g;
     const int64_t Q = p->max_Q;
     const uint32_t S = g->S;
-    const Geom G = make_geom(g);
+    const mg_dtype weights = std::is_same<AT, __half>::value          ? MG_F16
+                             : std::is_same<AT, __nv_bfloat16>::value ? MG_BF16
+                                                                      : MG_F32;
+    const Geom G = make_geom(g, tile_levels(g, weights));
     unsigned* status = g->status.as<unsigned>();
     const Lim lim{p->Qd, p->cap_blocks, p->cap_chunks};
     Buf acc_b, ncube, blk_off, chunk_off, blk, chunk_q, chunk_b, tiles, ticket;
@@ -2488,6 +2688,9 @@ mg_status plan_enqueue(mg_query_plan* p, const Alloc& al, cudaStream_t s) {
     A.P.ab32 = g->ab32.as<uint2>();
     A.P.lut_meta = g->lut_meta.as<uint2>();
     A.P.lut = g->lut.as<uint2>();
+    const int w16 = weights == MG_BF16;
+    A.P.rec = weights == MG_F32 ? g->lut_rec.as<uint4>() : g->rec16[w16].as<uint4>();
+    A.P.frac = weights == MG_F32 ? nullptr : g->frac16[w16].as<float>();
     A.P.alpha = std::is_same<AT, __half>::value ? g->alpha16.p : std::is_same<AT, __nv_bfloat16>::value ? g->alphab16.p
                                                                                                           : g->alpha.p;
     A.P.S = S;
@@ -2524,6 +2727,16 @@ mg_status plan_enqueue(mg_query_plan* p, const Alloc& al, cudaStream_t s) {
 }  // namespace mg
 
 namespace mg {
+PlanChunk plan_chunk(const mg_graph* g, int hist_type, int chunk_cubes, int64_t max_Q, uint64_t cap_chunks) {
+    const int tuned = g->tuned_chunk[hist_type == MG_HIST_F32];
+    if (chunk_cubes > 0) return PlanChunk{(uint32_t)chunk_cubes, 1};
+    if (tuned > 0) return PlanChunk{(uint32_t)tuned, 1};
+    const uint32_t c = default_chunk(g->S, max_Q), scale = kDefaultChunk / c;
+    // the map of the shorter chunks, 8 bytes each, stays within 64 MiB
+    if (cap_chunks * scale > (1u << 23)) return PlanChunk{kDefaultChunk, 1};
+    return PlanChunk{c, scale};
+}
+
 PlanParts plan_parts(const mg_query_plan* p) {
     return PlanParts{p->boxes, p->Qd, p->result, p->exec, p->chunk, p->cap_blocks, p->cap_chunks};
 }
@@ -2564,11 +2777,13 @@ MG_API mg_status mg_query_plan_create(mg_graph* g, int64_t max_Q, const mg_query
         p->g = g;
         p->max_Q = max_Q;
         p->fp = FP;
-        const int tc = g->tuned_chunk[FP], tt = g->tuned_threads[FP];
-        p->chunk = o.chunk_cubes > 0 ? (uint32_t)o.chunk_cubes : tc > 0 ? (uint32_t)tc : 2048u;
+        const int tt = g->tuned_threads[FP];
         p->threads = o.block_threads > 0 ? o.block_threads : tt > 0 ? tt : 256;
         p->cap_blocks = max_blocks > 0 ? (uint64_t)max_blocks : (uint64_t)max_Q * 1024;
         p->cap_chunks = max_chunks > 0 ? (uint64_t)max_chunks : (uint64_t)max_Q * 256;
+        const PlanChunk pc = plan_chunk(g, o.hist_type, o.chunk_cubes, max_Q, p->cap_chunks);
+        p->chunk = pc.chunk;
+        p->cap_chunks *= pc.scale;
         if (p->cap_blocks >= (1ull << 32) || p->cap_chunks >= (1ull << 32))
             st = fail(MG_ERR_UNSUPPORTED, "plan capacities must be below 2^32");
     }
@@ -2599,6 +2814,7 @@ MG_API mg_status mg_query_plan_create(mg_graph* g, int64_t max_Q, const mg_query
         }
     }
     if (st == MG_OK && p->fp && o.alpha_dtype != MG_F32) st = ensure_alpha16(g, (mg_dtype)o.alpha_dtype, nullptr);
+    if (st == MG_OK && p->fp && o.alpha_dtype != MG_F32) st = ensure_records16(g, (mg_dtype)o.alpha_dtype, nullptr);
     if (st == MG_OK) {
         cudaError_t e = cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking);
         if (e != cudaSuccess) st = cuda_fail(e, "cudaStreamCreateWithFlags");
