@@ -100,8 +100,8 @@ void arena_free(void* ctx, void* p, size_t bytes, mg_stream s) {
 }
 }  // namespace
 
-mg_status arena_begin(mg_graph* g, cudaStream_t s, Arena** out) {
-    std::lock_guard<std::mutex> lk(g->arena_mu);
+// the arena of a stream, made on first use (arena_mu held)
+static mg_status arena_of(mg_graph* g, cudaStream_t s, Arena** out) {
     auto& slot = g->arenas[s];
     if (!slot) {
         slot.reset(new (std::nothrow) Arena());
@@ -116,7 +116,31 @@ mg_status arena_begin(mg_graph* g, cudaStream_t s, Arena** out) {
             slot->pinned = nullptr;
         }
     }
-    Arena* a = slot.get();
+    *out = slot.get();
+    return MG_OK;
+}
+
+mg_status prop_sync_words(mg_graph* g, cudaStream_t s, int words, unsigned** out) {
+    std::lock_guard<std::mutex> lk(g->arena_mu);
+    Arena* a = nullptr;
+    MG_TRY(arena_of(g, s, &a));
+    if (!a->sync.p) MG_TRY(a->sync.alloc(&g->al, (size_t)words * sizeof(unsigned), s));
+    // a captured launch zeroes them itself: the graph may run before or after
+    // any other launch on the stream
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    MG_CUDA(cudaStreamIsCapturing(s, &cap));
+    if (cap != cudaStreamCaptureStatusNone || !a->sync_zero) {
+        MG_CUDA(cudaMemsetAsync(a->sync.p, 0, (size_t)words * sizeof(unsigned), s));
+        a->sync_zero = cap == cudaStreamCaptureStatusNone;
+    }
+    *out = a->sync.as<unsigned>();
+    return MG_OK;
+}
+
+mg_status arena_begin(mg_graph* g, cudaStream_t s, Arena** out) {
+    std::lock_guard<std::mutex> lk(g->arena_mu);
+    Arena* a = nullptr;
+    MG_TRY(arena_of(g, s, &a));
     if (a->need > a->buf.bytes) {
         a->buf.release();   // stream-ordered after the previous call on s
         MG_TRY(a->buf.alloc(&g->al, a->need + a->need / 4, s));
@@ -130,7 +154,7 @@ void arena_drop(mg_graph* g, cudaStream_t s) {
     std::lock_guard<std::mutex> lk(g->arena_mu);
     auto it = g->arenas.find(s);
     if (it == g->arenas.end()) return;
-    it->second->buf.s = nullptr;   // the caller has synchronised the device
+    it->second->buf.s = it->second->sync.s = nullptr;   // the caller has synchronised the device
     g->arenas.erase(it);
 }
 
@@ -426,7 +450,7 @@ MG_API void mg_free(mg_graph* g) {
     if (!g) return;
     DeviceGuard dg(g->device);
     cudaDeviceSynchronize();
-    for (auto& kv : g->arenas) kv.second->buf.s = nullptr;   // the device is idle; the call streams may be gone
+    for (auto& kv : g->arenas) kv.second->buf.s = kv.second->sync.s = nullptr;   // the device is idle; the call streams may be gone
     delete g;
 }
 

@@ -104,6 +104,8 @@ struct Arena {
     const Alloc* fallback = nullptr;
     Alloc view;                  // an Alloc whose alloc/free go through this arena
     uint64_t* pinned = nullptr;  // 8 pinned host words for readbacks on this stream
+    Buf sync;                    // the propagation's ticket and counters, zero between launches
+    bool sync_zero = false;      // they have been zeroed once
     ~Arena() {
         if (pinned) cudaFreeHost(pinned);
     }
@@ -252,6 +254,9 @@ mg_status query_boxes(const mg_graph* g, const int32_t* boxes, int64_t Q, const 
 mg_status query_timing(const mg_graph* g, float* plan_ms, float* main_ms, float* out_ms);
 // the arena of `s` on graph g, reset for a new call (grown if the last call overflowed)
 mg_status arena_begin(mg_graph* g, cudaStream_t s, Arena** out);
+// the propagation's words of stream `s` (zeroed when first handed out; every
+// launch leaves them zero)
+mg_status prop_sync_words(mg_graph* g, cudaStream_t s, int words, unsigned** out);
 // release the arena of a stream that is about to be destroyed (device idle)
 void arena_drop(mg_graph* g, cudaStream_t s);
 mg_status count_cubes(const mg_graph* g, const int32_t* boxes, int64_t Q, uint64_t* cubes,

@@ -3,19 +3,32 @@
 // Sources take the TF row of their segment; then, level by level (nodes of a
 // level are contiguous and independent), every node lerps the rows of its two
 // predecessors:  v = v_p + alpha * (v_q - v_p), fp32.  Node records are SoA:
-// (p, q) as one 8-byte load, alpha as 4 (or 2) bytes; value rows are gathered
-// as one vector load per predecessor.
+// (p, q) as one 8-byte load, alpha as 4 (or 2) bytes.
 //
-// One persistent launch covers all levels: CTAs take tiles of nodes from a
-// global ticket in level order, and a tile of level d first waits until every
-// tile of level d-1 has signalled (a per-level counter).  Tiles are handed out
-// in order, so every tile waited on belongs to a CTA that is already running:
-// the wait always ends.  It is bounded all the same; past the bound the
-// kernel records MG_ERR_TIMEOUT and returns.  Rows written in this launch are
-// read through L2 (ld.global.cg), never through the read-only cache.
+// An item is one vector (16 or 8 bytes) of one node's row, so neighbouring
+// threads read and write whole rows however long they are (a thread per row
+// took one 16-byte piece of 32 different rows per load: 8 RGBA TFs of a
+// 217,000-node graph 104 -> 29 us).
+//
+// One persistent launch covers all levels: CTAs take tiles of items from a
+// global ticket in level order, and a tile first waits until every tile of the
+// wave before it has signalled (a counter per wave).  Tiles are handed out in
+// order, so every tile waited on belongs to a CTA that is already running: the
+// wait always ends.  It is bounded all the same; past the bound the kernel
+// records MG_ERR_TIMEOUT and returns.  Waves: the sources and, for fp32 RGBA,
+// level 1, whose nodes read the transfer function itself, so that the largest
+// level waits for nothing; then one level each; the last levels, a few nodes
+// each, are one tile, whose CTA walks them with no hand-off but its own barrier.
+//
+// Rows are gathered through L1 (nodes of a level are ordered by predecessor, so
+// neighbours share rows): a CTA has acquired a wave's counter before it reads
+// the wave's rows, which orders its plain loads after the stores and drops
+// older lines.  The read-only path (ld.global.nc) is for the node table only.
 #include "mg_internal.cuh"
 
 #include <algorithm>
+#include <atomic>
+#include <type_traits>
 
 namespace mg {
 namespace {
@@ -34,97 +47,42 @@ template <> struct Cvt<__nv_bfloat16> {
     static __device__ __forceinline__ __nv_bfloat16 from(float x) { return __float2bfloat16_rn(x); }
 };
 
-// load / store one row of C values: as 16-byte vectors when the row is a
-// multiple of 16 bytes, 8-byte ones when it is a multiple of 8, else element
-// by element.  kL2 loads go through L2 only (rows written earlier in the same
-// launch are never read through the read-only cache).
-template <bool kL2, typename V>
-__device__ __forceinline__ V ld_vec(const V* p) {
-    if constexpr (kL2) return __ldcg(p);
-    else return __ldg(p);
-}
-
-template <typename ST, int C, bool kL2>
-__device__ __forceinline__ void load_row_t(const ST* __restrict__ base, int64_t row, float (&v)[C]) {
-    const ST* r = base + row * C;
-    constexpr int B = (int)sizeof(ST) * C;
-    if constexpr (B % 16 == 0) {
-        constexpr int E = 16 / (int)sizeof(ST);
+// One vector of E consecutive channels of a row, held as it is stored until
+// the lerp: 16 or 8 bytes, or E elements where their size is neither.
+template <typename ST, int E, int B = (int)sizeof(ST) * E> struct Vec {
+    ST e[E];
+    __device__ __forceinline__ void load(const ST* p) {
 #pragma unroll
-        for (int w = 0; w < B / 16; w++) {
-            const uint4 u = ld_vec<kL2>(reinterpret_cast<const uint4*>(r) + w);
-            const ST* e = reinterpret_cast<const ST*>(&u);
-#pragma unroll
-            for (int c = 0; c < E; c++) v[w * E + c] = Cvt<ST>::to(e[c]);
-        }
-    } else if constexpr (B % 8 == 0) {
-        constexpr int E = 8 / (int)sizeof(ST);
-#pragma unroll
-        for (int w = 0; w < B / 8; w++) {
-            const uint2 u = ld_vec<kL2>(reinterpret_cast<const uint2*>(r) + w);
-            const ST* e = reinterpret_cast<const ST*>(&u);
-#pragma unroll
-            for (int c = 0; c < E; c++) v[w * E + c] = Cvt<ST>::to(e[c]);
-        }
-    } else if constexpr (sizeof(ST) == 4) {
-#pragma unroll
-        for (int c = 0; c < C; c++) v[c] = ld_vec<kL2>(reinterpret_cast<const float*>(r) + c);
-    } else {
-#pragma unroll
-        for (int c = 0; c < C; c++) {
-            const unsigned short u = ld_vec<kL2>(reinterpret_cast<const unsigned short*>(r) + c);
-            v[c] = Cvt<ST>::to(*reinterpret_cast<const ST*>(&u));
-        }
+        for (int c = 0; c < E; c++) e[c] = p[c];
     }
-}
-
-template <typename ST, int C>
-__device__ __forceinline__ void load_row(const ST* __restrict__ base, int64_t row, float (&v)[C]) {
-    load_row_t<ST, C, false>(base, row, v);
-}
-
-template <typename ST, int C>
-__device__ __forceinline__ void load_row_cg(const ST* __restrict__ base, int64_t row, float (&v)[C]) {
-    load_row_t<ST, C, true>(base, row, v);
-}
-
-template <typename ST, int C>
-__device__ __forceinline__ void store_row(ST* __restrict__ base, int64_t row, const float (&v)[C]) {
-    ST* r = base + row * C;
-    constexpr int B = (int)sizeof(ST) * C;
-    if constexpr (B % 16 == 0 || B % 8 == 0) {
-        constexpr int VB = B % 16 == 0 ? 16 : 8;
-        constexpr int E = VB / (int)sizeof(ST);
+    __device__ __forceinline__ void store(ST* p) const {
 #pragma unroll
-        for (int w = 0; w < B / VB; w++) {
-            ST e[E];
-#pragma unroll
-            for (int c = 0; c < E; c++) e[c] = Cvt<ST>::from(v[w * E + c]);
-            if constexpr (VB == 16)
-                reinterpret_cast<uint4*>(r)[w] = *reinterpret_cast<const uint4*>(e);
-            else
-                reinterpret_cast<uint2*>(r)[w] = *reinterpret_cast<const uint2*>(e);
-        }
-    } else {
-#pragma unroll
-        for (int c = 0; c < C; c++) r[c] = Cvt<ST>::from(v[c]);
+        for (int c = 0; c < E; c++) p[c] = e[c];
     }
-}
+    __device__ __forceinline__ float get(int c) const { return Cvt<ST>::to(e[c]); }
+    __device__ __forceinline__ void set(int c, float x) { e[c] = Cvt<ST>::from(x); }
+};
+template <typename ST, int E, typename W> struct WideVec {
+    union {
+        W w;
+        ST e[E];
+    };
+    __device__ __forceinline__ WideVec() {}
+    __device__ __forceinline__ void load(const ST* p) { w = *reinterpret_cast<const W*>(p); }
+    __device__ __forceinline__ void store(ST* p) const { *reinterpret_cast<W*>(p) = w; }
+    __device__ __forceinline__ float get(int c) const { return Cvt<ST>::to(e[c]); }
+    __device__ __forceinline__ void set(int c, float x) { e[c] = Cvt<ST>::from(x); }
+};
+template <typename ST, int E> struct Vec<ST, E, 16> : WideVec<ST, E, uint4> {};
+template <typename ST, int E> struct Vec<ST, E, 8> : WideVec<ST, E, uint2> {};
 
-// channel c of source n: k transfer functions of cin channels each, TF j at
-// tf + j * S * cin (k = 1: the row-major S x C table)
-__device__ __forceinline__ float tf_value(const float* __restrict__ tf, int64_t n, int c, int cin, int64_t tf_stride) {
-    return tf[(int64_t)(c / cin) * tf_stride + n * cin + (c % cin)];
-}
-
-template <typename ST, int C>
-__global__ void sources_kernel(const float* __restrict__ tf, uint32_t S, int cin, ST* __restrict__ vals) {
-    for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < S; s += (int64_t)gridDim.x * blockDim.x) {
-        float v[C];
+// v_p + alpha (v_q - v_p) in fp32, rounded to the storage type
+template <typename ST, int E>
+__device__ __forceinline__ Vec<ST, E> lerp_vec(const Vec<ST, E>& p, const Vec<ST, E>& q, float al) {
+    Vec<ST, E> out;
 #pragma unroll
-        for (int c = 0; c < C; c++) v[c] = tf_value(tf, s, c, cin, (int64_t)S * cin);
-        store_row<ST, C>(vals, s, v);
-    }
+    for (int c = 0; c < E; c++) out.set(c, fmaf(al, q.get(c) - p.get(c), p.get(c)));
+    return out;
 }
 
 // node weight: fp32 alpha, or a signed 16-bit alpha whose sign says p and q
@@ -136,166 +94,226 @@ template <> struct Weight<float> {
     using T = float;
 };
 
-template <typename ST, int C>
-__global__ void level_kernel(const uint2* __restrict__ pq, const typename Weight<ST>::T* __restrict__ alpha,
-                             int64_t lo, int64_t hi, ST* __restrict__ vals) {
-    const int64_t n = lo + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= hi) return;
-    const uint2 e = __ldg(pq + n);
-    uint32_t p = e.x, q = e.y;
-    float al = Cvt<typename Weight<ST>::T>::to(alpha[n]);
-    if (al < 0.f) {
-        al = -al;
-        const uint32_t t = p;
-        p = q;
-        q = t;
-    }
-    float vp[C], vq[C], out[C];
-    load_row<ST, C>(vals, p, vp);
-    load_row<ST, C>(vals, q, vq);
-#pragma unroll
-    for (int c = 0; c < C; c++) out[c] = fmaf(al, vq[c] - vp[c], vp[c]);
-    store_row<ST, C>(vals, n, out);
-}
-
 constexpr int kPropThreads = 256;
-constexpr int kPropTile = 1024;                 // nodes per tile
+constexpr int kPerThread = 2;                   // items of a tile per thread
+constexpr int kTileItems = kPropThreads * kPerThread;
+constexpr int kTailItems = 4 * kTileItems;      // levels up to this size may join the tail
 constexpr unsigned kSpinLimit = 1u << 22;       // polls before a wait gives up
 
-struct PropTiles {
-    int levels;                                 // D + 1, level 0 = the sources
-    int64_t tile0[MG_MAX_DEPTH + 2];            // first tile of every level (+ end)
-    int64_t first[MG_MAX_DEPTH + 1];            // first node of every level
-    int64_t count[MG_MAX_DEPTH + 1];            // nodes of every level
+// elements of an item and items of a row: the row as 16-byte vectors, else as
+// 8-byte ones, else whole
+template <typename ST, int C> struct RowShape {
+    static constexpr int B = (int)sizeof(ST) * C;
+    static constexpr int E = B % 16 == 0 ? 16 / (int)sizeof(ST) : B % 8 == 0 ? 8 / (int)sizeof(ST) : C;
+    static constexpr int items = C / E;
+    static constexpr int tile_nodes = kTileItems / items;
+    // resident CTAs: bound by load latency, as many as the registers allow
+    // without spills (11.8 M nodes, f32 / f16 x 4 TFs: 112 / 210 us with 4, 114 /
+    // 289 with 5, 118 / 202 with 3 of twice the items)
+    static constexpr int min_ctas = E <= 4 ? 5 : 4;
 };
 
-// level of tile t (tile0: first tile of every level)
-__device__ __forceinline__ int tile_level(const PropTiles& T, long long t) {
-    int d = 0;
-    while (t >= T.tile0[d + 1]) d++;
-    return d;
+// k transfer functions of cin channels each, TF j at tf + j * S * cin
+struct TfRows {
+    const float* tf;
+    int64_t stride;   // S * cin
+    int cin;
+};
+
+// segments of tiles in ticket order: the sources, the levels, the tail
+enum { kSources = 0, kFromTf = 1, kFromRows = 2, kTail = 3 };
+struct PropPlan {
+    int segs;
+    uint32_t tiles;
+    uint32_t tile0[MG_MAX_DEPTH + 2];           // first tile of every segment (+ end)
+    uint32_t first[MG_MAX_DEPTH + 1];           // first node
+    uint32_t count[MG_MAX_DEPTH + 1];           // nodes
+    int8_t kind[MG_MAX_DEPTH + 1];
+    int8_t wave[MG_MAX_DEPTH + 1];
+    uint32_t wave_tiles[MG_MAX_DEPTH + 1];      // tiles of every wave
+    int tail_first, tail_last;                  // levels of the tail
+    uint32_t bucket[MG_MAX_DEPTH + 2];
+};
+
+struct PropArgs {
+    const uint2* pq;
+    const void* alpha;
+    TfRows F;
+    void* vals;
+    unsigned* sync;        // words kLine apart: ticket, CTAs that have left, signalled tiles of every wave; zero between launches
+    unsigned* status;
+};
+// each word has a 128-byte line of its own: the polls of one wave's counter do
+// not meet the ticket's atomics
+constexpr int kLine = 32;
+constexpr int kSyncWords = (MG_MAX_DEPTH + 4) * kLine;
+
+// Poll *p (acquire) until it reaches `need`: at once for the first polls, then
+// with pauses; bounded like bounded_wait_geq.
+__device__ __forceinline__ bool wave_wait(const unsigned* p, unsigned need, unsigned* status) {
+    for (int i = 0; i < 32; i++)
+        if (ld_acquire_u32(p) >= need) return true;
+    return bounded_wait_geq(p, need, kSpinLimit, status);
 }
 
-// this thread's edges and weights of tile t: nodes lo + threadIdx.x + k * kPropThreads
-template <typename ST, int NT>
-__device__ __forceinline__ void tile_edges(const PropTiles& T, long long t, long long total,
-                                           const uint2* __restrict__ pq,
-                                           const typename Weight<ST>::T* __restrict__ alpha, uint2 (&e)[NT],
-                                           float (&al)[NT]) {
-#pragma unroll
-    for (int k = 0; k < NT; k++) {
-        e[k] = make_uint2(0u, 0u);
-        al[k] = 0.f;
-    }
-    if (t >= total) return;
-    const int d = tile_level(T, t);
-    if (d == 0) return;
-    const int64_t lo = T.first[d] + (t - T.tile0[d]) * kPropTile;
-    const int64_t hi = min(lo + kPropTile, T.first[d] + T.count[d]);
-#pragma unroll
-    for (int k = 0; k < NT; k++) {
-        const int64_t n = lo + threadIdx.x + (int64_t)k * kPropThreads;
-        if (n < hi) {
-            e[k] = __ldg(pq + n);
-            al[k] = Cvt<typename Weight<ST>::T>::to(alpha[n]);
-        }
-    }
-}
+// p and q in the order of the lerp (16-bit weights: sign = swapped)
+__device__ __forceinline__ uint2 lerp_order(uint2 e, float al) { return al < 0.f ? make_uint2(e.y, e.x) : e; }
 
 template <typename ST, int C>
-__global__ void __launch_bounds__(kPropThreads) single_pass_kernel(PropTiles T, const uint2* __restrict__ pq,
-                                                                   const typename Weight<ST>::T* __restrict__ alpha,
-                                                                   const float* __restrict__ tf, int cin,
-                                                                   ST* __restrict__ vals, unsigned* __restrict__ done,
-                                                                   unsigned long long* __restrict__ ticket,
-                                                                   unsigned* __restrict__ status) {
-    constexpr int NT = kPropTile / kPropThreads;      // nodes of a tile per thread
-    constexpr int NPT = C <= 4 ? 4 : C <= 8 ? 2 : 1;  // of them gathered at once
-    __shared__ long long s_next;
+__global__ void __launch_bounds__(kPropThreads, RowShape<ST, C>::min_ctas) propagate_kernel(const __grid_constant__ PropPlan T,
+                                                                 const __grid_constant__ PropArgs A) {
+    using R = RowShape<ST, C>;
+    using WT = typename Weight<ST>::T;
+    constexpr int E = R::E, I = R::items, TN = R::tile_nodes;
+    using V = Vec<ST, E>;
+    constexpr int NT = kPerThread;
+    __shared__ unsigned s_next[2];
     __shared__ int s_abort;
-    const long long total = T.tile0[T.levels];
+    ST* vals = static_cast<ST*>(A.vals);
+    const WT* __restrict__ alpha = static_cast<const WT*>(A.alpha);
+    unsigned* ticket = A.sync;
+    unsigned* done = A.sync + 2 * kLine;
+    const unsigned total = T.tiles;
     // thread 0 holds the ticket after next, taken two tiles ahead so that the
     // atomic's round trip is never waited on
-    long long ahead = 0;
-    int seen = 0;   // thread 0: every level below this one is known to be complete
+    unsigned ahead = 0;
+    int seen = 0;        // every wave below this one is known to be complete
+    int pending = -1;    // wave of the finished tile that is not yet signalled
+    unsigned turn = 0;
     if (threadIdx.x == 0) {
-        s_next = (long long)atomicAdd(ticket, 1ull);
-        ahead = (long long)atomicAdd(ticket, 1ull);
+        s_next[1] = atomicAdd(ticket, 1u);
+        ahead = atomicAdd(ticket, 1u);
+        s_abort = 0;
     }
     __syncthreads();
-    long long t = s_next;
+    unsigned t = s_next[1];
+    // thread 0, once every thread of the CTA has stored its part of the tile
+    auto signal = [&]() {
+        if (threadIdx.x == 0 && pending >= 0) {
+            __threadfence();
+            atomicAdd(done + pending * kLine, 1u);
+        }
+        pending = -1;
+    };
+    auto segment = [&](unsigned tile) {
+        int d = 0;
+        while (tile >= T.tile0[d + 1]) d++;
+        return d;
+    };
+    // item k of this thread in tile `tile` of segment d: node (past the end: none) and vector
+    auto item = [&](int d, unsigned tile, int k, uint32_t& n, int& ch) {
+        const uint32_t i = k * kPropThreads + threadIdx.x, r = i / I;
+        ch = (int)(i - r * I);
+        const uint32_t at = (tile - T.tile0[d]) * TN + r;
+        n = T.first[d] + at;
+        return r < TN && at < T.count[d];
+    };
+    auto edges = [&](unsigned tile, uint2 (&e)[NT], WT (&al)[NT]) {
+        const int d = tile < total ? segment(tile) : 0;
+        const bool live = tile < total && (T.kind[d] == kFromTf || T.kind[d] == kFromRows);
+#pragma unroll
+        for (int k = 0; k < NT; k++) {
+            uint32_t n;
+            int ch;
+            e[k] = make_uint2(0u, 0u);
+            al[k] = WT(0.f);
+            if (live && item(d, tile, k, n, ch)) {   // (nothing here waits for the loads)
+                e[k] = __ldg(A.pq + n);
+                al[k] = alpha[n];
+            }
+        }
+    };
     // Software pipeline over tiles: the next tile's ticket is known and its
     // (static) edges and weights are loaded while this tile waits and runs.
     // Tickets are taken in order and a tile only waits for smaller ones, so
     // the smallest unfinished ticket is always some CTA's current tile.
     uint2 e[NT];
-    float al[NT];
-    tile_edges<ST, NT>(T, t, total, pq, alpha, e, al);
+    WT al[NT];
+    edges(t, e, al);
     while (t < total) {
-        const int d = tile_level(T, t);
-        const int64_t lo = T.first[d] + (t - T.tile0[d]) * kPropTile;
-        const int64_t hi = min(lo + kPropTile, T.first[d] + T.count[d]);
-        __syncthreads();   // every thread has read s_next
-        if (threadIdx.x == 0) {
-            s_next = ahead;
-            ahead = (long long)atomicAdd(ticket, 1ull);
-            s_abort = 0;
-            if (d > seen) {   // level d-1 not yet seen complete
-                const unsigned need = (unsigned)(T.tile0[d] - T.tile0[d - 1]);
-                if (bounded_wait_geq(done + d - 1, need, kSpinLimit, status)) seen = d;
-                else s_abort = 1;
-            }
+        const int d = segment(t);
+        const int kind = T.kind[d], w = T.wave[d];
+        if (w > seen) {   // wave w - 1 not yet seen complete; it may lack this CTA's last tile
+            __syncthreads();
+            signal();
+            if (threadIdx.x == 0 && !wave_wait(done + (w - 1) * kLine, T.wave_tiles[w - 1], A.status)) s_abort = 1;
+            seen = w;
         }
+        if (threadIdx.x == 0) {
+            s_next[turn] = ahead;
+            ahead = atomicAdd(ticket, 1u);
+        }
+        // one barrier a tile: the last tile is stored, the next ticket known,
+        // the wave's rows acquired
         __syncthreads();
         if (s_abort) break;
-        const long long tn = s_next;
+        const unsigned tn = s_next[turn];
+        turn ^= 1u;
         uint2 en[NT];
-        float aln[NT];
-        tile_edges<ST, NT>(T, tn, total, pq, alpha, en, aln);
-        if (d == 0) {
-            for (int64_t n = lo + threadIdx.x; n < hi; n += kPropThreads) {
-                float out[C];
+        WT aln[NT];
+        edges(tn, en, aln);
+        if (kind == kSources) {
 #pragma unroll
-                for (int c = 0; c < C; c++) out[c] = tf_value(tf, n, c, cin, T.count[0] * cin);
-                store_row<ST, C>(vals, n, out);
+            for (int k = 0; k < NT; k++) {
+                uint32_t n;
+                int ch;
+                if (item(d, t, k, n, ch)) {
+                    V v;
+                    for (int c = 0; c < E; c++) {
+                        const int j = (ch * E + c) / A.F.cin;
+                        v.set(c, __ldg(A.F.tf + j * A.F.stride + (int64_t)n * A.F.cin + (ch * E + c - j * A.F.cin)));
+                    }
+                    v.store(vals + (int64_t)n * C + ch * E);
+                }
+            }
+        } else if (kind == kTail) {
+            signal();
+            for (int l = T.tail_first; l <= T.tail_last; l++) {
+                const uint32_t lo = T.bucket[l];
+                const int items = (int)(T.bucket[l + 1] - lo) * I;
+                for (int i = (int)threadIdx.x; i < items; i += kPropThreads) {
+                    const int r = i / I, ch = i - r * I;
+                    const float a = Cvt<WT>::to(alpha[lo + r]);
+                    const uint2 x = lerp_order(__ldg(A.pq + lo + r), a);
+                    V p, q;
+                    p.load(vals + (int64_t)x.x * C + ch * E);
+                    q.load(vals + (int64_t)x.y * C + ch * E);
+                    lerp_vec<ST, E>(p, q, fabsf(a)).store(vals + (int64_t)(lo + r) * C + ch * E);
+                }
+                __syncthreads();   // the next level reads these rows
             }
         } else {
-            // NPT nodes at a time: both predecessor rows of every node are
-            // loaded before any is stored (nodes of one level never read each other)
+            // both predecessor vectors of every item are loaded before any is
+            // stored (nodes of one level never read each other)
+            const ST* rows = vals;
+            int64_t pitch = C, tf_ch = E;   // elements between rows, and between a row's vectors
+            if (std::is_same<ST, float>::value && kind == kFromTf) {
+                rows = reinterpret_cast<const ST*>(A.F.tf);
+                pitch = E;
+                tf_ch = A.F.stride;
+            }
+            V p[NT], q[NT];   // (loaded before the last tile's signal, whose fence takes as long)
 #pragma unroll
-            for (int k0 = 0; k0 < NT; k0 += NPT) {
-                float vp[NPT][C], vq[NPT][C];
-#pragma unroll
-                for (int k = 0; k < NPT; k++) {
-                    const int64_t n = lo + threadIdx.x + (int64_t)(k0 + k) * kPropThreads;
-                    if (n < hi) {
-                        uint32_t p = e[k0 + k].x, q = e[k0 + k].y;
-                        if (al[k0 + k] < 0.f) {   // 16-bit weights: sign = p and q swapped
-                            p = e[k0 + k].y;
-                            q = e[k0 + k].x;
-                        }
-                        load_row_cg<ST, C>(vals, p, vp[k]);
-                        load_row_cg<ST, C>(vals, q, vq[k]);
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < NPT; k++) {
-                    const int64_t n = lo + threadIdx.x + (int64_t)(k0 + k) * kPropThreads;
-                    if (n < hi) {
-                        const float a = fabsf(al[k0 + k]);
-                        float out[C];
-#pragma unroll
-                        for (int c = 0; c < C; c++) out[c] = fmaf(a, vq[k][c] - vp[k][c], vp[k][c]);
-                        store_row<ST, C>(vals, n, out);
-                    }
+            for (int k = 0; k < NT; k++) {
+                uint32_t n;
+                int ch;
+                if (item(d, t, k, n, ch)) {
+                    const uint2 x = lerp_order(e[k], Cvt<WT>::to(al[k]));
+                    p[k].load(rows + (int64_t)x.x * pitch + ch * tf_ch);
+                    q[k].load(rows + (int64_t)x.y * pitch + ch * tf_ch);
                 }
             }
+            signal();
+#pragma unroll
+            for (int k = 0; k < NT; k++) {
+                uint32_t n;
+                int ch;
+                if (item(d, t, k, n, ch))
+                    lerp_vec<ST, E>(p[k], q[k], fabsf(Cvt<WT>::to(al[k]))).store(vals + (int64_t)n * C + ch * E);
+            }
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            atomicAdd(done + d, 1u);
-        }
+        signal();
+        pending = w;
         t = tn;
 #pragma unroll
         for (int k = 0; k < NT; k++) {
@@ -303,6 +321,18 @@ __global__ void __launch_bounds__(kPropThreads) single_pass_kernel(PropTiles T, 
             al[k] = aln[k];
         }
     }
+    __syncthreads();
+    signal();
+    // The last CTA to leave (no other reads or writes the words any more)
+    // zeroes them for the next launch on this stream.
+    __shared__ int s_last;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(A.sync + kLine, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (s_last)
+        for (int i = threadIdx.x; i < kSyncWords / kLine; i += kPropThreads) A.sync[i * kLine] = 0u;
 }
 
 __global__ void alpha16_kernel(const ulonglong2* __restrict__ ab, int64_t N, uint32_t S, int bf16,
@@ -344,51 +374,61 @@ int sm_count_prop(int dev) {
     return n > 0 ? n : 1;
 }
 
-template <typename ST, int C>
-mg_status run_single_pass(mg_graph* g, const float* tf, int cin, const void* alpha, ST* vals, cudaStream_t s) {
-    PropTiles T;
-    T.levels = g->D + 1;
-    int64_t tiles = 0;
-    for (int d = 0; d <= g->D; d++) {
-        T.tile0[d] = tiles;
-        T.first[d] = g->bucket[d];
-        T.count[d] = g->bucket[d + 1] - g->bucket[d];
-        tiles += (T.count[d] + kPropTile - 1) / kPropTile;
-    }
-    T.tile0[g->D + 1] = tiles;
-    Arena* arena = nullptr;
-    MG_TRY(arena_begin(g, s, &arena));
-    Buf sync;
-    MG_TRY(sync.alloc(&arena->view, (MG_MAX_DEPTH + 2) * sizeof(unsigned) + 16, s));
-    MG_CUDA(cudaMemsetAsync(sync.p, 0, (MG_MAX_DEPTH + 2) * sizeof(unsigned) + 16, s));
-    unsigned* done = sync.as<unsigned>();
-    auto* ticket = reinterpret_cast<unsigned long long*>(sync.as<unsigned char>() + (MG_MAX_DEPTH + 2) * sizeof(unsigned) +
-                                                        (8 - ((MG_MAX_DEPTH + 2) * sizeof(unsigned)) % 8) % 8);
-    using W = typename Weight<ST>::T;
-    auto k = single_pass_kernel<ST, C>;
-    int per_sm = 0;
-    MG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kPropThreads, 0));
-    const int64_t grid = std::min<int64_t>(tiles, (int64_t)std::max(per_sm, 1) * sm_count_prop(g->device));
-    k<<<(unsigned)std::max<int64_t>(grid, 1), kPropThreads, 0, s>>>(T, g->pq.as<uint2>(), static_cast<const W*>(alpha),
-                                                                    tf, cin, vals, done, ticket,
-                                                                    g->status.as<unsigned>());
-    MG_CUDA(cudaGetLastError());
-    return MG_OK;
-}
+bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
 template <typename ST, int C>
 mg_status run(mg_graph* g, const float* tf, int cin, const void* alpha, ST* vals, cudaStream_t s) {
-    if (g->D + 1 <= MG_MAX_DEPTH) return run_single_pass<ST, C>(g, tf, cin, alpha, vals, s);
-    sources_kernel<ST, C><<<grid_for(g->S, 256, 152 * 16), 256, 0, s>>>(tf, g->S, cin, vals);
-    MG_CUDA(cudaGetLastError());
-    using W = typename Weight<ST>::T;
-    for (int d = 1; d <= g->D; d++) {
-        const int64_t lo = g->bucket[d], hi = g->bucket[d + 1];
-        if (hi <= lo) continue;
-        level_kernel<ST, C><<<grid_for(hi - lo, 256), 256, 0, s>>>(g->pq.as<uint2>(), static_cast<const W*>(alpha),
-                                                                   lo, hi, vals);
-        MG_CUDA(cudaGetLastError());
+    using R = RowShape<ST, C>;
+    PropPlan T;
+    T.segs = 0;
+    T.tiles = 0;
+    int waves = 0;
+    auto add = [&](int kind, int wave, int64_t first, int64_t count, int64_t tiles) {
+        const int d = T.segs++;
+        T.kind[d] = (int8_t)kind;
+        T.wave[d] = (int8_t)wave;
+        T.first[d] = (uint32_t)first;
+        T.count[d] = (uint32_t)count;
+        T.tile0[d] = T.tiles;
+        T.tiles += (uint32_t)tiles;
+        if (wave == waves) T.wave_tiles[waves++] = 0;
+        T.wave_tiles[wave] += (uint32_t)tiles;
+    };
+    auto tiles_of = [](int64_t nodes) { return (nodes + R::tile_nodes - 1) / R::tile_nodes; };
+    // the levels after which none is larger than kTailItems
+    int tail = g->D + 1;
+    while (tail > 2 && (g->bucket[tail] - g->bucket[tail - 1]) * R::items <= kTailItems) tail--;
+    for (int d = 0; d <= g->D + 1; d++) T.bucket[d] = (uint32_t)g->bucket[d];
+    // level 1 from the transfer function: rows of four floats on 16 bytes, the
+    // vectors of a row one TF apart
+    const bool quad = std::is_same<ST, float>::value && R::E == 4 && cin == 4 && aligned(tf, 16);
+    for (int d = 0; d < tail && d <= g->D; d++) {
+        const int64_t n = g->bucket[d + 1] - g->bucket[d];
+        const bool from_tf = d == 1 && quad;
+        add(d == 0 ? kSources : from_tf ? kFromTf : kFromRows, from_tf ? 0 : d == 0 ? 0 : waves, g->bucket[d], n,
+            tiles_of(n));
     }
+    T.tail_first = tail;
+    T.tail_last = g->D;
+    if (tail <= g->D) add(kTail, waves, g->bucket[tail], g->bucket[g->D + 1] - g->bucket[tail], 1);
+    T.tile0[T.segs] = T.tiles;
+    PropArgs A;
+    A.pq = g->pq.as<uint2>();
+    A.alpha = alpha;
+    A.F = TfRows{tf, (int64_t)g->S * cin, cin};
+    A.vals = vals;
+    A.status = g->status.as<unsigned>();
+    MG_TRY(prop_sync_words(g, s, kSyncWords, &A.sync));
+    auto k = propagate_kernel<ST, C>;
+    static std::atomic<int> per_sm{0};   // of this kernel (one architecture)
+    int per = per_sm.load(std::memory_order_relaxed);
+    if (per == 0) {
+        MG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, kPropThreads, 0));
+        per_sm.store(std::max(per, 1), std::memory_order_relaxed);
+    }
+    const int64_t grid = std::min<int64_t>(T.tiles, (int64_t)std::max(per, 1) * sm_count_prop(g->device));
+    k<<<(unsigned)std::max<int64_t>(grid, 1), kPropThreads, 0, s>>>(T, A);
+    MG_CUDA(cudaGetLastError());
     return MG_OK;
 }
 
@@ -414,8 +454,6 @@ mg_status dispatch_c(mg_graph* g, const float* tf, int C, int cin, const void* a
     }
     return fail(MG_ERR_UNSUPPORTED, "channels per node (k * C) must be 1-8, 12, 16, 20, 24, 28 or 32");
 }
-
-bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
 }  // namespace
 
