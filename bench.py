@@ -61,7 +61,7 @@ def parse(argv=None):
     ap.add_argument("--threads", type=int, default=0)
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--no-cpu-baseline", action="store_true")
-    ap.add_argument("--no-plan", action="store_true", help="time direct calls instead of the captured plan")
+    ap.add_argument("--no-plan", action="store_true", help="time direct calls instead of the query plan")
     ap.add_argument("--no-forms", action="store_true", help="skip the plain/naive/16-bit extra measurements")
     ap.add_argument("--no-serve", action="store_true", help="skip the request-loop (serving mix) measurement")
     ap.add_argument("--no-large", action="store_true", help="skip the cylinder graph measurements")
@@ -418,9 +418,8 @@ def measure_step(mg, g, cfg_i, boxes_h, storage, args, dev, flush, stream, world
                       "propagate_alone": prop_alone, "propagate_with_tf_upload": prop_with_upload,
                       "lookup_alone": look_alone,
                       "note": "propagate/lookup run concurrently with the query; *_alone timed by themselves; "
-                              "query_plan = tile reset + fused plan kernel, query_main = histogram kernel (events "
-                              "in a timed copy of the plan's graph), query_rest = the rest of a batch (batch size "
-                              "and io slots, launch gaps)" if use_plan else
+                              "query_plan = fused plan kernel, query_main = histogram kernel (events of a timed "
+                              "plan's runs), query_rest = the rest of a batch (launch gaps)" if use_plan else
                               "propagate/lookup run concurrently with the query; *_alone timed by themselves; "
                               "query_rest includes the output stage"},
         "roofline_nominal": {"peak": NOMINAL_HBM_GBS, "unit": "GB/s", "frac": achieved / NOMINAL_HBM_GBS,
@@ -437,16 +436,15 @@ def measure_step(mg, g, cfg_i, boxes_h, storage, args, dev, flush, stream, world
                   "max_list": info["max_list"], "pairs": info["pairs"], "lut_entries": info["lut_entries"]},
         "e2e": e2e_rec,
         "autotune": tune,
-        "query_path": "captured plan (one CUDA graph launch per batch)" if use_plan else "direct calls",
+        "query_path": "query plan (two launches per batch)" if use_plan else "direct calls",
         "clocks": clk,
         "wall_s_timed": wall,
     }
-    # one persistent propagation launch (depth within the single pass), the lookup, and the query:
-    # batch size and io slots, tile reset, fused plan kernel, main kernel (plans)
-    launches_prop = 1 if info["depth"] + 1 <= 64 else 1 + sum(
-        1 for d in range(1, info["depth"] + 1) if info["bucket"][d + 1] > info["bucket"][d])
+    # one persistent propagation launch, the lookup, and the query: the fused plan kernel and the
+    # main kernel (plans)
+    launches_prop = 1
     if args.schedule == "batched" and use_plan:
-        launches_query = 4
+        launches_query = 2
     elif args.schedule == "batched":
         nscan = 1 if Q <= 2048 else 3
         launches_query = 1 + (1 if Q <= (1 << 18) else 2 * nscan + 1) + 1 + 1

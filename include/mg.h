@@ -247,19 +247,19 @@ MG_API mg_status mg_query_boxes_noalloc(const mg_graph *g, const int32_t *boxes,
 MG_API mg_status mg_query_timing(const mg_graph *g, float *plan_ms, float *main_ms, float *output_ms);
 
 /*
- * Query plans: the batched pipeline of mg_query_boxes for up to max_Q boxes,
- * captured once as a CUDA graph with every buffer preallocated, so that a run
- * is one small kernel (the batch size and the caller's buffers) and one graph
- * launch, with no copies and no host synchronisation.
+ * Query plans: the batched pipeline of mg_query_boxes for up to max_Q boxes
+ * with every buffer preallocated and the launch shape chosen once, so that a
+ * run is two launches (three for fp32 histograms), with no copies and no host
+ * synchronisation.
  * opts: dense layout and batched schedule only; hist_type, alpha_dtype and the
  *   launch shape (0 = the graph's tuned shape, else the defaults) as for
  *   mg_query_boxes.
  * max_blocks, max_chunks: footprint blocks and work chunks one run may need
  *   (0 = 1024 and 256 per box).  A run whose boxes need more writes zero
  *   histograms and sets MG_ERR_CAPACITY in the status word (mg_sync_status).
- * opts->timing set: the graph also records CUDA events around its plan stage
- *   (tile reset and the fused plan kernel) and its main kernel; read the
- *   durations of the last run with mg_query_plan_timing.
+ * opts->timing set: a run also records CUDA events around its plan stage (the
+ *   fused plan kernel) and its main kernel; read the durations of the last run
+ *   with mg_query_plan_timing.
  * The plan holds its memory (from the graph's allocator) until
  * mg_query_plan_free; runs of one plan share it, so runs of one plan on
  * different streams must not overlap.
@@ -268,7 +268,7 @@ typedef struct mg_query_plan mg_query_plan;
 MG_API mg_status mg_query_plan_create(mg_graph *g, int64_t max_Q, const mg_query_opts *opts, int64_t max_blocks,
                                       int64_t max_chunks, mg_query_plan **out);
 /* boxes: Q x 6 int32 (device), 0 <= Q <= max_Q; out: Q x S (uint32 or fp32),
- * both 4-byte aligned.  The graph reads `boxes` and writes `out` in the order
+ * both 4-byte aligned.  The run reads `boxes` and writes `out` in the order
  * of `stream`: they must stay valid until the run has completed on it. */
 MG_API mg_status mg_query_plan_run(mg_query_plan *p, const int32_t *boxes, int64_t Q, void *out, size_t out_capacity,
                                    mg_stream stream);

@@ -281,7 +281,7 @@ struct PlanParts {
     uint32_t chunk;
     uint64_t cap_blocks, cap_chunks;
 };
-PlanParts plan_parts(const mg_query_plan* p);
+mg_status plan_parts(mg_query_plan* p, PlanParts* out);
 // Work-chunk length of a plan, and the chunk-map entries it keeps per chunk of
 // the caller's capacity: an untuned plan for few boxes takes chunks `scale`
 // times shorter than the default, so that what fits the capacity in default

@@ -298,10 +298,9 @@ __device__ __forceinline__ uint64_t footprint_count(const Runs& R, uint32_t tile
     return n;
 }
 
-// Batch size and capacities read on the device, for query plans replayed as
-// CUDA graphs: the launches cover Q boxes, *Qd of them are live, and the
-// footprint must fit the plan's buffers.  Qd == nullptr: all Q are live and
-// the buffers were sized for this batch.
+// A batch planned by the fused kernel: the footprint must fit the buffers, and
+// the batch size is known (Qd == nullptr) or, for plans replayed as CUDA
+// graphs, read on the device: the launches then cover Q boxes, *Qd of them live.
 struct Lim {
     const int64_t* Qd;
     uint64_t cap_blocks, cap_chunks;
@@ -309,28 +308,15 @@ struct Lim {
 
 __device__ __forceinline__ int64_t live_q(const Lim& lim, int64_t Q) { return lim.Qd ? *lim.Qd : Q; }
 
-__device__ __forceinline__ bool over_cap(const Lim& lim, const uint64_t* blk_off, const uint64_t* chunk_off,
-                                         int64_t Qe) {
-    return lim.Qd && (blk_off[Qe] > lim.cap_blocks || chunk_off[Qe] > lim.cap_chunks);
-}
-
 // ---------------------------------------------------------------------------
 // plan
 // ---------------------------------------------------------------------------
 __global__ void plan_count_kernel(Geom G, const int32_t* __restrict__ boxes, int64_t Q, uint32_t chunk,
                                   uint32_t* __restrict__ nblk, uint64_t* __restrict__ ncube,
-                                  uint64_t* __restrict__ nchunk, unsigned* __restrict__ status, Lim lim, bool items) {
+                                  uint64_t* __restrict__ nchunk, unsigned* __restrict__ status, bool items) {
     const int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (q >= Q) return;
-    if (q >= live_q(lim, Q)) {
-        if (lane == 0) {
-            if (nblk) nblk[q] = 0;
-            ncube[q] = 0;
-            if (nchunk) nchunk[q] = 0;
-        }
-        return;
-    }
     int32_t b[6];
 #pragma unroll
     for (int k = 0; k < 6; k++) b[k] = boxes[q * 6 + k];
@@ -357,13 +343,12 @@ __global__ void plan_count_kernel(Geom G, const int32_t* __restrict__ boxes, int
 // Block records of every box, and for every work chunk of `chunk` cubes its
 // box and the block holding its first cube.
 __global__ void plan_write_kernel(Geom G, const int32_t* __restrict__ boxes, int64_t Q,
-                                  const uint64_t* __restrict__ blk_off, Blk* __restrict__ blk, Lim lim,
+                                  const uint64_t* __restrict__ blk_off, Blk* __restrict__ blk,
                                   const uint64_t* __restrict__ chunk_off, uint32_t chunk,
                                   uint32_t* __restrict__ chunk_q, uint32_t* __restrict__ chunk_b) {
     const int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    const int64_t Qe = live_q(lim, Q);
-    if (q >= Qe || over_cap(lim, blk_off, chunk_off, Qe)) return;
+    if (q >= Q) return;
     int32_t b[6];
 #pragma unroll
     for (int k = 0; k < 6; k++) b[k] = boxes[q * 6 + k];
@@ -416,7 +401,9 @@ __global__ void plan_write_kernel(Geom G, const int32_t* __restrict__ boxes, int
 // boxes in ticket order (tb chosen on the host so that the tiles of a full
 // batch fill the GPU once); a tile publishes its own totals, then sums its
 // predecessors' words backwards until it meets one that holds an inclusive
-// prefix, and publishes its own prefix.  Plans only (capacities in `lim`).
+// prefix, and publishes its own prefix.  The tile words and the ticket are zero
+// at launch: the main kernel, which starts reading once this one has ended,
+// zeroes them for the next batch.
 // ---------------------------------------------------------------------------
 constexpr int kTileMax = 64;                     // boxes per tile at most
 constexpr int kFusedThreads = 512;
@@ -437,15 +424,6 @@ int tile_boxes(int64_t Q, int sms) {
     return (int)std::min<int64_t>(kTileMax, std::max<int64_t>(1, (Q + slots - 1) / slots));
 }
 
-// zero the tile words of the live batch and both work tickets
-__global__ void plan_reset_kernel(const int64_t* __restrict__ Qd, int tb, uint64_t* __restrict__ tiles,
-                                  unsigned long long* __restrict__ tickets) {
-    const int64_t n = 2 * ((*Qd + tb - 1) / tb);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        tiles[i] = 0;
-    if (blockIdx.x == 0 && threadIdx.x < 2) tickets[threadIdx.x] = 0;
-}
-
 struct FusedOut {
     uint64_t* ncube;
     uint64_t* blk_off;
@@ -454,7 +432,7 @@ struct FusedOut {
     uint32_t* chunk_q;
     uint32_t* chunk_b;
     uint64_t* tiles;               // two words per tile: blocks, chunks
-    unsigned long long* ticket;    // tile order
+    unsigned long long* ticket;    // tile order; [1]: the main kernel's, zeroed here
     uint32_t* acc;                 // rows zeroed for the live batch
     float* accf;                   // likewise (fp32 histograms), or nullptr
     void* const* io;               // io[0]: the boxes; io[1]: the output (acc for u32, accf for fp32)
@@ -512,7 +490,10 @@ __global__ void __launch_bounds__(kFusedThreads, 2) plan_fused_kernel(const __gr
     __shared__ unsigned long long s_tile;
     __shared__ uint64_t s_pre_b, s_pre_c;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) s_tile = atomicAdd(F.ticket, 1ull);
+    if (threadIdx.x == 0) {
+        s_tile = gridDim.x == 1 ? 0ull : atomicAdd(F.ticket, 1ull);
+        if (s_tile == 0) F.ticket[1] = 0;
+    }
     // the main kernel may be scheduled once every tile has started; it waits
     // for this grid's completion before it reads anything written here
     grid_dependents_launch();
@@ -1049,7 +1030,10 @@ struct MainArgs {
     const uint32_t* chunk_q;     // box of every chunk
     const uint32_t* chunk_b;     // block holding every chunk's first cube
     unsigned long long total_chunks;
-    Lim lim;                     // device-side batch size (plans)
+    bool planned;                // by the fused kernel (lim holds its batch size and capacities)
+    Lim lim;
+    uint64_t* clean;             // its words to zero, but for [1], this kernel's ticket
+    uint32_t clean_words;
     int64_t Q;
     uint32_t chunk;
     unsigned long long* ticket;
@@ -1085,12 +1069,16 @@ constexpr uint32_t kQueueLong = 320, kQueueShort = 64;   // entries
 constexpr size_t queue_bytes(uint32_t cap) { return (size_t)cap * 8 + 16; }   // nodes, weights, counter
 constexpr size_t kMaxDynSmem = 227 * 1024;   // dynamic shared memory of one CTA at most
 
-// chunks of the launch: known on the host, or (plans) read on the device,
-// zero when the batch overflows the plan's buffers
+// chunks of the launch: known on the host, or (planned by the fused kernel) read
+// on the device, zero when the batch overflows the plan's buffers; the fused
+// kernel's words are left zero for its next launch
 __device__ __forceinline__ unsigned long long main_total(const MainArgs& A) {
-    if (!A.lim.Qd) return A.total_chunks;
-    const int64_t Qe = *A.lim.Qd;
-    return over_cap(A.lim, A.blk_off, A.chunk_off, Qe) ? 0ull : A.chunk_off[Qe];
+    if (!A.planned) return A.total_chunks;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < A.clean_words; i += gridDim.x * blockDim.x)
+        if (i != 1) A.clean[i] = 0;
+    const int64_t Qe = live_q(A.lim, A.Q);
+    const bool over = A.blk_off[Qe] > A.lim.cap_blocks || A.chunk_off[Qe] > A.lim.cap_chunks;
+    return over ? 0ull : A.chunk_off[Qe];
 }
 
 struct Queue {
@@ -1517,17 +1505,18 @@ __global__ void __launch_bounds__(NT, WarpKernelBounds<NT>::min_ctas) query_warp
     extern __shared__ __align__(16) uint8_t smem[];
     const uint32_t S = A.P.S;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const size_t hist_bytes = (size_t)S * 4 * (FP ? 2 : 1);
+    const uint32_t S4 = (S + 3) & ~3u;   // a histogram is flushed four bins at a time
+    const size_t hist_bytes = (size_t)S4 * 4 * (FP ? 2 : 1);
     Desc* desc = reinterpret_cast<Desc*>(smem + warp * kDescBytes);
     uint8_t* mine = smem + (blockDim.x >> 5) * kDescBytes + warp * (hist_bytes + (REC ? 0 : queue_bytes(A.qcap)));
     Hist<FP> H;
     H.h = reinterpret_cast<uint32_t*>(mine);
-    H.hf = FP ? reinterpret_cast<float*>(H.h + S) : nullptr;
+    H.hf = FP ? reinterpret_cast<float*>(H.h + S4) : nullptr;
     H.touched = nullptr;
     H.ntouched = nullptr;
     H.track = false;
     const Queue Qu = carve_queue(mine + hist_bytes, A.qcap);
-    for (uint32_t i = lane; i < S; i += 32) {
+    for (uint32_t i = lane; i < S4; i += 32) {
         H.h[i] = 0;
         if constexpr (FP) H.hf[i] = 0.f;
     }
@@ -1537,25 +1526,32 @@ __global__ void __launch_bounds__(NT, WarpKernelBounds<NT>::min_ctas) query_warp
     uint32_t* acc;
     float* accf;
     main_out<FP>(A, acc, accf);
-    const unsigned long long total = main_total(A);
-    for (;;) {
-        unsigned long long c = 0;
-        if (lane == 0) c = atomicAdd(A.ticket, 1ull);
-        c = __shfl_sync(0xffffffffu, c, 0);
-        if (c >= total) break;
+    const uint32_t total = (uint32_t)main_total(A);   // (below 2^32: the chunk map's bound)
+    // A warp's first chunk is its own number, the ticket hands out the rest.
+    // (Taking the next one while the current chunk runs left the last chunks
+    // to busy warps: 125 -> 140 us for 10,000 boxes of 512x512x384.)
+    const uint32_t all = gridDim.x * (NT / 32);
+    uint32_t c = blockIdx.x * (NT / 32) + warp;
+    while (c < total) {
         const uint32_t q = __ldg(A.chunk_q + c);
         const uint32_t ncube = (uint32_t)A.ncube[q];
-        const uint32_t c0 = (uint32_t)(c - A.chunk_off[q]) * A.chunk;
+        const uint32_t c0 = (c - (uint32_t)A.chunk_off[q]) * A.chunk;
         const uint32_t c1 = min(c0 + A.chunk, ncube);
         process_span<FP, AT, REC>(A, H, Qu, desc, c0, c1, __ldg(A.chunk_b + c), A.blk_off[q + 1], ncube);
         if constexpr (!REC) drain<FP, AT>(A.P, H, Qu, true);
-        for (uint32_t s = lane; s < S; s += 32) {
-            const uint32_t v = H.h[s];
-            if (v) {
-                H.h[s] = 0;
-                atomicAdd(acc + (size_t)q * S + s, v);
+        uint32_t* row = acc + (size_t)q * S;
+        for (uint32_t s = 4 * lane; s < S4; s += 128) {
+            const uint4 v = *reinterpret_cast<const uint4*>(H.h + s);
+            if (v.x | v.y | v.z | v.w) {
+                *reinterpret_cast<uint4*>(H.h + s) = make_uint4(0u, 0u, 0u, 0u);
+                if (v.x) atomicAdd(row + s, v.x);
+                if (v.y) atomicAdd(row + s + 1, v.y);
+                if (v.z) atomicAdd(row + s + 2, v.z);
+                if (v.w) atomicAdd(row + s + 3, v.w);
             }
-            if constexpr (FP) {
+        }
+        if constexpr (FP) {
+            for (uint32_t s = lane; s < S; s += 32) {
                 const float f = H.hf[s];
                 if (f != 0.f) {
                     H.hf[s] = 0.f;
@@ -1564,6 +1560,9 @@ __global__ void __launch_bounds__(NT, WarpKernelBounds<NT>::min_ctas) query_warp
             }
         }
         __syncwarp();
+        if (total <= all) break;
+        if (lane == 0) c = all + atomicAdd(reinterpret_cast<uint32_t*>(A.ticket), 1u);
+        c = __shfl_sync(0xffffffffu, c, 0);
     }
 }
 
@@ -1595,9 +1594,9 @@ __global__ void __launch_bounds__(512, 2) query_batched_kernel(const __grid_cons
     float* accf;
     main_out<FP>(A, acc, accf);
     const unsigned long long total = main_total(A);
-    for (;;) {
+    for (bool own = true;; own = false) {   // a CTA's first chunk is its own number
         if (threadIdx.x == 0) {
-            const unsigned long long c = atomicAdd(A.ticket, 1ull);
+            const unsigned long long c = own ? blockIdx.x : gridDim.x + atomicAdd(A.ticket, 1ull);
             s_chunk = c;
             s_next = 0;
             if (c < total) s_q = A.chunk_q[c];
@@ -1949,8 +1948,7 @@ constexpr int64_t kFusedScanMax = 1 << 18;
 __global__ void __launch_bounds__(kScanThreads) plan_scan_kernel(const uint32_t* __restrict__ nblk,
                                                                  const uint64_t* __restrict__ nchunk, int64_t Q,
                                                                  uint64_t* __restrict__ blk_off,
-                                                                 uint64_t* __restrict__ chunk_off, Lim lim,
-                                                                 unsigned* __restrict__ status) {
+                                                                 uint64_t* __restrict__ chunk_off) {
     __shared__ unsigned long long sb[32], sc[32];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     unsigned long long carry_b = 0, carry_c = 0;
@@ -2000,25 +1998,7 @@ __global__ void __launch_bounds__(kScanThreads) plan_scan_kernel(const uint32_t*
     if (t == 0) {
         blk_off[Q] = carry_b;
         chunk_off[Q] = carry_c;
-        if (lim.Qd && (carry_b > lim.cap_blocks || carry_c > lim.cap_chunks)) set_status(status, kStatCapacity);
     }
-}
-
-// the live batch size of a plan run, passed by value (no host staging)
-// and the caller's boxes and output named in the plan's io slots
-__global__ void set_batch_kernel(int64_t* __restrict__ Qd, int64_t Q, void** __restrict__ io, const void* boxes,
-                                 void* out) {
-    *Qd = Q;
-    io[0] = const_cast<void*>(boxes);
-    io[1] = out;
-}
-
-// zero the first *Qd rows of S counters (plans); n = rows * S bound
-template <typename T>
-__global__ void zero_rows_kernel(T* __restrict__ a, const int64_t* __restrict__ Qd, int64_t S) {
-    const int64_t n = *Qd * S;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        a[i] = T(0);
 }
 
 __global__ void widen_kernel(const uint32_t* __restrict__ a, uint64_t* __restrict__ b, int64_t n) {
@@ -2051,17 +2031,116 @@ uint32_t default_chunk(uint32_t S, int64_t Q) {
     return c;
 }
 
+// Most blocks and work chunks that Q boxes of the volume can have.  An axis of
+// d voxels splits into at most 2 ceil(log2(d + 1)) runs, two of each level; the
+// cubes of level l whose thickness lies on an axis are at most 2 (area across
+// it) / 4^l, so a footprint holds at most 8/3 of the three areas.
+uint64_t block_bound(const mg_graph* g, int64_t Q) {
+    uint64_t n = (uint64_t)Q;
+    for (int k = 0; k < 3; k++) {
+        int bits = 0;
+        while ((g->geom.dims[0][k] >> bits) > 0) bits++;
+        n *= 2 * (uint64_t)bits;
+    }
+    return n;
+}
+uint64_t chunk_bound(const mg_graph* g, int64_t Q, uint32_t chunk) {
+    const uint64_t x = g->geom.dims[0][0], y = g->geom.dims[0][1], z = g->geom.dims[0][2];
+    return (uint64_t)Q * ((3 * (x * y + y * z + z * x)) / chunk + 1);
+}
+
 template <typename K>
 mg_status prepare_kernel(K kernel, size_t smem) {
     MG_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     return MG_OK;
 }
 
-// pdl: launch the batched kernel with programmatic stream serialisation (its
-// CTAs start while the plan kernel finishes and wait for it on the device)
+size_t hist_smem(uint32_t S, bool FP) {   // histogram and touched list of a CTA
+    const size_t touched = (size_t)S * 2 * (FP ? 2 : 1);
+    return (size_t)S * 4 * (FP ? 2 : 1) + ((touched + 15) & ~(size_t)15) + 16;
+}
+
+// the batched kernel for a graph and a CTA size
+struct MainShape {
+    void (*k)(const MainArgs) = nullptr;
+    int threads = 0, full = 0;     // CTAs that fill the GPU
+    int chunks_per_cta = 1;        // chunks a CTA works on at a time
+    size_t smem = 0;
+    uint32_t qcap = 0;
+};
+
+template <bool FP, typename AT>
+mg_status main_shape(const mg_graph* g, bool rec, int threads, MainShape* out) {
+    // few segments: a private histogram per warp; else one per CTA (smem
+    // is then the histogram's part); the warps' block descriptors and, without
+    // node records, their queues come on top
+    int warps = threads / 32;
+    const size_t smem = hist_smem(g->S, FP);
+    const size_t hist_w = (size_t)g->S * 4 * (FP ? 2 : 1), hist_s = (size_t)((g->S + 3) & ~3u) * 4 * (FP ? 2 : 1);
+    const bool warp_mode =
+        g->S <= kWarpHistMax && threads <= 256 && (hist_w + queue_bytes(kQueueShort)) * warps <= 96 * 1024;
+    auto k = !warp_mode       ? (rec ? query_batched_kernel<FP, AT, true> : query_batched_kernel<FP, AT, false>)
+             : threads <= 128 ? (rec ? query_warp_kernel<FP, AT, 128, true> : query_warp_kernel<FP, AT, 128, false>)
+                              : (rec ? query_warp_kernel<FP, AT, 256, true> : query_warp_kernel<FP, AT, 256, false>);
+    auto smem_for = [&](uint32_t cap) {
+        const size_t each = kDescBytes + (rec ? 0 : queue_bytes(cap));
+        return warp_mode ? (hist_s + each) * warps : smem + warps * each;
+    };
+    int per_sm = 0, per_long = 0;
+    if (!warp_mode) {
+        // the shape asked for has to fit with its queues alone; the descriptors
+        // of the last few segment counts that do take fewer warps
+        if (smem + warps * queue_bytes(kQueueShort) > kMaxDynSmem)
+            return fail(MG_ERR_UNSUPPORTED, "query kernel does not fit on an SM");
+        while (warps > 1 && smem_for(kQueueShort) > kMaxDynSmem) warps /= 2;
+        threads = warps * 32;
+    }
+    // one limit for every launch of the kernel: callers of several shapes never
+    // lower each other's
+    MG_TRY(prepare_kernel(k, std::max(smem_for(kQueueShort), kMaxDynSmem - 1024)));
+    MG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem_for(kQueueShort)));
+    if (per_sm < 1) return fail(MG_ERR_UNSUPPORTED, "query kernel does not fit on an SM");
+    if (!rec && smem_for(kQueueLong) <= kMaxDynSmem - 1024)
+        MG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_long, k, threads, smem_for(kQueueLong)));
+    out->k = k;
+    out->threads = threads;
+    out->full = per_sm * sm_count(g->device);
+    out->chunks_per_cta = warp_mode ? warps : 1;
+    out->qcap = per_long >= per_sm ? kQueueLong : kQueueShort;
+    out->smem = smem_for(out->qcap);
+    return MG_OK;
+}
+
+// pdl: with programmatic stream serialisation (its CTAs start while the plan
+// kernel finishes and wait for it on the device)
+mg_status launch_shape(const mg_graph* g, const MainArgs& A, const MainShape& M, cudaStream_t s, bool pdl) {
+    MainArgs A2 = A;
+    A2.qcap = M.qcap;
+    // no more CTAs than chunks the batch can have
+    const uint64_t most = chunk_bound(g, A.Q, A.chunk);
+    const unsigned grid = (unsigned)std::min<uint64_t>(M.full, (most + M.chunks_per_cta - 1) / M.chunks_per_cta);
+    if (!pdl) {
+        M.k<<<grid, M.threads, M.smem, s>>>(A2);
+        MG_CUDA(cudaGetLastError());
+        return MG_OK;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3((unsigned)M.threads);
+    cfg.dynamicSmemBytes = M.smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    MG_CUDA(cudaLaunchKernelEx(&cfg, M.k, A2));
+    return MG_OK;
+}
+
 template <bool FP, typename AT>
 mg_status launch_main(const mg_graph* g, const MainArgs& A, const mg_query_opts& o, const int32_t* boxes,
-                      size_t smem, int threads, cudaStream_t s, bool pdl = false, const Alloc* scratch = nullptr) {
+                      size_t smem, int threads, cudaStream_t s, const Alloc* scratch) {
     if (o.schedule == MG_SCHED_NAIVE) {
         // slabs per box, their offsets, then one persistent launch
         if (!scratch) return fail(MG_ERR_INVALID_ARG, "naive schedule without scratch");
@@ -2094,7 +2173,7 @@ mg_status launch_main(const mg_graph* g, const MainArgs& A, const mg_query_opts&
         Buf cubes;
         MG_TRY(cubes.alloc(scratch, (size_t)A.Q * 8, s));
         plan_count_kernel<<<grid_for(A.Q * 32, kPlanThreads), kPlanThreads, 0, s>>>(
-            A.G, boxes, A.Q, 1, nullptr, cubes.as<uint64_t>(), nullptr, A.P.status, Lim{nullptr, 0, 0}, false);
+            A.G, boxes, A.Q, 1, nullptr, cubes.as<uint64_t>(), nullptr, A.P.status, false);
         MG_CUDA(cudaGetLastError());
         std::vector<uint64_t> nc((size_t)A.Q);
         MG_CUDA(cudaMemcpyAsync(nc.data(), cubes.p, (size_t)A.Q * 8, cudaMemcpyDeviceToHost, s));
@@ -2111,58 +2190,9 @@ mg_status launch_main(const mg_graph* g, const MainArgs& A, const mg_query_opts&
         MG_CUDA(cudaGetLastError());
         return MG_OK;
     }
-    // few segments: a private histogram per warp; else one per CTA (smem
-    // is then the histogram's part); the warps' block descriptors and, without
-    // node records, their queues come on top
-    int warps = threads / 32;
-    const size_t hist_w = (size_t)g->S * 4 * (FP ? 2 : 1);
-    const bool rec = A.P.rec != nullptr;
-    const bool warp_mode =
-        g->S <= kWarpHistMax && threads <= 256 && (hist_w + queue_bytes(kQueueShort)) * warps <= 96 * 1024;
-    auto k = !warp_mode       ? (rec ? query_batched_kernel<FP, AT, true> : query_batched_kernel<FP, AT, false>)
-             : threads <= 128 ? (rec ? query_warp_kernel<FP, AT, 128, true> : query_warp_kernel<FP, AT, 128, false>)
-                              : (rec ? query_warp_kernel<FP, AT, 256, true> : query_warp_kernel<FP, AT, 256, false>);
-    auto smem_for = [&](uint32_t cap) {
-        const size_t each = kDescBytes + (rec ? 0 : queue_bytes(cap));
-        return warp_mode ? (hist_w + each) * warps : smem + warps * each;
-    };
-    int per_sm = 0, per_long = 0;
-    if (!warp_mode) {
-        // the shape asked for has to fit with its queues alone; the descriptors
-        // of the last few segment counts that do take fewer warps
-        if (smem + warps * queue_bytes(kQueueShort) > kMaxDynSmem)
-            return fail(MG_ERR_UNSUPPORTED, "query kernel does not fit on an SM");
-        while (warps > 1 && smem_for(kQueueShort) > kMaxDynSmem) warps /= 2;
-        threads = warps * 32;
-    }
-    MG_TRY(prepare_kernel(k, smem_for(kQueueShort)));
-    MG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem_for(kQueueShort)));
-    if (per_sm < 1) return fail(MG_ERR_UNSUPPORTED, "query kernel does not fit on an SM");
-    if (smem_for(kQueueLong) <= kMaxDynSmem) {
-        MG_TRY(prepare_kernel(k, smem_for(kQueueLong)));
-        MG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_long, k, threads, smem_for(kQueueLong)));
-    }
-    MainArgs A2 = A;
-    A2.qcap = per_long >= per_sm ? kQueueLong : kQueueShort;
-    const size_t sm = smem_for(A2.qcap);
-    const int grid = per_sm * sm_count(g->device);
-    if (!pdl) {
-        k<<<grid, threads, sm, s>>>(A2);
-        MG_CUDA(cudaGetLastError());
-        return MG_OK;
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = sm;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    MG_CUDA(cudaLaunchKernelEx(&cfg, k, A2));
-    return MG_OK;
+    MainShape M;
+    MG_TRY((main_shape<FP, AT>(g, A.P.rec != nullptr, threads, &M)));
+    return launch_shape(g, A, M, s, false);
 }
 
 // Box histograms summed from the mixture table (Sec. 3.6) with error bars
@@ -2255,12 +2285,133 @@ mg_status query_lut(const mg_graph* g, const int32_t* boxes, int64_t Q, double* 
 mg_status count_cubes(const mg_graph* g, const int32_t* boxes, int64_t Q, uint64_t* cubes, cudaStream_t s) {
     const Geom G = make_geom(g, 0);
     plan_count_kernel<<<grid_for(Q * 32, kPlanThreads), kPlanThreads, 0, s>>>(G, boxes, Q, 1, nullptr, cubes, nullptr,
-                                                            g->status.as<unsigned>(), Lim{nullptr, 0, 0}, false);
+                                                            g->status.as<unsigned>(), false);
     MG_CUDA(cudaGetLastError());
     return MG_OK;
 }
 
 namespace {
+
+int64_t tile_count(int64_t Q, int dev) {
+    const int tb = tile_boxes(Q, sm_count(dev));
+    return (Q + tb - 1) / tb;
+}
+
+// buffers of a batch planned by the fused kernel
+struct QueryBufs {
+    uint64_t *ncube, *blk_off, *chunk_off;
+    Blk* blk;
+    uint32_t *chunk_q, *chunk_b;
+    uint64_t* words;        // two tickets (fused kernel, main kernel), then the tile words; zero between batches
+    uint32_t* acc;          // fp32 histograms: the integer part
+    uint64_t cap_blocks, cap_chunks;
+    uint32_t chunk;
+    MainShape shape;
+};
+
+// the batch itself: boxes, size and output given here (Qd, io null), or read on
+// the device from Qd and io = {boxes, output} (replayed graphs), Q the most
+struct BatchRun {
+    const int32_t* boxes;
+    int64_t Q;
+    const int64_t* Qd;
+    void* const* io;
+    void* out;
+};
+
+// The fused plan kernel and the main kernel, the latter launched with
+// programmatic stream serialisation; fp32 histograms then get their integer
+// part added (unless `parts`: the caller takes both parts).  ev: events after
+// the plan, after the main kernel.
+template <bool FP, typename AT>
+mg_status enqueue_batch(const mg_graph* g, const QueryBufs& B, const BatchRun& R, bool parts, cudaEvent_t* ev,
+                        cudaStream_t s) {
+    const mg_dtype weights = std::is_same<AT, __half>::value          ? MG_F16
+                             : std::is_same<AT, __nv_bfloat16>::value ? MG_BF16
+                                                                      : MG_F32;
+    const Geom G = make_geom(g, tile_levels(g, weights));
+    unsigned* status = g->status.as<unsigned>();
+    const Lim lim{R.Qd, B.cap_blocks, B.cap_chunks};
+    uint32_t* acc = FP ? B.acc : static_cast<uint32_t*>(R.out);
+    float* accf = FP ? static_cast<float*>(R.out) : nullptr;
+    const int64_t tiles = tile_count(R.Q, g->device);
+    const int tb = tile_boxes(R.Q, sm_count(g->device));
+    const int chunk_shift = (B.chunk & (B.chunk - 1)) == 0 ? __builtin_ctz(B.chunk) : -1;
+    FusedOut F;
+    F.ncube = B.ncube;
+    F.blk_off = B.blk_off;
+    F.chunk_off = B.chunk_off;
+    F.blk = B.blk;
+    F.chunk_q = B.chunk_q;
+    F.chunk_b = B.chunk_b;
+    F.tiles = B.words + 2;
+    F.ticket = reinterpret_cast<unsigned long long*>(B.words);
+    F.acc = acc;
+    F.accf = accf;
+    F.io = R.io;
+    plan_fused_kernel<<<(unsigned)tiles, kFusedThreads, 0, s>>>(G, R.boxes, R.Q, tb, B.chunk, chunk_shift, lim, F,
+                                                                status);
+    MG_CUDA(cudaGetLastError());
+    if (ev) MG_CUDA(cudaEventRecord(ev[0], s));
+
+    const int w16 = weights == MG_BF16;
+    MainArgs A;
+    A.G = G;
+    A.I = make_ids(g);
+    A.P.pq = g->pq.as<uint2>();
+    A.P.ab32 = g->ab32.as<uint2>();
+    A.P.lut_meta = g->lut_meta.as<uint2>();
+    A.P.lut = g->lut.as<uint2>();
+    A.P.rec = weights == MG_F32 ? g->lut_rec.as<uint4>() : g->rec16[w16].as<uint4>();
+    A.P.frac = weights == MG_F32 ? nullptr : g->frac16[w16].as<float>();
+    A.P.alpha = weights == MG_F16 ? g->alpha16.p : weights == MG_BF16 ? g->alphab16.p : g->alpha.p;
+    A.P.S = g->S;
+    A.P.status = status;
+    A.blk = B.blk;
+    A.blk_off = B.blk_off;
+    A.ncube = B.ncube;
+    A.chunk_off = B.chunk_off;
+    A.chunk_q = B.chunk_q;
+    A.chunk_b = B.chunk_b;
+    A.total_chunks = 0;
+    A.planned = true;
+    A.lim = lim;
+    A.clean = B.words;
+    A.clean_words = (uint32_t)(2 + 2 * tiles);
+    A.Q = R.Q;
+    A.chunk = B.chunk;
+    A.ticket = F.ticket + 1;
+    A.acc = acc;
+    A.accf = accf;
+    A.io = R.io;
+    A.qcap = 0;   // the shape's
+    MG_TRY(launch_shape(g, A, B.shape, s, !ev));
+    if (ev) MG_CUDA(cudaEventRecord(ev[1], s));
+    if (FP && !parts) {
+        const int64_t cells = R.Q * (int64_t)g->S;
+        const unsigned gb = grid_for(cells, 256, 152 * 64);
+        if (R.io) dense_f32_rows_kernel<<<gb, 256, 0, s>>>(acc, R.io, R.Qd, g->S);
+        else dense_f32_kernel<<<gb, 256, 0, s>>>(acc, accf, cells);
+        MG_CUDA(cudaGetLastError());
+    }
+    return MG_OK;
+}
+
+mg_status enqueue_any(const mg_graph* g, const QueryBufs& B, const BatchRun& R, bool FP, mg_dtype weights, bool parts,
+                      cudaEvent_t* ev, cudaStream_t s) {
+    if (!FP) return enqueue_batch<false, float>(g, B, R, parts, ev, s);
+    if (weights == MG_F16) return enqueue_batch<true, __half>(g, B, R, parts, ev, s);
+    if (weights == MG_BF16) return enqueue_batch<true, __nv_bfloat16>(g, B, R, parts, ev, s);
+    return enqueue_batch<true, float>(g, B, R, parts, ev, s);
+}
+
+mg_status shape_of(const mg_graph* g, bool FP, mg_dtype weights, int threads, MainShape* out) {
+    const bool rec = (weights == MG_F32 ? g->lut_rec : g->rec16[weights == MG_BF16]).p != nullptr;
+    if (!FP) return main_shape<false, float>(g, rec, threads, out);
+    if (weights == MG_F16) return main_shape<true, __half>(g, rec, threads, out);
+    if (weights == MG_BF16) return main_shape<true, __nv_bfloat16>(g, rec, threads, out);
+    return main_shape<true, float>(g, rec, threads, out);
+}
 
 // Scratch comes from `al`; `words` are two host words for readbacks; `room`,
 // when not null, returns the bytes `al` can still hand out (fixed pools).
@@ -2319,6 +2470,7 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
     }
 
     const mg_dtype weights = (mg_dtype)o.alpha_dtype;
+    const int w16 = weights == MG_BF16;
     MainArgs A;
     A.G = G;
     A.I = make_ids(g);
@@ -2326,7 +2478,6 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
     A.P.ab32 = g->ab32.as<uint2>();
     A.P.lut_meta = g->lut_meta.as<uint2>();
     A.P.lut = g->lut.as<uint2>();
-    const int w16 = weights == MG_BF16;
     A.P.rec = weights == MG_F32 ? g->lut_rec.as<uint4>() : g->rec16[w16].as<uint4>();
     A.P.frac = weights == MG_F32 ? nullptr : g->frac16[w16].as<float>();
     A.P.alpha = o.alpha_dtype == MG_F16 ? g->alpha16.p : o.alpha_dtype == MG_BF16 ? g->alphab16.p : g->alpha.p;
@@ -2344,15 +2495,50 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
     A.chunk_b = nullptr;
     A.total_chunks = 0;
     A.lim = Lim{nullptr, 0, 0};
+    A.planned = false;
+    A.clean = nullptr;
+    A.clean_words = 0;
     A.ticket = nullptr;
     A.io = nullptr;
     A.qcap = kQueueShort;
 
-    const size_t touched_bytes = (size_t)S * 2 * (FP ? 2 : 1);
-    const size_t smem = (size_t)S * 4 * (FP ? 2 : 1) + ((touched_bytes + 15) & ~(size_t)15) + 16;
+    const size_t smem = hist_smem(S, FP);
     if (smem > 220 * 1024) return fail(MG_ERR_UNSUPPORTED, "too many segments for the shared-memory histogram");
+    // Where the most that this many boxes can have fits a modest buffer, the
+    // footprint is planned in one launch and nothing is read back: 1,000 boxes
+    // of a 64^3 volume took 69 us with three plan kernels and the read-back of
+    // their totals, 34 with this.
+    const uint64_t most_blocks = block_bound(g, Q), most_chunks = chunk_bound(g, Q, chunk);
+    const bool fused = o.schedule == MG_SCHED_BATCHED && !room && most_blocks < (1u << 22) && most_chunks < (1u << 22);
     Buf nblk, ncube, nchunk, blk_off, chunk_off, blk, ticket, chunk_q, chunk_b;
-    if (o.schedule == MG_SCHED_BATCHED) {
+    if (fused) {
+        Buf tiles;
+        QueryBufs B;
+        B.cap_blocks = most_blocks;
+        B.cap_chunks = most_chunks;
+        B.chunk = chunk;
+        MG_TRY(shape_of(g, FP, weights, threads, &B.shape));
+        const size_t words_bytes = 16 + 16 * (size_t)tile_count(Q, g->device);
+        MG_TRY(ncube.alloc(&al, (size_t)Q * 8, s));
+        MG_TRY(blk_off.alloc(&al, (size_t)(Q + 1) * 8, s));
+        MG_TRY(chunk_off.alloc(&al, (size_t)(Q + 1) * 8, s));
+        MG_TRY(blk.alloc(&al, (size_t)most_blocks * sizeof(Blk), s));
+        MG_TRY(chunk_q.alloc(&al, (size_t)most_chunks * 4, s));
+        MG_TRY(chunk_b.alloc(&al, (size_t)most_chunks * 4, s));
+        MG_TRY(tiles.alloc(&al, words_bytes, s));
+        B.ncube = ncube.as<uint64_t>();
+        B.blk_off = blk_off.as<uint64_t>();
+        B.chunk_off = chunk_off.as<uint64_t>();
+        B.blk = blk.as<Blk>();
+        B.chunk_q = chunk_q.as<uint32_t>();
+        B.chunk_b = chunk_b.as<uint32_t>();
+        B.words = tiles.as<uint64_t>();
+        B.acc = acc;
+        MG_CUDA(cudaMemsetAsync(B.words, 0, words_bytes, s));
+        const BatchRun run{boxes, Q, nullptr, nullptr, FP ? static_cast<void*>(accf) : static_cast<void*>(acc)};
+        cudaEvent_t* ev = timed ? gm->qev + 1 : nullptr;
+        MG_TRY(enqueue_any(g, B, run, FP, weights, csr, ev, s));
+    } else if (o.schedule == MG_SCHED_BATCHED) {
         MG_TRY(nblk.alloc(&al, (size_t)Q * 4, s));
         MG_TRY(ncube.alloc(&al, (size_t)Q * 8, s));
         MG_TRY(nchunk.alloc(&al, (size_t)Q * 8, s));
@@ -2361,12 +2547,11 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
         MG_TRY(ticket.alloc(&al, 8, s));
         plan_count_kernel<<<grid_for(Q * 32, kPlanThreads), kPlanThreads, 0, s>>>(G, boxes, Q, chunk, nblk.as<uint32_t>(),
                                                                 ncube.as<uint64_t>(), nchunk.as<uint64_t>(),
-                                                                status, Lim{nullptr, 0, 0}, true);
+                                                                status, true);
         MG_CUDA(cudaGetLastError());
         if (Q <= kFusedScanMax) {
             plan_scan_kernel<<<1, kScanThreads, 0, s>>>(nblk.as<uint32_t>(), nchunk.as<uint64_t>(), Q,
-                                                        blk_off.as<uint64_t>(), chunk_off.as<uint64_t>(),
-                                                        Lim{nullptr, 0, 0}, status);
+                                                        blk_off.as<uint64_t>(), chunk_off.as<uint64_t>());
             MG_CUDA(cudaGetLastError());
         } else {
             // block offsets are 64-bit sums of the 32-bit per-box counts
@@ -2397,7 +2582,7 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
         MG_TRY(chunk_q.alloc(&al, (size_t)std::max<uint64_t>(totals[1], 1) * 4, s));
         MG_TRY(chunk_b.alloc(&al, (size_t)std::max<uint64_t>(totals[1], 1) * 4, s));
         plan_write_kernel<<<grid_for(Q * 32, kPlanThreads), kPlanThreads, 0, s>>>(
-            G, boxes, Q, blk_off.as<uint64_t>(), blk.as<Blk>(), Lim{nullptr, 0, 0}, chunk_off.as<uint64_t>(), chunk,
+            G, boxes, Q, blk_off.as<uint64_t>(), blk.as<Blk>(), chunk_off.as<uint64_t>(), chunk,
             chunk_q.as<uint32_t>(), chunk_b.as<uint32_t>());
         MG_CUDA(cudaGetLastError());
         A.chunk_q = chunk_q.as<uint32_t>();
@@ -2412,23 +2597,25 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
     }
     // the accumulators are cleared only once the footprint is known to fit, so
     // a refused call leaves the caller's output as it was
-    if (FP) MG_CUDA(cudaMemsetAsync(accf, 0, cells * 4, s));
-    MG_CUDA(cudaMemsetAsync(acc, 0, cells * 4, s));
-    if (timed) MG_CUDA(cudaEventRecord(gm->qev[1], s));
-    if (FP) {
+    if (!fused) {
+        if (FP) MG_CUDA(cudaMemsetAsync(accf, 0, cells * 4, s));
+        MG_CUDA(cudaMemsetAsync(acc, 0, cells * 4, s));
+        if (timed) MG_CUDA(cudaEventRecord(gm->qev[1], s));
+    }
+    if (!fused && FP) {
         if (o.alpha_dtype == MG_F16)
-            MG_TRY((launch_main<true, __half>(g, A, o, boxes, smem, threads, s, false, &al)));
+            MG_TRY((launch_main<true, __half>(g, A, o, boxes, smem, threads, s, &al)));
         else if (o.alpha_dtype == MG_BF16)
-            MG_TRY((launch_main<true, __nv_bfloat16>(g, A, o, boxes, smem, threads, s, false, &al)));
+            MG_TRY((launch_main<true, __nv_bfloat16>(g, A, o, boxes, smem, threads, s, &al)));
         else
-            MG_TRY((launch_main<true, float>(g, A, o, boxes, smem, threads, s, false, &al)));
-    } else {
-        MG_TRY((launch_main<false, float>(g, A, o, boxes, smem, threads, s, false, &al)));
+            MG_TRY((launch_main<true, float>(g, A, o, boxes, smem, threads, s, &al)));
+    } else if (!fused) {
+        MG_TRY((launch_main<false, float>(g, A, o, boxes, smem, threads, s, &al)));
     }
 
-    if (timed) MG_CUDA(cudaEventRecord(gm->qev[2], s));
+    if (timed && !fused) MG_CUDA(cudaEventRecord(gm->qev[2], s));
     if (!csr) {
-        if (FP) {
+        if (FP && !fused) {
             dense_f32_kernel<<<grid_for((int64_t)cells, 256, 152 * 64), 256, 0, s>>>(acc, accf, (int64_t)cells);
             MG_CUDA(cudaGetLastError());
         }
@@ -2593,17 +2780,17 @@ extern "C" MG_API mg_status mg_query_boxes_noalloc(const mg_graph* g, const int3
 }
 
 // ---------------------------------------------------------------------------
-// Query plans: the whole batched pipeline for up to max_Q boxes captured once
-// as a CUDA graph, with every buffer preallocated; a run copies the boxes in,
-// replays the graph and copies the histograms out, with no host sync.
+// Query plans: every buffer of a batch of up to max_Q boxes, allocated once; a
+// run is two launches (three for fp32 histograms) on the caller's boxes and
+// output, with no host synchronisation.  The request loop replays the same
+// launches as a CUDA graph on the plan's own buffers.
 // ---------------------------------------------------------------------------
 struct mg_query_plan {
     mg_graph* g = nullptr;
     int64_t max_Q = 0;
     bool fp = false;
-    uint32_t chunk = 0;
-    int threads = 0;
-    uint64_t cap_blocks = 0, cap_chunks = 0;
+    mg_dtype weights = MG_F32;
+    mg::QueryBufs bufs{};
     mg::Buf pool;
     mg::Pool bump{nullptr, 0, 0};
     int32_t* boxes = nullptr;
@@ -2625,108 +2812,6 @@ struct mg_query_plan {
 };
 
 namespace mg {
-namespace {
-
-template <bool FP, typename AT>
-mg_status plan_enqueue(mg_query_plan* p, const Alloc& al, cudaStream_t s) {
-    const mg_graph* g = p->g;
-    const int64_t Q = p->max_Q;
-    const uint32_t S = g->S;
-    const mg_dtype weights = std::is_same<AT, __half>::value          ? MG_F16
-                             : std::is_same<AT, __nv_bfloat16>::value ? MG_BF16
-                                                                      : MG_F32;
-    const Geom G = make_geom(g, tile_levels(g, weights));
-    unsigned* status = g->status.as<unsigned>();
-    const Lim lim{p->Qd, p->cap_blocks, p->cap_chunks};
-    Buf acc_b, ncube, blk_off, chunk_off, blk, chunk_q, chunk_b, tiles, ticket;
-    uint32_t* acc = nullptr;
-    float* accf = nullptr;
-    if (FP) {
-        MG_TRY(acc_b.alloc(&al, (size_t)Q * S * 4, s));
-        acc = acc_b.as<uint32_t>();
-        accf = static_cast<float*>(p->result);
-    } else {
-        acc = static_cast<uint32_t*>(p->result);
-    }
-    const int tb = tile_boxes(Q, sm_count(g->device));
-    const int64_t ntiles = (Q + tb - 1) / tb;
-    const int chunk_shift = (p->chunk & (p->chunk - 1)) == 0 ? __builtin_ctz(p->chunk) : -1;
-    MG_TRY(ncube.alloc(&al, (size_t)Q * 8, s));
-    MG_TRY(blk_off.alloc(&al, (size_t)(Q + 1) * 8, s));
-    MG_TRY(chunk_off.alloc(&al, (size_t)(Q + 1) * 8, s));
-    MG_TRY(blk.alloc(&al, (size_t)p->cap_blocks * sizeof(Blk), s));
-    MG_TRY(chunk_q.alloc(&al, (size_t)p->cap_chunks * 4, s));
-    MG_TRY(chunk_b.alloc(&al, (size_t)p->cap_chunks * 4, s));
-    MG_TRY(tiles.alloc(&al, (size_t)ntiles * 16, s));
-    MG_TRY(ticket.alloc(&al, 16, s));   // tile order, main-kernel chunks
-
-    if (p->timed) MG_CUDA(cudaEventRecordWithFlags(p->ev[0], s, cudaEventRecordExternal));
-    plan_reset_kernel<<<grid_for(2 * ntiles, 256, 152 * 4), 256, 0, s>>>(p->Qd, tb, tiles.as<uint64_t>(),
-                                                                         ticket.as<unsigned long long>());
-    MG_CUDA(cudaGetLastError());
-    FusedOut F;
-    F.ncube = ncube.as<uint64_t>();
-    F.blk_off = blk_off.as<uint64_t>();
-    F.chunk_off = chunk_off.as<uint64_t>();
-    F.blk = blk.as<Blk>();
-    F.chunk_q = chunk_q.as<uint32_t>();
-    F.chunk_b = chunk_b.as<uint32_t>();
-    F.tiles = tiles.as<uint64_t>();
-    F.ticket = ticket.as<unsigned long long>();
-    F.acc = acc;
-    F.accf = accf;
-    F.io = p->io;
-    plan_fused_kernel<<<(unsigned)ntiles, kFusedThreads, 0, s>>>(G, p->boxes, Q, tb, p->chunk, chunk_shift, lim, F,
-                                                                 status);
-    MG_CUDA(cudaGetLastError());
-    if (p->timed) MG_CUDA(cudaEventRecordWithFlags(p->ev[1], s, cudaEventRecordExternal));
-
-    MainArgs A;
-    A.G = G;
-    A.I = make_ids(g);
-    A.P.pq = g->pq.as<uint2>();
-    A.P.ab32 = g->ab32.as<uint2>();
-    A.P.lut_meta = g->lut_meta.as<uint2>();
-    A.P.lut = g->lut.as<uint2>();
-    const int w16 = weights == MG_BF16;
-    A.P.rec = weights == MG_F32 ? g->lut_rec.as<uint4>() : g->rec16[w16].as<uint4>();
-    A.P.frac = weights == MG_F32 ? nullptr : g->frac16[w16].as<float>();
-    A.P.alpha = std::is_same<AT, __half>::value ? g->alpha16.p : std::is_same<AT, __nv_bfloat16>::value ? g->alphab16.p
-                                                                                                          : g->alpha.p;
-    A.P.S = S;
-    A.P.status = status;
-    A.blk = blk.as<Blk>();
-    A.blk_off = blk_off.as<uint64_t>();
-    A.ncube = ncube.as<uint64_t>();
-    A.chunk_off = chunk_off.as<uint64_t>();
-    A.chunk_q = chunk_q.as<uint32_t>();
-    A.chunk_b = chunk_b.as<uint32_t>();
-    A.total_chunks = 0;
-    A.lim = lim;
-    A.Q = Q;
-    A.chunk = p->chunk;
-    A.ticket = ticket.as<unsigned long long>() + 1;
-    A.acc = acc;
-    A.accf = accf;
-    A.io = p->io;
-    A.qcap = kQueueShort;
-    mg_query_opts o{};
-    o.hist_type = FP ? MG_HIST_F32 : MG_HIST_U32;
-    const size_t touched_bytes = (size_t)S * 2 * (FP ? 2 : 1);
-    const size_t smem = (size_t)S * 4 * (FP ? 2 : 1) + ((touched_bytes + 15) & ~(size_t)15) + 16;
-    MG_TRY((launch_main<FP, AT>(g, A, o, nullptr, smem, p->threads, s, !p->timed)));
-    if (p->timed) MG_CUDA(cudaEventRecordWithFlags(p->ev[2], s, cudaEventRecordExternal));
-    if (FP) {
-        dense_f32_rows_kernel<<<grid_for(Q * S, 256, 152 * 64), 256, 0, s>>>(acc, p->io, p->Qd, S);
-        MG_CUDA(cudaGetLastError());
-    }
-    return MG_OK;
-}
-
-}  // namespace
-}  // namespace mg
-
-namespace mg {
 PlanChunk plan_chunk(const mg_graph* g, int hist_type, int chunk_cubes, int64_t max_Q, uint64_t cap_chunks) {
     const int tuned = g->tuned_chunk[hist_type == MG_HIST_F32];
     if (chunk_cubes > 0) return PlanChunk{(uint32_t)chunk_cubes, 1};
@@ -2737,8 +2822,19 @@ PlanChunk plan_chunk(const mg_graph* g, int hist_type, int chunk_cubes, int64_t 
     return PlanChunk{c, scale};
 }
 
-PlanParts plan_parts(const mg_query_plan* p) {
-    return PlanParts{p->boxes, p->Qd, p->result, p->exec, p->chunk, p->cap_blocks, p->cap_chunks};
+mg_status plan_parts(mg_query_plan* p, PlanParts* out) {
+    if (!p->exec) {
+        MG_CUDA(cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
+        MG_CUDA(cudaStreamBeginCapture(p->cap_stream, cudaStreamCaptureModeThreadLocal));
+        const BatchRun run{p->boxes, p->max_Q, p->Qd, p->io, p->result};
+        const mg_status st = enqueue_any(p->g, p->bufs, run, p->fp, p->weights, false, nullptr, p->cap_stream);
+        const cudaError_t e = cudaStreamEndCapture(p->cap_stream, &p->graph);
+        if (st != MG_OK) return st;
+        if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
+        MG_CUDA(cudaGraphInstantiate(&p->exec, p->graph, 0));
+    }
+    *out = PlanParts{p->boxes, p->Qd, p->result, p->exec, p->bufs.chunk, p->bufs.cap_blocks, p->bufs.cap_chunks};
+    return MG_OK;
 }
 }  // namespace mg
 
@@ -2777,77 +2873,61 @@ MG_API mg_status mg_query_plan_create(mg_graph* g, int64_t max_Q, const mg_query
         p->g = g;
         p->max_Q = max_Q;
         p->fp = FP;
-        const int tt = g->tuned_threads[FP];
-        p->threads = o.block_threads > 0 ? o.block_threads : tt > 0 ? tt : 256;
-        p->cap_blocks = max_blocks > 0 ? (uint64_t)max_blocks : (uint64_t)max_Q * 1024;
-        p->cap_chunks = max_chunks > 0 ? (uint64_t)max_chunks : (uint64_t)max_Q * 256;
-        const PlanChunk pc = plan_chunk(g, o.hist_type, o.chunk_cubes, max_Q, p->cap_chunks);
-        p->chunk = pc.chunk;
-        p->cap_chunks *= pc.scale;
-        if (p->cap_blocks >= (1ull << 32) || p->cap_chunks >= (1ull << 32))
+        p->weights = (mg_dtype)o.alpha_dtype;
+        QueryBufs& B = p->bufs;
+        B.cap_blocks = max_blocks > 0 ? (uint64_t)max_blocks : (uint64_t)max_Q * 1024;
+        B.cap_chunks = max_chunks > 0 ? (uint64_t)max_chunks : (uint64_t)max_Q * 256;
+        const PlanChunk pc = plan_chunk(g, o.hist_type, o.chunk_cubes, max_Q, B.cap_chunks);
+        B.chunk = pc.chunk;
+        B.cap_chunks *= pc.scale;
+        if (B.cap_blocks >= (1ull << 32) || B.cap_chunks >= (1ull << 32))
             st = fail(MG_ERR_UNSUPPORTED, "plan capacities must be below 2^32");
     }
     if (st == MG_OK) {
+        QueryBufs& B = p->bufs;
         const size_t S = g->S, Q = (size_t)max_Q;
         auto r = [](size_t n) { return (n + 255) & ~(size_t)255; };
-        // boxes, batch size, results (+ u32 scratch), cube counts, both offset
-        // arrays, blocks, chunk map, tile words, tickets
-        const size_t tiles = Q;   // at most one tile word pair per box
+        // boxes, batch size, io slots, results (+ the integer part of fp32
+        // ones), cube counts, both offset arrays, blocks, chunk map, tile words
+        // (a pair per box at most), tickets
         const size_t bytes = r(Q * 24) + r(8) + r(16) + r(Q * S * 4) * (p->fp ? 2 : 1) + r(8 * Q) + 2 * r(8 * (Q + 1)) +
-                             r(p->cap_blocks * sizeof(Blk)) + 2 * r(p->cap_chunks * 4) + r(16 * tiles) + r(16) +
-                             65536;
+                             r(B.cap_blocks * sizeof(Blk)) + 2 * r(B.cap_chunks * 4) + r(16 * Q + 16) + 65536;
         st = p->pool.alloc(&g->al, bytes, nullptr);
         if (st == MG_OK) {
-            cudaError_t e = cudaStreamSynchronize(nullptr);
-            if (e != cudaSuccess) st = cuda_fail(e, "plan pool");
-            p->pool.s = nullptr;
-        }
-        if (st == MG_OK) {
             p->bump = Pool{p->pool.as<unsigned char>(), p->pool.bytes, 0};
-            p->boxes = static_cast<int32_t*>(pool_alloc(&p->bump, Q * 24, nullptr));
-            p->Qd = static_cast<int64_t*>(pool_alloc(&p->bump, 8, nullptr));
-            p->result = pool_alloc(&p->bump, Q * S * 4, nullptr);
-            p->io = static_cast<void**>(pool_alloc(&p->bump, 16, nullptr));
+            auto take = [&](size_t n) { return pool_alloc(&p->bump, n, nullptr); };
+            p->boxes = static_cast<int32_t*>(take(Q * 24));
+            p->Qd = static_cast<int64_t*>(take(8));
+            p->result = take(Q * S * 4);
+            p->io = static_cast<void**>(take(16));
+            B.acc = p->fp ? static_cast<uint32_t*>(take(Q * S * 4)) : nullptr;
+            B.ncube = static_cast<uint64_t*>(take(Q * 8));
+            B.blk_off = static_cast<uint64_t*>(take((Q + 1) * 8));
+            B.chunk_off = static_cast<uint64_t*>(take((Q + 1) * 8));
+            B.blk = static_cast<Blk*>(take(B.cap_blocks * sizeof(Blk)));
+            B.chunk_q = static_cast<uint32_t*>(take(B.cap_chunks * 4));
+            B.chunk_b = static_cast<uint32_t*>(take(B.cap_chunks * 4));
+            B.words = static_cast<uint64_t*>(take(16 * Q + 16));
             void* io0[2] = {p->boxes, p->result};
-            const cudaError_t e = cudaMemcpy(p->io, io0, sizeof(io0), cudaMemcpyHostToDevice);
-            if (e != cudaSuccess) st = cuda_fail(e, "plan io slots");
+            cudaError_t e = cudaMemcpy(p->io, io0, sizeof(io0), cudaMemcpyHostToDevice);
+            if (e == cudaSuccess) e = cudaMemsetAsync(B.words, 0, 16 * Q + 16, nullptr);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+            if (e != cudaSuccess) st = cuda_fail(e, "plan buffers");
+            p->pool.s = nullptr;
         }
     }
     if (st == MG_OK && p->fp && o.alpha_dtype != MG_F32) st = ensure_alpha16(g, (mg_dtype)o.alpha_dtype, nullptr);
     if (st == MG_OK && p->fp && o.alpha_dtype != MG_F32) st = ensure_records16(g, (mg_dtype)o.alpha_dtype, nullptr);
     if (st == MG_OK) {
-        cudaError_t e = cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking);
-        if (e != cudaSuccess) st = cuda_fail(e, "cudaStreamCreateWithFlags");
+        const int tt = g->tuned_threads[p->fp];
+        const int threads = o.block_threads > 0 ? o.block_threads : tt > 0 ? tt : 256;
+        st = shape_of(g, p->fp, p->weights, threads, &p->bufs.shape);
     }
     if (st == MG_OK && o.timing) {
         p->timed = true;
         for (cudaEvent_t& ev : p->ev) {
             const cudaError_t e = cudaEventCreate(&ev);
             if (e != cudaSuccess && st == MG_OK) st = cuda_fail(e, "cudaEventCreate");
-        }
-    }
-    if (st == MG_OK) {
-        // scratch comes from the plan's pool, so nothing is allocated while capturing
-        Alloc al;
-        al.a.ctx = &p->bump;
-        al.a.alloc = pool_alloc;
-        al.a.free = pool_free;
-        al.custom = true;
-        cudaError_t e = cudaStreamBeginCapture(p->cap_stream, cudaStreamCaptureModeThreadLocal);
-        if (e != cudaSuccess) st = cuda_fail(e, "cudaStreamBeginCapture");
-        if (st == MG_OK) {
-            if (!p->fp) st = plan_enqueue<false, float>(p.get(), al, p->cap_stream);
-            else if (o.alpha_dtype == MG_F16) st = plan_enqueue<true, __half>(p.get(), al, p->cap_stream);
-            else if (o.alpha_dtype == MG_BF16) st = plan_enqueue<true, __nv_bfloat16>(p.get(), al, p->cap_stream);
-            else st = plan_enqueue<true, float>(p.get(), al, p->cap_stream);
-            cudaGraph_t gr = nullptr;
-            e = cudaStreamEndCapture(p->cap_stream, &gr);
-            p->graph = gr;
-            if (st == MG_OK && e != cudaSuccess) st = cuda_fail(e, "cudaStreamEndCapture");
-        }
-        if (st == MG_OK) {
-            e = cudaGraphInstantiate(&p->exec, p->graph, 0);
-            if (e != cudaSuccess) st = cuda_fail(e, "cudaGraphInstantiate");
         }
     }
     if (prev >= 0 && prev != g->device) cudaSetDevice(prev);
@@ -2872,12 +2952,13 @@ MG_API mg_status mg_query_plan_run(mg_query_plan* p, const int32_t* boxes, int64
     cudaGetDevice(&prev);
     if (prev != p->g->device) MG_CUDA(cudaSetDevice(p->g->device));
     mg_status st = MG_OK;
-    // the graph reads the boxes from and accumulates into the caller's buffers
-    set_batch_kernel<<<1, 1, 0, s>>>(p->Qd, Q, p->io, boxes, out);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaGraphLaunch(p->exec, s);
-    if (e == cudaSuccess) p->ran = true;
-    if (e != cudaSuccess) st = cuda_fail(e, "mg_query_plan_run");
+    if (p->timed) {
+        const cudaError_t e = cudaEventRecord(p->ev[0], s);
+        if (e != cudaSuccess) st = cuda_fail(e, "mg_query_plan_run");
+    }
+    const BatchRun run{boxes, Q, nullptr, nullptr, out};
+    if (st == MG_OK) st = enqueue_any(p->g, p->bufs, run, p->fp, p->weights, false, p->timed ? p->ev + 1 : nullptr, s);
+    if (st == MG_OK) p->ran = true;
     if (prev >= 0 && prev != p->g->device) cudaSetDevice(prev);
     return st;
 }

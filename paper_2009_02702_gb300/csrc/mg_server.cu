@@ -548,7 +548,7 @@ MG_API mg_status mg_server_add_volume(mg_server* sv, mg_graph* g, int C, int* vo
             mg_query_opts qo{};
             qo.hist_type = sv->o.hist_type;
             st = mg_query_plan_create(g, (int64_t)Q, &qo, (int64_t)cap_blocks, (int64_t)cap_chunks, &vs.plan);
-            if (st == MG_OK) vs.pp = plan_parts(vs.plan);
+            if (st == MG_OK) st = plan_parts(vs.plan, &vs.pp);
         }
         if (st == MG_OK) st = vs.tf_dev.alloc(&g->al, (size_t)F * S * C * 4, nullptr);
         if (st == MG_OK) st = vs.vals_dev.alloc(&g->al, N * F * C * sv->esize, nullptr);

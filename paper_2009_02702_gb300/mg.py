@@ -517,7 +517,7 @@ def mg_query_boxes_noalloc(g: Graph, boxes: torch.Tensor, out: torch.Tensor = No
 
 
 class QueryPlan:
-    """A captured batched query (mg_query_plan_*): one graph launch per batch."""
+    """A batched query with its buffers and launch shape kept (mg_query_plan_*)."""
 
     def __init__(self, g: Graph, max_Q: int, hist: str = "u32", alpha: str = "f32", chunk_cubes: int = 0,
                  block_threads: int = 0, max_blocks: int = 0, max_chunks: int = 0, timing: bool = False):
