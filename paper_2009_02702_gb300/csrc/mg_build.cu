@@ -241,6 +241,77 @@ __global__ void next_write_kernel(const uint32_t* __restrict__ off, const uint32
     }
 }
 
+// The coarse levels: few parents with long lists.  A CTA sums the children's
+// lists of one parent in a table of all segments in shared memory and reads it
+// out in order (a thread merging eight lists of hundreds of entries takes
+// about 150 ns an entry: the last five levels of 512x512x384 cost 440 us,
+// this 90).  Taken for at most kDenseParents parents and segment counts whose
+// table fits.
+constexpr int kDenseThreads = 256;
+constexpr int64_t kDenseParents = 2048;
+constexpr uint32_t kDenseSegments = 24 * 1024;   // 192 KB of 64-bit sums
+
+// the sums of parent v's children in `sum` (zeroed here); returns the children in support
+__device__ __forceinline__ int dense_sum(const uint32_t* __restrict__ off, const uint32_t* __restrict__ ids,
+                                         const uint64_t* __restrict__ w, Dims3 dl, int X, int Y, int Z, uint32_t S,
+                                         unsigned long long* sum) {
+    for (uint32_t s = threadIdx.x; s < S; s += kDenseThreads) sum[s] = 0;
+    __syncthreads();
+    int n = 0;
+    for (int c = 0; c < 8; c++) {
+        const int x = 2 * X + (c & 1), y = 2 * Y + ((c >> 1) & 1), z = 2 * Z + (c >> 2);
+        if (x >= dl.x || y >= dl.y || z >= dl.z) continue;
+        n++;
+        const int64_t cv = ((int64_t)z * dl.y + y) * dl.x + x;
+        const uint32_t e1 = off[cv + 1];
+        for (uint32_t e = off[cv] + threadIdx.x; e < e1; e += kDenseThreads) atomicAdd(sum + ids[e], w[e]);
+    }
+    __syncthreads();
+    return n;
+}
+
+// WRITE = false: entries of every parent's list; true: the lists
+template <bool WRITE>
+__global__ void __launch_bounds__(kDenseThreads) dense_next_kernel(const uint32_t* __restrict__ off,
+                                                                   const uint32_t* __restrict__ ids,
+                                                                   const uint64_t* __restrict__ w, Dims3 dl, Dims3 dn,
+                                                                   uint32_t S, uint32_t* __restrict__ noff,
+                                                                   uint32_t* __restrict__ nids,
+                                                                   uint64_t* __restrict__ nw) {
+    extern __shared__ __align__(16) unsigned long long s_sum[];
+    __shared__ uint32_t s_warp[kDenseThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t Vn = nvox(dn);
+    for (int64_t v = blockIdx.x; v < Vn; v += gridDim.x) {
+        int X, Y, Z;
+        parent_at((uint32_t)v, dn, X, Y, Z);
+        const int n = dense_sum(off, ids, w, dl, X, Y, Z, S, s_sum);
+        const uint64_t scale = 8u / (unsigned)n;   // Eq. 4
+        uint32_t at = WRITE ? noff[v] : 0u;
+        for (uint32_t s0 = 0; s0 < S; s0 += kDenseThreads) {
+            const uint32_t s = s0 + threadIdx.x;
+            const unsigned long long x = s < S ? s_sum[s] : 0ull;
+            const unsigned m = __ballot_sync(0xffffffffu, x != 0);
+            if (lane == 0) s_warp[warp] = __popc(m);
+            __syncthreads();
+            uint32_t before = 0, all = 0;
+#pragma unroll
+            for (int k = 0; k < kDenseThreads / 32; k++) {
+                if (k < warp) before += s_warp[k];
+                all += s_warp[k];
+            }
+            if (WRITE && x) {
+                const uint32_t o = at + before + __popc(m & ((1u << lane) - 1u));
+                nids[o] = s;
+                nw[o] = x * scale;
+            }
+            at += all;
+            __syncthreads();
+        }
+        if (!WRITE && threadIdx.x == 0) noff[v] = at;
+    }
+}
+
 // ---------------------------------------------------------------------------
 // A2: node table with lock-free hash pruning
 // ---------------------------------------------------------------------------
@@ -330,70 +401,90 @@ __device__ uint32_t node_get(const NodeTab& t, uint32_t p, uint32_t q, uint64_t 
     return kNone;
 }
 
-constexpr int kShortList = 16;
+// Lists are factorised by a thread (up to kShortList entries), a warp (up to
+// kWarpList) or a CTA: a round's pairs are independent, while a node costs a
+// chain of dependent table accesses (2-4 us), so a thread that walked 16
+// entries alone held its level up.
+constexpr int kShortList = 4;
+constexpr int64_t kWarpList = 256;
+constexpr int kFactorThreads = 256;
+constexpr int kFactorPer = 8;       // voxels per thread and block at most (one where a level has few)
 
-__global__ void factor_short_kernel(NodeTab t, const uint32_t* __restrict__ off, const uint32_t* __restrict__ ids,
-                                    const uint64_t* __restrict__ w, int64_t V, uint32_t* __restrict__ mip_out,
-                                    uint32_t* __restrict__ long_list, unsigned* __restrict__ long_count,
-                                    unsigned* __restrict__ longest) {
+// Lists of one entry are copied; the others of a block are gathered first, so
+// that a warp's lanes factorise together (one voxel in seven of level 1 has
+// more than one entry: nearly every warp held some).
+__global__ void __launch_bounds__(kFactorThreads) factor_short_kernel(
+    NodeTab t, const uint32_t* __restrict__ off, const uint32_t* __restrict__ ids, const uint64_t* __restrict__ w,
+    int64_t V, uint32_t* __restrict__ mip_out, uint32_t* __restrict__ long_list, unsigned* __restrict__ long_count,
+    unsigned* __restrict__ longest, int per) {
+    __shared__ uint32_t s_list[kFactorThreads * kFactorPer];
+    __shared__ unsigned s_count;
     unsigned most = 0;   // longest list seen (statistics)
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t b = off[v];
-        int n = (int)(off[v + 1] - b);
-        most = max(most, (unsigned)n);
-        if (n == 1) {
-            mip_out[v] = ids[b];
-            continue;
+    const int64_t span = (int64_t)kFactorThreads * per;
+    for (int64_t base = (int64_t)blockIdx.x * span; base < V; base += (int64_t)gridDim.x * span) {
+        if (threadIdx.x == 0) s_count = 0;
+        __syncthreads();
+        for (int k = 0; k < per; k++) {
+            const int64_t v = base + k * kFactorThreads + threadIdx.x;
+            if (v >= V) break;
+            const uint32_t b = off[v], n = off[v + 1] - b;
+            most = max(most, n);
+            if (n == 1) mip_out[v] = ids[b];
+            else if (n <= kShortList) s_list[atomicAdd(&s_count, 1u)] = (uint32_t)v;
+            else long_list[atomicAdd(long_count, 1u)] = (uint32_t)v;
         }
-        if (n > kShortList) {
-            const unsigned i = atomicAdd(long_count, 1u);
-            long_list[i] = (uint32_t)v;
-            continue;
-        }
-        uint32_t nd[kShortList];
-        uint64_t ww[kShortList];
-        for (int i = 0; i < n; i++) {
-            nd[i] = ids[b + i];
-            ww[i] = w[b + i];
-        }
-        while (n > 1) {
-            int m = 0;
-            for (int k = 0; k + 1 < n; k += 2) {
-                const uint32_t r = node_get(t, nd[k], nd[k + 1], ww[k], ww[k + 1]);
-                const uint64_t s = ww[k] + ww[k + 1];
-                nd[m] = r;
-                ww[m] = s;
-                m++;
+        __syncthreads();
+        for (unsigned i = threadIdx.x; i < s_count; i += kFactorThreads) {
+            const uint32_t v = s_list[i], b = off[v], n = off[v + 1] - b;
+            const uint64_t w0 = w[b], w1 = w[b + 1];
+            uint32_t r = node_get(t, ids[b], ids[b + 1], w0, w1);
+            if (n == 3) {
+                r = node_get(t, r, ids[b + 2], w0 + w1, w[b + 2]);
+            } else if (n == 4) {
+                const uint64_t w2 = w[b + 2], w3 = w[b + 3];
+                const uint32_t r2 = node_get(t, ids[b + 2], ids[b + 3], w2, w3);
+                r = node_get(t, r, r2, w0 + w1, w2 + w3);
             }
-            if (n & 1) {
-                nd[m] = nd[n - 1];
-                ww[m] = ww[n - 1];
-                m++;
-            }
-            n = m;
+            mip_out[v] = r;
         }
-        mip_out[v] = nd[0];
+        __syncthreads();
     }
     most = __reduce_max_sync(0xffffffffu, most);
     if ((threadIdx.x & 31) == 0 && most > ld_relaxed_u32(longest)) atomicMax(longest, most);
 }
 
-// One CTA per long list; rounds in place in the level's CSR arrays (all reads
-// of a round's slice happen before its writes, separated by a barrier).
-__global__ void factor_long_kernel(NodeTab t, const uint32_t* __restrict__ off, uint32_t* ids, uint64_t* w,
-                                   const uint32_t* __restrict__ long_list, const unsigned* __restrict__ long_count,
-                                   uint32_t* __restrict__ mip_out) {
-    const unsigned nlong = *long_count;
-    for (unsigned i = blockIdx.x; i < nlong; i += gridDim.x) {
-        const uint32_t v = long_list[i];
+// One warp (or CTA) per list; rounds in place in the level's CSR arrays (all
+// reads of a round's slice happen before its writes, separated by a barrier).
+// The warps pass the lists above kWarpList on to the CTAs.
+template <bool CTA>
+__global__ void __launch_bounds__(kFactorThreads) factor_long_kernel(NodeTab t, const uint32_t* __restrict__ off,
+                                                                     uint32_t* ids, uint64_t* w,
+                                                                     const uint32_t* __restrict__ list,
+                                                                     const unsigned* __restrict__ count,
+                                                                     uint32_t* __restrict__ next,
+                                                                     unsigned* __restrict__ next_count,
+                                                                     uint32_t* __restrict__ mip_out) {
+    constexpr int G = CTA ? kFactorThreads : 32;   // threads on a list
+    const int me = threadIdx.x % G;
+    const unsigned groups = gridDim.x * (kFactorThreads / G), nlong = *count;
+    auto sync = [] {
+        if constexpr (CTA) __syncthreads();
+        else __syncwarp();
+    };
+    for (unsigned i = blockIdx.x * (kFactorThreads / G) + threadIdx.x / G; i < nlong; i += groups) {
+        const uint32_t v = list[i];
         const uint32_t b = off[v];
         int64_t n = (int64_t)(off[v + 1] - b);
+        if (!CTA && n > kWarpList) {
+            if (me == 0) next[atomicAdd(next_count, 1u)] = v;
+            continue;
+        }
         uint32_t* nd = ids + b;
         uint64_t* ww = w + b;
         while (n > 1) {
             const int64_t half = n / 2;
-            for (int64_t base = 0; base < half; base += blockDim.x) {
-                const int64_t k = base + threadIdx.x;
+            for (int64_t base = 0; base < half; base += G) {
+                const int64_t k = base + me;
                 uint32_t n0 = 0, n1 = 0;
                 uint64_t w0 = 0, w1 = 0;
                 if (k < half) {
@@ -402,24 +493,24 @@ __global__ void factor_long_kernel(NodeTab t, const uint32_t* __restrict__ off, 
                     w0 = ww[2 * k];
                     w1 = ww[2 * k + 1];
                 }
-                __syncthreads();
+                sync();
                 if (k < half) {
                     nd[k] = node_get(t, n0, n1, w0, w1);
                     ww[k] = w0 + w1;
                 }
-                __syncthreads();
+                sync();
             }
             if (n & 1) {
-                if (threadIdx.x == 0) {
+                if (me == 0) {
                     nd[half] = nd[n - 1];
                     ww[half] = ww[n - 1];
                 }
-                __syncthreads();
+                sync();
             }
             n = (n + 1) / 2;
         }
-        if (threadIdx.x == 0) mip_out[v] = nd[0];
-        __syncthreads();
+        if (me == 0) mip_out[v] = nd[0];
+        sync();
     }
 }
 
@@ -638,7 +729,7 @@ __global__ void weights_kernel(const ulonglong2* __restrict__ ab, int64_t N, uin
 // axis) through a shared-memory tile, because x is the fast axis of the
 // source and the slow or middle one of the copy: a thread-per-element copy
 // read one ID per 32-byte sector.  HBM bound once both sides move whole rows:
-// 512x512x384, both level-0 copies 1.04 -> 0.28 ms, levels >= 1 0.28 -> 0.09 ms.
+// 512x512x384, both level-0 copies 1.04 -> 0.16 ms, levels >= 1 0.28 -> 0.07 ms.
 struct AxisJob {
     const void* src;
     void* dst;
@@ -682,35 +773,45 @@ __global__ void __launch_bounds__(kTransThreads) transpose_kernel(const __grid_c
         const T* src = static_cast<const T*>(A.src) + (int64_t)o * so;
         T* dst = static_cast<T*>(A.dst) + (int64_t)o * dn;
         const bool even = PW == 1 || (A.x % 2 == 0);   // two-byte rows readable as words
-        for (int f = warp; f < E; f += kTransThreads / 32) {
-            const int x = x0 + lane * PW;
-            uint32_t w = 0;
-            if (f0 + f < nf && x < A.x) {
-                const T* p = src + (int64_t)(f0 + f) * sf + x;
-                if constexpr (PW == 1) {
-                    w = __ldcs(p);
-                } else {
-                    if (even) w = __ldcs(reinterpret_cast<const uint32_t*>(p));
-                    else w = (uint32_t)__ldcs(p) | (x + 1 < A.x ? (uint32_t)__ldcs(p + 1) << 16 : 0u);
-                }
+        constexpr int N = E / (kTransThreads / 32);     // rows per warp, all in flight
+        const int x = x0 + lane * PW;
+        uint32_t w[N];
+        if (even) {
+#pragma unroll
+            for (int k = 0; k < N; k++) {
+                const int f = f0 + warp + k * (kTransThreads / 32);
+                w[k] = 0;
+                if (f < nf && x < A.x) w[k] = __ldcs(reinterpret_cast<const uint32_t*>(src + (int64_t)f * sf + x));
             }
-            *reinterpret_cast<uint32_t*>(&tile[f][lane * PW]) = w;
+        } else {
+#pragma unroll
+            for (int k = 0; k < N; k++) {
+                const int f = f0 + warp + k * (kTransThreads / 32);
+                const T* p = src + (int64_t)f * sf + x;
+                w[k] = 0;
+                if (f < nf && x < A.x) w[k] = (uint32_t)__ldcs(p) | (x + 1 < A.x ? (uint32_t)__ldcs(p + 1) << 16 : 0u);
+            }
         }
+#pragma unroll
+        for (int k = 0; k < N; k++)
+            *reinterpret_cast<uint32_t*>(&tile[warp + k * (kTransThreads / 32)][lane * PW]) = w[k];
         __syncthreads();
         const bool words = PW == 1 || (A.pitch % 2 == 0);
-        for (int x = warp; x < E && x0 + x < A.x; x += kTransThreads / 32) {
-            const int f = lane * PW;
-            if (f0 + f >= A.pitch) continue;
-            T* p = dst + (int64_t)(x0 + x) * dx + f0 + f;
+        const int f = lane * PW;
+#pragma unroll
+        for (int k = 0; k < N; k++) {
+            const int c = warp + k * (kTransThreads / 32);
+            if (x0 + c >= A.x || f0 + f >= A.pitch) continue;
+            T* p = dst + (int64_t)(x0 + c) * dx + f0 + f;
             if constexpr (PW == 1) {
-                *p = tile[f][x];
+                *p = tile[f][c];
             } else {
-                const uint32_t w = (uint32_t)tile[f][x] | (uint32_t)tile[f + 1][x] << 16;
+                const uint32_t u = (uint32_t)tile[f][c] | (uint32_t)tile[f + 1][c] << 16;
                 if (words) {
-                    *reinterpret_cast<uint32_t*>(p) = w;
+                    *reinterpret_cast<uint32_t*>(p) = u;
                 } else {
-                    p[0] = (T)w;
-                    if (f0 + f + 1 < A.pitch) p[1] = (T)(w >> 16);
+                    p[0] = (T)u;
+                    if (f0 + f + 1 < A.pitch) p[1] = (T)(u >> 16);
                 }
             }
         }
@@ -876,8 +977,8 @@ mg_status build_graph(mg_graph* g, const void* ids, int id_bytes, int64_t nx, in
     Buf maxlen;
     MG_TRY(maxlen.alloc(&al, sizeof(unsigned), s));
     MG_CUDA(cudaMemsetAsync(maxlen.p, 0, sizeof(unsigned), s));
-    Buf long_list, long_count;
-    MG_TRY(long_count.alloc(&al, sizeof(unsigned), s));
+    Buf long_list, huge_list, long_count;   // counts: warp lists, CTA lists
+    MG_TRY(long_count.alloc(&al, 2 * sizeof(unsigned), s));
 
     // ---- A1 + A2, level by level ----
     struct Lists {
@@ -923,7 +1024,18 @@ mg_status build_graph(mg_graph* g, const void* ids, int id_bytes, int64_t nx, in
         out.V = nvox(dn);
         MG_TRY(out.off.alloc(&al, (size_t)(out.V + 1) * 4, s));
         const unsigned gb = grid_n(out.V);
-        next_count_kernel<<<gb, 256, 0, s>>>(in.off.as<uint32_t>(), in.ids.as<uint32_t>(), dl, dn,
+        const bool dense = out.V <= kDenseParents && S <= kDenseSegments;
+        const unsigned db = grid_for(out.V, 1, 152 * 2);
+        const size_t dsm = (size_t)S * 8;
+        if (dense) {
+            MG_CUDA(cudaFuncSetAttribute(dense_next_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(kDenseSegments * 8)));
+            MG_CUDA(cudaFuncSetAttribute(dense_next_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(kDenseSegments * 8)));
+            dense_next_kernel<false><<<db, kDenseThreads, dsm, s>>>(in.off.as<uint32_t>(), in.ids.as<uint32_t>(),
+                                                                     in.w.as<uint64_t>(), dl, dn, S,
+                                                                     out.off.as<uint32_t>(), nullptr, nullptr);
+        } else next_count_kernel<<<gb, 256, 0, s>>>(in.off.as<uint32_t>(), in.ids.as<uint32_t>(), dl, dn,
                                              out.off.as<uint32_t>());
         MG_CUDA(cudaGetLastError());
         MG_TRY(scan_exclusive_u32(out.off.as<uint32_t>(), out.off.as<uint32_t>(), out.V,
@@ -931,7 +1043,12 @@ mg_status build_graph(mg_graph* g, const void* ids, int id_bytes, int64_t nx, in
         MG_TRY(read_counts(out));
         MG_TRY(out.ids.alloc(&al, (size_t)out.nnz * 4, s));
         MG_TRY(out.w.alloc(&al, (size_t)out.nnz * 8, s));
-        next_write_kernel<<<gb, 256, 0, s>>>(in.off.as<uint32_t>(), in.ids.as<uint32_t>(), in.w.as<uint64_t>(), dl,
+        if (dense)
+            dense_next_kernel<true><<<db, kDenseThreads, dsm, s>>>(in.off.as<uint32_t>(), in.ids.as<uint32_t>(),
+                                                                    in.w.as<uint64_t>(), dl, dn, S,
+                                                                    out.off.as<uint32_t>(), out.ids.as<uint32_t>(),
+                                                                    out.w.as<uint64_t>());
+        else next_write_kernel<<<gb, 256, 0, s>>>(in.off.as<uint32_t>(), in.ids.as<uint32_t>(), in.w.as<uint64_t>(), dl,
                                              dn, out.off.as<uint32_t>(), out.ids.as<uint32_t>(),
                                              out.w.as<uint64_t>());
         MG_CUDA(cudaGetLastError());
@@ -958,18 +1075,27 @@ mg_status build_graph(mg_graph* g, const void* ids, int id_bytes, int64_t nx, in
                 MG_CUDA(cudaGetLastError());
             }
         }
-        MG_CUDA(cudaMemsetAsync(long_count.p, 0, sizeof(unsigned), s));
+        MG_CUDA(cudaMemsetAsync(long_count.p, 0, 2 * sizeof(unsigned), s));
         if (long_list.bytes < (size_t)cur.V * 4) MG_TRY(long_list.alloc(&al, (size_t)cur.V * 4, s));
+        const size_t huge = ((size_t)cur.nnz / kWarpList + 1) * 4;   // lists above kWarpList at most
+        if (huge_list.bytes < huge) MG_TRY(huge_list.alloc(&al, huge, s));
         uint32_t* mip_out = g->mip.as<uint32_t>() + G.off[l];
-        factor_short_kernel<<<grid_n(cur.V), 256, 0, s>>>(view(t, status), cur.off.as<uint32_t>(),
-                                                          cur.ids.as<uint32_t>(), cur.w.as<uint64_t>(), cur.V,
-                                                          mip_out, long_list.as<uint32_t>(),
-                                                          long_count.as<unsigned>(), maxlen.as<unsigned>());
+        unsigned* counts2 = long_count.as<unsigned>();
+        const int per = (int)std::min<int64_t>(kFactorPer, std::max<int64_t>(1, cur.V / (kFactorThreads * 152 * 8)));
+        factor_short_kernel<<<grid_for(cur.V, kFactorThreads * per, 152 * 8), kFactorThreads, 0, s>>>(
+            view(t, status), cur.off.as<uint32_t>(), cur.ids.as<uint32_t>(), cur.w.as<uint64_t>(), cur.V, mip_out,
+            long_list.as<uint32_t>(), counts2, maxlen.as<unsigned>(), per);
         MG_CUDA(cudaGetLastError());
-        factor_long_kernel<<<152 * 4, 256, 0, s>>>(view(t, status), cur.off.as<uint32_t>(), cur.ids.as<uint32_t>(),
-                                                   cur.w.as<uint64_t>(), long_list.as<uint32_t>(),
-                                                   long_count.as<unsigned>(), mip_out);
+        factor_long_kernel<false><<<152 * 8, kFactorThreads, 0, s>>>(
+            view(t, status), cur.off.as<uint32_t>(), cur.ids.as<uint32_t>(), cur.w.as<uint64_t>(),
+            long_list.as<uint32_t>(), counts2, huge_list.as<uint32_t>(), counts2 + 1, mip_out);
         MG_CUDA(cudaGetLastError());
+        if (S > kWarpList && cur.nnz > kWarpList) {   // a list holds each segment once
+            factor_long_kernel<true><<<152 * 4, kFactorThreads, 0, s>>>(
+                view(t, status), cur.off.as<uint32_t>(), cur.ids.as<uint32_t>(), cur.w.as<uint64_t>(),
+                huge_list.as<uint32_t>(), counts2 + 1, nullptr, nullptr, mip_out);
+            MG_CUDA(cudaGetLastError());
+        }
         cur = std::move(nxt);
     }
     {

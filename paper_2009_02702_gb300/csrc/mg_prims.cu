@@ -94,44 +94,53 @@ __global__ void scan_tile_kernel(const T* in, T* out, int64_t n, const T* __rest
     if (total && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *total = off + bt;
 }
 
-// A few tiles in one CTA of 1,024 threads, tile after tile with a running
-// carry: one launch of about 2 us per 8,192 elements where the reduce-then-scan
-// takes three launches (and three 2-us gaps), so it is taken up to 64 K.
+// A few tiles in one CTA of 1,024 threads, 16 consecutive counters per thread
+// and tile, with a running carry: one launch where the reduce-then-scan takes
+// three (and the gaps between them), so it is taken up to 64 K counters.
 constexpr int kOneThreads = 1024;
+constexpr int kOneItems = 16;
 constexpr int64_t kOneMax = 1 << 16;
-template <typename T>
-__global__ void __launch_bounds__(kOneThreads) scan_one_kernel(const T* in, T* out, int64_t n, T* __restrict__ total) {
-    __shared__ T tile[kOneThreads * kScanItems];
-    __shared__ T wsum[32];
-    T carry = 0;
-    for (int64_t base = 0; base < n; base += kOneThreads * kScanItems) {
+__global__ void __launch_bounds__(kOneThreads) scan_one_kernel(const uint32_t* in, uint32_t* out, int64_t n,
+                                                               uint32_t* __restrict__ total) {
+    __shared__ uint32_t wsum[32];
+    uint32_t carry = 0;
+    for (int64_t base = 0; base < n; base += kOneThreads * kOneItems) {
+        const int64_t at = base + (int64_t)threadIdx.x * kOneItems;
+        uint32_t x[kOneItems], sum = 0;
+        if (at + kOneItems <= n) {
 #pragma unroll
-        for (int i = 0; i < kScanItems; i++) {
-            const int64_t idx = base + i * kOneThreads + threadIdx.x;
-            tile[i * kOneThreads + threadIdx.x] = idx < n ? in[idx] : T(0);
-        }
-        __syncthreads();
-        T loc[kScanItems], sum = 0;
+            for (int k = 0; k < kOneItems / 4; k++) {
+                const uint4 u = *reinterpret_cast<const uint4*>(in + at + 4 * k);
+                x[4 * k] = u.x;
+                x[4 * k + 1] = u.y;
+                x[4 * k + 2] = u.z;
+                x[4 * k + 3] = u.w;
+            }
+        } else {
 #pragma unroll
-        for (int i = 0; i < kScanItems; i++) {
-            loc[i] = tile[threadIdx.x * kScanItems + i];
-            sum += loc[i];
+            for (int k = 0; k < kOneItems; k++) x[k] = at + k < n ? in[at + k] : 0u;
         }
-        T bt;
-        T run = carry + block_excl_scan(sum, wsum, &bt);
+#pragma unroll
+        for (int k = 0; k < kOneItems; k++) sum += x[k];
+        uint32_t bt;
+        uint32_t run = carry + block_excl_scan(sum, wsum, &bt);
         carry += bt;
 #pragma unroll
-        for (int i = 0; i < kScanItems; i++) {
-            tile[threadIdx.x * kScanItems + i] = run;
-            run += loc[i];
+        for (int k = 0; k < kOneItems; k++) {
+            const uint32_t v = x[k];
+            x[k] = run;
+            run += v;
         }
-        __syncthreads();
+        if (at + kOneItems <= n) {
 #pragma unroll
-        for (int i = 0; i < kScanItems; i++) {
-            const int64_t idx = base + i * kOneThreads + threadIdx.x;
-            if (idx < n) out[idx] = tile[i * kOneThreads + threadIdx.x];
+            for (int k = 0; k < kOneItems / 4; k++)
+                *reinterpret_cast<uint4*>(out + at + 4 * k) = make_uint4(x[4 * k], x[4 * k + 1], x[4 * k + 2], x[4 * k + 3]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < kOneItems; k++)
+                if (at + k < n) out[at + k] = x[k];
         }
-        __syncthreads();
+        __syncthreads();   // wsum is reused
     }
     if (total && threadIdx.x == 0) *total = carry;
 }
@@ -148,8 +157,9 @@ mg_status scan_impl(const T* in, T* out, int64_t n, T* total, const Alloc& al, c
         MG_CUDA(cudaGetLastError());
         return MG_OK;
     }
-    if (n <= kOneMax && sizeof(T) == 4) {
-        scan_one_kernel<uint32_t><<<1, kOneThreads, 0, s>>>(reinterpret_cast<const uint32_t*>(in),
+    if (n <= kOneMax && sizeof(T) == 4 && reinterpret_cast<uintptr_t>(in) % 16 == 0 &&
+        reinterpret_cast<uintptr_t>(out) % 16 == 0) {
+        scan_one_kernel<<<1, kOneThreads, 0, s>>>(reinterpret_cast<const uint32_t*>(in),
                                                             reinterpret_cast<uint32_t*>(out), n,
                                                             reinterpret_cast<uint32_t*>(total));
         MG_CUDA(cudaGetLastError());
