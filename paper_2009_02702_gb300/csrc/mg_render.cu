@@ -15,47 +15,83 @@ struct Geom {
     int64_t off[MG_MAX_LEVELS];
 };
 
-__device__ __forceinline__ int64_t floor_coord(float x, int32_t d0) {
+__device__ __forceinline__ int32_t floor_coord(float x, int32_t d0) {
     float xc = x;
     if (!(xc >= 0.f)) xc = 0.f;                  // negatives and NaN
     if (xc > (float)d0) xc = (float)d0;
-    return (int64_t)xc;                         // truncation is the floor for xc >= 0
+    return (int32_t)xc;                         // truncation is the floor for xc >= 0
 }
 
 // 128-thread CTAs of at most 32 registers a thread: one fits beside a
 // persistent query kernel that leaves 4,096 registers of an SM free, so a
 // lookup issued on another stream runs concurrently with it
 constexpr int kLookupThreads = 128;
+// samples per thread: a lookup is three dependent loads (sample, ID, row), and
+// two chains in flight per thread hide more of them than one
+constexpr int kLookupSamples = 2;
 
-template <typename RowT>
-__global__ void __launch_bounds__(kLookupThreads, 16) lookup_kernel(Geom G, const void* __restrict__ mip0, const uint32_t* __restrict__ mip,
-                              const float4* __restrict__ samples, int64_t P, const RowT* __restrict__ vals,
-                              int words, RowT* __restrict__ out) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= P) return;
-    const float4 smp = __ldg(samples + i);
+// index of the voxel of a sample in its level (32-bit: a volume holds fewer
+// than 2^32 voxels), and the level
+__device__ __forceinline__ uint32_t sample_voxel(const Geom& G, const float4& smp, int& l) {
     const float t = smp.w + 0.5f;                 // nearest level
-    int l;
     if (!(t >= 0.f)) l = 0;
     else if (t >= (float)(G.L - 1)) l = G.L - 1;
     else l = (int)t;
-    int64_t v[3];
+    uint32_t v[3];
     const float c[3] = {smp.x, smp.y, smp.z};
 #pragma unroll
-    for (int k = 0; k < 3; k++) {
-        const int64_t x = floor_coord(c[k], G.dims[0][k]) >> l;
-        v[k] = min(x, (int64_t)G.dims[l][k] - 1);
-    }
-    const int64_t idx = (v[2] * G.dims[l][1] + v[1]) * G.dims[l][0] + v[0];
-    uint32_t node;
+    for (int k = 0; k < 3; k++)
+        v[k] = (uint32_t)min(floor_coord(c[k], G.dims[0][k]) >> l, G.dims[l][k] - 1);
+    return (v[2] * (uint32_t)G.dims[l][1] + v[1]) * (uint32_t)G.dims[l][0] + v[0];
+}
+
+__device__ __forceinline__ uint32_t voxel_node(const Geom& G, const void* __restrict__ mip0,
+                                               const uint32_t* __restrict__ mip, int l, uint32_t idx) {
     if (l == 0)
-        node = G.id0_bytes == 2 ? (uint32_t)__ldg(static_cast<const uint16_t*>(mip0) + idx)
+        return G.id0_bytes == 2 ? (uint32_t)__ldg(static_cast<const uint16_t*>(mip0) + idx)
                                 : __ldg(static_cast<const uint32_t*>(mip0) + idx);
-    else
-        node = __ldg(mip + G.off[l] + idx);
-    const RowT* src = vals + (int64_t)node * words;
-    RowT* dst = out + i * words;
-    for (int w = 0; w < words; w++) dst[w] = __ldg(src + w);
+    return __ldg(mip + G.off[l] + idx);
+}
+
+template <typename RowT>
+__global__ void __launch_bounds__(kLookupThreads, 16) lookup_kernel(const __grid_constant__ Geom G,
+                                                                    const void* __restrict__ mip0,
+                                                                    const uint32_t* __restrict__ mip,
+                                                                    const float4* __restrict__ samples, int64_t P,
+                                                                    const RowT* __restrict__ vals, int words,
+                                                                    RowT* __restrict__ out) {
+    constexpr int N = kLookupSamples;
+    const int64_t i0 = (int64_t)blockIdx.x * (kLookupThreads * N) + threadIdx.x;
+    uint32_t node[N];
+    {
+        float4 smp[N];
+#pragma unroll
+        for (int k = 0; k < N; k++)
+            smp[k] = i0 + k * kLookupThreads < P ? __ldcs(samples + i0 + k * kLookupThreads) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < N; k++) {
+            int l;
+            const uint32_t idx = sample_voxel(G, smp[k], l);
+            node[k] = voxel_node(G, mip0, mip, l, idx);   // (past the end: the volume's first voxel)
+        }
+    }
+    if (words == 1) {
+        RowT v[N];
+#pragma unroll
+        for (int k = 0; k < N; k++) v[k] = __ldg(vals + node[k]);
+#pragma unroll
+        for (int k = 0; k < N; k++)
+            if (i0 + k * kLookupThreads < P) out[i0 + k * kLookupThreads] = v[k];
+        return;
+    }
+#pragma unroll
+    for (int k = 0; k < N; k++) {
+        const int64_t i = i0 + k * kLookupThreads;
+        if (i >= P) return;
+        const RowT* src = vals + (int64_t)node[k] * words;
+        RowT* dst = out + i * words;
+        for (int w = 0; w < words; w++) dst[w] = __ldg(src + w);
+    }
 }
 
 // k frames in one launch: samples [off[j], off[j+1]) belong to frame j and
@@ -77,26 +113,9 @@ __global__ void __launch_bounds__(kLookupThreads, 16) lookup_multi_kernel(Geom G
     if (i >= F.off[k]) return;
     int j = 0;
     while (j + 1 < k && F.off[j + 1] <= i) j++;
-    const float4 smp = __ldg(samples + i);
-    const float t = smp.w + 0.5f;
     int l;
-    if (!(t >= 0.f)) l = 0;
-    else if (t >= (float)(G.L - 1)) l = G.L - 1;
-    else l = (int)t;
-    int64_t v[3];
-    const float c[3] = {smp.x, smp.y, smp.z};
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        const int64_t x = floor_coord(c[a], G.dims[0][a]) >> l;
-        v[a] = min(x, (int64_t)G.dims[l][a] - 1);
-    }
-    const int64_t idx = (v[2] * G.dims[l][1] + v[1]) * G.dims[l][0] + v[0];
-    uint32_t node;
-    if (l == 0)
-        node = G.id0_bytes == 2 ? (uint32_t)__ldg(static_cast<const uint16_t*>(mip0) + idx)
-                                : __ldg(static_cast<const uint32_t*>(mip0) + idx);
-    else
-        node = __ldg(mip + G.off[l] + idx);
+    const uint32_t idx = sample_voxel(G, __ldg(samples + i), l);
+    const uint32_t node = voxel_node(G, mip0, mip, l, idx);
     const RowT* src = vals + ((int64_t)node * k + j) * words;
     RowT* dst = out + i * words;
     for (int w = 0; w < words; w++) dst[w] = __ldg(src + w);
@@ -156,7 +175,7 @@ mg_status render_lookup(const mg_graph* g, const void* vals, int C, mg_dtype dt,
     if (!aligned(samples, 16)) return fail(MG_ERR_INVALID_ARG, "samples must be 16-byte aligned");
     const Geom G = render_geom(g);
     const size_t row = (size_t)C * (dt == MG_F32 ? 4 : 2);
-    const unsigned grid = grid_for(P, kLookupThreads);
+    const unsigned grid = grid_for(P, kLookupThreads * kLookupSamples);
     const float4* sm = reinterpret_cast<const float4*>(samples);
     const uint32_t* mip = g->mip.as<uint32_t>();
     if (row % 16 == 0 && aligned(vals, 16) && aligned(out, 16))
