@@ -144,6 +144,8 @@ _lock = threading.Lock()
 def lib():
     """The loaded libmg.so; raises if it has not been built."""
     global _lib
+    if _lib is not None:   # (the lock and the checks are for the first call only)
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -273,8 +275,15 @@ def _check(st: int):
         raise MGError(st, mg_last_error())
 
 
+# the current stream as a raw handle: 0.3 us where building a Stream object
+# takes 2 us, which a call of a few microseconds on the device waits for
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream=None) -> int:
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream
@@ -396,7 +405,7 @@ def mg_graph_copy_mip(g: Graph, level: int, stream=None):
 def _check_out(out, shape, dtype, device, name="out"):
     """A caller's output tensor is written through its data pointer: it must be
     contiguous, with the shape, dtype and device of the result."""
-    if (not isinstance(out, torch.Tensor) or out.dtype != dtype or tuple(out.shape) != tuple(shape)
+    if (not isinstance(out, torch.Tensor) or out.dtype != dtype or out.shape != shape
             or out.device != device or not out.is_contiguous()):
         raise ValueError("%s must be a contiguous %s tensor of shape %s on %s" % (name, dtype, tuple(shape), device))
     return out
