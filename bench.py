@@ -170,6 +170,27 @@ def cube_levels(boxes, dims):
     return out
 
 
+def footprint_items(boxes, dims):
+    """What the batched query reads for these boxes: (tile records, level-0
+    IDs, higher-level IDs).  A block one cube of a level <= 3 thick whose other
+    extents reach 8 cubes is read as records of 8 x 8 cubes (16 x 16 where both
+    reach 16, levels 0-2); a narrower one at least 16 long, levels 1-3, as
+    records of 16 cubes in a line; all else as IDs."""
+    rec = ids0 = ids = 0
+    for b in boxes:
+        r = [_runs(int(b[k]), int(b[k + 3]), dims[k]) for k in range(3)]
+        L = np.stack([a.ravel() for a in np.meshgrid(*r, indexing="ij")])
+        l = L.min(0)
+        e = np.sort(L - l, 0)
+        cubes = np.left_shift(1, e.sum(0))
+        edge = np.where(l < 3, 4, np.where(l < 4, 3, 0))
+        T = np.where(e[1] >= 3, np.minimum(e[1], edge), np.where((l >= 1) & (l < 4) & (e[2] >= 4), 2, 0))
+        rec += int((cubes >> (2 * T))[T > 0].sum())
+        ids0 += int(cubes[(T == 0) & (l == 0)].sum())
+        ids += int(cubes[(T == 0) & (l > 0)].sum())
+    return rec, ids0, ids
+
+
 def measured_traffic(kernel, cfg_i, Q):
     """DRAM bytes per launch from the committed ncu records (profiles/
     traffic.json: one record per kernel and workload), only while the kernel's
@@ -243,12 +264,13 @@ def query_kernel_name(S, threads, hist="u32"):
 
 
 def query_bytes(boxes_h, dims, S):
-    """Algorithmic bytes of one query launch: the box, every footprint cube's
-    node ID (uint16 at level 0, uint32 above) and the dense u32 row out."""
+    """Algorithmic bytes of one query launch: the box, the tile records and the
+    IDs that cover its footprint (16 bytes a record, 2 a level-0 ID, 4 a higher
+    one) and the dense u32 row out; and the footprint's cubes."""
     lv = cube_levels(boxes_h, dims)
-    id0 = 2 if S <= 65536 else 4
+    rec, ids0, ids = footprint_items(boxes_h, dims)
     Q = len(boxes_h)
-    return 24 * Q + id0 * int(lv[0]) + 4 * int(lv[1:].sum()) + 4 * Q * S, int(lv.sum()), lv
+    return 24 * Q + 16 * rec + 2 * ids0 + 4 * ids + 4 * Q * S, int(lv.sum()), lv
 
 
 def build_graph(mg, cfg_i, dev, dims=None):
