@@ -109,3 +109,24 @@ def test_most_segments_of_a_float_histogram(mg, threads):
     mg.mg_sync_status(g)
     assert np.array_equal(h.astype(np.int64), oracle.box_hist(vol, S, bx).astype(np.int64))
     g.close()
+
+
+@pytest.mark.parametrize("dims,S,third", [((64, 48, 40), 16384, 0.0), ((64, 48, 40), 5, 0.01), ((61, 47, 39), 997, 0.004)])
+def test_tiles_of_two_segments(mg, dims, S, third):
+    # pairs that share and differ in any bits, one segment a single voxel or all but one, and strays among them
+    rng = np.random.default_rng([S, *dims])
+    nx, ny, nz = dims
+    cell = tuple((n + 7) // 8 for n in (nz, ny, nx))
+
+    def spread(v):
+        return v.repeat(8, 0).repeat(8, 1).repeat(8, 2)[:nz, :ny, :nx]
+
+    a, b, share = (spread(v) for v in (rng.integers(0, S, cell), rng.integers(0, S, cell), rng.random(cell) ** 3))
+    vol = np.where(rng.random((nz, ny, nx)) < share, a, b)
+    vol = np.where(rng.random(vol.shape) < third, rng.integers(0, S, vol.shape), vol).astype(np.uint16)
+    g = mg.mg_build(torch.from_numpy(vol).cuda(), S)
+    bx = boxes_at_edges(dims, rng)
+    h = mg.mg_query_boxes(g, torch.from_numpy(bx).cuda()).cpu().numpy()
+    mg.mg_sync_status(g)
+    assert np.array_equal(h.astype(np.int64), oracle.box_hist(vol, S, bx).astype(np.int64))
+    g.close()
