@@ -359,11 +359,33 @@ __device__ __forceinline__ uint64_t gcd64(uint64_t u, uint64_t v) {
     return u << shift;
 }
 
+__device__ __forceinline__ uint32_t gcd32(uint32_t u, uint32_t v) {
+    if (u == 0) return v;
+    if (v == 0) return u;
+    const int shift = __ffs((int)(u | v)) - 1;
+    u >>= __ffs((int)u) - 1;
+    do {
+        v >>= __ffs((int)v) - 1;
+        const uint32_t lo = min(u, v);
+        v = max(u, v) - lo;
+        u = lo;
+    } while (v);
+    return u << shift;
+}
+
 // Eq. 5-6 with Sec. 3.3 re-use: node for the lerp of (p, wp) and (q, wq).
 __device__ uint32_t node_get(const NodeTab& t, uint32_t p, uint32_t q, uint64_t wp, uint64_t wq) {
     if (p >= kDead || q >= kDead) return kNone;   // an earlier failure propagates
-    const uint64_t g = gcd64(wp, wq);
-    const uint64_t a = wp / g, b = wq / g;
+    uint64_t a, b;
+    if (((wp | wq) >> 32) == 0) {   // nearly all: a fraction of the 64-bit steps' latency
+        const uint32_t g = gcd32((uint32_t)wp, (uint32_t)wq);
+        a = (uint32_t)wp / g;
+        b = (uint32_t)wq / g;
+    } else {
+        const uint64_t g = gcd64(wp, wq);
+        a = wp / g;
+        b = wq / g;
+    }
     uint64_t h = key_hash(p, q, a, b) & t.mask;
     uint32_t mine = kNone;
     for (uint64_t probe = 0; probe <= t.mask; probe++) {
