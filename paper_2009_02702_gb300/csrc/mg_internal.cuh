@@ -289,7 +289,8 @@ mg_status plan_parts(mg_query_plan* p, PlanParts* out);
 struct PlanChunk {
     uint32_t chunk, scale;
 };
-PlanChunk plan_chunk(const mg_graph* g, int hist_type, int chunk_cubes, int64_t max_Q, uint64_t cap_chunks);
+PlanChunk plan_chunk(const mg_graph* g, int hist_type, mg_dtype weights, int chunk_cubes, int64_t max_Q,
+                     uint64_t cap_chunks);
 
 // ---------------------------------------------------------------------------
 // small device helpers

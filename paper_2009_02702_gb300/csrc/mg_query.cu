@@ -2024,10 +2024,16 @@ int sm_count(int dev) {
 // 10,000 there 205 / 135 / 104 / 104 / 121; 100,000 on 2048x2048x300 - / - /
 // 1580 / 1290 / 1120.  Below 128 the per-chunk flush outweighs it.  A histogram
 // shared by a CTA (many segments) has 16 warps on a chunk already.
+//
+// With 16-bit weights a chunk flushes two bins a segment and its items touch
+// more of them: it holds at least one item per two segments (1,000 boxes, 1,182
+// segments: 355 / 309 / 303 / 305 us at 256 / 512 / 1,024 / 2,048 items; 300
+// boxes, 353 segments: 113 / 68 / 101 at 128 / 256 / 1,024).
 constexpr uint32_t kDefaultChunk = 2048, kMinChunk = 128;
-uint32_t default_chunk(uint32_t S, int64_t Q) {
+uint32_t default_chunk(uint32_t S, int64_t Q, mg_dtype weights) {
     uint32_t c = kDefaultChunk;
-    while (S <= kWarpHistMax && c > kMinChunk && (int64_t)c > Q * 2 / 7) c /= 2;
+    const uint32_t least = weights == MG_F32 ? kMinChunk : std::max(kMinChunk, (S + 1) / 2);
+    while (S <= kWarpHistMax && c / 2 >= least && (int64_t)c > Q * 2 / 7) c /= 2;
     return c;
 }
 
@@ -2413,6 +2419,23 @@ mg_status shape_of(const mg_graph* g, bool FP, mg_dtype weights, int threads, Ma
     return main_shape<true, float>(g, rec, threads, out);
 }
 
+// Threads of an untuned batch's CTAs.  256 have the smaller register budget and
+// the faster loop; where their histograms leave shared memory for a quarter
+// fewer warps per SM than CTAs of 128 (the loop is bound by latency, so resident
+// warps count), 128.  fp32 histograms of 1,182 segments, 16 against 20 warps:
+// 100,000 boxes 2.98 -> 2.60 ms, with 16-bit weights 17.7 -> 14.7, 1,000 boxes
+// 307 -> 274 us; uint32 counts, 32 against 36: 1.66 at 256, 1.70 at 128; fp32
+// histograms of 353, 40 against 36: 547 us at 256, 574 at 128 (10,000 boxes).
+int default_threads(const mg_graph* g, bool FP, mg_dtype weights) {
+    const bool rec = (weights == MG_F32 ? g->lut_rec : g->rec16[weights == MG_BF16]).p != nullptr;
+    const size_t bins = FP ? 2 : 1, queue = queue_bytes(kQueueShort);
+    if ((g->S * 4 * bins + queue) * 8 > 96 * 1024) return 256;   // a histogram per CTA
+    const size_t each = ((g->S + 3) & ~(size_t)3) * 4 * bins + kDescBytes + (rec ? 0 : queue);
+    const size_t sm = kMaxDynSmem + 1024;                        // a CTA takes 1 KiB more than it asks for
+    auto warps = [&](size_t w, size_t most) { return w * std::min<size_t>(most, sm / (w * each + 1024)); };
+    return 4 * warps(4, WarpKernelBounds<128>::min_ctas) >= 5 * warps(8, WarpKernelBounds<256>::min_ctas) ? 128 : 256;
+}
+
 // Scratch comes from `al`; `words` are two host words for readbacks; `room`,
 // when not null, returns the bytes `al` can still hand out (fixed pools).
 mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, const mg_query_opts& o, void* out,
@@ -2436,8 +2459,11 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
     const uint32_t chunk = o.chunk_cubes > 0 ? (uint32_t)o.chunk_cubes
                            : tuned_c > 0     ? (uint32_t)tuned_c
                            : room            ? kDefaultChunk
-                                             : default_chunk(S, Q);
-    const int threads = o.block_threads > 0 ? o.block_threads : tuned_t > 0 ? tuned_t : 256;
+                                             : default_chunk(S, Q, FP ? (mg_dtype)o.alpha_dtype : MG_F32);
+    const int threads = o.block_threads > 0                ? o.block_threads
+                        : tuned_t > 0                      ? tuned_t
+                        : o.schedule == MG_SCHED_BATCHED   ? default_threads(g, FP, (mg_dtype)o.alpha_dtype)
+                                                           : 256;
     const Geom G = make_geom(g, tile_levels(g, (mg_dtype)o.alpha_dtype));
     unsigned* status = g->status.as<unsigned>();
     mg_graph* gm = const_cast<mg_graph*>(g);
@@ -2812,11 +2838,12 @@ struct mg_query_plan {
 };
 
 namespace mg {
-PlanChunk plan_chunk(const mg_graph* g, int hist_type, int chunk_cubes, int64_t max_Q, uint64_t cap_chunks) {
+PlanChunk plan_chunk(const mg_graph* g, int hist_type, mg_dtype weights, int chunk_cubes, int64_t max_Q,
+                     uint64_t cap_chunks) {
     const int tuned = g->tuned_chunk[hist_type == MG_HIST_F32];
     if (chunk_cubes > 0) return PlanChunk{(uint32_t)chunk_cubes, 1};
     if (tuned > 0) return PlanChunk{(uint32_t)tuned, 1};
-    const uint32_t c = default_chunk(g->S, max_Q), scale = kDefaultChunk / c;
+    const uint32_t c = default_chunk(g->S, max_Q, hist_type == MG_HIST_F32 ? weights : MG_F32), scale = kDefaultChunk / c;
     // the map of the shorter chunks, 8 bytes each, stays within 64 MiB
     if (cap_chunks * scale > (1u << 23)) return PlanChunk{kDefaultChunk, 1};
     return PlanChunk{c, scale};
@@ -2877,7 +2904,7 @@ MG_API mg_status mg_query_plan_create(mg_graph* g, int64_t max_Q, const mg_query
         QueryBufs& B = p->bufs;
         B.cap_blocks = max_blocks > 0 ? (uint64_t)max_blocks : (uint64_t)max_Q * 1024;
         B.cap_chunks = max_chunks > 0 ? (uint64_t)max_chunks : (uint64_t)max_Q * 256;
-        const PlanChunk pc = plan_chunk(g, o.hist_type, o.chunk_cubes, max_Q, B.cap_chunks);
+        const PlanChunk pc = plan_chunk(g, o.hist_type, p->weights, o.chunk_cubes, max_Q, B.cap_chunks);
         B.chunk = pc.chunk;
         B.cap_chunks *= pc.scale;
         if (B.cap_blocks >= (1ull << 32) || B.cap_chunks >= (1ull << 32))
@@ -2920,7 +2947,7 @@ MG_API mg_status mg_query_plan_create(mg_graph* g, int64_t max_Q, const mg_query
     if (st == MG_OK && p->fp && o.alpha_dtype != MG_F32) st = ensure_records16(g, (mg_dtype)o.alpha_dtype, nullptr);
     if (st == MG_OK) {
         const int tt = g->tuned_threads[p->fp];
-        const int threads = o.block_threads > 0 ? o.block_threads : tt > 0 ? tt : 256;
+        const int threads = o.block_threads > 0 ? o.block_threads : tt > 0 ? tt : default_threads(g, p->fp, p->weights);
         st = shape_of(g, p->fp, p->weights, threads, &p->bufs.shape);
     }
     if (st == MG_OK && o.timing) {

@@ -130,3 +130,24 @@ def test_tiles_of_two_segments(mg, dims, S, third):
     mg.mg_sync_status(g)
     assert np.array_equal(h.astype(np.int64), oracle.box_hist(vol, S, bx).astype(np.int64))
     g.close()
+
+
+@pytest.mark.parametrize("S", [352, 1040, 1100, 1200, 1480, 2048])
+def test_default_shapes_of_float_histograms(mg, S):
+    # both CTA sizes that an untuned batch can take, and its chunk lengths; the bound of the 16-bit weights as above
+    dims = (96, 64, 48)
+    rng = np.random.default_rng(S)
+    vol = volume("bricks", dims, S, rng)
+    g = mg.mg_build(torch.from_numpy(vol).cuda(), S)
+    for n in (1, 40, 900):
+        bx = boxes_at_edges(dims, rng, n)
+        ref = oracle.box_hist(vol, S, bx).astype(np.float64)
+        t = torch.from_numpy(bx).cuda()
+        assert np.array_equal(mg.mg_query_boxes(g, t, hist="f32").cpu().numpy().astype(np.float64), ref)
+        plan = mg.QueryPlan(g, max_Q=len(bx), hist="f32", alpha="f16", max_blocks=len(bx) * 4096, max_chunks=len(bx) * 4096)
+        for h in (mg.mg_query_boxes(g, t, hist="f32", alpha="f16"), plan.run(t)):
+            h = h.cpu().numpy().astype(np.float64)
+            assert (np.abs(h - ref).sum(1) <= 1.5 * g.info["depth"] * 2.0 ** -11 * ref.sum(1)).all()
+        mg.mg_sync_status(g)
+        plan.close()
+    g.close()
