@@ -100,8 +100,9 @@ void arena_free(void* ctx, void* p, size_t bytes, mg_stream s) {
 }
 }  // namespace
 
-// the arena of a stream, made on first use (arena_mu held)
-static mg_status arena_of(mg_graph* g, cudaStream_t s, Arena** out) {
+// The arena of a stream, made on first use (arena_mu held).  What it keeps is
+// allocated by the first calls that are not captured; *capturing tells them apart.
+static mg_status arena_of(mg_graph* g, cudaStream_t s, Arena** out, bool* capturing) {
     auto& slot = g->arenas[s];
     if (!slot) {
         slot.reset(new (std::nothrow) Arena());
@@ -111,37 +112,61 @@ static mg_status arena_of(mg_graph* g, cudaStream_t s, Arena** out) {
         slot->view.a.alloc = arena_alloc;
         slot->view.a.free = arena_free;
         slot->view.custom = true;
-        if (cudaMallocHost(&slot->pinned, 8 * sizeof(uint64_t)) != cudaSuccess) {
+    }
+    Arena* a = slot.get();
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    MG_CUDA(cudaStreamIsCapturing(s, &cap));
+    *capturing = cap != cudaStreamCaptureStatusNone;
+    if (!*capturing) {
+        if (!a->pinned && cudaMallocHost(&a->pinned, 8 * sizeof(uint64_t)) != cudaSuccess) {
             cudaGetLastError();
-            slot->pinned = nullptr;
+            a->pinned = nullptr;
+        }
+        if (!a->sync.p) {   // (a propagation without them reports the failure)
+            void* p = g->al.get(2 * kPropWords * sizeof(unsigned), s);
+            if (p) {
+                a->sync.al = &g->al;
+                a->sync.s = s;
+                a->sync.p = p;
+                a->sync.bytes = 2 * kPropWords * sizeof(unsigned);
+            }
         }
     }
-    *out = slot.get();
+    *out = a;
     return MG_OK;
 }
 
-mg_status prop_sync_words(mg_graph* g, cudaStream_t s, int words, unsigned** out) {
+mg_status prop_sync_words(mg_graph* g, cudaStream_t s, Buf& own, unsigned** out) {
+    constexpr size_t bytes = kPropWords * sizeof(unsigned);
     std::lock_guard<std::mutex> lk(g->arena_mu);
     Arena* a = nullptr;
-    MG_TRY(arena_of(g, s, &a));
-    if (!a->sync.p) MG_TRY(a->sync.alloc(&g->al, (size_t)words * sizeof(unsigned), s));
-    // a captured launch zeroes them itself: the graph may run before or after
-    // any other launch on the stream
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    MG_CUDA(cudaStreamIsCapturing(s, &cap));
-    if (cap != cudaStreamCaptureStatusNone || !a->sync_zero) {
-        MG_CUDA(cudaMemsetAsync(a->sync.p, 0, (size_t)words * sizeof(unsigned), s));
-        a->sync_zero = cap == cudaStreamCaptureStatusNone;
+    bool capturing = false;
+    MG_TRY(arena_of(g, s, &a, &capturing));
+    if (!a->sync.p) {
+        if (!capturing) return fail(MG_ERR_OOM, "device allocation of the propagation's counters failed");
+        MG_TRY(own.alloc(&g->al, bytes, s));
     }
-    *out = a->sync.as<unsigned>();
+    unsigned* w = !a->sync.p ? own.as<unsigned>() : a->sync.as<unsigned>() + (capturing ? kPropWords : 0);
+    // a captured launch zeroes its words itself: nothing is known of the
+    // launches before a replay
+    if (capturing || !a->sync_zero) {
+        MG_CUDA(cudaMemsetAsync(w, 0, bytes, s));
+        if (!capturing) a->sync_zero = true;
+    }
+    *out = w;
     return MG_OK;
 }
 
 mg_status arena_begin(mg_graph* g, cudaStream_t s, Arena** out) {
     std::lock_guard<std::mutex> lk(g->arena_mu);
     Arena* a = nullptr;
-    MG_TRY(arena_of(g, s, &a));
-    if (a->need > a->buf.bytes) {
+    bool capturing = false;
+    MG_TRY(arena_of(g, s, &a, &capturing));
+    if (capturing) {
+        a->captured = a->captured || a->buf.p;
+    } else if (a->need > a->buf.bytes) {
+        if (a->captured) a->kept.push_back(std::move(a->buf));
+        a->captured = false;
         a->buf.release();   // stream-ordered after the previous call on s
         MG_TRY(a->buf.alloc(&g->al, a->need + a->need / 4, s));
     }
@@ -154,7 +179,7 @@ void arena_drop(mg_graph* g, cudaStream_t s) {
     std::lock_guard<std::mutex> lk(g->arena_mu);
     auto it = g->arenas.find(s);
     if (it == g->arenas.end()) return;
-    it->second->buf.s = it->second->sync.s = nullptr;   // the caller has synchronised the device
+    it->second->unbind();   // the caller has synchronised the device
     g->arenas.erase(it);
 }
 
@@ -450,7 +475,7 @@ MG_API void mg_free(mg_graph* g) {
     if (!g) return;
     DeviceGuard dg(g->device);
     cudaDeviceSynchronize();
-    for (auto& kv : g->arenas) kv.second->buf.s = kv.second->sync.s = nullptr;   // the device is idle; the call streams may be gone
+    for (auto& kv : g->arenas) kv.second->unbind();   // the device is idle; the call streams may be gone
     delete g;
 }
 

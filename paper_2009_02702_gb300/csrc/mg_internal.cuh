@@ -10,6 +10,7 @@
 #include <memory>
 #include <mutex>
 #include <string>
+#include <vector>
 
 #include "mg.h"
 
@@ -26,6 +27,11 @@ enum : unsigned {
     kStatTimeout = 1u << 2,    // bounded wait expired
     kStatInexact = 1u << 3,    // integer push met W % (a+b) != 0
 };
+
+// words of a propagation launch: ticket, CTAs that have left, a counter per
+// wave, each on a 128-byte line of its own
+constexpr int kPropLine = 32;
+constexpr int kPropWords = (MG_MAX_DEPTH + 4) * kPropLine;
 
 constexpr uint32_t kNone = 0xFFFFFFFFu;   // no predecessor
 constexpr uint32_t kDead = 0xFFFFFFFEu;   // node slot lost a publication race
@@ -98,14 +104,28 @@ struct Buf {
 // buffer, reset at the start of every call.  What does not fit comes from the
 // graph's allocator; the next call on the stream grows the buffer to the
 // high-water mark.  Calls on one stream run in order, so reuse is safe.
+//
+// A captured call leaves addresses in its graph.  So nothing that outlives the
+// call is allocated while the stream captures (stream-ordered memory of a
+// capture belongs to the graph), and a buffer that a captured call has used is
+// kept, not released, when it is grown.
 struct Arena {
     Buf buf;
+    bool captured = false;       // a captured call has used buf
+    std::vector<Buf> kept;       // former buffers that captured calls have used
     size_t used = 0, need = 0;
     const Alloc* fallback = nullptr;
     Alloc view;                  // an Alloc whose alloc/free go through this arena
     uint64_t* pinned = nullptr;  // 8 pinned host words for readbacks on this stream
-    Buf sync;                    // the propagation's ticket and counters, zero between launches
-    bool sync_zero = false;      // they have been zeroed once
+    // the propagation's ticket and counters: those of eager launches, zero
+    // between them, then those of captured launches, which zero them themselves
+    Buf sync;
+    bool sync_zero = false;      // the first have been zeroed once
+    // the device is idle and the stream may be gone: release on the legacy stream
+    void unbind() {
+        buf.s = sync.s = nullptr;
+        for (Buf& b : kept) b.s = nullptr;
+    }
     ~Arena() {
         if (pinned) cudaFreeHost(pinned);
     }
@@ -254,9 +274,10 @@ mg_status query_boxes(const mg_graph* g, const int32_t* boxes, int64_t Q, const 
 mg_status query_timing(const mg_graph* g, float* plan_ms, float* main_ms, float* out_ms);
 // the arena of `s` on graph g, reset for a new call (grown if the last call overflowed)
 mg_status arena_begin(mg_graph* g, cudaStream_t s, Arena** out);
-// the propagation's words of stream `s` (zeroed when first handed out; every
-// launch leaves them zero)
-mg_status prop_sync_words(mg_graph* g, cudaStream_t s, int words, unsigned** out);
+// the propagation's words for a launch on stream `s`, zero when it starts; a
+// captured launch on a stream that has none takes them from `own`, which the
+// caller releases in stream order after the launch
+mg_status prop_sync_words(mg_graph* g, cudaStream_t s, Buf& own, unsigned** out);
 // release the arena of a stream that is about to be destroyed (device idle)
 void arena_drop(mg_graph* g, cudaStream_t s);
 mg_status count_cubes(const mg_graph* g, const int32_t* boxes, int64_t Q, uint64_t* cubes,

@@ -145,8 +145,7 @@ struct PropArgs {
 };
 // each word has a 128-byte line of its own: the polls of one wave's counter do
 // not meet the ticket's atomics
-constexpr int kLine = 32;
-constexpr int kSyncWords = (MG_MAX_DEPTH + 4) * kLine;
+constexpr int kLine = kPropLine, kSyncWords = kPropWords;
 
 // Poll *p (acquire) until it reaches `need`: at once for the first polls, then
 // with pauses; bounded like bounded_wait_geq.
@@ -418,7 +417,8 @@ mg_status run(mg_graph* g, const float* tf, int cin, const void* alpha, ST* vals
     A.F = TfRows{tf, (int64_t)g->S * cin, cin};
     A.vals = vals;
     A.status = g->status.as<unsigned>();
-    MG_TRY(prop_sync_words(g, s, kSyncWords, &A.sync));
+    Buf own;
+    MG_TRY(prop_sync_words(g, s, own, &A.sync));
     auto k = propagate_kernel<ST, C>;
     static std::atomic<int> per_sm{0};   // of this kernel (one architecture)
     int per = per_sm.load(std::memory_order_relaxed);
