@@ -2392,7 +2392,7 @@ mg_status enqueue_batch(const mg_graph* g, const QueryBufs& B, const BatchRun& R
     plan_fused_kernel<<<(unsigned)tiles, kFusedThreads, 0, s>>>(G, R.boxes, R.Q, tb, B.chunk, chunk_shift, lim, F,
                                                                 status);
     MG_CUDA(cudaGetLastError());
-    if (ev) MG_CUDA(cudaEventRecord(ev[0], s));
+    const cudaError_t mark = ev ? cudaEventRecord(ev[0], s) : cudaSuccess;
 
     const int w16 = weights == MG_BF16;
     MainArgs A;
@@ -2425,7 +2425,12 @@ mg_status enqueue_batch(const mg_graph* g, const QueryBufs& B, const BatchRun& R
     A.accf = accf;
     A.io = R.io;
     A.qcap = 0;   // the shape's
-    MG_TRY(launch_shape(g, A, B.shape, s, !ev));
+    const mg_status st =
+        mark == cudaSuccess ? launch_shape(g, A, B.shape, s, !ev) : cuda_fail(mark, "cudaEventRecord");
+    if (st != MG_OK) {   // it is the main kernel that zeroes the words for the next batch
+        cudaMemsetAsync(B.words, 0, (size_t)A.clean_words * 8, s);
+        return st;
+    }
     if (ev) MG_CUDA(cudaEventRecord(ev[1], s));
     if (FP && !parts) {
         const int64_t cells = R.Q * (int64_t)g->S;

@@ -1,0 +1,55 @@
+"""Launch shapes of the batched box query at the limits of shared memory, and
+plans whose launches were refused.  Counts are whole numbers, equal to the
+oracle's."""
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mg():
+    from paper_2009_02702_gb300 import mg as _mg
+    _mg.lib()
+    return _mg
+
+
+def noise(dims, S, seed):
+    rng = np.random.default_rng(seed)
+    return rng.integers(0, S, dims[::-1]).astype(np.uint16)
+
+
+def some_boxes(dims, n, seed):
+    rng = np.random.default_rng(seed)
+    d = np.array(dims)
+    lo = rng.integers(0, d, (n, 3))
+    return np.concatenate([lo, rng.integers(1, d - lo + 1)], 1).astype(np.int32)
+
+
+def test_a_plan_goes_on_after_a_refused_launch(mg):
+    """Two graphs whose fp32 histograms take the same kernel, one of them nearly
+    all shared memory of an SM: should a run of its plan be refused after the
+    other graph's calls, the next run starts from clean counters."""
+    dims, S = (40, 32, 24), 18620
+    vol = noise(dims, S, 1)
+    g = mg.mg_build(torch.from_numpy(vol).cuda(), S)
+    other = mg.mg_build(torch.from_numpy(noise(dims, 2500, 2)).cuda(), 2500)
+    batches = [some_boxes(dims, 60, k) for k in range(3)]
+    t = [torch.from_numpy(b).cuda() for b in batches]
+    plan = mg.QueryPlan(g, max_Q=60, hist="f32")
+    mg.mg_query_boxes(other, t[0], hist="f32")
+    try:
+        plan.run(t[0])
+    except mg.MGError as e:
+        assert e.status == mg.MG_ERR_CUDA
+    mg.mg_query_boxes(g, t[1], hist="f32")
+    for k in (2, 0):
+        h = plan.run(t[k]).cpu().numpy()
+        assert np.array_equal(h.astype(np.int64), oracle.box_hist(vol, S, batches[k]).astype(np.int64)), k
+    mg.mg_sync_status(g)
+    plan.close()
+    g.close()
+    other.close()
