@@ -1067,7 +1067,10 @@ __device__ __forceinline__ void main_out(const MainArgs& A, uint32_t*& acc, floa
 // latency, so resident warps count for more where shared memory limits them.
 constexpr uint32_t kQueueLong = 320, kQueueShort = 64;   // entries
 constexpr size_t queue_bytes(uint32_t cap) { return (size_t)cap * 8 + 16; }   // nodes, weights, counter
-constexpr size_t kMaxDynSmem = 227 * 1024;   // dynamic shared memory of one CTA at most
+constexpr size_t kMaxDynSmem = 227 * 1024;   // shared memory of one CTA at most
+// dynamic shared memory of the batched kernels at most: 256 bytes are left for
+// the static variables of query_batched_kernel
+constexpr size_t kMaxMainSmem = kMaxDynSmem - 256;
 
 // chunks of the launch: known on the host, or (planned by the fused kernel) read
 // on the device, zero when the batch overflows the plan's buffers; the fused
@@ -2132,15 +2135,15 @@ mg_status main_shape(const mg_graph* g, bool rec, int threads, MainShape* out) {
         // of the last few segment counts that do take fewer warps
         if (smem + warps * queue_bytes(kQueueShort) > kMaxDynSmem)
             return fail(MG_ERR_UNSUPPORTED, "query kernel does not fit on an SM");
-        while (warps > 1 && smem_for(kQueueShort) > kMaxDynSmem) warps /= 2;
+        while (warps > 1 && smem_for(kQueueShort) > kMaxMainSmem) warps /= 2;
         threads = warps * 32;
     }
-    // one limit for every launch of the kernel: callers of several shapes never
-    // lower each other's
-    MG_TRY(prepare_kernel(k, std::max(smem_for(kQueueShort), kMaxDynSmem - 1024)));
+    // one limit for every launch of the kernel, the most that any shape asks
+    // for: callers of several shapes never lower each other's
+    MG_TRY(prepare_kernel(k, kMaxMainSmem));
     MG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem_for(kQueueShort)));
     if (per_sm < 1) return fail(MG_ERR_UNSUPPORTED, "query kernel does not fit on an SM");
-    if (!rec && smem_for(kQueueLong) <= kMaxDynSmem - 1024)
+    if (!rec && smem_for(kQueueLong) <= kMaxMainSmem)
         MG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_long, k, threads, smem_for(kQueueLong)));
     out->k = k;
     out->threads = threads;

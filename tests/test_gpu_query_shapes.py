@@ -53,3 +53,41 @@ def test_a_plan_goes_on_after_a_refused_launch(mg):
     plan.close()
     g.close()
     other.close()
+
+
+# 18002-18004 at 512 threads and 18685-18686 at 256: dynamic shared memory fits
+# an SM by itself, but not with the kernel's static variables
+@pytest.mark.parametrize("S", [17299, 18003, 18333, 18602, 18686])
+def test_every_shape_of_the_largest_float_histograms(mg, S):
+    dims = (40, 32, 24)
+    vol = noise(dims, S, S)
+    g = mg.mg_build(torch.from_numpy(vol).cuda(), S)
+    bx = some_boxes(dims, 40, S)
+    t = torch.from_numpy(bx).cuda()
+    ref = oracle.box_hist(vol, S, bx).astype(np.int64)
+    most = 512 if S < 18660 else 256   # 16 warps' queues fit beside the histogram up to there
+    for threads in (0, 128, 256, 512)[:3 + (most == 512)]:
+        h = mg.mg_query_boxes(g, t, hist="f32", block_threads=threads)
+        assert np.array_equal(h.cpu().numpy().astype(np.int64), ref), threads
+    if most == 512:
+        assert mg.mg_query_autotune(g, t, hist="f32")["block_threads"] in (128, 256, 512)
+    assert np.array_equal(mg.mg_query_boxes(g, t, hist="f32").cpu().numpy().astype(np.int64), ref)
+    mg.mg_sync_status(g)
+    g.close()
+
+
+def test_plans_of_two_graphs_keep_their_shared_memory(mg):
+    """The limit of a kernel's shared memory is the same for every caller."""
+    dims, S = (40, 32, 24), 18620
+    vol = noise(dims, S, 1)
+    g = mg.mg_build(torch.from_numpy(vol).cuda(), S)
+    other = mg.mg_build(torch.from_numpy(noise(dims, 2500, 2)).cuda(), 2500)
+    bx = some_boxes(dims, 60, 5)
+    t = torch.from_numpy(bx).cuda()
+    plan = mg.QueryPlan(g, max_Q=60, hist="f32")
+    mg.mg_query_boxes(other, t, hist="f32")
+    h = plan.run(t).cpu().numpy()
+    assert np.array_equal(h.astype(np.int64), oracle.box_hist(vol, S, bx).astype(np.int64))
+    plan.close()
+    g.close()
+    other.close()
