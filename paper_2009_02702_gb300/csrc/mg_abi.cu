@@ -100,6 +100,15 @@ void arena_free(void* ctx, void* p, size_t bytes, mg_stream s) {
 }
 }  // namespace
 
+bool is_capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return cap != cudaStreamCaptureStatusNone;
+}
+
 // The arena of a stream, made on first use (arena_mu held).  What it keeps is
 // allocated by the first calls that are not captured; *capturing tells them apart.
 static mg_status arena_of(mg_graph* g, cudaStream_t s, Arena** out, bool* capturing) {

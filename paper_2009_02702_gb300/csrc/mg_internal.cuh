@@ -202,6 +202,7 @@ struct mg_graph {
     mg::Buf lut_meta;
     mg::Buf lut;
     mg::Buf lut_rec;   // uint4 record per node (mg_tiles.cu; empty if there was no room)
+    std::mutex alpha16_mu;
     // the same for 16-bit weights (0: f16, 1: bf16), built on first use: the
     // share of a node's weight that every entry of its row receives, and the
     // nodes' records
@@ -272,6 +273,8 @@ mg_status query_boxes(const mg_graph* g, const int32_t* boxes, int64_t Q, const 
                       void* out, size_t cap, uint32_t* seg, uint64_t* offsets, size_t* required,
                       cudaStream_t s);
 mg_status query_timing(const mg_graph* g, float* plan_ms, float* main_ms, float* out_ms);
+// whether `s` is being captured into a CUDA graph (also when it cannot be asked)
+bool is_capturing(cudaStream_t s);
 // the arena of `s` on graph g, reset for a new call (grown if the last call overflowed)
 mg_status arena_begin(mg_graph* g, cudaStream_t s, Arena** out);
 // the propagation's words for a launch on stream `s`, zero when it starts; a

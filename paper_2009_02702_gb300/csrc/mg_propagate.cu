@@ -459,17 +459,22 @@ mg_status dispatch_c(mg_graph* g, const float* tf, int C, int cin, const void* a
 
 mg_status ensure_alpha16(mg_graph* g, mg_dtype dt, cudaStream_t s) {
     Buf& b = dt == MG_BF16 ? g->alphab16 : g->alpha16;
+    std::lock_guard<std::mutex> lk(g->alpha16_mu);   // until the weights are there: other threads read them at once
     if (b.p) return MG_OK;
-    MG_TRY(b.alloc(&g->al, (size_t)g->N * 2, s));
+    if (is_capturing(s))
+        return fail(MG_ERR_CUDA, "the first call with 16-bit weights makes them and cannot be captured");
+    Buf made;
+    MG_TRY(made.alloc(&g->al, (size_t)g->N * 2, s));
     if (g->quantised)
         alpha16_from_f32_kernel<<<grid_for(g->N, 256, 152 * 32), 256, 0, s>>>(g->alpha.as<float>(), g->N, g->S,
-                                                                              dt == MG_BF16, b.p);
+                                                                              dt == MG_BF16, made.p);
     else
         alpha16_kernel<<<grid_for(g->N, 256, 152 * 32), 256, 0, s>>>(g->ab.as<ulonglong2>(), g->N, g->S,
-                                                                    dt == MG_BF16, b.p);
+                                                                    dt == MG_BF16, made.p);
     MG_CUDA(cudaGetLastError());
     MG_CUDA(cudaStreamSynchronize(s));
-    b.s = nullptr;
+    made.s = nullptr;
+    b = std::move(made);
     return MG_OK;
 }
 

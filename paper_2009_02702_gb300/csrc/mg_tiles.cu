@@ -585,7 +585,7 @@ mg_status ensure_records16(mg_graph* g, mg_dtype dt, cudaStream_t s) {
     if (!g->lut_meta.p || g->quantised || g->S > kMaxSharedSegments) return MG_OK;
     const int k = dt == MG_BF16;
     std::lock_guard<std::mutex> lk(g->rec16_mu);
-    if (g->rec16[k].p) return MG_OK;
+    if (g->rec16[k].p || is_capturing(s)) return MG_OK;
     Buf frac, rec;
     if (!try_alloc(frac, &g->al, (size_t)std::max<int64_t>(g->lut_entries, 1) * 4, s) ||
         !try_alloc(rec, &g->al, (size_t)g->N * sizeof(uint4), s))

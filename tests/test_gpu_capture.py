@@ -1,7 +1,8 @@
 """Calls captured into CUDA graphs: what a captured call leaves behind (the
 propagation's counters, the scratch of a stream) serves later eager calls and
 every replay, in any order."""
-import numpy as np
+import threading
+
 import pytest
 
 from paper_2009_02702_gb300 import synth
@@ -100,3 +101,60 @@ def test_scratch_outlives_its_growth(mg, own_allocator):
     mg.mg_sync_status(g)
     del graph
     g.close()
+
+
+@pytest.mark.parametrize("storage", ["f16", "bf16"])
+def test_first_16_bit_call_captured(mg, storage):
+    """The weights it would make cannot come from a capture: it is refused, and
+    nothing of it is kept."""
+    ref = mg.mg_propagate_tf(build(mg, True), torch.from_numpy(synth.make_tf(3, S, 4)).cuda(), storage=storage)
+    g = build(mg, True)
+    tf = torch.from_numpy(synth.make_tf(3, S, 4)).cuda()
+    out = torch.empty_like(ref)
+    s = torch.cuda.Stream()
+    with pytest.raises(mg.MGError) as e:
+        capture(lambda: mg.mg_propagate_tf(g, tf, storage=storage, out=out, stream=s), s)
+    assert e.value.status == mg.MG_ERR_CUDA
+    got = mg.mg_propagate_tf(g, tf, storage=storage, stream=s)
+    torch.cuda.synchronize()
+    assert torch.equal(got, ref)
+    graph = capture(lambda: mg.mg_propagate_tf(g, tf, storage=storage, out=out, stream=s), s)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, ref)
+    mg.mg_sync_status(g)
+    del graph
+    g.close()
+
+
+def test_first_16_bit_calls_of_several_threads(mg):
+    """Weights and records are made once and read only when they are there."""
+    tf = torch.from_numpy(synth.make_tf(3, S, 4)).cuda()
+    boxes = torch.from_numpy(synth.make_boxes(1, Q=50, dims=DIMS, box_max=61)).cuda()
+    work = [lambda g, s: mg.mg_propagate_tf(g, tf, storage="f16", stream=s),
+            lambda g, s: mg.mg_query_boxes(g, boxes, hist="f32", alpha="f16", stream=s)]
+    g = build(mg, True)
+    ref = [f(g, None) for f in work]
+    torch.cuda.synchronize()
+    g.close()
+    for _ in range(5):
+        g = build(mg, True)
+        streams = [torch.cuda.Stream() for _ in range(8)]
+        out = [None] * 8
+        gate = threading.Barrier(8)
+
+        def go(k):
+            gate.wait()
+            out[k] = work[k % 2](g, streams[k])
+
+        threads = [threading.Thread(target=go, args=(k,)) for k in range(8)]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        torch.cuda.synchronize()
+        for k in range(8):
+            # (the order of the fp32 sums of a histogram differs from run to run)
+            assert torch.equal(out[k], ref[0]) if k % 2 == 0 else torch.allclose(out[k], ref[1], rtol=1e-4, atol=1e-3), k
+        mg.mg_sync_status(g)
+        g.close()
