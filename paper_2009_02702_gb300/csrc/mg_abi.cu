@@ -88,8 +88,9 @@ void* arena_alloc(void* ctx, size_t bytes, mg_stream s) {
         if (a->used > a->need) a->need = a->used;
         return p;
     }
-    if (a->used + n > a->need) a->need = a->used + n;
-    return a->fallback->get(bytes, reinterpret_cast<cudaStream_t>(s));
+    void* p = a->fallback->get(bytes, reinterpret_cast<cudaStream_t>(s));
+    if (p && a->used + n > a->need) a->need = a->used + n;
+    return p;
 }
 
 void arena_free(void* ctx, void* p, size_t bytes, mg_stream s) {
@@ -177,7 +178,10 @@ mg_status arena_begin(mg_graph* g, cudaStream_t s, Arena** out) {
         if (a->captured) a->kept.push_back(std::move(a->buf));
         a->captured = false;
         a->buf.release();   // stream-ordered after the previous call on s
-        MG_TRY(a->buf.alloc(&g->al, a->need + a->need / 4, s));
+        if (a->buf.alloc(&g->al, a->need + a->need / 4, s) != MG_OK) {   // this call's allocations are its own again
+            a->need = 0;
+            set_error("");
+        }
     }
     a->used = 0;
     *out = a;

@@ -2577,23 +2577,27 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
     // of a 64^3 volume took 69 us with three plan kernels and the read-back of
     // their totals, 34 with this.
     const uint64_t most_blocks = block_bound(g, Q), most_chunks = chunk_bound(g, Q, chunk);
-    const bool fused = o.schedule == MG_SCHED_BATCHED && !room && most_blocks < (1u << 22) && most_chunks < (1u << 22);
-    Buf nblk, ncube, nchunk, blk_off, chunk_off, blk, ticket, chunk_q, chunk_b;
+    bool fused = o.schedule == MG_SCHED_BATCHED && !room && most_blocks < (1u << 22) && most_chunks < (1u << 22);
+    Buf nblk, ncube, nchunk, blk_off, chunk_off, blk, ticket, chunk_q, chunk_b, tiles;
+    const size_t words_bytes = 16 + 16 * (size_t)tile_count(Q, g->device);
     if (fused) {
-        Buf tiles;
+        // buffers of that size are more than the batch needs: where there is no
+        // memory for them, it is planned with a read-back
+        auto got = [&](Buf& b, size_t n) { return b.alloc(&al, n, s) == MG_OK; };
+        fused = got(ncube, (size_t)Q * 8) && got(blk_off, (size_t)(Q + 1) * 8) && got(chunk_off, (size_t)(Q + 1) * 8) &&
+                got(blk, (size_t)most_blocks * sizeof(Blk)) && got(chunk_q, (size_t)most_chunks * 4) &&
+                got(chunk_b, (size_t)most_chunks * 4) && got(tiles, words_bytes);
+        if (!fused) {
+            for (Buf* b : {&ncube, &blk_off, &chunk_off, &blk, &chunk_q, &chunk_b, &tiles}) b->release();
+            set_error("");
+        }
+    }
+    if (fused) {
         QueryBufs B;
         B.cap_blocks = most_blocks;
         B.cap_chunks = most_chunks;
         B.chunk = chunk;
         MG_TRY(shape_of(g, FP, weights, threads, &B.shape));
-        const size_t words_bytes = 16 + 16 * (size_t)tile_count(Q, g->device);
-        MG_TRY(ncube.alloc(&al, (size_t)Q * 8, s));
-        MG_TRY(blk_off.alloc(&al, (size_t)(Q + 1) * 8, s));
-        MG_TRY(chunk_off.alloc(&al, (size_t)(Q + 1) * 8, s));
-        MG_TRY(blk.alloc(&al, (size_t)most_blocks * sizeof(Blk), s));
-        MG_TRY(chunk_q.alloc(&al, (size_t)most_chunks * 4, s));
-        MG_TRY(chunk_b.alloc(&al, (size_t)most_chunks * 4, s));
-        MG_TRY(tiles.alloc(&al, words_bytes, s));
         B.ncube = ncube.as<uint64_t>();
         B.blk_off = blk_off.as<uint64_t>();
         B.chunk_off = chunk_off.as<uint64_t>();

@@ -1,6 +1,8 @@
 """Launch shapes of the batched box query at the limits of shared memory, and
 plans whose launches were refused.  Counts are whole numbers, equal to the
 oracle's."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -91,3 +93,66 @@ def test_plans_of_two_graphs_keep_their_shared_memory(mg):
     plan.close()
     g.close()
     other.close()
+
+
+@pytest.mark.parametrize("layout", ["dense", "csr"])
+def test_direct_batch_within_a_small_allocator(mg, layout):
+    """1,000 boxes of 64^3 could have 2.7 M blocks (33 MB) and have under
+    200,000: without memory for the worst case the batch is planned exactly."""
+    dims, S = (64, 64, 64), 64
+    vol = (np.arange(64 ** 3).reshape(64, 64, 64) // 97 % S).astype(np.uint16)
+    ids = torch.from_numpy(vol).cuda()
+    state = {"most": 1 << 40, "refused": 0}
+
+    def alloc(ctx, nbytes, stream):
+        if nbytes > state["most"]:
+            state["refused"] += 1
+            return None
+        return torch.cuda.caching_allocator_alloc(int(nbytes), 0, int(stream or 0))
+
+    def free(ctx, ptr, nbytes, stream):
+        torch.cuda.caching_allocator_delete(int(ptr))
+
+    a = mg.mg_allocator(None, mg.ALLOC_FN(alloc), mg.FREE_FN(free))
+    h = ctypes.c_void_p()
+    st = mg.lib().mg_build(ids.data_ptr(), *dims, S, ctypes.byref(mg.mg_build_opts(2)), ctypes.byref(a),
+                           torch.cuda.current_stream().cuda_stream, ctypes.byref(h))
+    assert st == mg.MG_OK
+    g = mg.Graph(h.value, 0, a)
+    bx = some_boxes(dims, 1000, 7)
+    t = torch.from_numpy(bx).cuda()
+    ref = oracle.box_hist(vol, S, bx)
+    state["most"] = 8 << 20
+    for k in range(3):   # (the scratch of a stream grows to what its calls took)
+        if layout == "dense":
+            got = mg.mg_query_boxes(g, t).cpu().numpy()
+        else:
+            off, seg, cnt = (x.cpu().numpy() for x in mg.mg_query_boxes(g, t, layout="csr"))
+            got = np.zeros_like(ref)
+            for q in range(len(bx)):
+                got[q, seg[off[q]:off[q + 1]]] = cnt[off[q]:off[q + 1]]
+        assert np.array_equal(got, ref), k
+    assert state["refused"] > 0
+    mg.mg_sync_status(g)
+    g.close()
+
+
+@pytest.mark.parametrize("hist,alpha", [("u32", "f32"), ("f32", "f32"), ("f32", "f16")])
+def test_direct_batches_on_both_sides_of_the_worst_case_bound(mg, hist, alpha):
+    """1,528 boxes of 64^3 have fewer than 2^22 blocks whatever they are and are
+    planned in one launch; 1,529 boxes are not."""
+    dims, S = (64, 64, 64), 64
+    assert 1528 * 14 ** 3 < 1 << 22 <= 1529 * 14 ** 3
+    vol = (np.arange(64 ** 3).reshape(64, 64, 64) // 97 % S).astype(np.uint16)
+    g = mg.mg_build(torch.from_numpy(vol).cuda(), S)
+    bx = some_boxes(dims, 1529, 8)
+    t = torch.from_numpy(bx).cuda()
+    one = mg.mg_query_boxes(g, t[:1528].contiguous(), hist=hist, alpha=alpha).cpu().numpy().astype(np.float64)
+    many = mg.mg_query_boxes(g, t, hist=hist, alpha=alpha).cpu().numpy().astype(np.float64)
+    mg.mg_sync_status(g)
+    ref = oracle.box_hist(vol, S, bx).astype(np.float64)
+    if alpha == "f32":
+        assert np.array_equal(one, ref[:1528]) and np.array_equal(many, ref)
+    else:   # the same shares, at most one a cube (8/3 of the three areas), summed in another order
+        assert (np.abs(one - many[:1528]) <= 8 * 64 ** 2 * 2.0 ** -24 * np.maximum(one, many[:1528])).all()
+    g.close()
