@@ -1598,7 +1598,10 @@ __global__ void __launch_bounds__(NT, WarpKernelBounds<NT>::min_ctas) query_warp
         }
         __syncwarp();
         if (total <= all) break;
-        if (lane == 0) c = all + atomicAdd(reinterpret_cast<uint32_t*>(A.ticket), 1u);
+        if (lane == 0) {   // (compared before the sum, which could pass 2^32)
+            const uint32_t t = atomicAdd(reinterpret_cast<uint32_t*>(A.ticket), 1u);
+            c = t < total - all ? all + t : total;
+        }
         c = __shfl_sync(0xffffffffu, c, 0);
     }
 }
