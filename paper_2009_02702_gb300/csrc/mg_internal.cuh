@@ -306,15 +306,16 @@ struct PlanParts {
     uint64_t cap_blocks, cap_chunks;
 };
 mg_status plan_parts(mg_query_plan* p, PlanParts* out);
-// Work-chunk length of a plan, and the chunk-map entries it keeps per chunk of
-// the caller's capacity: an untuned plan for few boxes takes chunks `scale`
-// times shorter than the default, so that what fits the capacity in default
-// chunks fits its map.
+// Work-chunk length of a plan, and the entries of its chunk map.  An untuned
+// plan for few boxes takes shorter chunks than the default, and entries for
+// all that fits the caller's capacity in default chunks, or for the most that
+// max_Q boxes can have if that is less: 64 MiB at most, or the caller's own.
 struct PlanChunk {
-    uint32_t chunk, scale;
+    uint32_t chunk;
+    uint64_t cap_chunks;
 };
-PlanChunk plan_chunk(const mg_graph* g, int hist_type, mg_dtype weights, int chunk_cubes, int64_t max_Q,
-                     uint64_t cap_chunks);
+PlanChunk plan_chunk(const mg_graph* g, int hist_type, mg_dtype weights, int chunk_cubes, int block_threads,
+                     int64_t max_Q, uint64_t cap_chunks);
 
 // ---------------------------------------------------------------------------
 // small device helpers

@@ -29,6 +29,7 @@
 #include "mg_internal.cuh"
 
 #include <algorithm>
+#include <cmath>
 #include <mutex>
 #include <type_traits>
 #include <vector>
@@ -2055,25 +2056,47 @@ int sm_count(int dev) {
     return cache[dev] ? cache[dev] : 1;
 }
 
-// Items per work chunk of an untuned batch of Q boxes.  A small batch is bound
-// by the latency of the longest chunk (one warp walks it alone), so its chunks
-// shrink until the batch holds a few per resident warp.  Histogram kernel, us
-// at 128 / 256 / 512 / 1,024 / 2,048 items a chunk: 1,000 boxes of a 64^3
-// volume 16 / 18 / 24 / 35 / 46; 777 of a 251x187x113 volume 20 / 24 / 28 / 37
-// / 61; 2,000 with 16-bit weights on 512x512x384 - / 120 / 106 / 118 / 151;
-// 10,000 there 205 / 135 / 104 / 104 / 121; 100,000 on 2048x2048x300 - / - /
-// 1580 / 1290 / 1120.  Below 128 the per-chunk flush outweighs it.  A histogram
-// shared by a CTA (many segments) has 16 warps on a chunk already.
-//
-// With 16-bit weights a chunk flushes two bins a segment and its items touch
-// more of them: it holds at least one item per two segments (1,000 boxes, 1,182
-// segments: 355 / 309 / 303 / 305 us at 256 / 512 / 1,024 / 2,048 items; 300
-// boxes, 353 segments: 113 / 68 / 101 at 128 / 256 / 1,024).
-constexpr uint32_t kDefaultChunk = 2048, kMinChunk = 128;
-uint32_t default_chunk(uint32_t S, int64_t Q, mg_dtype weights) {
+// Whether a CTA's warps have a histogram each (few segments) or share one.
+bool warp_hists(const mg_graph* g, bool FP, int threads) {
+    const size_t hist = (size_t)g->S * 4 * (FP ? 2 : 1);
+    return g->S <= kWarpHistMax && threads <= 256 && (hist + queue_bytes(kQueueShort)) * (threads / 32) <= 96 * 1024;
+}
+
+// Items per work chunk of an untuned batch of Q boxes.  A batch is bound by the
+// latency of its longest chunk (one warp walks it alone, or a CTA whose warps
+// share a histogram) until it holds enough chunks to fill the GPU, then by what
+// each chunk costs beyond its items (descriptors, the flush).  The best length
+// grows with the square root of Q, and more slowly with the area of the volume's
+// sides, which a box's items follow.  us of a plan run at 128 / 256 / 512 /
+// 1,024 / 2,048 items, the rule's choice in brackets, uint32 counts:
+//   64^3, 64 segments: 1,000 boxes [24] / 26 / 32 / 41 / 52; 10,000 boxes
+//     55 / [50] / 48 / 55 / 67; 30,000 boxes 135 / 108 / [101] / 101 / 113
+//   251x187x113, 90 segments: 777 boxes [31] / 32 / 36 / 46 / 58; 10,000 boxes
+//     113 / 87 / [77] / 83 / 96
+//   512x512x384, 353 segments: 100 boxes [23] / 26 / 31 / 39 / 55; 1,000 boxes
+//     42 / [40] / 46 / 65 / 86; 10,000 boxes 212 / 150 / [127] / 127 / 134
+//   2048x2048x300, 1,182 segments: 1,000 boxes 57 / [49] / 52 / 58 / 85; 10,000
+//     boxes 377 / 255 / 197 / [181] / 190; 100,000 boxes - / - / - / 1472 / [1328]
+//   614x961x600, 15,917 segments, a histogram per CTA: 10 boxes 33 / [32] / 35 /
+//     44 / 52; 100 boxes 84 / 66 / [60] / 58 / 74; 1,000 boxes - / - / 446 /
+//     409 / [398]
+// fp32 histograms flush two bins a segment: a third longer (2048x2048x300,
+// 10,000 boxes: - / - / 335 / 289 / [283]).  With 16-bit weights a chunk's items
+// touch more bins too: longer in proportion above 750 segments, and at least one
+// item per five segments in a warp's (1,182 segments: 100 boxes 64 / [52] / 58 /
+// 85 / 108, 1,000 boxes 337 / 241 / 194 / [186] / 197; 64^3, 10,000 boxes 77 /
+// [77] / 86 / 98 / 134).
+constexpr uint32_t kDefaultChunk = 2048, kMinChunk = 128, kMinSharedChunk = 256;
+uint32_t default_chunk(const mg_graph* g, bool FP, mg_dtype weights, int threads, int64_t Q) {
+    const bool own = warp_hists(g, FP, threads);
+    const double x = g->geom.dims[0][0], y = g->geom.dims[0][1], z = g->geom.dims[0][2];
+    const double per = !own ? (FP ? 3.6 : 2.0) : !FP ? 0.33 : weights == MG_F32 ? 0.45 : 0.45 * std::max(1.0, g->S / 750.0);
+    const double best = per * std::sqrt((double)Q * std::sqrt(x * y + y * z + z * x));
+    const uint32_t least = !own                ? kMinSharedChunk
+                           : weights == MG_F32 ? kMinChunk
+                                               : std::max(kMinChunk, g->S / 5);
     uint32_t c = kDefaultChunk;
-    const uint32_t least = weights == MG_F32 ? kMinChunk : std::max(kMinChunk, (S + 1) / 2);
-    while (S <= kWarpHistMax && c / 2 >= least && (int64_t)c > Q * 2 / 7) c /= 2;
+    while (c / 2 >= least && c > best) c /= 2;
     return c;
 }
 
@@ -2122,9 +2145,8 @@ mg_status main_shape(const mg_graph* g, bool rec, int threads, MainShape* out) {
     // node records, their queues come on top
     int warps = threads / 32;
     const size_t smem = hist_smem(g->S, FP);
-    const size_t hist_w = (size_t)g->S * 4 * (FP ? 2 : 1), hist_s = (size_t)((g->S + 3) & ~3u) * 4 * (FP ? 2 : 1);
-    const bool warp_mode =
-        g->S <= kWarpHistMax && threads <= 256 && (hist_w + queue_bytes(kQueueShort)) * warps <= 96 * 1024;
+    const size_t hist_s = (size_t)((g->S + 3) & ~3u) * 4 * (FP ? 2 : 1);
+    const bool warp_mode = warp_hists(g, FP, threads);
     auto k = !warp_mode       ? (rec ? query_batched_kernel<FP, AT, true> : query_batched_kernel<FP, AT, false>)
              : threads <= 128 ? (rec ? query_warp_kernel<FP, AT, 128, true> : query_warp_kernel<FP, AT, 128, false>)
                               : (rec ? query_warp_kernel<FP, AT, 256, true> : query_warp_kernel<FP, AT, 256, false>);
@@ -2500,15 +2522,29 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
         MG_TRY(ensure_records16(const_cast<mg_graph*>(g), (mg_dtype)o.alpha_dtype, s));
     }
     const int tuned_c = g->tuned_chunk[FP ? 1 : 0], tuned_t = g->tuned_threads[FP ? 1 : 0];
-    // a fixed pool keeps the long chunks: its room is counted in them
-    const uint32_t chunk = o.chunk_cubes > 0 ? (uint32_t)o.chunk_cubes
-                           : tuned_c > 0     ? (uint32_t)tuned_c
-                           : room            ? kDefaultChunk
-                                             : default_chunk(S, Q, FP ? (mg_dtype)o.alpha_dtype : MG_F32);
     const int threads = o.block_threads > 0                ? o.block_threads
                         : tuned_t > 0                      ? tuned_t
                         : o.schedule == MG_SCHED_BATCHED   ? default_threads(g, FP, (mg_dtype)o.alpha_dtype)
                                                            : 256;
+    // a fixed pool keeps the long chunks: its room is counted in them
+    uint32_t chunk = o.chunk_cubes > 0 ? (uint32_t)o.chunk_cubes
+                     : tuned_c > 0     ? (uint32_t)tuned_c
+                     : room            ? kDefaultChunk
+                                       : default_chunk(g, FP, (mg_dtype)o.alpha_dtype, threads, Q);
+    // Where the most that this many boxes can have fits a modest buffer, the
+    // footprint is planned in one launch and nothing is read back: 1,000 boxes
+    // of a 64^3 volume took 69 us with three plan kernels and the read-back of
+    // their totals, 34 with this.  That is worth somewhat longer chunks (300
+    // boxes of 512x512x384, 16-bit weights: 97 us with 128 items and the
+    // read-back, 59 with 256).
+    constexpr uint64_t kMostUnread = 1u << 22;
+    const uint64_t most_blocks = block_bound(g, Q);
+    bool fused = o.schedule == MG_SCHED_BATCHED && !room && most_blocks < kMostUnread;
+    while (fused && o.chunk_cubes <= 0 && tuned_c <= 0 && chunk < kDefaultChunk &&
+           chunk_bound(g, Q, chunk) >= kMostUnread)
+        chunk *= 2;
+    const uint64_t most_chunks = chunk_bound(g, Q, chunk);
+    fused = fused && most_chunks < kMostUnread;
     const Geom G = make_geom(g, tile_levels(g, (mg_dtype)o.alpha_dtype));
     unsigned* status = g->status.as<unsigned>();
     mg_graph* gm = const_cast<mg_graph*>(g);
@@ -2575,12 +2611,6 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
 
     const size_t smem = hist_smem(S, FP);
     if (smem > 220 * 1024) return fail(MG_ERR_UNSUPPORTED, "too many segments for the shared-memory histogram");
-    // Where the most that this many boxes can have fits a modest buffer, the
-    // footprint is planned in one launch and nothing is read back: 1,000 boxes
-    // of a 64^3 volume took 69 us with three plan kernels and the read-back of
-    // their totals, 34 with this.
-    const uint64_t most_blocks = block_bound(g, Q), most_chunks = chunk_bound(g, Q, chunk);
-    bool fused = o.schedule == MG_SCHED_BATCHED && !room && most_blocks < (1u << 22) && most_chunks < (1u << 22);
     Buf nblk, ncube, nchunk, blk_off, chunk_off, blk, ticket, chunk_q, chunk_b, tiles;
     const size_t words_bytes = 16 + 16 * (size_t)tile_count(Q, g->device);
     if (fused) {
@@ -2887,15 +2917,26 @@ struct mg_query_plan {
 };
 
 namespace mg {
-PlanChunk plan_chunk(const mg_graph* g, int hist_type, mg_dtype weights, int chunk_cubes, int64_t max_Q,
-                     uint64_t cap_chunks) {
-    const int tuned = g->tuned_chunk[hist_type == MG_HIST_F32];
-    if (chunk_cubes > 0) return PlanChunk{(uint32_t)chunk_cubes, 1};
-    if (tuned > 0) return PlanChunk{(uint32_t)tuned, 1};
-    const uint32_t c = default_chunk(g->S, max_Q, hist_type == MG_HIST_F32 ? weights : MG_F32), scale = kDefaultChunk / c;
-    // the map of the shorter chunks, 8 bytes each, stays within 64 MiB
-    if (cap_chunks * scale > (1u << 23)) return PlanChunk{kDefaultChunk, 1};
-    return PlanChunk{c, scale};
+namespace {
+// threads of a plan's CTAs: the caller's, else the tuned ones, else the default
+int plan_threads(const mg_graph* g, bool FP, mg_dtype weights, int block_threads) {
+    const int tuned = g->tuned_threads[FP];
+    return block_threads > 0 ? block_threads : tuned > 0 ? tuned : default_threads(g, FP, weights);
+}
+}  // namespace
+
+PlanChunk plan_chunk(const mg_graph* g, int hist_type, mg_dtype weights, int chunk_cubes, int block_threads,
+                     int64_t max_Q, uint64_t cap_chunks) {
+    const bool FP = hist_type == MG_HIST_F32;
+    const int tuned = g->tuned_chunk[FP];
+    if (chunk_cubes > 0) return PlanChunk{(uint32_t)chunk_cubes, cap_chunks};
+    if (tuned > 0) return PlanChunk{(uint32_t)tuned, cap_chunks};
+    const int threads = plan_threads(g, FP, weights, block_threads);
+    for (uint32_t c = default_chunk(g, FP, FP ? weights : MG_F32, threads, max_Q); c < kDefaultChunk; c *= 2) {
+        const uint64_t n = std::min(cap_chunks * (kDefaultChunk / c), chunk_bound(g, max_Q, c));
+        if (n <= std::max<uint64_t>(cap_chunks, 1u << 23)) return PlanChunk{c, n};
+    }
+    return PlanChunk{kDefaultChunk, cap_chunks};
 }
 
 mg_status plan_parts(mg_query_plan* p, PlanParts* out) {
@@ -2944,6 +2985,10 @@ MG_API mg_status mg_query_plan_create(mg_graph* g, int64_t max_Q, const mg_query
     if (prev != g->device) MG_CUDA(cudaSetDevice(g->device));
     std::unique_ptr<mg_query_plan> p(new (std::nothrow) mg_query_plan());
     mg_status st = p ? MG_OK : fail(MG_ERR_OOM, "host allocation failed");
+    if (st == MG_OK && o.hist_type == MG_HIST_F32 && o.alpha_dtype != MG_F32) {   // (the launch shape depends on them)
+        st = ensure_alpha16(g, (mg_dtype)o.alpha_dtype, nullptr);
+        if (st == MG_OK) st = ensure_records16(g, (mg_dtype)o.alpha_dtype, nullptr);
+    }
     if (st == MG_OK) {
         const bool FP = o.hist_type == MG_HIST_F32;
         p->g = g;
@@ -2953,9 +2998,9 @@ MG_API mg_status mg_query_plan_create(mg_graph* g, int64_t max_Q, const mg_query
         QueryBufs& B = p->bufs;
         B.cap_blocks = max_blocks > 0 ? (uint64_t)max_blocks : (uint64_t)max_Q * 1024;
         B.cap_chunks = max_chunks > 0 ? (uint64_t)max_chunks : (uint64_t)max_Q * 256;
-        const PlanChunk pc = plan_chunk(g, o.hist_type, p->weights, o.chunk_cubes, max_Q, B.cap_chunks);
+        const PlanChunk pc = plan_chunk(g, o.hist_type, p->weights, o.chunk_cubes, o.block_threads, max_Q, B.cap_chunks);
         B.chunk = pc.chunk;
-        B.cap_chunks *= pc.scale;
+        B.cap_chunks = pc.cap_chunks;
         if (B.cap_blocks >= (1ull << 32) || B.cap_chunks >= (1ull << 32))
             st = fail(MG_ERR_UNSUPPORTED, "plan capacities must be below 2^32");
     }
@@ -2992,13 +3037,8 @@ MG_API mg_status mg_query_plan_create(mg_graph* g, int64_t max_Q, const mg_query
             p->pool.s = nullptr;
         }
     }
-    if (st == MG_OK && p->fp && o.alpha_dtype != MG_F32) st = ensure_alpha16(g, (mg_dtype)o.alpha_dtype, nullptr);
-    if (st == MG_OK && p->fp && o.alpha_dtype != MG_F32) st = ensure_records16(g, (mg_dtype)o.alpha_dtype, nullptr);
-    if (st == MG_OK) {
-        const int tt = g->tuned_threads[p->fp];
-        const int threads = o.block_threads > 0 ? o.block_threads : tt > 0 ? tt : default_threads(g, p->fp, p->weights);
-        st = shape_of(g, p->fp, p->weights, threads, &p->bufs.shape);
-    }
+    if (st == MG_OK)
+        st = shape_of(g, p->fp, p->weights, plan_threads(g, p->fp, p->weights, o.block_threads), &p->bufs.shape);
     if (st == MG_OK && o.timing) {
         p->timed = true;
         for (cudaEvent_t& ev : p->ev) {

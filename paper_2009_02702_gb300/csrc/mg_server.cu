@@ -529,7 +529,7 @@ MG_API mg_status mg_server_add_volume(mg_server* sv, mg_graph* g, int C, int* vo
     const size_t query_bytes =
         sv->o.plain ? round_up(Q * 24) + round_up(Q * S * 4) + 2 * Q * S * 4
                     : Q * 24 + Q * S * 4 * (sv->o.hist_type == MG_HIST_F32 ? 2 : 1) + Q * 64 + cap_blocks * 12 +
-                          cap_chunks * 8 * plan_chunk(g, sv->o.hist_type, MG_F32, 0, (int64_t)Q, cap_chunks).scale;
+                          8 * plan_chunk(g, sv->o.hist_type, MG_F32, 0, 0, (int64_t)Q, cap_chunks).cap_chunks;
     const int64_t need = (int64_t)((tf_bytes + query_bytes) * sv->slots.size()) + g->device_bytes();
     if (sv->o.memory_budget > 0 && sv->budget_used + need > sv->o.memory_budget)
         return fail(MG_ERR_CAPACITY, "volume not admitted: it needs " + std::to_string(need >> 20) + " MiB and " +

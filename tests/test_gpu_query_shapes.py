@@ -156,3 +156,24 @@ def test_direct_batches_on_both_sides_of_the_worst_case_bound(mg, hist, alpha):
     else:   # the same shares, at most one a cube (8/3 of the three areas), summed in another order
         assert (np.abs(one - many[:1528]) <= 8 * 64 ** 2 * 2.0 ** -24 * np.maximum(one, many[:1528])).all()
     g.close()
+
+
+@pytest.mark.parametrize("S", [64, 1182, 2500])
+def test_chunks_of_every_length_the_default_takes(mg, S):
+    """Batches whose default chunks run from 128 items to 2,048, direct and by a
+    plan made for just as many boxes: few and many, histograms per warp and per CTA."""
+    dims = (160, 96, 80)
+    z, y, x = np.meshgrid(*(np.arange(n) // k for n, k in zip(dims[::-1], (9, 7, 11))), indexing="ij")
+    vol = ((x * 7919 + y * 104729 + z * 1299709) % S).astype(np.uint16)
+    g = mg.mg_build(torch.from_numpy(vol).cuda(), S)
+    for Q in (1, 60, 700, 9000):
+        bx = some_boxes(dims, Q, Q)
+        t = torch.from_numpy(bx).cuda()
+        ref = oracle.box_hist(vol, S, bx).astype(np.int64)
+        for hist in ("u32", "f32"):
+            plan = mg.QueryPlan(g, max_Q=Q, hist=hist, max_blocks=4096 * Q)
+            for h in (mg.mg_query_boxes(g, t, hist=hist), plan.run(t)):
+                assert np.array_equal(h.cpu().numpy().astype(np.int64), ref), (Q, hist)
+            plan.close()
+    mg.mg_sync_status(g)
+    g.close()
