@@ -1304,6 +1304,36 @@ __device__ __forceinline__ void add_record(const PushArgs& P, const Hist<FP>& H,
     }
 }
 
+// Rows of more entries than this are added by the whole warp: a lane's loop over
+// one holds the others up (a cube of level 3 of a volume of noise has 512; 100
+// boxes of such a 64^3 volume with 32,768 segments 621 -> 144 us).
+constexpr uint32_t kLongRow = 32;
+template <typename AT> __device__ __forceinline__ bool long_row(uint4 r) {
+    return std::is_same<AT, float>::value ? r.x == kTileList && r.z > kLongRow : r.w == kFracList && r.y > kLongRow;
+}
+
+// the long rows among the warp's cubes (record r, zero for none, level l)
+template <bool FP, typename AT>
+__device__ __forceinline__ void add_long_rows(const PushArgs& P, const Hist<FP>& H, uint4 r, uint32_t l) {
+    const int lane = threadIdx.x & 31;
+    for (unsigned m = __ballot_sync(0xffffffffu, long_row<AT>(r)); m; m &= m - 1) {
+        const int j = __ffs(m) - 1;
+        const uint32_t lj = 3 * __shfl_sync(0xffffffffu, l, j);
+        if constexpr (std::is_same<AT, float>::value) {
+            const uint32_t first = __shfl_sync(0xffffffffu, r.y, j), n = __shfl_sync(0xffffffffu, r.z, j);
+            const uint32_t sh = lj - __shfl_sync(0xffffffffu, r.w, j);
+            for (uint32_t e = lane; e < n; e += 32) {
+                const uint2 t = __ldg(P.lut + first + e);
+                H.add_int(t.x, t.y << sh);
+            }
+        } else {
+            const uint32_t first = __shfl_sync(0xffffffffu, r.x, j), n = __shfl_sync(0xffffffffu, r.y, j);
+            const float W = (float)(1u << lj);
+            for (uint32_t e = lane; e < n; e += 32) H.add_frac(__ldg(P.lut + first + e).x, W * __ldg(P.frac + first + e));
+        }
+    }
+}
+
 // Items [w0, w1) of one box by one warp, b the block holding item w0.
 //
 // The span is a flat stream of units.  A window holds the records of 31
@@ -1328,7 +1358,12 @@ __device__ __forceinline__ void add_record(const PushArgs& P, const Hist<FP>& H,
 // Only in the 128-thread instantiation, whose registers it fits: 100,000 boxes
 // with 1,182 segments 14.7 -> 12.0 ms; at 256 threads it spills (2,000 boxes
 // with 353 segments 189 -> 205 us).
-template <bool FP, typename AT, bool REC, bool PAIRS>
+//
+// LONG: rows above kLongRow by the whole warp.  Only where a CTA shares a
+// histogram: with up to 2,048 segments the rows are shorter and the chunks of
+// a warp many, 2 to 12 times faster on noise than the queues without it, and
+// the loop has no register to spare.
+template <bool FP, typename AT, bool REC, bool PAIRS, bool LONG>
 __device__ __forceinline__ void process_span(const MainArgs& A, const Hist<FP>& H, const Queue& Qu, Desc* desc,
                                              uint32_t w0, uint32_t w1, uint64_t b, uint64_t b1, uint32_t ncube) {
     const int lane = threadIdx.x & 31;
@@ -1485,10 +1520,14 @@ __device__ __forceinline__ void process_span(const MainArgs& A, const Hist<FP>& 
 #pragma unroll
                     for (int r = 0; r < R; r++) {
                         if (id[r] < S) run_add(id[r], 1u << (3 * lv[r]));
-                        else if (id[r] != kNone) {
+                        else if (id[r] != kNone && !(LONG && long_row<AT>(rec[r]))) {
                             if (PAIRS && rec[r].w == kFracPair) pair_add(rec[r], (float)(1u << (3 * lv[r])));
                             else add_record<FP, AT>(A.P, H, rec[r], id[r], lv[r]);
                         }
+                    }
+                    if constexpr (LONG) {
+#pragma unroll
+                        for (int r = 0; r < R; r++) add_long_rows<FP, AT>(A.P, H, rec[r], lv[r]);
                     }
                 } else {
 #pragma unroll
@@ -1575,7 +1614,7 @@ __global__ void __launch_bounds__(NT, WarpKernelBounds<NT>::min_ctas) query_warp
         const uint32_t ncube = (uint32_t)A.ncube[q];
         const uint32_t c0 = (c - (uint32_t)A.chunk_off[q]) * A.chunk;
         const uint32_t c1 = min(c0 + A.chunk, ncube);
-        process_span<FP, AT, REC, kPairs>(A, H, Qu, desc, c0, c1, __ldg(A.chunk_b + c), A.blk_off[q + 1], ncube);
+        process_span<FP, AT, REC, kPairs, false>(A, H, Qu, desc, c0, c1, __ldg(A.chunk_b + c), A.blk_off[q + 1], ncube);
         if constexpr (!REC) drain<FP, AT>(A.P, H, Qu, true);
         uint32_t* row = acc + (size_t)q * S;
         for (uint32_t s = 4 * lane; s < S4; s += 128) {
@@ -1671,7 +1710,7 @@ __global__ void __launch_bounds__(512, 2) query_batched_kernel(const __grid_cons
             }
             b = __shfl_sync(0xffffffffu, b, 0);
             bhint = b;
-            process_span<FP, AT, REC, false>(A, H, Qu, desc, w0, w1, b, b1, ncube);
+            process_span<FP, AT, REC, false, true>(A, H, Qu, desc, w0, w1, b, b1, ncube);
         }
         if constexpr (!REC) drain<FP, AT>(A.P, H, Qu, true);
         __syncthreads();

@@ -177,3 +177,25 @@ def test_chunks_of_every_length_the_default_takes(mg, S):
             plan.close()
     mg.mg_sync_status(g)
     g.close()
+
+
+@pytest.mark.parametrize("S", [2049, 3000, 18000])
+def test_rows_of_many_segments(mg, S):
+    """Noise: a cube of level 2 holds some 64 segments, one of level 3 some 500, at
+    every place of a warp's step, added by all its lanes."""
+    dims = (64, 48, 40)
+    vol = noise(dims, S, S)
+    g = mg.mg_build(torch.from_numpy(vol).cuda(), S)
+    bx = np.concatenate([some_boxes(dims, 200, S), [[0, 0, 0, *dims], [8, 8, 8, 16, 16, 16], [3, 0, 0, 5, 48, 40]]])
+    bx = bx.astype(np.int32)
+    t = torch.from_numpy(bx).cuda()
+    ref = oracle.box_hist(vol, S, bx).astype(np.float64)
+    for hist in ("u32", "f32"):
+        for kw in (dict(), dict(chunk_cubes=37), dict(schedule="plain")):
+            assert np.array_equal(mg.mg_query_boxes(g, t, hist=hist, **kw).cpu().numpy().astype(np.float64), ref)
+    for alpha, u in (("f16", 2.0 ** -11), ("bf16", 2.0 ** -8)):   # each unit crosses at most D rounded weights
+        h = mg.mg_query_boxes(g, t, hist="f32", alpha=alpha).cpu().numpy().astype(np.float64)
+        assert (np.abs(h - ref).sum(1) <= 1.5 * g.info["depth"] * u * ref.sum(1)).all()
+        assert ((h != 0) <= (ref != 0)).all()
+    mg.mg_sync_status(g)
+    g.close()
