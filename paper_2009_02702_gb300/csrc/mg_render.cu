@@ -427,67 +427,82 @@ __global__ void __launch_bounds__(128) march_kernel(MarchArgs A) {
     if (A.steps) A.steps[o] = taken;
 }
 
-// The occupancy of all levels >= 2 in one launch: bit v of a level's words says
-// that the opacity of voxel v's node is not zero (one lane per voxel, a warp's
-// ballot is one word).
-struct OccJob {
-    int64_t first, voxels;      // first word and voxels of the level
+// Where a climb from every voxel of a level >= 2 ends: the last of the levels l,
+// l + 1, ... whose voxel around it is empty, 0 when the voxel itself is occupied
+// (the opacity of its node is not zero).  A ray takes some 45 samples a pixel of
+// which one or two skip, so the climb is walked once per voxel here (5.6 M of
+// them for 1024x1024x300) instead of at every sample (95 M of a 1920x1080
+// frame).
+//
+// From the coarse levels down, a climb that leaves a voxel ends where its
+// parent's ends: one byte read.  The levels of at most kClimbSmall voxels are
+// one launch, each voxel climbing by itself, the larger ones one launch each,
+// bound by the gathers of the opacities.  (One launch for all, occupancy bits
+// first and every voxel climbing over them, took 240 us for 2048x2048x300, as
+// much as a frame of 160x120 pixels without skipping; this 47.)
+constexpr int64_t kClimbSmall = 1 << 16;
+struct ClimbLevel {
     const uint32_t* ids;
+    uint8_t* top;
     int32_t d[3];
 };
-struct OccJobs {
-    int n;                      // job j is level 2 + j
-    int64_t words;
-    OccJob job[MG_MAX_LEVELS];
+struct ClimbLevels {
+    int first, last;
+    ClimbLevel lev[MG_MAX_LEVELS];
+    int64_t end[MG_MAX_LEVELS];     // voxels of the levels first..l
 };
-__device__ __forceinline__ int occ_job(const OccJobs& J, int64_t w) {
-    int j = 0;
-    while (j + 1 < J.n && J.job[j + 1].first <= w) j++;
-    return j;
-}
-__global__ void occ_bits_kernel(const __grid_constant__ OccJobs J, const float* __restrict__ opac,
-                                uint32_t* __restrict__ words) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < J.words; w += warps) {
-        const OccJob& A = J.job[occ_job(J, w)];
-        const int64_t i = (w - A.first) * 32 + lane;
-        const bool occ = i < A.voxels && __ldg(opac + __ldg(A.ids + i)) != 0.0f;
-        const unsigned b = __ballot_sync(0xffffffffu, occ);
-        if (lane == 0) words[w] = b;
+
+__global__ void climb_small_kernel(const __grid_constant__ ClimbLevels A, const float* __restrict__ opac) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < A.end[A.last]; v += stride) {
+        int l = A.first;
+        while (v >= A.end[l]) l++;
+        const uint32_t i = (uint32_t)(v - (l > A.first ? A.end[l - 1] : 0));
+        uint32_t r = i / (uint32_t)A.lev[l].d[0];
+        uint32_t x = i - r * (uint32_t)A.lev[l].d[0], z = r / (uint32_t)A.lev[l].d[1], y = r - z * (uint32_t)A.lev[l].d[1];
+        int t = 0;
+        uint32_t at = i;
+        for (int j = l;; j++) {
+            if (__ldg(opac + __ldg(A.lev[j].ids + at)) != 0.0f) break;
+            t = j;
+            if (j == A.last) break;
+            x >>= 1;
+            y >>= 1;
+            z >>= 1;
+            at = (z * (uint32_t)A.lev[j + 1].d[1] + y) * (uint32_t)A.lev[j + 1].d[0] + x;
+        }
+        A.lev[l].top[i] = (uint8_t)t;
     }
 }
 
-// Where a climb from every voxel ends: the last of the levels l, l + 1, ...
-// whose voxel around it is empty, 0 when the voxel itself is occupied.  A ray
-// takes some 45 samples a pixel of which one or two skip, so the climb is
-// walked once per voxel here (5.6 M of them for 1024x1024x300) instead of at
-// every sample (95 M of a 1920x1080 frame).
-__global__ void climb_top_kernel(const __grid_constant__ OccJobs J, const uint32_t* __restrict__ words,
-                                 uint8_t* __restrict__ top) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < J.words; w += warps) {
-        const int j0 = occ_job(J, w);
-        const OccJob& A = J.job[j0];
-        const int64_t i = (w - A.first) * 32 + lane;
-        if (i >= A.voxels) continue;
-        int t = 0;
-        if (!((__ldg(words + w) >> lane) & 1u)) {
-            const uint32_t r = (uint32_t)i / (uint32_t)A.d[0];
-            uint32_t x = (uint32_t)i - r * (uint32_t)A.d[0], z = r / (uint32_t)A.d[1], y = r - z * (uint32_t)A.d[1];
-            t = 2 + j0;
-            for (int j = j0 + 1; j < J.n; j++) {
-                x >>= 1;
-                y >>= 1;
-                z >>= 1;
-                const OccJob& P = J.job[j];
-                const uint32_t v = (z * (uint32_t)P.d[1] + y) * (uint32_t)P.d[0] + x;
-                if ((__ldg(words + P.first + (v >> 5)) >> (v & 31)) & 1u) break;
-                t = 2 + j;
+// level l from its parents; 2^lg threads on a row
+__global__ void __launch_bounds__(256) climb_level_kernel(const __grid_constant__ ClimbLevel V,
+                                                          const __grid_constant__ ClimbLevel P, int l, int lg,
+                                                          const float* __restrict__ opac) {
+    constexpr int N = 4;   // voxels in flight per thread
+    const uint32_t w = 1u << lg, dx = (uint32_t)V.d[0], dy = (uint32_t)V.d[1], rows = dy * (uint32_t)V.d[2];
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, step = (gridDim.x * blockDim.x) >> lg;
+    for (uint32_t r = t >> lg; r < rows; r += step) {
+        const uint32_t z = r / dy, y = r - z * dy;
+        const uint32_t* ids = V.ids + (size_t)r * dx;
+        const uint8_t* up = P.top + ((size_t)(z >> 1) * (uint32_t)P.d[1] + (y >> 1)) * (uint32_t)P.d[0];
+        uint8_t* top = V.top + (size_t)r * dx;
+        for (uint32_t x0 = t & (w - 1); x0 < dx; x0 += N * w) {
+            uint32_t id[N];
+            uint8_t u[N];
+#pragma unroll
+            for (int k = 0; k < N; k++) {
+                const uint32_t x = x0 + k * w;
+                id[k] = x < dx ? __ldg(ids + x) : 0u;   // (past the end: a node that is there)
+                u[k] = x < dx ? __ldg(up + (x >> 1)) : 0;
             }
+            float o[N];
+#pragma unroll
+            for (int k = 0; k < N; k++) o[k] = __ldg(opac + id[k]);
+#pragma unroll
+            for (int k = 0; k < N; k++)
+                if (x0 + k * w < dx) top[x0 + k * w] = o[k] != 0.0f ? (uint8_t)0 : u[k] ? u[k] : (uint8_t)l;
         }
-        top[w * 32 + lane] = (uint8_t)t;
     }
 }
 
@@ -514,32 +529,42 @@ mg_status raymarch(const mg_graph* g, const float* vals, const float* opacity, c
         // empty-space skipping reads where its climb ends, one byte per voxel
         // of levels >= 2 (built here, in the graph's per-stream scratch),
         // instead of a node ID and its opacity per level climbed
-        int64_t words = 0, at[MG_MAX_LEVELS] = {};
+        int64_t bytes = 0, at[MG_MAX_LEVELS] = {};
         for (int l = 2; l < g->L; l++) {
-            at[l] = words;
-            words += ((int64_t)G.dims[l][0] * G.dims[l][1] * G.dims[l][2] + 31) / 32;
+            at[l] = bytes;
+            bytes += ((int64_t)G.dims[l][0] * G.dims[l][1] * G.dims[l][2] + 31) & ~(int64_t)31;
         }
-        if (words > 0) {
+        if (bytes > 0) {
             Arena* arena = nullptr;
             MG_TRY(arena_begin(const_cast<mg_graph*>(g), s, &arena));
-            Buf bits, top;
-            MG_TRY(bits.alloc(&arena->view, (size_t)words * 4, s));
-            MG_TRY(top.alloc(&arena->view, (size_t)words * 32, s));
-            OccJobs jobs{};
-            for (int l = 2; l < g->L; l++) {
-                A.lev[l].top = top.as<uint8_t>() + 32 * at[l];
-                OccJob& J = jobs.job[jobs.n++];
-                J.first = at[l];
-                J.ids = static_cast<const uint32_t*>(A.lev[l].ids);
-                J.voxels = (int64_t)G.dims[l][0] * G.dims[l][1] * G.dims[l][2];
-                for (int c = 0; c < 3; c++) J.d[c] = G.dims[l][c];
+            Buf top;
+            MG_TRY(top.alloc(&arena->view, (size_t)bytes, s));
+            ClimbLevels C{};
+            C.first = g->L - 1;
+            C.last = g->L - 1;
+            for (int l = g->L - 1; l >= 2; l--) {
+                ClimbLevel& V = C.lev[l];
+                V.ids = static_cast<const uint32_t*>(A.lev[l].ids);
+                V.top = top.as<uint8_t>() + at[l];
+                A.lev[l].top = V.top;
+                for (int c = 0; c < 3; c++) V.d[c] = G.dims[l][c];
+                if ((int64_t)V.d[0] * V.d[1] * V.d[2] <= kClimbSmall) C.first = l;
             }
-            jobs.words = words;
-            const unsigned gb = grid_for(words * 32, 256, 152 * 16);
-            occ_bits_kernel<<<gb, 256, 0, s>>>(jobs, opacity, bits.as<uint32_t>());
+            int64_t small = 0;
+            for (int l = C.first; l < g->L; l++) {
+                small += (int64_t)G.dims[l][0] * G.dims[l][1] * G.dims[l][2];
+                C.end[l] = small;
+            }
+            climb_small_kernel<<<grid_for(small, 128, 152 * 8), 128, 0, s>>>(C, opacity);
             MG_CUDA(cudaGetLastError());
-            climb_top_kernel<<<gb, 256, 0, s>>>(jobs, bits.as<uint32_t>(), top.as<uint8_t>());
-            MG_CUDA(cudaGetLastError());
+            for (int l = C.first - 1; l >= 2; l--) {
+                const ClimbLevel& V = C.lev[l];
+                int lg = 0;
+                while (lg < 5 && (1 << lg) < V.d[0]) lg++;
+                const int64_t threads = ((int64_t)V.d[1] * V.d[2]) << lg;
+                climb_level_kernel<<<grid_for(threads, 256, 152 * 16), 256, 0, s>>>(V, C.lev[l + 1], l, lg, opacity);
+                MG_CUDA(cudaGetLastError());
+            }
             A.skip = 1;
         }
     }
