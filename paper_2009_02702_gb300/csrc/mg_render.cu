@@ -26,9 +26,12 @@ __device__ __forceinline__ int32_t floor_coord(float x, int32_t d0) {
 // persistent query kernel that leaves 4,096 registers of an SM free, so a
 // lookup issued on another stream runs concurrently with it
 constexpr int kLookupThreads = 128;
-// samples per thread: a lookup is three dependent loads (sample, ID, row), and
-// two chains in flight per thread hide more of them than one
-constexpr int kLookupSamples = 2;
+// Samples per thread: a lookup is three dependent loads (sample, ID, row), and
+// two chains in flight per thread hide more of them than one.  Rows of 32 bytes
+// and more are bound by the copy, and a second one only spreads a warp's writes
+// (2.07 M samples of 512x512x384: 4-byte rows 20.6 us with one, 14.4 with two;
+// 64-byte rows 45.6 and 49.7).
+constexpr int lookup_samples(size_t row) { return row < 32 ? 2 : 1; }
 
 // index of the voxel of a sample in its level (32-bit: a volume holds fewer
 // than 2^32 voxels), and the level
@@ -53,14 +56,13 @@ __device__ __forceinline__ uint32_t voxel_node(const Geom& G, const void* __rest
     return __ldg(mip + G.off[l] + idx);
 }
 
-template <typename RowT>
+template <typename RowT, int N>
 __global__ void __launch_bounds__(kLookupThreads, 16) lookup_kernel(const __grid_constant__ Geom G,
                                                                     const void* __restrict__ mip0,
                                                                     const uint32_t* __restrict__ mip,
                                                                     const float4* __restrict__ samples, int64_t P,
                                                                     const RowT* __restrict__ vals, int words,
                                                                     RowT* __restrict__ out) {
-    constexpr int N = kLookupSamples;
     const int64_t i0 = (int64_t)blockIdx.x * (kLookupThreads * N) + threadIdx.x;
     uint32_t node[N];
     {
@@ -175,21 +177,21 @@ mg_status render_lookup(const mg_graph* g, const void* vals, int C, mg_dtype dt,
     if (!aligned(samples, 16)) return fail(MG_ERR_INVALID_ARG, "samples must be 16-byte aligned");
     const Geom G = render_geom(g);
     const size_t row = (size_t)C * (dt == MG_F32 ? 4 : 2);
-    const unsigned grid = grid_for(P, kLookupThreads * kLookupSamples);
+    const int each = lookup_samples(row);
+    const unsigned grid = grid_for(P, kLookupThreads * each);
     const float4* sm = reinterpret_cast<const float4*>(samples);
     const uint32_t* mip = g->mip.as<uint32_t>();
-    if (row % 16 == 0 && aligned(vals, 16) && aligned(out, 16))
-        lookup_kernel<uint4><<<grid, kLookupThreads, 0, s>>>(G, g->mip0.p, mip, sm, P, (const uint4*)vals, (int)(row / 16),
-                                                  (uint4*)out);
-    else if (row % 8 == 0 && aligned(vals, 8) && aligned(out, 8))
-        lookup_kernel<uint2><<<grid, kLookupThreads, 0, s>>>(G, g->mip0.p, mip, sm, P, (const uint2*)vals, (int)(row / 8),
-                                                  (uint2*)out);
-    else if (row % 4 == 0 && aligned(vals, 4) && aligned(out, 4))
-        lookup_kernel<uint32_t><<<grid, kLookupThreads, 0, s>>>(G, g->mip0.p, mip, sm, P, (const uint32_t*)vals,
-                                                     (int)(row / 4), (uint32_t*)out);
-    else
-        lookup_kernel<uint16_t><<<grid, kLookupThreads, 0, s>>>(G, g->mip0.p, mip, sm, P, (const uint16_t*)vals,
-                                                     (int)(row / 2), (uint16_t*)out);
+    auto launch = [&](auto k, auto* v, auto* o) {
+        k<<<grid, kLookupThreads, 0, s>>>(G, g->mip0.p, mip, sm, P, v, (int)(row / sizeof(*v)), o);
+    };
+    auto run = [&](auto word) {
+        using W = decltype(word);
+        launch(each == 2 ? lookup_kernel<W, 2> : lookup_kernel<W, 1>, static_cast<const W*>(vals), static_cast<W*>(out));
+    };
+    if (row % 16 == 0 && aligned(vals, 16) && aligned(out, 16)) run(uint4{});
+    else if (row % 8 == 0 && aligned(vals, 8) && aligned(out, 8)) run(uint2{});
+    else if (row % 4 == 0 && aligned(vals, 4) && aligned(out, 4)) run(uint32_t{});
+    else run(uint16_t{});
     MG_CUDA(cudaGetLastError());
     return MG_OK;
 }
