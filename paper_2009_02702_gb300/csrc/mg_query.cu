@@ -2565,11 +2565,12 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
                         : tuned_t > 0                      ? tuned_t
                         : o.schedule == MG_SCHED_BATCHED   ? default_threads(g, FP, (mg_dtype)o.alpha_dtype)
                                                            : 256;
-    // a fixed pool keeps the long chunks: its room is counted in them
     uint32_t chunk = o.chunk_cubes > 0 ? (uint32_t)o.chunk_cubes
                      : tuned_c > 0     ? (uint32_t)tuned_c
-                     : room            ? kDefaultChunk
                                        : default_chunk(g, FP, (mg_dtype)o.alpha_dtype, threads, Q);
+    // the room of a fixed pool is counted in long chunks: shorter ones are taken
+    // where the batch fits with them too, and there is one scan to repeat
+    if (room && Q > kFusedScanMax) chunk = std::max(chunk, kDefaultChunk);
     // Where the most that this many boxes can have fits a modest buffer, the
     // footprint is planned in one launch and nothing is read back: 1,000 boxes
     // of a 64^3 volume took 69 us with three plan kernels and the read-back of
@@ -2689,39 +2690,47 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
         MG_TRY(blk_off.alloc(&al, (size_t)(Q + 1) * 8, s));
         MG_TRY(chunk_off.alloc(&al, (size_t)(Q + 1) * 8, s));
         MG_TRY(ticket.alloc(&al, 8, s));
-        plan_count_kernel<<<grid_for(Q * 32, kPlanThreads), kPlanThreads, 0, s>>>(G, boxes, Q, chunk, nblk.as<uint32_t>(),
-                                                                ncube.as<uint64_t>(), nchunk.as<uint64_t>(),
-                                                                status, true);
-        MG_CUDA(cudaGetLastError());
-        if (Q <= kFusedScanMax) {
-            plan_scan_kernel<<<1, kScanThreads, 0, s>>>(nblk.as<uint32_t>(), nchunk.as<uint64_t>(), Q,
-                                                        blk_off.as<uint64_t>(), chunk_off.as<uint64_t>());
-            MG_CUDA(cudaGetLastError());
-        } else {
-            // block offsets are 64-bit sums of the 32-bit per-box counts
-            MG_TRY(scan_exclusive_u64(nchunk.as<uint64_t>(), chunk_off.as<uint64_t>(), Q,
-                                      chunk_off.as<uint64_t>() + Q, al, s));
-            Buf nb64;
-            MG_TRY(nb64.alloc(&al, (size_t)Q * 8, s));
-            widen_kernel<<<grid_for(Q, 256, 152 * 64), 256, 0, s>>>(nblk.as<uint32_t>(), nb64.as<uint64_t>(), Q);
-            MG_CUDA(cudaGetLastError());
-            MG_TRY(scan_exclusive_u64(nb64.as<uint64_t>(), blk_off.as<uint64_t>(), Q, blk_off.as<uint64_t>() + Q, al,
-                                      s));
-        }
         uint64_t* totals = words;   // blocks, chunks
-        MG_CUDA(cudaMemcpyAsync(&totals[0], blk_off.as<uint64_t>() + Q, 8, cudaMemcpyDeviceToHost, s));
-        MG_CUDA(cudaMemcpyAsync(&totals[1], chunk_off.as<uint64_t>() + Q, 8, cudaMemcpyDeviceToHost, s));
-        MG_CUDA(cudaStreamSynchronize(s));
-        if (totals[0] >= (1ull << 32) || totals[1] >= (1ull << 32))
-            return fail(MG_ERR_UNSUPPORTED, "more than 2^32 footprint blocks or work chunks in one call");
-        if (room) {
-            const size_t need = (((size_t)std::max<uint64_t>(totals[0], 1) * sizeof(Blk) + 255) & ~(size_t)255) +
-                                2 * (((size_t)std::max<uint64_t>(totals[1], 1) * 4 + 255) & ~(size_t)255);
-            if (need > room(al))
-                return fail(MG_ERR_CAPACITY, "these boxes need " + std::to_string(need >> 10) +
-                                                 " KiB of footprint scratch; " + std::to_string(room(al) >> 10) +
-                                                 " KiB of the fixed scratch remain: split the batch");
+        for (;;) {
+            plan_count_kernel<<<grid_for(Q * 32, kPlanThreads), kPlanThreads, 0, s>>>(G, boxes, Q, chunk, nblk.as<uint32_t>(),
+                                                                    ncube.as<uint64_t>(), nchunk.as<uint64_t>(),
+                                                                    status, true);
+            MG_CUDA(cudaGetLastError());
+            if (Q <= kFusedScanMax) {
+                plan_scan_kernel<<<1, kScanThreads, 0, s>>>(nblk.as<uint32_t>(), nchunk.as<uint64_t>(), Q,
+                                                            blk_off.as<uint64_t>(), chunk_off.as<uint64_t>());
+                MG_CUDA(cudaGetLastError());
+            } else {
+                // block offsets are 64-bit sums of the 32-bit per-box counts
+                MG_TRY(scan_exclusive_u64(nchunk.as<uint64_t>(), chunk_off.as<uint64_t>(), Q,
+                                          chunk_off.as<uint64_t>() + Q, al, s));
+                Buf nb64;
+                MG_TRY(nb64.alloc(&al, (size_t)Q * 8, s));
+                widen_kernel<<<grid_for(Q, 256, 152 * 64), 256, 0, s>>>(nblk.as<uint32_t>(), nb64.as<uint64_t>(), Q);
+                MG_CUDA(cudaGetLastError());
+                MG_TRY(scan_exclusive_u64(nb64.as<uint64_t>(), blk_off.as<uint64_t>(), Q, blk_off.as<uint64_t>() + Q, al,
+                                          s));
+            }
+            MG_CUDA(cudaMemcpyAsync(&totals[0], blk_off.as<uint64_t>() + Q, 8, cudaMemcpyDeviceToHost, s));
+            MG_CUDA(cudaMemcpyAsync(&totals[1], chunk_off.as<uint64_t>() + Q, 8, cudaMemcpyDeviceToHost, s));
+            MG_CUDA(cudaStreamSynchronize(s));
+            if (totals[0] >= (1ull << 32) || totals[1] >= (1ull << 32))
+                return fail(MG_ERR_UNSUPPORTED, "more than 2^32 footprint blocks or work chunks in one call");
+            if (room) {
+                const size_t need = (((size_t)std::max<uint64_t>(totals[0], 1) * sizeof(Blk) + 255) & ~(size_t)255) +
+                                    2 * (((size_t)std::max<uint64_t>(totals[1], 1) * 4 + 255) & ~(size_t)255);
+                if (need > room(al) && chunk < kDefaultChunk && o.chunk_cubes <= 0 && tuned_c <= 0) {
+                    chunk = kDefaultChunk;
+                    continue;
+                }
+                if (need > room(al))
+                    return fail(MG_ERR_CAPACITY, "these boxes need " + std::to_string(need >> 10) +
+                                                     " KiB of footprint scratch; " + std::to_string(room(al) >> 10) +
+                                                     " KiB of the fixed scratch remain: split the batch");
+            }
+            break;
         }
+        A.chunk = chunk;
         MG_TRY(blk.alloc(&al, (size_t)std::max<uint64_t>(totals[0], 1) * sizeof(Blk), s));
         MG_TRY(chunk_q.alloc(&al, (size_t)std::max<uint64_t>(totals[1], 1) * 4, s));
         MG_TRY(chunk_b.alloc(&al, (size_t)std::max<uint64_t>(totals[1], 1) * 4, s));

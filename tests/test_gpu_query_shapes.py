@@ -199,3 +199,39 @@ def test_rows_of_many_segments(mg, S):
         assert ((h != 0) <= (ref != 0)).all()
     mg.mg_sync_status(g)
     g.close()
+
+
+def test_fixed_scratch_filled_to_its_limit(mg):
+    """The scratch-free call takes short chunks for small batches; a batch whose
+    blocks leave no room for them is planned with long ones before it is refused."""
+    dims, S = (255, 255, 255), 50
+    z, y, x = np.meshgrid(*(np.arange(n) // 32 for n in dims), indexing="ij")
+    vol = ((x + 8 * y + 64 * z) % S).astype(np.uint16)
+    g = mg.mg_build(torch.from_numpy(vol).cuda(), S)
+    one = np.array([[1, 1, 1, 253, 253, 253]], np.int32)
+    ref = oracle.box_hist(vol, S, one)[0]
+    out = torch.empty((4000, S), dtype=torch.uint32, device="cuda")
+
+    def fits(Q):
+        t = torch.from_numpy(one.repeat(Q, 0)).cuda()
+        try:
+            mg.mg_query_boxes_noalloc(g, t, out=out[:Q])
+        except mg.MGError as e:
+            assert e.status == mg.MG_ERR_CAPACITY
+            return False
+        return True
+
+    lo, hi = 1, 4000
+    while hi - lo > 1:
+        mid = (lo + hi) // 2
+        lo, hi = (mid, hi) if fits(mid) else (lo, mid)
+    for Q in (1, lo - 20, lo):
+        assert fits(Q)
+        got = out[:Q].cpu().numpy()
+        assert (got == ref).all(), Q
+    # 12 bytes a block and 8 a chunk, at most one chunk a box more than its cubes fill
+    blocks = 13 ** 3
+    cubes = int(mg.mg_count_cubes(g, torch.from_numpy(one).cuda()).cpu().numpy()[0])
+    assert (lo + 1) * (12 * blocks + 8 * (cubes // 2048 + 1)) > (60 << 20)
+    mg.mg_sync_status(g)
+    g.close()
