@@ -25,19 +25,24 @@
 // blocks of such words at `first` in the pool.
 //
 // Edge-8 tiles of level 0 and lines of level 1 are counted from the IDs: a
-// thread reads its tile, settles it when it is one segment, reads it again and
-// settles it when it is two (four in five of the mixed tiles of a volume of
-// cells): the second segment differs from the first in some bit, and that bit
-// of an ID says which of the two it has to be, so a word of two IDs costs five
-// instructions and no branch.  The warp takes the other tiles one by one, its
-// lanes finding the distinct segments together, a chain of warp reductions.
-// 512x512x384, edge-8 tiles / lines: 186 / 295 us with only one-segment tiles
-// settled by their thread, 125 / 163 with two-segment ones too (per-thread
-// lists of up to four segments took 385 us for the edge-8 tiles: a warp nearly
-// always holds a mixed tile, so all of it walked the list code for every
-// voxel).  An edge-16 tile is the sum of four edge-8 ones, an edge-8 tile of
-// level l + 1 the sum of two edge-16 ones of level l, and a line of level
-// l + 1 the sum of eight lines.
+// thread holds its tile in registers and takes its segments in ascending order,
+// one pass over the tile each that counts the IDs equal to this segment and
+// finds the least ID above it (three instructions a word of two IDs and the
+// sum), so that a warp's 32 tiles advance together whatever they hold.  Tiles
+// of more than kOwnSegments segments are left to the warp, which counts one at
+// a time in a table in shared memory.  Edge-8 tiles / lines, us: 512x512x384
+// cells 118 / 125, 614x961x600 fibres 1,062 / 903, 255x256x257 bricks of five to
+// eight segments a tile 49 / 79 (125 / 163, 3,101 / 3,403 and 264 / 843 with the
+// warp counting all tiles of more than two segments, by reductions).
+//
+// An edge-16 tile is the sum of four edge-8 ones, an edge-8 tile of level l + 1
+// the sum of two edge-16 ones of level l, and a line of level l + 1 the sum of
+// eight lines: a thread collects its children's words, the warp those of tiles
+// with more than kOwnWords (the fibres, all merges: 3,360 -> 1,780 us; 12, 16
+// and 24 words 2,201 / 1,834 / 1,767), or of every list where there are few tiles.
+//
+// A stage whose lists find no room in the pool ends there, and those made from
+// it at once: they are not used.
 #include "mg_internal.cuh"
 
 #include <algorithm>
@@ -49,6 +54,8 @@ namespace {
 constexpr int kThreads = 128;
 constexpr int kWarps = kThreads / 32;
 constexpr uint32_t kReserve = 32;       // pool blocks a warp reserves at a time
+constexpr uint32_t kOwnSegments = 16;   // segments that a thread counts by itself
+constexpr uint32_t kOwnWords = 24;      // distinct words that a thread collects by itself
 constexpr uint32_t kMaxMerge = 256;     // words merged into distinct segments; longer lists are joined as they are
 constexpr uint32_t kSegMask = 0xFFFFu;
 
@@ -57,46 +64,18 @@ struct Counters {
     unsigned failed[kTileStages];       // a list of the stage did not fit the pool
 };
 
-// up to four (segment, count) words built one occurrence at a time
-struct Few {
-    uint32_t id[4], n[4];
-    bool over;
-    __device__ __forceinline__ Few() : over(false) {
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            id[k] = 0x10000u;   // no segment
-            n[k] = 0;
-        }
-    }
-    __device__ __forceinline__ void add(uint32_t s, uint32_t c) {
-        bool hit = false;
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            const bool take = !hit && (id[k] == s || n[k] == 0);
-            if (take) {
-                id[k] = s;
-                n[k] += c;
-            }
-            hit = hit || take;
-        }
-        over = over || !hit;
-    }
-    __device__ __forceinline__ uint4 record() const {
-        uint32_t w[4];
-#pragma unroll
-        for (int k = 0; k < 4; k++) w[k] = n[k] ? (id[k] | n[k] << 16) : 0u;
-        return make_uint4(w[0], w[1], w[2], w[3]);
-    }
-};
-
 // a warp's part of the pool: [cur, end), refilled by one atomic per kReserve blocks
 struct PoolCursor {
     uint4* pool;
     unsigned long long cap, cur, end;
     Counters* cnt;
     int stage;
+    bool full;   // no room for a list: the stage is not used, its warps leave
+    __device__ __forceinline__ PoolCursor(uint4* p, unsigned long long c, Counters* n, int st)
+        : pool(p), cap(c), cur(0), end(0), cnt(n), stage(st), full(false) {}
     // `need` blocks (same value in every lane), or ~0 when the pool is full
     __device__ __forceinline__ unsigned long long take(uint32_t need) {
+        if (full) return ~0ull;
         if (cur + need > end) {
             const uint32_t r = max(need, kReserve);
             unsigned long long b = 0;
@@ -104,6 +83,7 @@ struct PoolCursor {
             b = __shfl_sync(0xffffffffu, b, 0);
             if (b + r > cap) {
                 if ((threadIdx.x & 31) == 0) cnt->failed[stage] = 1u;
+                full = true;
                 return ~0ull;
             }
             cur = b;
@@ -115,31 +95,40 @@ struct PoolCursor {
     }
 };
 
-// The distinct segments of the warp's words (K per lane, segment | count << 16
-// with count 0 for none), ascending, with summed counts, into buf; returns
-// their number.
-template <int K>
-__device__ __forceinline__ uint32_t distinct(uint32_t (&w)[K], int used, uint32_t* buf) {
-    uint32_t n = 0;
-    for (;;) {
-        uint32_t m = 0xFFFFFFFFu;
-#pragma unroll
-        for (int j = 0; j < K; j++)
-            if (j < used && (w[j] >> 16)) m = min(m, w[j] & kSegMask);
-        m = __reduce_min_sync(0xffffffffu, m);
-        if (m == 0xFFFFFFFFu) return n;
-        uint32_t c = 0;
-#pragma unroll
-        for (int j = 0; j < K; j++)
-            if (j < used && (w[j] >> 16) && (w[j] & kSegMask) == m) {
-                c += w[j] >> 16;
-                w[j] = 0;
+// A warp's table of segments: words segment | count << 16 at the segment's hash
+// or the next free place, zero where there is none and between tiles.  It holds
+// at most half of its 2^lg places.
+struct Table {
+    uint32_t* at;
+    int lg;
+    __device__ __forceinline__ void add(uint32_t w) const {
+        const uint32_t mask = (1u << lg) - 1u, s = w & kSegMask;
+        for (uint32_t h = (s * 0x9E3779B1u) >> (32 - lg);; h = (h + 1) & mask) {
+            const uint32_t old = atomicCAS(at + h, 0u, w);
+            if (old == 0u) return;
+            if ((old & kSegMask) == s) {
+                atomicAdd(at + h, w & ~kSegMask);
+                return;
             }
-        c = __reduce_add_sync(0xffffffffu, c);
-        if ((threadIdx.x & 31) == 0) buf[n] = m | c << 16;
-        n++;
+        }
     }
-}
+    // its words into buf (warp); returns their number
+    __device__ __forceinline__ uint32_t take(uint32_t* buf) const {
+        const int lane = threadIdx.x & 31;
+        uint32_t n = 0;
+        __syncwarp();
+        for (uint32_t h = lane; h < 1u << lg; h += 32) {
+            const uint32_t w = at[h];
+            const unsigned m = __ballot_sync(0xffffffffu, w != 0u);
+            if (w) {
+                buf[n + __popc(m & ((1u << lane) - 1u))] = w;
+                at[h] = 0u;
+            }
+            n += __popc(m);
+        }
+        return n;
+    }
+};
 
 // the record of a tile whose n words are in buf (warp)
 __device__ __forceinline__ uint4 finish(PoolCursor& P, const uint32_t* buf, uint32_t n) {
@@ -158,6 +147,40 @@ __device__ __forceinline__ uint4 finish(PoolCursor& P, const uint32_t* buf, uint
         }
     }
     __syncwarp();
+    return rec;
+}
+
+// The records of the warp's tiles, each with n words at w (shared memory,
+// kThreads apart): lists of more than four go to the pool, with one atomic for
+// the warp.  n = 0: none (the warp path's).
+__device__ __forceinline__ uint4 emit(PoolCursor& P, const uint32_t* w, uint32_t n) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t need = n > 4 ? (n + 3) / 4 : 0u;
+    uint4 rec = make_uint4(n > 0 ? w[0] : 0u, n > 1 ? w[kThreads] : 0u, n > 2 ? w[2 * kThreads] : 0u,
+                           n > 3 ? w[3 * kThreads] : 0u);
+    if (__any_sync(0xffffffffu, need != 0u)) {
+        uint32_t incl = need;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+        unsigned long long base = 0;
+        if (lane == 0) base = atomicAdd(&P.cnt->used, (unsigned long long)total);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (base + total > P.cap) {
+            if (lane == 0) P.cnt->failed[P.stage] = 1u;
+            P.full = true;
+        } else if (need) {
+            const uint32_t first = (uint32_t)base + incl - need;
+            for (uint32_t k = 0; k < n; k += 4)
+                P.pool[first + k / 4] = make_uint4(w[k * kThreads], k + 1 < n ? w[(k + 1) * kThreads] : 0u,
+                                                   k + 2 < n ? w[(k + 2) * kThreads] : 0u,
+                                                   k + 3 < n ? w[(k + 3) * kThreads] : 0u);
+            rec = make_uint4(kTileList, first, need, 0u);
+        }
+    }
     return rec;
 }
 
@@ -181,66 +204,82 @@ __global__ void __launch_bounds__(kThreads) tile_ids_kernel(const __grid_constan
     constexpr int ROWS = LINE ? 4 : 8, VECS = LINE ? 4 : 1;   // rows of a tile, 16-byte vectors of a row
     constexpr int PER = LINE ? 4 : 2;                         // IDs per lane of a warp's tile
     constexpr uint32_t VOX = ROWS * VECS * 8;
-    __shared__ uint32_t s_buf[kWarps][VOX];
+    constexpr int LG = LINE ? 8 : 7;                          // places of the warp's table: twice the IDs
+    static_assert(2 * VOX == 1u << LG, "a table is at most half full");
+    constexpr int WORDS = VOX / 2;
+    if (cnt->used >= cap) {   // no list has room
+        if (threadIdx.x == 0) cnt->failed[stage] = 1u;
+        return;
+    }
+    __shared__ uint32_t s_buf[kWarps][VOX], s_tab[kWarps][1 << LG], s_own[kOwnSegments * kThreads];
+    uint32_t* own = s_own + threadIdx.x;
     const int c = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t tiles = A.tiles[c], na = A.na[c], nb = A.nb[c], st1 = A.st1[c];
     const int64_t st2 = A.st2[c];
     auto row = [&](int k) -> int64_t {
         return LINE ? (int64_t)(k >> 1) * st2 + (int64_t)(k & 1) * st1 : (int64_t)k * st1;
     };
-    PoolCursor P{pool, cap, 0, 0, cnt, stage};
+    PoolCursor P(pool, cap, cnt, stage);
+    const Table table{s_tab[warp], LG};
+    for (int h = lane; h < 1 << LG; h += 32) s_tab[warp][h] = 0u;
+    __syncwarp();
     const uint32_t step = gridDim.x * kWarps * per;
-    for (uint32_t i0 = (blockIdx.x * kWarps + warp) * per; i0 < tiles; i0 += step) {
+    for (uint32_t i0 = (blockIdx.x * kWarps + warp) * per; i0 < tiles && !P.full; i0 += step) {
         const uint32_t i = (uint32_t)lane < per ? i0 + lane : tiles;
         const uint16_t* p = A.ids[c];
-        uint32_t d = 0, s0 = 0;
+        uint32_t x[WORDS];
         if (i < tiles) {
             const uint32_t a = i % na, r = i / na, b = r % nb, t = r / nb;
             p += LINE ? (int64_t)(2 * t) * st2 + (int64_t)(2 * b) * st1 + 32 * a
                       : (int64_t)t * st2 + (int64_t)(8 * b) * st1 + 8 * a;
-            s0 = (uint32_t)__ldg(p);
-            const uint32_t pat = s0 * 0x10001u;
             if (A.vec[c]) {
 #pragma unroll
                 for (int k = 0; k < ROWS; k++)
 #pragma unroll
                     for (int v = 0; v < VECS; v++) {
                         const uint4 u = __ldg(reinterpret_cast<const uint4*>(p + row(k)) + v);
-                        const uint32_t x[4] = {u.x ^ pat, u.y ^ pat, u.z ^ pat, u.w ^ pat};
-#pragma unroll
-                        for (int e = 0; e < 4; e++) d = x[e] ? x[e] : d;
+                        const int e = 4 * (k * VECS + v);
+                        x[e] = u.x;
+                        x[e + 1] = u.y;
+                        x[e + 2] = u.z;
+                        x[e + 3] = u.w;
                     }
             } else {
+#pragma unroll
                 for (int k = 0; k < ROWS; k++)
-                    for (int v = 0; v < 8 * VECS; v++) d |= (uint32_t)__ldg(p + row(k) + v) ^ s0;
+#pragma unroll
+                    for (int v = 0; v < 4 * VECS; v++)
+                        x[4 * k * VECS + v] = (uint32_t)__ldg(p + row(k) + 2 * v) |
+                                              (uint32_t)__ldg(p + row(k) + 2 * v + 1) << 16;
             }
+        } else {
+#pragma unroll
+            for (int e = 0; e < WORDS; e++) x[e] = 0u;
         }
-        uint4 rec = make_uint4(s0 | VOX << 16, 0u, 0u, 0u);
-        if (d != 0 && A.vec[c]) {
-            // a second segment s0 ^ e: of two-segment tiles every ID ^ s0 is 0 or e, told apart by one bit of e
-            const uint32_t pat = s0 * 0x10001u, e = (d & kSegMask) ? d & kSegMask : d >> 16, bit = __ffs(e) - 1;
-            uint32_t other = 0, n2 = 0;
+        // the least ID, then the segments in ascending order
+        uint32_t m2 = x[0], cur = 0, n = 0;
 #pragma unroll
-            for (int k = 0; k < ROWS; k++)
+        for (int e = 1; e < WORDS; e++) m2 = __vminu2(m2, x[e]);
+        cur = min(m2 & kSegMask, m2 >> 16);
+        bool more = true;
+        while (more && n < kOwnSegments) {
+            const uint32_t pat = cur * 0x10001u, below = ((0xFFFFu - cur) & kSegMask) * 0x10001u;
+            uint32_t other = 0, above = 0xFFFFFFFFu;
 #pragma unroll
-                for (int v = 0; v < VECS; v++) {
-                    const uint4 u = __ldg(reinterpret_cast<const uint4*>(p + row(k)) + v);
-                    const uint32_t x[4] = {u.x ^ pat, u.y ^ pat, u.z ^ pat, u.w ^ pat};
-#pragma unroll
-                    for (int q = 0; q < 4; q++) {
-                        const uint32_t y = (x[q] >> bit) & 0x10001u;   // a 1 per ID with e's bit
-                        n2 += y;
-                        other |= x[q] ^ y * e;
-                    }
-                }
-            if (other == 0) {
-                const uint32_t n = (n2 & kSegMask) + (n2 >> 16), s1 = s0 ^ e;
-                const uint32_t w0 = s0 | (VOX - n) << 16, w1 = s1 | n << 16;
-                rec = s0 < s1 ? make_uint4(w0, w1, 0u, 0u) : make_uint4(w1, w0, 0u, 0u);
-                d = 0;
+            for (int e = 0; e < WORDS; e++) {
+                other += __vminu2(x[e] ^ pat, 0x10001u);                // 1 per ID that is not cur
+                above = __viaddmin_u16x2(x[e], below, above);           // ID - cur - 1 modulo 2^16
             }
+            own[n * kThreads] = cur | (VOX - (other & kSegMask) - (other >> 16)) << 16;
+            n++;
+            const uint32_t next = min(above & kSegMask, above >> 16) + cur + 1u;   // past 2^16: none above cur
+            more = next <= kSegMask;
+            cur = next;
         }
-        for (unsigned m = __ballot_sync(0xffffffffu, d != 0); m; m &= m - 1) {
+        const uint32_t d = more ? 1u : 0u;   // the warp counts it
+        uint4 rec = emit(P, own, more || i >= tiles ? 0u : n);
+        if (P.full) break;
+        for (unsigned m = __ballot_sync(0xffffffffu, d != 0); m && !P.full; m &= m - 1) {
             const int j = __ffs(m) - 1;
             const uint16_t* q = reinterpret_cast<const uint16_t*>(
                 __shfl_sync(0xffffffffu, (unsigned long long)reinterpret_cast<uintptr_t>(p), j));
@@ -251,14 +290,25 @@ __global__ void __launch_bounds__(kThreads) tile_ids_kernel(const __grid_constan
 #pragma unroll
                 for (int e = 0; e < PER; e += 2) {
                     const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(q) + e / 2);
-                    v[e] = (w & kSegMask) | 1u << 16;
-                    v[e + 1] = (w >> 16) | 1u << 16;
+                    v[e] = w & kSegMask;
+                    v[e + 1] = w >> 16;
                 }
             } else {
 #pragma unroll
-                for (int e = 0; e < PER; e++) v[e] = (uint32_t)__ldg(q + e) | 1u << 16;
+                for (int e = 0; e < PER; e++) v[e] = (uint32_t)__ldg(q + e);
             }
-            const uint4 lr = finish(P, s_buf[warp], distinct<PER>(v, PER, s_buf[warp]));
+            uint32_t run = v[0] | 1u << 16;
+#pragma unroll
+            for (int e = 1; e < PER; e++) {
+                if (v[e] == (run & kSegMask)) {
+                    run += 1u << 16;
+                } else {
+                    table.add(run);
+                    run = v[e] | 1u << 16;
+                }
+            }
+            table.add(run);
+            const uint4 lr = finish(P, s_buf[warp], table.take(s_buf[warp]));
             if (lane == j) rec = lr;
         }
         if (i < tiles) A.out[c][i] = rec;
@@ -278,16 +328,26 @@ struct Merge {
 template <int CH>
 __global__ void __launch_bounds__(kThreads) tile_merge_kernel(const __grid_constant__ Merge A, uint4* pool,
                                                               unsigned long long cap, Counters* cnt, int stage,
-                                                              uint32_t per) {
-    __shared__ uint32_t s_buf[kWarps][kMaxMerge];
+                                                              int from, uint32_t per) {
+    if (cnt->failed[from] || cnt->used >= cap) {   // the records read here are not all there, or no list has room
+        if (threadIdx.x == 0) cnt->failed[stage] = 1u;
+        return;
+    }
+    __shared__ uint32_t s_buf[kWarps][kMaxMerge], s_tab[kWarps][2 * kMaxMerge], s_own[kOwnWords * kThreads];
+    uint32_t* own = s_own + threadIdx.x;
     const int c = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t tiles = A.tiles[c], na = A.na[c], nb = A.nb[c];
-    PoolCursor P{pool, cap, 0, 0, cnt, stage};
+    PoolCursor P(pool, cap, cnt, stage);
+    for (uint32_t h = lane; h < 2 * kMaxMerge; h += 32) s_tab[warp][h] = 0u;
+    __syncwarp();
     const uint32_t step = gridDim.x * kWarps * per;
-    for (uint32_t i0 = (blockIdx.x * kWarps + warp) * per; i0 < tiles; i0 += step) {
+    for (uint32_t i0 = (blockIdx.x * kWarps + warp) * per; i0 < tiles && !P.full; i0 += step) {
         const uint32_t i = (uint32_t)lane < per ? i0 + lane : tiles;
         uint4 in[CH];
-        Few f;
+        // (where a warp has few tiles, its lanes are better spent on one each time)
+        const uint32_t most = per == 32 ? kOwnWords : 4u;
+        uint32_t n = 0, total = 0;
+        bool over = false;
 #pragma unroll
         for (int k = 0; k < CH; k++) in[k] = make_uint4(0u, 0u, 0u, 0u);
         if (i < tiles) {
@@ -300,23 +360,42 @@ __global__ void __launch_bounds__(kThreads) tile_merge_kernel(const __grid_const
                 in[k] = __ldg(A.in[c] + at);
             }
 #pragma unroll
-            for (int k = 0; k < CH; k++) {
-                const uint32_t w[4] = {in[k].x, in[k].y, in[k].z, in[k].w};
-                if (w[0] == kTileList) {
-                    f.over = true;
-                } else {
+            for (int k = 0; k < CH; k++) total += in[k].x == kTileList ? 4u * in[k].z : 4u;
+            over = total > 4 * most;
+        }
+        auto collect = [&](uint32_t w) {
+            if (!(w >> 16)) return;
+            uint32_t q = 0;
+            while (q < n && ((own[q * kThreads] ^ w) & kSegMask)) q++;
+            if (q < n) {
+                own[q * kThreads] += w & ~kSegMask;
+            } else if (n < most) {
+                own[n * kThreads] = w;
+                n++;
+            } else {
+                over = true;
+            }
+        };
 #pragma unroll
-                    for (int e = 0; e < 4; e++)
-                        if (w[e] >> 16) f.add(w[e] & kSegMask, w[e] >> 16);
-                }
+        for (int k = 0; k < CH; k++) {
+            const bool list = in[k].x == kTileList;
+            const uint32_t blocks = over ? 0u : list ? in[k].z : 1u;
+            for (uint32_t q = 0; q < blocks && !over; q++) {
+                const uint4 w = list ? pool[in[k].y + q] : in[k];
+                collect(w.x);
+                collect(w.y);
+                collect(w.z);
+                collect(w.w);
             }
         }
-        uint4 rec = f.record();
-        for (unsigned m = __ballot_sync(0xffffffffu, f.over); m; m &= m - 1) {
+        uint4 rec = emit(P, own, over ? 0u : n);
+        if (P.full) break;
+        for (unsigned m = __ballot_sync(0xffffffffu, over); m && !P.full; m &= m - 1) {
             const int j = __ffs(m) - 1;
             // the children's words as one sequence: four of an inline record, the pool's of a list
             uint4 ch[CH];
-            uint32_t end[CH], total = 0;
+            uint32_t end[CH];
+            total = 0;
 #pragma unroll
             for (int k = 0; k < CH; k++) {
                 ch[k] = make_uint4(__shfl_sync(0xffffffffu, in[k].x, j), __shfl_sync(0xffffffffu, in[k].y, j),
@@ -339,13 +418,12 @@ __global__ void __launch_bounds__(kThreads) tile_merge_kernel(const __grid_const
             };
             uint4 lr;
             if (total <= kMaxMerge) {
-                constexpr int K = kMaxMerge / 32;
-                const int used = (int)(total + 31) / 32;
-                uint32_t v[K];
-#pragma unroll
-                for (int q = 0; q < K; q++) v[q] = q < used && (uint32_t)(lane + 32 * q) < total ? word(lane + 32 * q) : 0u;
-                const uint32_t n = distinct<K>(v, used, s_buf[warp]);
-                lr = finish(P, s_buf[warp], n);
+                const Table table{s_tab[warp], max(5, 32 - __clz(2 * total - 1))};
+                for (uint32_t e = lane; e < total; e += 32) {
+                    const uint32_t w = word(e);
+                    if (w >> 16) table.add(w);
+                }
+                lr = finish(P, s_buf[warp], table.take(s_buf[warp]));
             } else {
                 // long lists are joined: a segment may appear twice, its counts still add up
                 const unsigned long long at = P.take(total / 4);
@@ -507,13 +585,13 @@ mg_status build_tiles(mg_graph* g, cudaStream_t s) {
     // room for lists of 2 bytes per voxel (noise would need 12 and gets no
     // tiles); the part that is used is kept
     const unsigned long long cap = (unsigned long long)std::max<int64_t>(V / 8, 1 << 16);
-    Buf cnt_b, pool;
-    if (!try_alloc(g->tiles, &g->al, (size_t)total * sizeof(uint4), s) || !try_alloc(cnt_b, &g->al, sizeof(Counters), s) ||
-        !try_alloc(pool, &g->al, (size_t)cap * sizeof(uint4), s)) {
+    Buf pool;   // the blocks, then the counters
+    if (!try_alloc(g->tiles, &g->al, (size_t)total * sizeof(uint4), s) ||
+        !try_alloc(pool, &g->al, (size_t)cap * sizeof(uint4) + sizeof(Counters), s)) {
         g->tiles.release();
         return MG_OK;
     }
-    Counters* cnt = cnt_b.as<Counters>();
+    Counters* cnt = reinterpret_cast<Counters*>(pool.as<uint4>() + cap);
     MG_CUDA(cudaMemsetAsync(cnt, 0, sizeof(Counters), s));
     uint4* rec = g->tiles.as<uint4>();
     for (size_t k = 0; k < stages.size(); k++) {
@@ -552,7 +630,9 @@ mg_status build_tiles(mg_graph* g, cudaStream_t s) {
                 A.tiles[c] = (uint32_t)st.count[c];
             }
             auto kernel = st.kind == 0 ? tile_merge_kernel<2> : st.kind == 1 ? tile_merge_kernel<4> : tile_merge_kernel<8>;
-            kernel<<<grid, kThreads, 0, s>>>(A, pool.as<uint4>(), cap, cnt, (int)k, per);
+            int from = 0;
+            while (stages[from].kind != st.from_kind || stages[from].l != st.from_l) from++;
+            kernel<<<grid, kThreads, 0, s>>>(A, pool.as<uint4>(), cap, cnt, (int)k, from, per);
         }
         MG_CUDA(cudaGetLastError());
     }
@@ -560,6 +640,7 @@ mg_status build_tiles(mg_graph* g, cudaStream_t s) {
     MG_CUDA(cudaMemcpyAsync(&h, cnt, sizeof(h), cudaMemcpyDeviceToHost, s));
     MG_CUDA(cudaStreamSynchronize(s));
     // a stage whose lists did not fit, and those made from it, are not used
+    // (nor read: their records are not all written)
     bool ok[kTileLevels][3] = {};
     for (size_t k = 0; k < stages.size(); k++) {
         const Stage& st = stages[k];
@@ -574,7 +655,8 @@ mg_status build_tiles(mg_graph* g, cudaStream_t s) {
     }
     const size_t kept = (size_t)std::min(h.used, cap) * sizeof(uint4);
     if (kept == 0) return MG_OK;
-    if (kept < pool.bytes / 4 * 3 && try_alloc(g->tile_pool, &g->al, kept, s))
+    // (a megabyte is not worth another allocation and copy: importing 64^3 takes 0.2 ms)
+    if (kept < pool.bytes / 4 * 3 && pool.bytes - kept > (1u << 20) && try_alloc(g->tile_pool, &g->al, kept, s))
         MG_CUDA(cudaMemcpyAsync(g->tile_pool.p, pool.p, kept, cudaMemcpyDeviceToDevice, s));
     else
         g->tile_pool = std::move(pool);
