@@ -468,10 +468,12 @@ __global__ void climb_small_kernel(const __grid_constant__ ClimbLevels A, const 
             if (__ldg(opac + __ldg(A.lev[j].ids + at)) != 0.0f) break;
             t = j;
             if (j == A.last) break;
-            x >>= 1;
-            y >>= 1;
-            z >>= 1;
-            at = (z * (uint32_t)A.lev[j + 1].d[1] + y) * (uint32_t)A.lev[j + 1].d[0] + x;
+            // (clamped: an imported image may claim any extents)
+            const int32_t(&d)[3] = A.lev[j + 1].d;
+            x = min(x >> 1, (uint32_t)d[0] - 1u);
+            y = min(y >> 1, (uint32_t)d[1] - 1u);
+            z = min(z >> 1, (uint32_t)d[2] - 1u);
+            at = (z * (uint32_t)d[1] + y) * (uint32_t)d[0] + x;
         }
         A.lev[l].top[i] = (uint8_t)t;
     }
@@ -487,7 +489,8 @@ __global__ void __launch_bounds__(256) climb_level_kernel(const __grid_constant_
     for (uint32_t r = t >> lg; r < rows; r += step) {
         const uint32_t z = r / dy, y = r - z * dy;
         const uint32_t* ids = V.ids + (size_t)r * dx;
-        const uint8_t* up = P.top + ((size_t)(z >> 1) * (uint32_t)P.d[1] + (y >> 1)) * (uint32_t)P.d[0];
+        const uint32_t uz = min(z >> 1, (uint32_t)P.d[2] - 1u), uy = min(y >> 1, (uint32_t)P.d[1] - 1u);
+        const uint8_t* up = P.top + ((size_t)uz * (uint32_t)P.d[1] + uy) * (uint32_t)P.d[0];
         uint8_t* top = V.top + (size_t)r * dx;
         for (uint32_t x0 = t & (w - 1); x0 < dx; x0 += N * w) {
             uint32_t id[N];
@@ -496,7 +499,7 @@ __global__ void __launch_bounds__(256) climb_level_kernel(const __grid_constant_
             for (int k = 0; k < N; k++) {
                 const uint32_t x = x0 + k * w;
                 id[k] = x < dx ? __ldg(ids + x) : 0u;   // (past the end: a node that is there)
-                u[k] = x < dx ? __ldg(up + (x >> 1)) : 0;
+                u[k] = x < dx ? __ldg(up + min(x >> 1, (uint32_t)P.d[0] - 1u)) : 0;
             }
             float o[N];
 #pragma unroll

@@ -444,12 +444,13 @@ __global__ void __launch_bounds__(kThreads) tile_merge_kernel(const __grid_const
 // covers: up to four segments inline, so that a cube costs one gather instead
 // of the row header and then its entries; longer rows {0xFFFF, first entry,
 // entries, 3 lmin} in the table; zero for nodes without a row.  Rows average
-// two entries; lmin <= 5 for an inline record, whose counts have 16 bits.
-__global__ void node_records_kernel(const uint2* __restrict__ meta, const uint2* __restrict__ lut, int64_t N,
-                                    uint4* __restrict__ rec) {
+// two entries; lmin <= 5 for an inline record, whose counts have 16 bits.  Rows
+// past the table's `entries` (a damaged image) are not read.
+__global__ void node_records_kernel(const uint2* __restrict__ meta, const uint2* __restrict__ lut, int64_t entries,
+                                    int64_t N, uint4* __restrict__ rec) {
     for (int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (int64_t)gridDim.x * blockDim.x) {
         const uint2 m = meta[n];
-        const uint32_t len = m.y >> 8, lmin = m.y & 255u;
+        const uint32_t lmin = m.y & 255u, len = m.x + (int64_t)(m.y >> 8) <= entries ? m.y >> 8 : 0u;
         uint4 r = make_uint4(0u, 0u, 0u, 0u);
         if (len > 4 || (len && lmin > 5)) {
             r = make_uint4(kTileList, m.x, len, 3 * lmin);
@@ -477,12 +478,13 @@ __global__ void node_records_kernel(const uint2* __restrict__ meta, const uint2*
 // saved.  Two-source rows, the most frequent, are whole in the record.
 template <typename AT>
 __global__ void node_shares_kernel(const uint2* __restrict__ pq, const AT* __restrict__ alpha,
-                                   const uint2* __restrict__ meta, int64_t N, uint32_t S, float* __restrict__ frac,
+                                   const uint2* __restrict__ meta, int64_t entries, int64_t N, uint32_t S,
+                                   float* __restrict__ frac,
                                    uint4* __restrict__ rec) {
     constexpr int kStack = 64;
     for (int64_t n0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; n0 < N; n0 += (int64_t)gridDim.x * blockDim.x) {
         const uint2 m = meta[n0];
-        const uint32_t len = m.y >> 8;
+        const uint32_t len = m.x + (int64_t)(m.y >> 8) <= entries ? m.y >> 8 : 0u;
         uint4 r = make_uint4(0u, 0u, 0u, 0u);
         if (len) {
             uint32_t sn[kStack];
@@ -550,7 +552,7 @@ mg_status build_tiles(mg_graph* g, cudaStream_t s) {
     if (g->id0_bytes != 2 || g->S > kMaxSharedSegments) return MG_OK;   // no box queries on such graphs
     if (g->lut_meta.p && !g->quantised && try_alloc(g->lut_rec, &g->al, (size_t)g->N * sizeof(uint4), s)) {
         node_records_kernel<<<grid_for(g->N, 256, 152 * 32), 256, 0, s>>>(g->lut_meta.as<uint2>(), g->lut.as<uint2>(),
-                                                                         g->N, g->lut_rec.as<uint4>());
+                                                                         g->lut_entries, g->N, g->lut_rec.as<uint4>());
         MG_CUDA(cudaGetLastError());
     }
     // levels >= 1 replace pushes through exact nodes with table rows
@@ -675,10 +677,10 @@ mg_status ensure_records16(mg_graph* g, mg_dtype dt, cudaStream_t s) {
     const unsigned gb = grid_for(g->N, 256, 152 * 32);
     if (k)
         node_shares_kernel<<<gb, 256, 0, s>>>(g->pq.as<uint2>(), g->alphab16.as<__nv_bfloat16>(), g->lut_meta.as<uint2>(),
-                                              g->N, g->S, frac.as<float>(), rec.as<uint4>());
+                                              g->lut_entries, g->N, g->S, frac.as<float>(), rec.as<uint4>());
     else
-        node_shares_kernel<<<gb, 256, 0, s>>>(g->pq.as<uint2>(), g->alpha16.as<__half>(), g->lut_meta.as<uint2>(), g->N,
-                                              g->S, frac.as<float>(), rec.as<uint4>());
+        node_shares_kernel<<<gb, 256, 0, s>>>(g->pq.as<uint2>(), g->alpha16.as<__half>(), g->lut_meta.as<uint2>(),
+                                              g->lut_entries, g->N, g->S, frac.as<float>(), rec.as<uint4>());
     MG_CUDA(cudaGetLastError());
     MG_CUDA(cudaStreamSynchronize(s));   // read from other streams from here on
     frac.s = rec.s = nullptr;

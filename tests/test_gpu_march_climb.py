@@ -65,3 +65,23 @@ def test_values_that_are_not_finite(mg):
     assert np.abs(img[fin] - ref[fin]).max() <= 2e-5
     mg.mg_sync_status(g)
     g.close()
+
+
+def test_extents_that_an_image_only_claims(mg):
+    """An imported image may give a level's extents in another order: climbs stay
+    inside the levels' arrays, as the samples do."""
+    dims, S = (64, 64, 8), 12
+    g = mg.mg_build(torch.from_numpy(synth.make_volume(1, dims=dims, S=S)).cuda(), S)
+    img = np.array(mg.mg_graph_export(g))
+    at = 64   # the header's extents, three int32 a level
+    ext = img[at:at + 12 * g.info["levels"]].view(np.int32).reshape(-1, 3)
+    assert ext.tolist() == [list(d) for d in g.info["dims"]] and ext[2].tolist() == [16, 16, 2]
+    ext[2] = (2, 16, 16)
+    h = mg.mg_graph_import(img)
+    vals = mg.mg_propagate_tf(h, torch.from_numpy(synth.make_tf(1, S, 4)).cuda())
+    cam = synth.orbit_camera(1, dims=dims, width=33, height=17, lod_bias=0, ert=2.0, base_step=0.5)
+    out = mg.mg_raymarch(h, vals, cam, opacity=torch.zeros(h.N, device="cuda"))
+    mg.mg_sync_status(h)
+    assert bool(torch.isfinite(out).all())
+    g.close()
+    h.close()
