@@ -179,7 +179,9 @@ typedef struct {
                            MG_SCHED_PLAIN: one launch per query, one CTA (baseline);
                            MG_SCHED_NAIVE: no footprint assembly, every level-0 voxel
                            of the box counted (brute-force baseline, same results) */
-    int chunk_cubes;    /* batched: cubes per work item (0 = tuned default) */
+    int chunk_cubes;    /* batched: footprint items per work chunk (0 = tuned or default).  An item
+                           is a cube, or a tile record of 16, 64 or 256 cubes (mg_count_cubes
+                           counts cubes) */
     int block_threads;  /* batched: threads per CTA, 128/256/512 (0 = tuned default) */
     int timing;         /* nonzero: record CUDA events around the plan, main and output
                            stages on `stream` (read them with mg_query_timing) */
@@ -255,7 +257,8 @@ MG_API mg_status mg_query_timing(const mg_graph *g, float *plan_ms, float *main_
  *   launch shape (0 = the graph's tuned shape, else the defaults) as for
  *   mg_query_boxes.
  * max_blocks, max_chunks: footprint blocks and work chunks one run may need
- *   (0 = 1024 and 256 per box).  A run whose boxes need more writes zero
+ *   (0 = 1024 and 256 per box; chunks of opts->chunk_cubes items, or of the tuned
+ *   length, else of 2048, also where the plan takes shorter ones).  A run whose boxes need more writes zero
  *   histograms and sets MG_ERR_CAPACITY in the status word (mg_sync_status).
  * opts->timing set: a run also records CUDA events around its plan stage (the
  *   fused plan kernel) and its main kernel; read the durations of the last run
@@ -279,15 +282,18 @@ MG_API mg_status mg_query_plan_timing(const mg_query_plan *p, float *plan_ms, fl
 MG_API void mg_query_plan_free(mg_query_plan *p);
 
 /* Autotuner of the batched query: times every work-chunk size in
- * {1024, 2048, 4096, 8192, 16384} cubes with CTAs of 128, 256 and 512 threads on the
+ * {1024, 2048, 4096, 8192, 16384} items with CTAs of 128, 256 and 512 threads on the
  * given batch (dense layout; opts->hist_type and alpha_dtype as the caller
  * will use them), writes the fastest into opts->chunk_cubes/block_threads and
- * keeps it in the graph for later calls and plans that leave them 0.
+ * keeps it in the graph for later calls and plans with these weights that leave
+ * them 0.  Batches and plans so small that the default chunk is below 1024 items
+ * keep the default.
  * *best_ms (may be NULL) receives the fastest time of one call.
  * Synchronises `stream`. */
 MG_API mg_status mg_query_autotune(mg_graph *g, const int32_t *boxes, int64_t Q, mg_query_opts *opts,
                                    float *best_ms, mg_stream stream);
-/* Record a tuned launch shape for a histogram type (e.g. from a cache file). */
+/* Record a tuned launch shape for a histogram type (e.g. from a cache file),
+ * used as the autotuner's, with any weights. */
 MG_API mg_status mg_query_set_tuning(mg_graph *g, int hist_type, int chunk_cubes, int block_threads);
 
 /* Number of footprint-assembly cubes (mipmap fetches) of each box, uint64[Q]

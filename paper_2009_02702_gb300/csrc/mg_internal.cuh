@@ -221,6 +221,7 @@ struct mg_graph {
     // launch shape chosen by mg_query_autotune, per histogram type (0 = none yet)
     int tuned_chunk[2] = {0, 0};
     int tuned_threads[2] = {0, 0};
+    int tuned_weights = -1;   // the weights (mg_dtype) of the fp32 histograms' shape, -1: any
     // per-stream scratch arenas of query calls
     std::mutex arena_mu;
     std::map<cudaStream_t, std::unique_ptr<mg::Arena>> arenas;
@@ -306,13 +307,14 @@ struct PlanParts {
     uint64_t cap_blocks, cap_chunks;
 };
 mg_status plan_parts(mg_query_plan* p, PlanParts* out);
-// Work-chunk length of a plan, and the entries of its chunk map.  An untuned
-// plan for few boxes takes shorter chunks than the default, and entries for
-// all that fits the caller's capacity in default chunks, or for the most that
-// max_Q boxes can have if that is less: 64 MiB at most, or the caller's own.
+// Work-chunk length of a plan, and the entries of its chunk map.  A plan for few
+// boxes takes shorter chunks than the default's 2,048 items or the tuned ones,
+// and entries for all that fits the caller's capacity in those, or for the most
+// that max_Q boxes can have if that is less: 64 MiB at most, or the caller's own.
 struct PlanChunk {
     uint32_t chunk;
     uint64_t cap_chunks;
+    int threads;   // of a CTA
 };
 PlanChunk plan_chunk(const mg_graph* g, int hist_type, mg_dtype weights, int chunk_cubes, int block_threads,
                      int64_t max_Q, uint64_t cap_chunks);

@@ -2542,6 +2542,37 @@ int default_threads(const mg_graph* g, bool FP, mg_dtype weights) {
     return 4 * warps(4, WarpKernelBounds<128>::min_ctas) >= 5 * warps(8, WarpKernelBounds<256>::min_ctas) ? 128 : 256;
 }
 
+// The launch shape of a batch: what the caller names, else what
+// mg_query_autotune or mg_query_set_tuning recorded, else the defaults.  The
+// tuner's shape holds for the weights it was tuned with (16-bit weights want
+// other CTAs and longer chunks than fp32 ones).  It tries 1,024 items and more:
+// where the default is well below that, a batch has too few such chunks, and
+// CTAs of 512 threads only make up for that, whatever batch they were tuned on
+// (1,000 boxes of 64^3: 25 us a run with 128 items, 41 tuned; of 512x512x384 40
+// and 65; with a histogram per CTA 100 boxes 53 with 512 items, 51 tuned).
+struct Shape {
+    int threads;
+    uint32_t chunk;
+    uint32_t longest;   // the chunks that capacities are counted in
+};
+Shape launch_shape_of(const mg_graph* g, bool FP, mg_dtype weights, int chunk_cubes, int block_threads, int64_t Q) {
+    if (!FP) weights = MG_F32;
+    const bool told = !FP || g->tuned_weights < 0 || g->tuned_weights == (int)weights;
+    uint32_t tuned = told ? (uint32_t)g->tuned_chunk[FP] : 0u;
+    int threads = told ? g->tuned_threads[FP] : 0;
+    const int usual = default_threads(g, FP, weights);
+    Shape R;
+    R.longest = chunk_cubes > 0 ? (uint32_t)chunk_cubes : tuned ? tuned : kDefaultChunk;
+    const uint32_t c = default_chunk(g, FP, weights, block_threads > 0 ? block_threads : usual, Q);
+    if (chunk_cubes <= 0 && tuned > c && c < (warp_hists(g, FP, usual) ? 1024u : 512u)) {
+        tuned = 0;
+        threads = 0;
+    }
+    R.threads = block_threads > 0 ? block_threads : threads > 0 ? threads : usual;
+    R.chunk = chunk_cubes > 0 ? R.longest : tuned ? tuned : default_chunk(g, FP, weights, R.threads, Q);
+    return R;
+}
+
 // Scratch comes from `al`; `words` are two host words for readbacks; `room`,
 // when not null, returns the bytes `al` can still hand out (fixed pools).
 mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, const mg_query_opts& o, void* out,
@@ -2560,17 +2591,15 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
         MG_TRY(ensure_alpha16(const_cast<mg_graph*>(g), (mg_dtype)o.alpha_dtype, s));
         MG_TRY(ensure_records16(const_cast<mg_graph*>(g), (mg_dtype)o.alpha_dtype, s));
     }
-    const int tuned_c = g->tuned_chunk[FP ? 1 : 0], tuned_t = g->tuned_threads[FP ? 1 : 0];
-    const int threads = o.block_threads > 0                ? o.block_threads
-                        : tuned_t > 0                      ? tuned_t
-                        : o.schedule == MG_SCHED_BATCHED   ? default_threads(g, FP, (mg_dtype)o.alpha_dtype)
-                                                           : 256;
-    uint32_t chunk = o.chunk_cubes > 0 ? (uint32_t)o.chunk_cubes
-                     : tuned_c > 0     ? (uint32_t)tuned_c
-                                       : default_chunk(g, FP, (mg_dtype)o.alpha_dtype, threads, Q);
+    const Shape shape = launch_shape_of(g, FP, (mg_dtype)o.alpha_dtype, o.chunk_cubes, o.block_threads, Q);
+    const int threads = o.schedule == MG_SCHED_BATCHED || o.block_threads > 0 ? shape.threads
+                        : g->tuned_threads[FP] > 0                            ? g->tuned_threads[FP]
+                                                                              : 256;
+    const uint32_t longest = shape.longest;
+    uint32_t chunk = shape.chunk;
     // the room of a fixed pool is counted in long chunks: shorter ones are taken
     // where the batch fits with them too, and there is one scan to repeat
-    if (room && Q > kFusedScanMax) chunk = std::max(chunk, kDefaultChunk);
+    if (room && Q > kFusedScanMax) chunk = longest;
     // Where the most that this many boxes can have fits a modest buffer, the
     // footprint is planned in one launch and nothing is read back: 1,000 boxes
     // of a 64^3 volume took 69 us with three plan kernels and the read-back of
@@ -2580,9 +2609,7 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
     constexpr uint64_t kMostUnread = 1u << 22;
     const uint64_t most_blocks = block_bound(g, Q);
     bool fused = o.schedule == MG_SCHED_BATCHED && !room && most_blocks < kMostUnread;
-    while (fused && o.chunk_cubes <= 0 && tuned_c <= 0 && chunk < kDefaultChunk &&
-           chunk_bound(g, Q, chunk) >= kMostUnread)
-        chunk *= 2;
+    while (fused && chunk < longest && chunk_bound(g, Q, chunk) >= kMostUnread) chunk = std::min(2 * chunk, longest);
     const uint64_t most_chunks = chunk_bound(g, Q, chunk);
     fused = fused && most_chunks < kMostUnread;
     const Geom G = make_geom(g, tile_levels(g, (mg_dtype)o.alpha_dtype));
@@ -2719,8 +2746,8 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
             if (room) {
                 const size_t need = (((size_t)std::max<uint64_t>(totals[0], 1) * sizeof(Blk) + 255) & ~(size_t)255) +
                                     2 * (((size_t)std::max<uint64_t>(totals[1], 1) * 4 + 255) & ~(size_t)255);
-                if (need > room(al) && chunk < kDefaultChunk && o.chunk_cubes <= 0 && tuned_c <= 0) {
-                    chunk = kDefaultChunk;
+                if (need > room(al) && chunk < longest) {
+                    chunk = longest;
                     continue;
                 }
                 if (need > room(al))
@@ -2943,6 +2970,7 @@ struct mg_query_plan {
     int64_t max_Q = 0;
     bool fp = false;
     mg_dtype weights = MG_F32;
+    int threads = 0;
     mg::QueryBufs bufs{};
     mg::Buf pool;
     mg::Pool bump{nullptr, 0, 0};
@@ -2965,26 +2993,14 @@ struct mg_query_plan {
 };
 
 namespace mg {
-namespace {
-// threads of a plan's CTAs: the caller's, else the tuned ones, else the default
-int plan_threads(const mg_graph* g, bool FP, mg_dtype weights, int block_threads) {
-    const int tuned = g->tuned_threads[FP];
-    return block_threads > 0 ? block_threads : tuned > 0 ? tuned : default_threads(g, FP, weights);
-}
-}  // namespace
-
 PlanChunk plan_chunk(const mg_graph* g, int hist_type, mg_dtype weights, int chunk_cubes, int block_threads,
                      int64_t max_Q, uint64_t cap_chunks) {
-    const bool FP = hist_type == MG_HIST_F32;
-    const int tuned = g->tuned_chunk[FP];
-    if (chunk_cubes > 0) return PlanChunk{(uint32_t)chunk_cubes, cap_chunks};
-    if (tuned > 0) return PlanChunk{(uint32_t)tuned, cap_chunks};
-    const int threads = plan_threads(g, FP, weights, block_threads);
-    for (uint32_t c = default_chunk(g, FP, FP ? weights : MG_F32, threads, max_Q); c < kDefaultChunk; c *= 2) {
-        const uint64_t n = std::min(cap_chunks * (kDefaultChunk / c), chunk_bound(g, max_Q, c));
-        if (n <= std::max<uint64_t>(cap_chunks, 1u << 23)) return PlanChunk{c, n};
+    const Shape R = launch_shape_of(g, hist_type == MG_HIST_F32, weights, chunk_cubes, block_threads, max_Q);
+    for (uint32_t c = R.chunk; c < R.longest; c *= 2) {
+        const uint64_t n = std::min(cap_chunks * ((R.longest + c - 1) / c), chunk_bound(g, max_Q, c));
+        if (n <= std::max<uint64_t>(cap_chunks, 1u << 23)) return PlanChunk{c, n, R.threads};
     }
-    return PlanChunk{kDefaultChunk, cap_chunks};
+    return PlanChunk{R.longest, cap_chunks, R.threads};
 }
 
 mg_status plan_parts(mg_query_plan* p, PlanParts* out) {
@@ -3049,6 +3065,7 @@ MG_API mg_status mg_query_plan_create(mg_graph* g, int64_t max_Q, const mg_query
         const PlanChunk pc = plan_chunk(g, o.hist_type, p->weights, o.chunk_cubes, o.block_threads, max_Q, B.cap_chunks);
         B.chunk = pc.chunk;
         B.cap_chunks = pc.cap_chunks;
+        p->threads = pc.threads;
         if (B.cap_blocks >= (1ull << 32) || B.cap_chunks >= (1ull << 32))
             st = fail(MG_ERR_UNSUPPORTED, "plan capacities must be below 2^32");
     }
@@ -3086,7 +3103,7 @@ MG_API mg_status mg_query_plan_create(mg_graph* g, int64_t max_Q, const mg_query
         }
     }
     if (st == MG_OK)
-        st = shape_of(g, p->fp, p->weights, plan_threads(g, p->fp, p->weights, o.block_threads), &p->bufs.shape);
+        st = shape_of(g, p->fp, p->weights, p->threads, &p->bufs.shape);
     if (st == MG_OK && o.timing) {
         p->timed = true;
         for (cudaEvent_t& ev : p->ev) {
@@ -3217,6 +3234,7 @@ extern "C" MG_API mg_status mg_query_autotune(mg_graph* g, const int32_t* boxes,
     if (st == MG_OK) {
         g->tuned_chunk[FP ? 1 : 0] = best_c;
         g->tuned_threads[FP ? 1 : 0] = best_t;
+        if (FP) g->tuned_weights = opts->alpha_dtype;
         opts->chunk_cubes = best_c;
         opts->block_threads = best_t;
         if (best_ms) *best_ms = best / 2.f;
@@ -3234,5 +3252,6 @@ extern "C" MG_API mg_status mg_query_set_tuning(mg_graph* g, int hist_type, int 
         return fail(MG_ERR_INVALID_ARG, "bad launch shape");
     g->tuned_chunk[hist_type] = chunk_cubes;
     g->tuned_threads[hist_type] = block_threads;
+    if (hist_type == MG_HIST_F32) g->tuned_weights = -1;
     return MG_OK;
 }

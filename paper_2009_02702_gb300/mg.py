@@ -585,7 +585,9 @@ def mg_query_autotune(g: Graph, boxes: torch.Tensor, hist: str = "u32", alpha: s
     the same GPU name and key is reused without timing."""
     import json
     dev = torch.cuda.get_device_name(g.device)
-    full_key = "%s|%s|%s" % (dev, key, hist) if key else None
+    # (chunks are counted in footprint items: shapes kept from when they were
+    # counted in cubes are not these)
+    full_key = "%s|%s|%s|%s|items" % (dev, key, hist, alpha) if key else None
     ht = MG_HIST_F32 if hist == "f32" else MG_HIST_U32
     if cache and full_key and os.path.exists(cache):
         try:

@@ -235,3 +235,49 @@ def test_fixed_scratch_filled_to_its_limit(mg):
     assert (lo + 1) * (12 * blocks + 8 * (cubes // 2048 + 1)) > (60 << 20)
     mg.mg_sync_status(g)
     g.close()
+
+
+@pytest.mark.parametrize("chunk,threads", [(16384, 256), (3000, 128), (100, 256), (1024, 512), (0, 0)])
+def test_recorded_shapes_and_small_batches(mg, chunk, threads):
+    """A recorded length is for batches that fill it; what fits a plan's capacity in
+    recorded chunks fits it in shorter ones (noise: items are cubes)."""
+    dims, S = (64, 64, 64), 700
+    vol = noise(dims, S, 3)
+    g = mg.mg_build(torch.from_numpy(vol).cuda(), S)
+    one = np.array([[1, 1, 1, 62, 62, 62]], np.int32)
+    cubes = int(mg.mg_count_cubes(g, torch.from_numpy(one).cuda()).cpu().numpy()[0])
+    for hist in (0, 1):
+        assert mg.lib().mg_query_set_tuning(g.handle, hist, chunk, threads) == mg.MG_OK
+    fits = -(-cubes // (chunk or 2048))
+    for hist, alpha in (("u32", "f32"), ("f32", "f32"), ("f32", "bf16")):
+        for bx in (one, some_boxes(dims, 50, 1), some_boxes(dims, 3000, 2)):
+            t = torch.from_numpy(bx).cuda()
+            ref = oracle.box_hist(vol, S, bx).astype(np.float64)
+            plan = mg.QueryPlan(g, max_Q=len(bx), hist=hist, alpha=alpha, max_blocks=4096 * len(bx),
+                                max_chunks=fits * len(bx))
+            for h in (mg.mg_query_boxes(g, t, hist=hist, alpha=alpha), plan.run(t)):
+                h = h.cpu().numpy().astype(np.float64)
+                if alpha == "f32":
+                    assert np.array_equal(h, ref)
+                else:
+                    assert (np.abs(h - ref).sum(1) <= 1.5 * g.info["depth"] * 2.0 ** -8 * ref.sum(1)).all()
+            plan.close()
+    mg.mg_sync_status(g)
+    g.close()
+
+
+def test_a_shape_tuned_for_some_weights(mg):
+    dims, S = (64, 64, 64), 700
+    vol = noise(dims, S, 4)
+    g = mg.mg_build(torch.from_numpy(vol).cuda(), S)
+    bx = some_boxes(dims, 4000, 4)
+    t = torch.from_numpy(bx).cuda()
+    ref = oracle.box_hist(vol, S, bx).astype(np.float64)
+    for alpha in ("f16", "f32"):
+        r = mg.mg_query_autotune(g, t, hist="f32", alpha=alpha)
+        assert r["chunk_cubes"] in (1024, 2048, 4096, 8192, 16384) and r["block_threads"] in (128, 256, 512)
+        for other, u in (("f32", 0.0), ("f16", 2.0 ** -11), ("bf16", 2.0 ** -8)):
+            h = mg.mg_query_boxes(g, t, hist="f32", alpha=other).cpu().numpy().astype(np.float64)
+            assert (np.abs(h - ref).sum(1) <= 1.5 * g.info["depth"] * u * ref.sum(1)).all()
+    mg.mg_sync_status(g)
+    g.close()
