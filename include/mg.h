@@ -394,7 +394,9 @@ MG_API mg_status mg_raymarch(const mg_graph *g, const float *vals, const float *
  * buffers (device and pinned host) sized by the options.  A volume whose
  * graph plus these buffers would take the server past memory_budget is not
  * admitted (MG_ERR_CAPACITY), so resident volumes never compete for memory
- * at run time.
+ * at run time.  Where the budget is short, a graph that no query has read yet
+ * gives back the tile and node records that only speed queries up, and the
+ * plans take smaller chunk maps, before a volume is refused.
  */
 typedef struct mg_server mg_server;   /* opaque */
 

@@ -6,6 +6,7 @@
 #include <cuda_bf16.h>
 #include <cstdint>
 #include <cstddef>
+#include <atomic>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -189,6 +190,15 @@ struct mg_graph {
     mg::Buf tiles;      // uint4 records
     mg::Buf tile_pool;  // uint4 blocks of the lists
     mg::TileGeom tgeom{};
+    // Tiles and records may be given back until a query or a plan first reads
+    // them: after that, launches and captured graphs hold their addresses.
+    std::mutex tiles_mu;
+    std::atomic<bool> tiles_held{false};
+    void hold_tiles() {
+        if (tiles_held.load(std::memory_order_acquire)) return;
+        std::lock_guard<std::mutex> lk(tiles_mu);
+        tiles_held.store(true, std::memory_order_release);
+    }
     // node table, canonical order, N entries
     mg::Buf pq;       // uint2 (p, q); (kNone, kNone) for sources
     mg::Buf ab;       // ulonglong2 (a, b) exact coprime weights
@@ -266,6 +276,10 @@ mg_status build_query_copies(mg_graph* g, cudaStream_t s);
 mg_status build_tiles(mg_graph* g, cudaStream_t s);
 // box histograms summed from the mixture table, with error bars (Sec. 3.5-3.6)
 mg_status query_lut(const mg_graph* g, const int32_t* boxes, int64_t Q, double* hist, double* err, cudaStream_t s);
+// bytes that a graph no query has read could give back, and giving them back
+// (false: they are held)
+int64_t spare_tile_bytes(mg_graph* g);
+bool drop_tiles(mg_graph* g);
 mg_status ensure_alpha16(mg_graph* g, mg_dtype dt, cudaStream_t s);
 // the nodes' shares and records for 16-bit weights (after ensure_alpha16); the
 // queries walk the lerp trees where there is no memory for them
@@ -307,6 +321,8 @@ struct PlanParts {
     uint64_t cap_blocks, cap_chunks;
 };
 mg_status plan_parts(mg_query_plan* p, PlanParts* out);
+// The longest chunk that an untold plan takes: its map is the smallest.
+uint32_t longest_chunk(const mg_graph* g, int hist_type);
 // Work-chunk length of a plan, and the entries of its chunk map.  A plan for few
 // boxes takes shorter chunks than the default's 2,048 items or the tuned ones,
 // and entries for all that fits the caller's capacity in those, or for the most

@@ -2582,6 +2582,7 @@ mg_status query_boxes_impl(const mg_graph* g, const int32_t* boxes, int64_t Q, c
     const bool FP = o.hist_type == MG_HIST_F32;
     const bool csr = o.layout == MG_LAYOUT_CSR;
     if (S > kMaxSharedSegments) return fail(MG_ERR_UNSUPPORTED, "more than 32768 segments");
+    const_cast<mg_graph*>(g)->hold_tiles();
     if (required) *required = 0;
     if (Q == 0) {
         if (csr) MG_CUDA(cudaMemsetAsync(offsets, 0, sizeof(uint64_t), s));
@@ -2993,6 +2994,11 @@ struct mg_query_plan {
 };
 
 namespace mg {
+uint32_t longest_chunk(const mg_graph* g, int hist_type) {
+    const int tuned = g->tuned_chunk[hist_type == MG_HIST_F32];
+    return tuned > 0 ? (uint32_t)tuned : kDefaultChunk;
+}
+
 PlanChunk plan_chunk(const mg_graph* g, int hist_type, mg_dtype weights, int chunk_cubes, int block_threads,
                      int64_t max_Q, uint64_t cap_chunks) {
     const Shape R = launch_shape_of(g, hist_type == MG_HIST_F32, weights, chunk_cubes, block_threads, max_Q);
@@ -3049,6 +3055,7 @@ MG_API mg_status mg_query_plan_create(mg_graph* g, int64_t max_Q, const mg_query
     if (prev != g->device) MG_CUDA(cudaSetDevice(g->device));
     std::unique_ptr<mg_query_plan> p(new (std::nothrow) mg_query_plan());
     mg_status st = p ? MG_OK : fail(MG_ERR_OOM, "host allocation failed");
+    g->hold_tiles();
     if (st == MG_OK && o.hist_type == MG_HIST_F32 && o.alpha_dtype != MG_F32) {   // (the launch shape depends on them)
         st = ensure_alpha16(g, (mg_dtype)o.alpha_dtype, nullptr);
         if (st == MG_OK) st = ensure_records16(g, (mg_dtype)o.alpha_dtype, nullptr);

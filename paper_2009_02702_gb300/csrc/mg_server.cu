@@ -528,13 +528,28 @@ MG_API mg_status mg_server_add_volume(mg_server* sv, mg_graph* g, int C, int* vo
                             round_up((size_t)F * ms * 16) + round_up((size_t)F * ms * C * sv->esize);
     const size_t query_bytes =
         sv->o.plain ? round_up(Q * 24) + round_up(Q * S * 4) + 2 * Q * S * 4
-                    : Q * 24 + Q * S * 4 * (sv->o.hist_type == MG_HIST_F32 ? 2 : 1) + Q * 64 + cap_blocks * 12 +
-                          8 * plan_chunk(g, sv->o.hist_type, MG_F32, 0, 0, (int64_t)Q, cap_chunks).cap_chunks;
-    const int64_t need = (int64_t)((tf_bytes + query_bytes) * sv->slots.size()) + g->device_bytes();
-    if (sv->o.memory_budget > 0 && sv->budget_used + need > sv->o.memory_budget)
+                    : Q * 24 + Q * S * 4 * (sv->o.hist_type == MG_HIST_F32 ? 2 : 1) + Q * 64 + cap_blocks * 12;
+    // where the budget is short, the plans take long chunks, whose map is the
+    // caller's capacity, and a graph that no query has read gives back its tiles:
+    // slower queries for a volume that would not be there at all
+    mg_query_opts qo{};
+    qo.hist_type = sv->o.hist_type;
+    auto bytes_needed = [&](int chunk) {
+        const size_t map =
+            sv->o.plain ? 0 : 8 * plan_chunk(g, qo.hist_type, MG_F32, chunk, 0, (int64_t)Q, cap_chunks).cap_chunks;
+        return (int64_t)((tf_bytes + query_bytes + map) * sv->slots.size()) + g->device_bytes();
+    };
+    int64_t need = bytes_needed(0);
+    const int64_t room = sv->o.memory_budget > 0 ? sv->o.memory_budget - sv->budget_used : INT64_MAX;
+    const int longest = (int)longest_chunk(g, qo.hist_type);
+    if (need > room && bytes_needed(longest) < need) {
+        qo.chunk_cubes = longest;
+        need = bytes_needed(longest);
+    }
+    if (need > room && need - spare_tile_bytes(g) <= room && drop_tiles(g)) need = bytes_needed(qo.chunk_cubes);
+    if (need > room)
         return fail(MG_ERR_CAPACITY, "volume not admitted: it needs " + std::to_string(need >> 20) + " MiB and " +
-                                         std::to_string((sv->o.memory_budget - sv->budget_used) >> 20) +
-                                         " MiB of the budget remain");
+                                         std::to_string(room >> 20) + " MiB of the budget remain");
     if (sv->o.storage != MG_F32) MG_TRY(ensure_alpha16(g, (mg_dtype)sv->o.storage, nullptr));
     const size_t pin_bytes = pinned_bytes(Q, S, C, F, ms, sv->esize);
     std::vector<VolSlot> made(sv->slots.size());
@@ -545,8 +560,6 @@ MG_API mg_status mg_server_add_volume(mg_server* sv, mg_graph* g, int C, int* vo
             st = vs.boxes_dev.alloc(&g->al, Q * 24, nullptr);
             if (st == MG_OK) st = vs.out_dev.alloc(&g->al, Q * S * 4, nullptr);
         } else {
-            mg_query_opts qo{};
-            qo.hist_type = sv->o.hist_type;
             st = mg_query_plan_create(g, (int64_t)Q, &qo, (int64_t)cap_blocks, (int64_t)cap_chunks, &vs.plan);
             if (st == MG_OK) st = plan_parts(vs.plan, &vs.pp);
         }

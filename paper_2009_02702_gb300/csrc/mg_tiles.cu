@@ -665,6 +665,21 @@ mg_status build_tiles(mg_graph* g, cudaStream_t s) {
     return MG_OK;
 }
 
+int64_t spare_tile_bytes(mg_graph* g) {
+    std::lock_guard<std::mutex> lk(g->tiles_mu);
+    return g->tiles_held ? 0 : (int64_t)(g->tiles.bytes + g->tile_pool.bytes + g->lut_rec.bytes);
+}
+
+bool drop_tiles(mg_graph* g) {
+    std::lock_guard<std::mutex> lk(g->tiles_mu);
+    if (g->tiles_held) return false;
+    g->tgeom = TileGeom{};
+    g->tiles.release();
+    g->tile_pool.release();
+    g->lut_rec.release();
+    return true;
+}
+
 mg_status ensure_records16(mg_graph* g, mg_dtype dt, cudaStream_t s) {
     if (!g->lut_meta.p || g->quantised || g->S > kMaxSharedSegments) return MG_OK;
     const int k = dt == MG_BF16;
