@@ -12,6 +12,8 @@ have finished.  Per-kernel rooflines use each kernel timed alone.
 The graph build (A1-A3, the paper's offline encoder) runs once per volume
 before the timed region and is reported as build_ms.
 
+One line of JSON is printed, the headline; all other measurements go to the file
+of --detail.
 value = box-histogram queries per second over whole steps (all ranks).
 e2e   = the same through the public API with host buffers: boxes, TF and
         samples copied host->device and histograms and looked-up colours
@@ -67,6 +69,8 @@ def parse(argv=None):
     ap.add_argument("--no-large", action="store_true", help="skip the cylinder graph measurements")
     ap.add_argument("--no-ext", action="store_true",
                     help="skip ray marching, bitstream, greedy factorisation and error-table measurements")
+    ap.add_argument("--detail", default="bench_detail.json",
+                    help="file for everything measured, of which the printed line holds the headline ('': none)")
     ap.add_argument("--serve-requests", type=int, default=0)
     ap.add_argument("--serve-rate", type=float, default=0.0)
     return ap.parse_args(argv)
@@ -693,11 +697,39 @@ def run_ours(args):
     if cpu is not None:
         line["cpu_baseline"] = cpu
     if rank == 0:
-        print(json.dumps(line))
+        print(json.dumps(short_line(line, args.detail)))
     for c, gg in graphs.items():
         gg.close()
     if world > 1:
         dist.destroy_process_group()
+
+
+# --------------------------------------------------------------------------
+# the printed line
+# --------------------------------------------------------------------------
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "gpu_launches", "config", "e2e", "clocks", "roofline", "cpu_baseline",
+             "tf_propagations_per_s", "samples_per_s", "latency_ms")
+LINE_MOST = 6000    # characters; readers of a log's last lines see the whole of it
+
+
+def short_line(line, detail=None):
+    """The line that is printed: the headline's keys.  All that was measured goes
+    to the file `detail`, which the line names; below the headline's keys, what
+    makes the line too long is left to the file."""
+    short = {k: line[k] for k in LINE_KEYS if k in line}
+    if detail:
+        try:
+            with open(detail, "w") as f:
+                json.dump(line, f, indent=1)
+            short["detail"] = detail
+        except OSError as e:
+            print("bench: no detail file: %s" % e, file=sys.stderr)
+    for k in ("latency_ms", "samples_per_s", "tf_propagations_per_s", "roofline", "cpu_baseline"):
+        if len(json.dumps(short)) <= LINE_MOST:
+            break
+        short.pop(k, None)
+    return short
 
 
 # --------------------------------------------------------------------------
