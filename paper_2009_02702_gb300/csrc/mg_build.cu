@@ -245,7 +245,7 @@ __global__ void next_write_kernel(const uint32_t* __restrict__ off, const uint32
 // lists of one parent in a table of all segments in shared memory and reads it
 // out in order (a thread merging eight lists of hundreds of entries takes
 // about 150 ns an entry: the last five levels of 512x512x384 cost 440 us,
-// this 90).  Taken for at most kDenseParents parents and segment counts whose
+// this 78).  Taken for at most kDenseParents parents and segment counts whose
 // table fits.
 constexpr int kDenseThreads = 256;
 constexpr int64_t kDenseParents = 2048;

@@ -2116,9 +2116,9 @@ bool warp_hists(const mg_graph* g, bool FP, int threads) {
 //     42 / [40] / 46 / 65 / 86; 10,000 boxes 212 / 150 / [127] / 127 / 134
 //   2048x2048x300, 1,182 segments: 1,000 boxes 57 / [49] / 52 / 58 / 85; 10,000
 //     boxes 377 / 255 / 197 / [181] / 190; 100,000 boxes - / - / - / 1472 / [1328]
-//   614x961x600, 15,917 segments, a histogram per CTA: 10 boxes 33 / [32] / 35 /
-//     44 / 52; 100 boxes 84 / 66 / [60] / 58 / 74; 1,000 boxes - / - / 446 /
-//     409 / [398]
+//   614x961x600, 15,917 segments, a histogram per CTA: 10 boxes 33 / [33] / 35 /
+//     41 / 53; 100 boxes 76 / 59 / [52] / 50 / 63; 1,000 boxes - / - / 311 /
+//     250 / [229]
 // fp32 histograms flush two bins a segment: a third longer (2048x2048x300,
 // 10,000 boxes: - / - / 335 / 289 / [283]).  With 16-bit weights a chunk's items
 // touch more bins too: longer in proportion above 750 segments, and at least one
@@ -2352,9 +2352,14 @@ __global__ void __launch_bounds__(256) query_lut_kernel(Geom G, Ids I, const int
             const Blk B = make_blk(G, 0, R.sx[i], R.sy[j], R.sz[k], R.lx[i], R.ly[j], R.lz[k], 0);
             const uint32_t n = block_cubes(R.lx[i], R.ly[j], R.lz[k]);
             const uint32_t per = (n + 31) / 32, o0 = min(n, lane * per), o1 = min(n, o0 + per);
+            const int lv = B.meta & 63, cp = (B.meta >> 6) & 3;
+            const uint32_t bits = (B.meta >> 8) & 1023u, st1 = G.st1[lv][cp], st2 = G.st2[lv][cp];
+            const uint16_t* ids16 = static_cast<const uint16_t*>(I.l0[cp]) + B.base;
+            const uint32_t* ids32 = (lv ? I.hi[cp] + G.off[lv][cp] : static_cast<const uint32_t*>(I.l0[cp])) + B.base;
+            const bool half = lv == 0 && G.id0_bytes == 2;
             for (uint32_t o = o0; o < o1; o++) {
-                int lv = 0;
-                const uint32_t node = cube_node(G, I, B, o, lv);
+                const uint32_t at = item_at(o, bits, st1, st2);
+                const uint32_t node = half ? (uint32_t)__ldg(ids16 + at) : __ldg(ids32 + at);
                 if (node == rn && lv == rl) {
                     rc++;
                 } else {
