@@ -311,12 +311,14 @@ mg_status raymarch(const mg_graph* g, const float* vals, const float* opacity, c
 
 // A query plan's own buffers, executable graph and footprint capacities, for
 // the request loop, which stages boxes straight into them: a run is the boxes
-// in `boxes`, Q in `Qd`, a launch of `exec`, and Q x S values in `result`.
+// in `boxes`, Q in `Qd`, a launch of `exec` (of `exec_few` for at most kFewBoxes,
+// whose chunks suit them), and Q x S values in `result`.
+constexpr int kFewBoxes = 64;
 struct PlanParts {
     int32_t* boxes;
     int64_t* Qd;
     void* result;
-    cudaGraphExec_t exec;
+    cudaGraphExec_t exec, exec_few;
     uint32_t chunk;
     uint64_t cap_blocks, cap_chunks;
 };
@@ -330,7 +332,8 @@ uint32_t longest_chunk(const mg_graph* g, int hist_type);
 struct PlanChunk {
     uint32_t chunk;
     uint64_t cap_chunks;
-    int threads;   // of a CTA
+    int threads;     // of a CTA
+    bool recorded;   // the chunk is a recorded one
 };
 PlanChunk plan_chunk(const mg_graph* g, int hist_type, mg_dtype weights, int chunk_cubes, int block_threads,
                      int64_t max_Q, uint64_t cap_chunks);

@@ -2559,7 +2559,10 @@ struct Shape {
     int threads;
     uint32_t chunk;
     uint32_t longest;   // the chunks that capacities are counted in
+    bool recorded;      // the chunk is a recorded one
 };
+// default chunks below this are better than any recorded one
+uint32_t recorded_least(const mg_graph* g, bool FP, int threads) { return warp_hists(g, FP, threads) ? 1024u : 512u; }
 Shape launch_shape_of(const mg_graph* g, bool FP, mg_dtype weights, int chunk_cubes, int block_threads, int64_t Q) {
     if (!FP) weights = MG_F32;
     const bool told = !FP || g->tuned_weights < 0 || g->tuned_weights == (int)weights;
@@ -2569,11 +2572,12 @@ Shape launch_shape_of(const mg_graph* g, bool FP, mg_dtype weights, int chunk_cu
     Shape R;
     R.longest = chunk_cubes > 0 ? (uint32_t)chunk_cubes : tuned ? tuned : kDefaultChunk;
     const uint32_t c = default_chunk(g, FP, weights, block_threads > 0 ? block_threads : usual, Q);
-    if (chunk_cubes <= 0 && tuned > c && c < (warp_hists(g, FP, usual) ? 1024u : 512u)) {
+    if (chunk_cubes <= 0 && tuned > c && c < recorded_least(g, FP, usual)) {
         tuned = 0;
         threads = 0;
     }
     R.threads = block_threads > 0 ? block_threads : threads > 0 ? threads : usual;
+    R.recorded = chunk_cubes <= 0 && tuned != 0;
     R.chunk = chunk_cubes > 0 ? R.longest : tuned ? tuned : default_chunk(g, FP, weights, R.threads, Q);
     return R;
 }
@@ -2977,6 +2981,7 @@ struct mg_query_plan {
     bool fp = false;
     mg_dtype weights = MG_F32;
     int threads = 0;
+    bool told = false, recorded = false;   // the chunk is the caller's, a recorded one
     mg::QueryBufs bufs{};
     mg::Buf pool;
     mg::Pool bump{nullptr, 0, 0};
@@ -2985,15 +2990,17 @@ struct mg_query_plan {
     void* result = nullptr;   // max_Q x S, uint32 or fp32
     void** io = nullptr;      // device slots: the run's boxes and output (default: boxes, result)
     cudaStream_t cap_stream = nullptr;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
+    cudaGraph_t graph[2] = {nullptr, nullptr};         // any batch; a few boxes
+    cudaGraphExec_t exec[2] = {nullptr, nullptr};
     bool timed = false, ran = false;
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};   // graph start, plan done, main done
     ~mg_query_plan() {
         for (cudaEvent_t e : ev)
             if (e) cudaEventDestroy(e);
-        if (exec) cudaGraphExecDestroy(exec);
-        if (graph) cudaGraphDestroy(graph);
+        for (cudaGraphExec_t e : exec)
+            if (e) cudaGraphExecDestroy(e);
+        for (cudaGraph_t e : graph)
+            if (e) cudaGraphDestroy(e);
         if (cap_stream) cudaStreamDestroy(cap_stream);
     }
 };
@@ -3009,23 +3016,42 @@ PlanChunk plan_chunk(const mg_graph* g, int hist_type, mg_dtype weights, int chu
     const Shape R = launch_shape_of(g, hist_type == MG_HIST_F32, weights, chunk_cubes, block_threads, max_Q);
     for (uint32_t c = R.chunk; c < R.longest; c *= 2) {
         const uint64_t n = std::min(cap_chunks * ((R.longest + c - 1) / c), chunk_bound(g, max_Q, c));
-        if (n <= std::max<uint64_t>(cap_chunks, 1u << 23)) return PlanChunk{c, n, R.threads};
+        if (n <= std::max<uint64_t>(cap_chunks, 1u << 23)) return PlanChunk{c, n, R.threads, R.recorded};
     }
-    return PlanChunk{R.longest, cap_chunks, R.threads};
+    return PlanChunk{R.longest, cap_chunks, R.threads, R.recorded};
+}
+
+// Chunk length of a run of Q boxes: the plan's, or a shorter one that suits so
+// few boxes where the plan's chunk map holds the most that they can have (one
+// box with 15,917 segments and fp32 histograms by a plan for 10,000: 55 -> 33 us).
+static uint32_t run_chunk(const mg_query_plan* p, int64_t Q) {
+    const QueryBufs& B = p->bufs;
+    if (p->told || Q == p->max_Q) return B.chunk;
+    const int threads = B.shape.threads;
+    uint32_t c = default_chunk(p->g, p->fp, p->fp ? p->weights : MG_F32, threads, Q);
+    if (p->recorded && c >= recorded_least(p->g, p->fp, threads)) return B.chunk;
+    while (c < B.chunk && chunk_bound(p->g, Q, c) > B.cap_chunks) c *= 2;
+    return std::min(c, B.chunk);
 }
 
 mg_status plan_parts(mg_query_plan* p, PlanParts* out) {
-    if (!p->exec) {
+    if (!p->exec[0]) {
         MG_CUDA(cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
-        MG_CUDA(cudaStreamBeginCapture(p->cap_stream, cudaStreamCaptureModeThreadLocal));
-        const BatchRun run{p->boxes, p->max_Q, p->Qd, p->io, p->result};
-        const mg_status st = enqueue_any(p->g, p->bufs, run, p->fp, p->weights, false, nullptr, p->cap_stream);
-        const cudaError_t e = cudaStreamEndCapture(p->cap_stream, &p->graph);
-        if (st != MG_OK) return st;
-        if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
-        MG_CUDA(cudaGraphInstantiate(&p->exec, p->graph, 0));
+        for (int k = 0; k < 2; k++) {
+            const int64_t Q = k == 0 ? p->max_Q : std::min<int64_t>(p->max_Q, kFewBoxes);
+            QueryBufs B = p->bufs;
+            if (k == 1) B.chunk = run_chunk(p, Q);
+            MG_CUDA(cudaStreamBeginCapture(p->cap_stream, cudaStreamCaptureModeThreadLocal));
+            const BatchRun run{p->boxes, Q, p->Qd, p->io, p->result};
+            const mg_status st = enqueue_any(p->g, B, run, p->fp, p->weights, false, nullptr, p->cap_stream);
+            const cudaError_t e = cudaStreamEndCapture(p->cap_stream, &p->graph[k]);
+            if (st != MG_OK) return st;
+            if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
+            MG_CUDA(cudaGraphInstantiate(&p->exec[k], p->graph[k], 0));
+        }
     }
-    *out = PlanParts{p->boxes, p->Qd, p->result, p->exec, p->bufs.chunk, p->bufs.cap_blocks, p->bufs.cap_chunks};
+    *out = PlanParts{p->boxes, p->Qd, p->result, p->exec[0], p->exec[1],
+                     p->bufs.chunk, p->bufs.cap_blocks, p->bufs.cap_chunks};
     return MG_OK;
 }
 }  // namespace mg
@@ -3078,6 +3104,8 @@ MG_API mg_status mg_query_plan_create(mg_graph* g, int64_t max_Q, const mg_query
         B.chunk = pc.chunk;
         B.cap_chunks = pc.cap_chunks;
         p->threads = pc.threads;
+        p->told = o.chunk_cubes > 0;
+        p->recorded = pc.recorded;
         if (B.cap_blocks >= (1ull << 32) || B.cap_chunks >= (1ull << 32))
             st = fail(MG_ERR_UNSUPPORTED, "plan capacities must be below 2^32");
     }
@@ -3150,7 +3178,9 @@ MG_API mg_status mg_query_plan_run(mg_query_plan* p, const int32_t* boxes, int64
         if (e != cudaSuccess) st = cuda_fail(e, "mg_query_plan_run");
     }
     const BatchRun run{boxes, Q, nullptr, nullptr, out};
-    if (st == MG_OK) st = enqueue_any(p->g, p->bufs, run, p->fp, p->weights, false, p->timed ? p->ev + 1 : nullptr, s);
+    QueryBufs B = p->bufs;
+    B.chunk = run_chunk(p, Q);
+    if (st == MG_OK) st = enqueue_any(p->g, B, run, p->fp, p->weights, false, p->timed ? p->ev + 1 : nullptr, s);
     if (st == MG_OK) p->ran = true;
     if (prev >= 0 && prev != p->g->device) cudaSetDevice(prev);
     return st;

@@ -308,7 +308,7 @@ mg_status launch(mg_server* sv, Slot& sl, std::vector<Req>& w) {
             MG_TRY(cuda_ok(cudaMemcpyAsync(vs.pp.boxes, vs.pin_boxes, (size_t)Q * 24, cudaMemcpyHostToDevice, s),
                            "box upload"));
             MG_TRY(cuda_ok(cudaMemcpyAsync(vs.pp.Qd, vs.pin_q, 8, cudaMemcpyHostToDevice, s), "batch size upload"));
-            MG_TRY(cuda_ok(cudaGraphLaunch(vs.pp.exec, s), "plan launch"));
+            MG_TRY(cuda_ok(cudaGraphLaunch(Q <= kFewBoxes ? vs.pp.exec_few : vs.pp.exec, s), "plan launch"));
             result = vs.pp.result;
         }
         MG_TRY(cuda_ok(cudaMemcpyAsync(vs.pin_out, result, (size_t)Q * S * 4, cudaMemcpyDeviceToHost, s),

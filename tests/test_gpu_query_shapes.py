@@ -281,3 +281,48 @@ def test_a_shape_tuned_for_some_weights(mg):
             assert (np.abs(h - ref).sum(1) <= 1.5 * g.info["depth"] * u * ref.sum(1)).all()
     mg.mg_sync_status(g)
     g.close()
+
+
+@pytest.mark.parametrize("S,hist,alpha", [(64, "u32", "f32"), (64, "f32", "f16"), (2500, "f32", "f32"), (15000, "u32", "f32")])
+@pytest.mark.parametrize("max_chunks", [0, 40000])
+def test_plan_made_for_many_boxes_runs_few(mg, S, hist, alpha, max_chunks):
+    """Runs take chunks by their own size, where the plan's chunk map holds them."""
+    dims = (96, 80, 64)
+    vol = noise(dims, S, 9)
+    g = mg.mg_build(torch.from_numpy(vol).cuda(), S)
+    bx = some_boxes(dims, 5000, 9)
+    t = torch.from_numpy(bx).cuda()
+    plan = mg.QueryPlan(g, max_Q=5000, hist=hist, alpha=alpha, max_blocks=5000 * 2048, max_chunks=max_chunks)
+    for Q in (1, 5000, 7, 64, 65, 900, 5000, 2):
+        b = bx[:Q]
+        h = plan.run(t[:Q].contiguous()).cpu().numpy().astype(np.float64)
+        ref = oracle.box_hist(vol, S, b).astype(np.float64)
+        u = 2.0 ** -11 if alpha == "f16" else 0.0
+        assert (np.abs(h - ref).sum(1) <= 1.5 * g.info["depth"] * u * ref.sum(1)).all(), Q
+        mg.mg_sync_status(g)
+    plan.close()
+    g.close()
+
+
+def test_server_batches_of_few_and_of_many(mg):
+    dims, S = (96, 80, 64), 2500
+    vol = noise(dims, S, 10)
+    g = mg.mg_build(torch.from_numpy(vol).cuda(), S)
+    bx = some_boxes(dims, 1200, 10)
+    ref = oracle.box_hist(vol, S, bx)
+    for hist in ("u32", "f32"):
+        srv = mg.Server(slots=2, max_batch=512, hist=hist)
+        v = srv.add_volume(g, 4)
+        late = [srv.submit_box(v, b) for b in bx[:1100]]   # queued before the start: full batches
+        srv.start()
+        for k, (ticket, out) in enumerate(late):
+            srv.wait(ticket, timeout=60.0)
+            assert np.array_equal(out.astype(np.int64), ref[k].astype(np.int64)), k
+        for k in range(1100, 1200):                        # one by one
+            ticket, out = srv.submit_box(v, bx[k])
+            srv.wait(ticket, timeout=60.0)
+            assert np.array_equal(out.astype(np.int64), ref[k].astype(np.int64)), k
+        st = srv.stats()
+        assert st["max_batch_seen"] > 64 and st["failed"] == 0
+        srv.close()
+    g.close()
