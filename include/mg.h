@@ -286,8 +286,8 @@ MG_API void mg_query_plan_free(mg_query_plan *p);
  * given batch (dense layout; opts->hist_type and alpha_dtype as the caller
  * will use them), writes the fastest into opts->chunk_cubes/block_threads and
  * keeps it in the graph for later calls and plans with these weights that leave
- * them 0.  Batches and plans so small that the default chunk is below 1024 items
- * keep the default.
+ * them 0.  Batches and plans so small that shorter chunks than these suit them
+ * keep the defaults.
  * *best_ms (may be NULL) receives the fastest time of one call.
  * Synchronises `stream`. */
 MG_API mg_status mg_query_autotune(mg_graph *g, const int32_t *boxes, int64_t Q, mg_query_opts *opts,

@@ -2126,11 +2126,14 @@ bool warp_hists(const mg_graph* g, bool FP, int threads) {
 // 85 / 108, 1,000 boxes 337 / 241 / 194 / [186] / 197; 64^3, 10,000 boxes 77 /
 // [77] / 86 / 98 / 134).
 constexpr uint32_t kDefaultChunk = 2048, kMinChunk = 128, kMinSharedChunk = 256;
-uint32_t default_chunk(const mg_graph* g, bool FP, mg_dtype weights, int threads, int64_t Q) {
-    const bool own = warp_hists(g, FP, threads);
+double ideal_chunk(const mg_graph* g, bool FP, mg_dtype weights, bool own, int64_t Q) {
     const double x = g->geom.dims[0][0], y = g->geom.dims[0][1], z = g->geom.dims[0][2];
     const double per = !own ? (FP ? 3.6 : 2.0) : !FP ? 0.33 : weights == MG_F32 ? 0.45 : 0.45 * std::max(1.0, g->S / 750.0);
-    const double best = per * std::sqrt((double)Q * std::sqrt(x * y + y * z + z * x));
+    return per * std::sqrt((double)Q * std::sqrt(x * y + y * z + z * x));
+}
+uint32_t default_chunk(const mg_graph* g, bool FP, mg_dtype weights, int threads, int64_t Q) {
+    const bool own = warp_hists(g, FP, threads);
+    const double best = ideal_chunk(g, FP, weights, own, Q);
     const uint32_t least = !own                ? kMinSharedChunk
                            : weights == MG_F32 ? kMinChunk
                                                : std::max(kMinChunk, g->S / 5);
@@ -2551,18 +2554,22 @@ int default_threads(const mg_graph* g, bool FP, mg_dtype weights) {
 // mg_query_autotune or mg_query_set_tuning recorded, else the defaults.  The
 // tuner's shape holds for the weights it was tuned with (16-bit weights want
 // other CTAs and longer chunks than fp32 ones).  It tries 1,024 items and more:
-// where the default is well below that, a batch has too few such chunks, and
-// CTAs of 512 threads only make up for that, whatever batch they were tuned on
-// (1,000 boxes of 64^3: 25 us a run with 128 items, 41 tuned; of 512x512x384 40
-// and 65; with a histogram per CTA 100 boxes 53 with 512 items, 51 tuned).
+// where the best length is nearer to 512 (or below 512 with a histogram per CTA,
+// whose CTAs of 512 threads gain on long chunks), a batch has too few of those,
+// whatever batch they were tuned on (us a run untuned / tuned: 1,000 boxes of
+// 64^3 25 / 41, of 512x512x384 40 / 65, 3,000 of these 61 / 69, 10,000 beside a
+// frame's propagation 160 / 150; 15,917 segments, 100 boxes 53 / 44).
 struct Shape {
     int threads;
     uint32_t chunk;
     uint32_t longest;   // the chunks that capacities are counted in
     bool recorded;      // the chunk is a recorded one
 };
-// default chunks below this are better than any recorded one
-uint32_t recorded_least(const mg_graph* g, bool FP, int threads) { return warp_hists(g, FP, threads) ? 1024u : 512u; }
+// whether a batch has enough recorded chunks
+bool takes_recorded(const mg_graph* g, bool FP, mg_dtype weights, int threads, int64_t Q) {
+    const bool own = warp_hists(g, FP, threads);
+    return ideal_chunk(g, FP, weights, own, Q) >= (own ? 1024 / std::sqrt(2.0) : 512.0);
+}
 Shape launch_shape_of(const mg_graph* g, bool FP, mg_dtype weights, int chunk_cubes, int block_threads, int64_t Q) {
     if (!FP) weights = MG_F32;
     const bool told = !FP || g->tuned_weights < 0 || g->tuned_weights == (int)weights;
@@ -2572,7 +2579,7 @@ Shape launch_shape_of(const mg_graph* g, bool FP, mg_dtype weights, int chunk_cu
     Shape R;
     R.longest = chunk_cubes > 0 ? (uint32_t)chunk_cubes : tuned ? tuned : kDefaultChunk;
     const uint32_t c = default_chunk(g, FP, weights, block_threads > 0 ? block_threads : usual, Q);
-    if (chunk_cubes <= 0 && tuned > c && c < recorded_least(g, FP, usual)) {
+    if (chunk_cubes <= 0 && tuned > c && !takes_recorded(g, FP, weights, usual, Q)) {
         tuned = 0;
         threads = 0;
     }
@@ -3029,7 +3036,7 @@ static uint32_t run_chunk(const mg_query_plan* p, int64_t Q) {
     if (p->told || Q == p->max_Q) return B.chunk;
     const int threads = B.shape.threads;
     uint32_t c = default_chunk(p->g, p->fp, p->fp ? p->weights : MG_F32, threads, Q);
-    if (p->recorded && c >= recorded_least(p->g, p->fp, threads)) return B.chunk;
+    if (p->recorded && takes_recorded(p->g, p->fp, p->fp ? p->weights : MG_F32, threads, Q)) return B.chunk;
     while (c < B.chunk && chunk_bound(p->g, Q, c) > B.cap_chunks) c *= 2;
     return std::min(c, B.chunk);
 }
