@@ -20,6 +20,11 @@
  *     Errors only the device can see (an ID >= num_segments, a malformed box,
  *     an inexact integer push) set the graph's device status word, which
  *     mg_sync_status() reads and clears.
+ *   - Calls that neither synchronise nor say otherwise can be captured into CUDA
+ *     graphs.  Replays use the scratch of the stream they were captured on: they
+ *     run in order with each other and with that graph handle's later calls on
+ *     that stream (mg_propagate_tf's counters are apart, so its replays may
+ *     overlap eager calls, but not each other).
  *   - Volumes are x-fastest: voxel (x, y, z) is element (z*ny + y)*nx + x.
  *     Each axis is at most 65535 voxels and nx*ny*nz < 2^32.
  *   - Node IDs: sources 0..S-1 are the segment IDs; internal nodes S..N-1 are
